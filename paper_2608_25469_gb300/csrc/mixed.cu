@@ -380,9 +380,7 @@ hsma_status_t r32_apply(const R32Plan &P, float *B, int64_t ldb, int64_t n, floa
   TcArgs sa{};
   {
     const uint8_t ps[6][2] = {{0, 0}, {0, 1}, {1, 0}, {0, 2}, {1, 1}, {2, 0}};
-    sa.nunits = 1;
-    sa.ubeg[0] = 0;
-    sa.ubeg[1] = 6;
+    sa.npairs = 6;
     for (int q = 0; q < 6; ++q) {
       sa.pa[q] = ps[q][0];
       sa.pb[q] = ps[q][1];
@@ -479,9 +477,7 @@ hsma_status_t r32_apply(const R32Plan &P, float *B, int64_t ldb, int64_t n, floa
     if (pair && (r & 1) == 1) {
       // panel r-1 from its row nb on and panel r cover the same rows, one
       // uniform stride apart; X_{r-1} and X_r sit in the two split buffers
-      a.nunits = 1;
-      a.ubeg[0] = 0;
-      a.ubeg[1] = 2;
+      a.npairs = 2;
       a.pa[0] = 0;
       a.pb[0] = 0;
       a.pa[1] = 1;
@@ -599,29 +595,19 @@ __global__ void check_kernel(double *sums, int *state, double alpha_abs, double 
 }
 
 // ---------------------------------------------------------------------------
-// FP64 products emulated on the BF16 tensor cores (Ozaki-style exact slices).
+// FP64 products emulated on the BF16 tensor cores (residue arithmetic in
+// oz_tables.cuh).
 //
 // Row i of the left operand is scaled by 2^-e_i and column j of the right
 // operand by 2^-f_j (powers of two with |entry| < 2^e), so every scaled entry
 // lies in (-1, 1).  It is rounded to the fixed-point integer I = a 2^(59 - e)
-// (bits below 2^-59 of the row or column scale are dropped) and cut from the
-// top into kOzS signed base-64 digits, I = sum_p d_p 2^(59 - b_p) with
-// b_p = 5 + 6(p-1) and d_p in [-32, 32], using integer operations only.  A
-// digit is exact in BF16 and a product of two digits is at most 2^10, so a sum
-// of g slice-pair products over K terms is an integer below 2^24 whenever
-// g K <= 2^14: the FP32 tensor-memory accumulation is exact.  Pairs with the
-// same p + q share the weight 2^-(b_p + b_q); they are grouped into
-// accumulation units of at most 2^14 / K pairs, and each unit is folded into
-// the FP64 result once, with weight 2^(e_i + f_j - b_p - b_q).  Pairs with
-// p + q > kOzS + 1 are dropped; they and the fixed-point rounding contribute
-// below 2^-59 of |row scale| |column scale| per product term.
+// (bits below 2^-59 of the row or column scale are dropped) and stored as its
+// residues modulo kOzP moduli, exact in BF16.  One tensor-core product per
+// modulus gives the residues of the exact integer product, which is converted
+// to FP64 with one rounding and added to the result.  The fixed-point rounding
+// contributes at most 2^-59 of |row scale| |column scale| per product term.
 // ---------------------------------------------------------------------------
-constexpr int kOzFrac = 59;
-constexpr int kOzMaxK = 1 << 14;
 constexpr int kOzExpEmpty = -1100;  // exponent of an all-zero row
-
-__host__ __device__ constexpr int oz_bits(int p) { return 5 + 6 * (p - 1); }
-static_assert(oz_bits(kOzS) == kOzFrac, "the last digit has weight 2^-kOzFrac");
 
 // e with |x| < 2^e, from the bits of |x| (x != 0)
 __device__ __forceinline__ int oz_exponent(uint64_t absbits) {
@@ -649,18 +635,23 @@ __device__ __forceinline__ int64_t oz_fixed(double a, int e) {
   return (bits >> 63) ? -I : I;
 }
 
-// the kOzS digits of I, slice p at out[(p-1) stride]
-__device__ __forceinline__ void oz_put_digits(int64_t I, __nv_bfloat16 *out, size_t stride) {
-#pragma unroll
-  for (int p = 1; p <= kOzS; ++p) {
-    const int sh = kOzFrac - oz_bits(p);
-    int64_t d = I;
-    if (sh > 0) {
-      d = (I + (1ll << (sh - 1))) >> sh;
-      I -= d << sh;
-    }
-    out[(size_t)(p - 1) * stride] = __float2bfloat16_rn((float)(int)d);
-  }
+// I (|I| <= 2^59) as four limbs, I = sum_j a[j] 2^(15 j): 15 bits each, the top one signed
+__device__ __forceinline__ void oz_limbs(int64_t I, float (&a)[4]) {
+  const uint32_t lo = (uint32_t)I, hi = (uint32_t)((uint64_t)I >> 30);
+  a[0] = __fadd_rn(__uint_as_float(0x4B000000u | (lo & 0x7fffu)), -8388608.0f);
+  a[1] = __fadd_rn(__uint_as_float(0x4B000000u | ((lo >> 15) & 0x7fffu)), -8388608.0f);
+  a[2] = __fadd_rn(__uint_as_float(0x4B000000u | (hi & 0x7fffu)), -8388608.0f);
+  a[3] = __fadd_rn(__uint_as_float(0x4B400000u + (uint32_t)(int32_t)(I >> 45)), -12582912.0f);
+}
+
+// balanced residue of sum_j a[j] w[j]: at most 3.5 2^15 2^7 < 2^24, exact in FP32
+__device__ __forceinline__ float oz_limb_residue(const float (&a)[4], const float (&w)[4], float mod, float inv) {
+  return oz_residue(fmaf(a[3], w[3], fmaf(a[2], w[2], fmaf(a[1], w[1], a[0] * w[0]))), mod, inv);
+}
+
+// two residues as a pair of BF16 (they have at most eight significant bits)
+__device__ __forceinline__ uint32_t oz_pair(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
 __device__ __forceinline__ uint64_t oz_absbits(double x) {
@@ -719,27 +710,22 @@ __global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__
   }
 }
 
-// Slices of a left operand: the rows x K block (mode as in oz_entry; complex
-// expanded to the real 2 rows x 2 K form with [re -im; im re] per entry),
-// balanced by 2^-g_k, as out[p][row][k], rows' x Kp row-major per slice (zero
-// beyond K'), plus the row exponents.  One CTA per 32 rows: a pass for the
-// exponents, a pass for the digits.
+// Row exponents of a left operand balanced by 2^-g_k (atomicMax over the
+// kOzExpEmpty fill): a CTA covers 32 rows x kOzRexpCols columns, lanes across
+// the rows.
+constexpr int kOzRexpCols = 128;
+
 template <bool CPLX>
-__global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
-                                                         int Kp, int mode, const int *__restrict__ kexp, int *rexp,
-                                                         __nv_bfloat16 *out, size_t sstride) {
+__global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
+                                                      int mode, const int *__restrict__ kexp, int *rexp) {
   constexpr int W = CPLX ? 2 : 1;
-  constexpr int KT = 32 / W;  // source columns per tile
-  __shared__ double sre[KT][33], sim[CPLX ? KT : 1][33];
-  __shared__ int sg[KT];
   __shared__ int red[8][32];
-  __shared__ int se[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int i0 = blockIdx.x * 32;
-  const int i = i0 + tx;
-  int ex = INT_MIN;
-  const int kend = mode != 0 ? min(K, i + 1) : K;
-  for (int k = ty; k < kend && i < rows; k += 8) {
+  const int i = blockIdx.x * 32 + tx, kb = blockIdx.y * kOzRexpCols;
+  if (mode != 0 && kb > blockIdx.x * 32 + 31) return;  // above the diagonal
+  int ex = kOzExpEmpty;
+#pragma unroll 4
+  for (int k = kb + ty; k < min(K, kb + kOzRexpCols); k += 8) {
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, i, k, re, im);
     const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
@@ -749,95 +735,110 @@ __global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restric
   __syncthreads();
   if (ty == 0) {
     for (int w = 1; w < 8; ++w) ex = max(ex, red[w][tx]);
-    const int e = ex == INT_MIN ? kOzExpEmpty : ex;
-    se[tx] = e;
-    if (i < rows) {
-      rexp[W * i] = e;
-      if (CPLX) rexp[W * i + 1] = e;
+    if (i < rows && ex != kOzExpEmpty) {
+      atomicMax(&rexp[W * i], ex);
+      if (CPLX) atomicMax(&rexp[W * i + 1], ex);
     }
-  }
-  __syncthreads();
-  for (int k0 = 0; k0 < Kp; k0 += 32) {
-    const int kc0 = k0 / W;
-    for (int kk = ty; kk < KT; kk += 8) {
-      double re, im;
-      oz_entry<CPLX>(A, lda, rows, K, mode, i, kc0 + kk, re, im);
-      sre[kk][tx] = re;
-      if (CPLX) sim[kk][tx] = im;
-    }
-    if (threadIdx.x < KT) sg[threadIdx.x] = kc0 + (int)threadIdx.x < K ? kexp[W * (kc0 + threadIdx.x)] : 0;
-    __syncthreads();
-    const int g = sg[tx / W];
-    for (int ii = ty; ii < 32; ii += 8) {
-      const int r = i0 + ii;
-      if (r >= rows) break;
-      const int e = se[ii];
-      const bool zero = e == kOzExpEmpty;
-      if (CPLX) {
-        const double re = sre[tx >> 1][ii], im = sim[tx >> 1][ii];
-        const bool first = (tx & 1) == 0;
-        oz_put_digits(zero ? 0 : oz_fixed(first ? re : -im, e + g), out + (size_t)(2 * r) * Kp + k0 + tx, sstride);
-        oz_put_digits(zero ? 0 : oz_fixed(first ? im : re, e + g), out + (size_t)(2 * r + 1) * Kp + k0 + tx,
-                      sstride);
-      } else {
-        oz_put_digits(zero ? 0 : oz_fixed(sre[tx][ii], e + g), out + (size_t)r * Kp + k0 + tx, sstride);
-      }
-    }
-    __syncthreads();
   }
 }
 
-// Slices of a right operand: K x N column-major (complex: its real view with
+// Residues of a left operand: the rows x K block (mode as in oz_entry; complex
+// expanded to the real 2 rows x 2 K form with [re -im; im re] per entry),
+// balanced by 2^-g_k, as out[l][row][k], rows' x Kp row-major per modulus (zero
+// beyond K').  One CTA per 32 source rows x 64 real columns: read as columns of
+// 32 rows, transposed through shared memory, written as pairs of consecutive k
+// (128 bytes per warp and modulus).  Tiles past the diagonal's 128-row tile,
+// which a triangular product does not read, are not written.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
+                                                         int Kp, int mode, const int *__restrict__ kexp,
+                                                         const int *__restrict__ rexp, uint32_t *out,
+                                                         size_t pstride) {
+  constexpr int W = CPLX ? 2 : 1;
+  constexpr int KT = 64 / W;  // source columns per tile
+  __shared__ double sre[KT][33], sim[CPLX ? KT : 1][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 64, kc0 = k0 / W;
+  if (mode != 0 && k0 >= (W * i0 / TC_BM + 1) * TC_BM) return;
+#pragma unroll
+  for (int q = 0; q < KT / 8; ++q) {
+    double re, im;
+    oz_entry<CPLX>(A, lda, rows, K, mode, i0 + tx, kc0 + ty + 8 * q, re, im);
+    sre[ty + 8 * q][tx] = re;
+    if (CPLX) sim[ty + 8 * q][tx] = im;
+  }
+  const int s0 = CPLX ? kc0 + tx : kc0 + 2 * tx, s1 = CPLX ? s0 : s0 + 1;  // source columns of this lane's pair
+  const int g0 = s0 < K ? kexp[W * s0] : 0, g1 = s1 < K ? kexp[W * s1] : 0;
+  __syncthreads();
+#pragma unroll 1
+  for (int ii = ty; ii < 32; ii += 8) {
+    const int r = i0 + ii;
+    if (r >= rows) break;
+    const int e = rexp[W * r];
+    const bool zero = e == kOzExpEmpty;
+    float a0[4], a1[4];
+    oz_limbs(zero ? 0 : oz_fixed(sre[CPLX ? tx : 2 * tx][ii], e + g0), a0);
+    oz_limbs(zero ? 0 : oz_fixed(CPLX ? sim[tx][ii] : sre[2 * tx + 1][ii], e + g1), a1);
+    uint32_t *o = out + (size_t)(W * r) * (Kp / 2) + k0 / 2 + tx;
+#pragma unroll
+    for (int l = 0; l < kOzP; ++l) {
+      const float r0 = oz_limb_residue(a0, c_oz.wa[l], c_oz.modf[l], c_oz.inv[l]);
+      const float r1 = oz_limb_residue(a1, c_oz.wa[l], c_oz.modf[l], c_oz.inv[l]);
+      if (CPLX) {
+        o[l * pstride] = oz_pair(r0, -r1);
+        o[l * pstride + Kp / 2] = oz_pair(r1, r0);
+      } else {
+        o[l * pstride] = oz_pair(r0, r1);
+      }
+    }
+  }
+}
+
+// Residues of a right operand: K x N column-major (complex: its real view with
 // 2K rows), balanced by 2^g_k (rows with g_k = kOzExpEmpty are ignored), as
-// out[q][j][k], N x Kp row-major per slice (zero beyond K), plus the column
-// exponents.  One warp per column; a lane handles two consecutive k, so each
-// slice is written 128 bytes per warp step.
+// out[l][j][k], N x Kp row-major per modulus (zero beyond K), plus the column
+// exponents.  One CTA per column: its largest exponent, then the residues, a
+// thread two consecutive k (128 bytes per warp and modulus).
 __global__ void __launch_bounds__(256) oz_slice_x_kernel(const double *__restrict__ X, int64_t ldx, int K, int N,
                                                          int Kp, const int *__restrict__ kexp, int *cexp,
-                                                         __nv_bfloat16 *out, size_t sstride, const int *skip) {
+                                                         uint32_t *out, size_t pstride, const int *skip) {
   if (skip != nullptr && *(volatile const int *)skip) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < N; j += nwarps) {
+  __shared__ int red[8];
+  const int tid = threadIdx.x;
+  for (int64_t j = blockIdx.x; j < N; j += gridDim.x) {
     const double *x = X + j * ldx;
     int ex = INT_MIN;
-    for (int k = lane; k < K; k += 32) {
+#pragma unroll 4
+    for (int k = tid; k < K; k += 256) {
       const uint64_t ab = oz_absbits(x[k]);
       const int g = kexp[k];
       if (ab != 0 && g != kOzExpEmpty) ex = max(ex, oz_exponent(ab) + g);
     }
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    if ((tid & 31) == 0) red[tid >> 5] = ex;
+    __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
+    for (int w = 0; w < 8; ++w) ex = max(ex, red[w]);
+    __syncthreads();  // red is rewritten by the next column
     const int e = ex == INT_MIN ? 0 : ex;
-    if (lane == 0) cexp[j] = e;
-    __nv_bfloat162 *o2 = reinterpret_cast<__nv_bfloat162 *>(out + (size_t)j * Kp);
-    for (int k = 2 * lane; k < Kp; k += 64) {
-      int64_t I[2];
+    if (tid == 0) cexp[j] = e;
+    uint32_t *o = out + (size_t)j * (Kp / 2);
+    for (int k = 2 * tid; k < Kp; k += 512) {
+      float a[2][4];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int g = k + h < K ? kexp[k + h] : kOzExpEmpty;
-        I[h] = g != kOzExpEmpty ? oz_fixed(x[k + h], e - g) : 0;
+        oz_limbs(g != kOzExpEmpty ? oz_fixed(x[k + h], e - g) : 0, a[h]);
       }
 #pragma unroll
-      for (int p = 1; p <= kOzS; ++p) {
-        const int sh = kOzFrac - oz_bits(p);
-        float d[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          int64_t v = I[h];
-          if (sh > 0) {
-            v = (I[h] + (1ll << (sh - 1))) >> sh;
-            I[h] -= v << sh;
-          }
-          d[h] = (float)(int)v;
-        }
-        o2[(size_t)(p - 1) * (sstride / 2) + k / 2] = __floats2bfloat162_rn(d[0], d[1]);
-      }
+      for (int l = 0; l < kOzP; ++l)
+        o[l * pstride + k / 2] = oz_pair(oz_limb_residue(a[0], c_oz.wx[l], c_oz.modf[l], c_oz.inv[l]),
+                                         oz_limb_residue(a[1], c_oz.wx[l], c_oz.modf[l], c_oz.inv[l]));
     }
   }
 }
 
-// One sliced operand: kOzS slices of rows x Kp BF16 digits, an exponent per
+// One sliced operand: kOzP planes of rows x Kp BF16 residues, an exponent per
 // row, and (left operands) the K-balancing exponents.
 struct OzOperand {
   __nv_bfloat16 *slices = nullptr;
@@ -849,7 +850,7 @@ struct OzOperand {
 int oz_kp(int64_t K) { return (int)((K + TC_BK - 1) / TC_BK) * TC_BK; }
 
 size_t oz_slices_bytes(int64_t rows, int Kp) {
-  return (kOzS * (size_t)rows * Kp * sizeof(__nv_bfloat16) + 1023) & ~(size_t)1023;
+  return (kOzP * (size_t)rows * Kp * sizeof(__nv_bfloat16) + 1023) & ~(size_t)1023;
 }
 
 size_t oz_operand_bytes(int64_t rows, int Kp) {
@@ -873,19 +874,24 @@ OzOperand oz_operand(void *ws, int64_t rows, int Kp) {
 hsma_status_t oz_slice_a(bool cplx, const double *A, int64_t lda, int rows, int K, int mode, OzOperand &o,
                          cudaStream_t st) {
   if (rows <= 0 || K <= 0) return HSMA_OK;
-  const size_t ss = (size_t)o.rows * o.Kp;
+  const int W = cplx ? 2 : 1;
   const dim3 kg((unsigned)((K + 31) / 32), (unsigned)((rows + 255) / 256));
-  if (kg.y > 65535) return HSMA_ERR_UNSUPPORTED;
-  const int kw = (cplx ? 2 : 1) * K;
-  oz_fill_kernel<<<(kw + 255) / 256, 256, 0, st>>>(o.kexp, kw, kOzExpEmpty);
+  const dim3 rg((unsigned)((rows + 31) / 32), (unsigned)((K + kOzRexpCols - 1) / kOzRexpCols));
+  const dim3 sg((unsigned)((rows + 31) / 32), (unsigned)(o.Kp / 64));
+  if (kg.y > 65535 || rg.y > 65535) return HSMA_ERR_UNSUPPORTED;
+  // row and K-balancing exponents lie one after the other
+  const int nfill = (int)(o.kexp + W * K - o.exps);
+  oz_fill_kernel<<<(nfill + 255) / 256, 256, 0, st>>>(o.exps, nfill, kOzExpEmpty);
+  uint32_t *out = reinterpret_cast<uint32_t *>(o.slices);
+  const size_t ps = (size_t)o.rows * o.Kp / 2;
   if (cplx) {
     oz_kexp_kernel<true><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp);
-    oz_slice_a_kernel<true><<<(rows + 31) / 32, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, o.slices,
-                                                               ss);
+    oz_rexp_kernel<true><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp, o.exps);
+    oz_slice_a_kernel<true><<<sg, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, out, ps);
   } else {
     oz_kexp_kernel<false><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp);
-    oz_slice_a_kernel<false><<<(rows + 31) / 32, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps,
-                                                                o.slices, ss);
+    oz_rexp_kernel<false><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp, o.exps);
+    oz_slice_a_kernel<false><<<sg, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, out, ps);
   }
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
@@ -896,100 +902,69 @@ hsma_status_t oz_slice_a(bool cplx, const double *A, int64_t lda, int rows, int 
 hsma_status_t oz_slice_x(const double *X, int64_t ldx, int K, const int *kexp, OzOperand &o, const int *skip,
                          cudaStream_t st) {
   if (o.rows <= 0) return HSMA_OK;
-  const int grid = std::min((o.rows + 7) / 8, hsma_sm_count() * 16);
-  oz_slice_x_kernel<<<grid, 256, 0, st>>>(X, ldx, K, o.rows, o.Kp, kexp, o.exps, o.slices, (size_t)o.rows * o.Kp,
-                                          skip);
+  const int grid = std::min(o.rows, hsma_sm_count() * 16);
+  oz_slice_x_kernel<<<grid, 256, 0, st>>>(X, ldx, K, o.rows, o.Kp, kexp, o.exps,
+                                          reinterpret_cast<uint32_t *>(o.slices), (size_t)o.rows * o.Kp / 2, skip);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
 }
 
-// Unit table: pairs of equal p + q, smallest weights first, at most
-// 2^14 / Kp pairs per unit (exact FP32 sums).
-void oz_units(int Kp, TcArgs &a) {
-  const int gmax = std::max(1, kOzMaxK / Kp);
-  int np = 0, nu = 0;
-  for (int s = kOzS + 1; s >= 2; --s) {
-    int in_unit = 0;
-    for (int p = std::max(1, s - kOzS); p <= std::min(kOzS, s - 1); ++p) {
-      if (in_unit == 0) {
-        a.ubeg[nu] = (uint8_t)np;
-        a.uexp[nu] = (int8_t)(-(oz_bits(p) + oz_bits(s - p)));
-        ++nu;
-      }
-      a.pa[np] = (uint8_t)(p - 1);
-      a.pb[np] = (uint8_t)(s - p - 1);
-      ++np;
-      if (++in_unit == gmax) in_unit = 0;
-    }
-  }
-  a.ubeg[nu] = (uint8_t)np;
-  a.nunits = nu;
+// Scratch of the emulated products of up to rows x cols results: the residue
+// bytes of one tile per CTA.
+constexpr int kEmuGemmMaxK = 1 << 14;      // hsma_gemm_f64_emulated
+constexpr int kOzResidualMaxM = 1 << 14;   // refinement residuals
+
+size_t oz_scratch_bytes(int64_t rows, int64_t cols) {
+  const int64_t tiles = ((rows + TC_BM - 1) / TC_BM) * ((cols + TC_BN - 1) / TC_BN);
+  return (size_t)std::min<int64_t>(tiles, hsma_sm_count()) * kOzTileWords * sizeof(uint32_t);
 }
 
 // C (M x N, column-major FP64) = (beta0 ? C : 0) -/+ L X in emulated FP64,
-// L and X given by their slices; tri: L is lower triangular.
+// L and X given by their residues; tri: L is lower triangular.  At most kOzMaxK
+// columns of L per launch, each launch one rounding and one addition to C.
 hsma_status_t oz_product(const OzOperand &L, const OzOperand &X, double *C, int64_t ldc, int beta0, int negate,
-                         int tri, const int *skip, const char *phase, cudaStream_t st) {
-  if (L.Kp != X.Kp || L.Kp > kOzMaxK) return HSMA_ERR_INVALID_ARG;
-  TcArgs a{};
-  a.C64 = C;
-  a.ldc = ldc;
-  a.beta0 = beta0;
-  a.negate = negate;
-  a.rexp = L.exps;
-  a.cexp = X.exps;
-  a.M = L.rows;
-  a.N = X.rows;
-  a.K = L.Kp;
-  a.tri = tri;
-  a.skip = skip;
-  oz_units(L.Kp, a);
-  return tc_gemm<TC_OZ>(L.slices, kOzS, X.slices, kOzS, a, phase, st);
+                         int tri, uint32_t *scratch, const int *skip, const char *phase, cudaStream_t st) {
+  if (L.Kp != X.Kp) return HSMA_ERR_INVALID_ARG;
+  for (int64_t c0 = 0; c0 < L.Kp; c0 += kOzMaxK) {
+    const int64_t i0 = tri ? c0 : 0;  // a triangular L has no entries above row c0 in these columns
+    if (i0 >= L.rows) break;
+    TcArgs a{};
+    a.C64 = C + i0;
+    a.ldc = ldc;
+    a.beta0 = beta0 != 0 || c0 > 0;
+    a.negate = negate;
+    a.rexp = L.exps + i0;
+    a.cexp = X.exps;
+    a.scratch = scratch;
+    a.M = (int)(L.rows - i0);
+    a.N = X.rows;
+    a.K = (int)std::min<int64_t>(kOzMaxK, L.Kp - c0);
+    a.tri = tri;
+    a.skip = skip;
+    SliceLayout la, lb;  // views into the full planes at row i0 and column c0
+    la.rows = L.rows - i0;
+    la.kext = L.Kp - c0;
+    la.ld = L.Kp;
+    la.sst = (int64_t)L.rows * L.Kp;
+    lb.rows = X.rows;
+    lb.kext = X.Kp - c0;
+    lb.ld = X.Kp;
+    lb.sst = (int64_t)X.rows * X.Kp;
+    hsma_status_t s = tc_gemm<TC_OZ>(L.slices + i0 * L.Kp + c0, kOzP, X.slices + c0, kOzP, a, phase, st, la, lb);
+    if (s != HSMA_OK) return s;
+  }
+  return HSMA_OK;
 }
 
 // R -= L X in emulated FP64 (R holds alpha B on entry); skip: device flag.
-// K runs in chunks of kOzResidualChunk columns of L: chunk c touches only rows
-// below its start (L is lower triangular) and each launch re-reads a chunk's
-// slices, which stay in L2, for all its slice pairs; one launch over the whole
-// K would stream every row tile's full slices from memory once per pair.
-constexpr int kOzResidualChunk = 1024;
-
 hsma_status_t oz_residual(const OzOperand &L, const double *X, int64_t ldx, double *R, int64_t ldr, OzOperand &Xo,
-                          const int *skip, cudaStream_t st) {
+                          uint32_t *scratch, const int *skip, cudaStream_t st) {
   {
     HsmaTraceScope ts("residual_slices", st);
     hsma_status_t s = oz_slice_x(X, ldx, L.rows, L.kexp, Xo, skip, st);
     if (s != HSMA_OK) return s;
   }
-  const int64_t m = L.rows, Kp = L.Kp;
-  for (int64_t c0 = 0; c0 < m; c0 += kOzResidualChunk) {
-    const int kc = (int)std::min<int64_t>(kOzResidualChunk, m - c0);
-    TcArgs a{};
-    a.C64 = R + c0;
-    a.ldc = ldr;
-    a.beta0 = 1;
-    a.negate = 0;
-    a.rexp = L.exps + c0;
-    a.cexp = Xo.exps;
-    a.M = (int)(m - c0);
-    a.N = Xo.rows;
-    a.K = oz_kp(kc);
-    a.tri = 1;  // rows c0 + i need chunk columns <= i only
-    a.skip = skip;
-    oz_units(a.K, a);
-    SliceLayout la, lb;  // views into the full slice stacks at row / K offset c0
-    la.rows = m - c0;
-    la.kext = Kp - c0;
-    la.ld = Kp;
-    la.sst = m * Kp;
-    lb.rows = Xo.rows;
-    lb.kext = Kp - c0;
-    lb.ld = Kp;
-    lb.sst = (int64_t)Xo.rows * Kp;
-    hsma_status_t s = tc_gemm<TC_OZ>(L.slices + c0 * Kp + c0, kOzS, Xo.slices + c0, kOzS, a, "residual", st, la, lb);
-    if (s != HSMA_OK) return s;
-  }
-  return HSMA_OK;
+  return oz_product(L, Xo, R, ldr, 1, 0, 1, scratch, skip, "residual", st);
 }
 
 __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, double ar, double ai, int cplx) {
@@ -1030,8 +1005,8 @@ __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, do
 struct EmuLayout {
   int W = 1, h = 1, Kpb = 0, Kpp = 0;
   int64_t P = 0;
-  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0;
-  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b; }
+  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0, sc_b = 0;
+  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b + sc_b; }
 };
 
 EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
@@ -1049,6 +1024,7 @@ EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
   L.pa_b = al(oz_operand_bytes((int64_t)L.W * m, L.Kpp));
   L.pd_b = al(oz_operand_bytes((int64_t)L.W * nb, L.Kpb));
   L.px_b = al(oz_operand_bytes(n, L.Kpp));
+  L.sc_b = al(oz_scratch_bytes(L.W * m, n));
   return L;
 }
 
@@ -1058,8 +1034,8 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
   const EmuLayout E = emu_layout(cplx, nb, panel_cols, m, n);
   const int W = E.W;
   const int64_t P = E.P;
-  const int Kpb = E.Kpb, Kpp = E.Kpp;
-  if (Kpp > kOzMaxK || (int64_t)W * m > INT32_MAX || n > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
+  const int Kpb = E.Kpb;
+  if ((int64_t)W * m > INT32_MAX || n > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
   const size_t eb = sizeof(double) * W;
   const size_t dinv_b = E.dinv_b, w_b = E.w_b, pa_b = E.pa_b;
   void *ws = nullptr;
@@ -1069,6 +1045,7 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
   double *Dinv = reinterpret_cast<double *>(base);
   double *Wb = reinterpret_cast<double *>(base + dinv_b);
   unsigned char *pa_mem = base + dinv_b + w_b, *px_mem = base + dinv_b + w_b + pa_b + E.pd_b;
+  uint32_t *scratch = reinterpret_cast<uint32_t *>(px_mem + E.px_b);
   // views of the operand buffers for a given K (the buffers hold the widest)
   auto view = [](unsigned char *mem, int64_t rows_cap, int Kp, int64_t rows) {
     OzOperand o = oz_operand(mem, rows_cap, Kp);
@@ -1082,12 +1059,12 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
     OzOperand Pa = view(pa_mem, (int64_t)W * m, Kp, (int64_t)W * rows);
     OzOperand Px = view(px_mem, n, Kp, n);
     {
-      HsmaTraceScope ts("slices", st, 4);  // oz_slice_a: 3 kernels, oz_slice_x: 1
+      HsmaTraceScope ts("slices", st, 5);  // oz_slice_a: 4 kernels, oz_slice_x: 1
       hsma_status_t e = oz_slice_a(cplx, A + W * (rb + c0 * lda), lda, (int)rows, k, 0, Pa, st);
       if (e == HSMA_OK) e = oz_slice_x(B + W * c0, (int64_t)W * ldb, W * k, Pa.kexp, Px, nullptr, st);
       if (e != HSMA_OK) return e;
     }
-    return oz_product(Pa, Px, B + W * rb, (int64_t)W * ldb, 1, 0, 0, nullptr, phase, st);
+    return oz_product(Pa, Px, B + W * rb, (int64_t)W * ldb, 1, 0, 0, scratch, nullptr, phase, st);
   };
   do {
     if ((s = hsma_diag_inverse(cplx ? HSMA_C128 : HSMA_R64, nb, A, lda, m, unit, Dinv, st)) != HSMA_OK) break;
@@ -1111,11 +1088,12 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
         Pd.rows = W * sr;
         OzOperand Px = view(px_mem, n, Kpb, n);
         {
-          HsmaTraceScope ts("slices", st, 4);
+          HsmaTraceScope ts("slices", st, 5);
           if ((s = oz_slice_a(cplx, Dinv + (size_t)W * r * nb * nb, nb, sr, sr, 1, Pd, st)) != HSMA_OK) break;
           if ((s = oz_slice_x(Wb, (int64_t)W * nb, W * sr, Pd.kexp, Px, nullptr, st)) != HSMA_OK) break;
         }
-        if ((s = oz_product(Pd, Px, B + W * r0, (int64_t)W * ldb, 0, 1, 1, nullptr, "solve_gemm", st)) != HSMA_OK)
+        if ((s = oz_product(Pd, Px, B + W * r0, (int64_t)W * ldb, 0, 1, 1, scratch, nullptr, "solve_gemm",
+                            st)) != HSMA_OK)
           break;
         // the panel's remaining rows
         const int64_t rin = R0 + PR - (r0 + sr);
@@ -1150,8 +1128,8 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   if (res_mode != 0 && res_mode != 1) return HSMA_ERR_INVALID_ARG;
   if (m > INT32_MAX || n > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
   // residual products: emulated FP64 on the BF16 tensor cores unless asked
-  // otherwise or K is beyond the exactness bound of the slice sums
-  const bool emulated = res_mode == 0 && m <= kOzMaxK;
+  // otherwise or m is beyond what the residues of L are kept for
+  const bool emulated = res_mode == 0 && m <= kOzResidualMaxM;
   auto al = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
   const size_t a32_b = sizeof(float) * (size_t)m * m;
   const size_t r32_b = sizeof(float) * (size_t)m * n;
@@ -1161,6 +1139,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   const int ozkp = oz_kp(m);
   const size_t ozl_b = emulated ? al(oz_operand_bytes(m, ozkp)) : 0;
   const size_t ozx_b = emulated ? al(oz_operand_bytes(n, ozkp)) : 0;
+  const size_t ozs_b = emulated ? al(oz_scratch_bytes(m, n)) : 0;
   // the FP32 inverses and BF16 panels of L, shared by the first solve and every correction
   R32Plan P;
   P.nb = nb < 32 ? 32 : nb;
@@ -1173,7 +1152,8 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   const size_t pan_b = al(sizeof(__nv_bfloat16) * r32_panels_elems(P.nb, terms, m));
   void *ws = nullptr;
   hsma_status_t s = hsma_ws_alloc(
-      &ws, al(a32_b) + al(r32_b) + al(b0_b) + al(r64_b) + st_b + ozl_b + ozx_b + dinv_b + pan_b, st);
+      &ws, al(a32_b) + al(r32_b) + al(b0_b) + al(r64_b) + st_b + ozl_b + ozx_b + ozs_b + dinv_b + pan_b,
+      st);
   if (s != HSMA_OK) return s;
   unsigned char *base = static_cast<unsigned char *>(ws);
   float *A32 = reinterpret_cast<float *>(base);
@@ -1186,7 +1166,8 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   void *ozx_ws = static_cast<unsigned char *>(ozl_ws) + ozl_b;
   OzOperand Lsl = oz_operand(ozl_ws, m, ozkp), Xsl = oz_operand(ozx_ws, n, ozkp);
   P.A = A32;
-  P.Dinv = reinterpret_cast<float *>(static_cast<unsigned char *>(ozx_ws) + ozx_b);
+  uint32_t *ozs = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(ozx_ws) + ozx_b);
+  P.Dinv = reinterpret_cast<float *>(static_cast<unsigned char *>(ozx_ws) + ozx_b + ozs_b);
   P.panels = reinterpret_cast<__nv_bfloat16 *>(reinterpret_cast<unsigned char *>(P.Dinv) + dinv_b);
   const dim3 grid = hsma_grid_rc(m, n);
   auto fail = [&](cudaError_t e) { return e == cudaSuccess ? HSMA_OK : hsma_from_cuda(e); };
@@ -1204,7 +1185,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
       if ((s = fail(cudaGetLastError())) != HSMA_OK) break;
     }
     if (emulated) {
-      HsmaTraceScope ts("residual_slices", st, 3);
+      HsmaTraceScope ts("residual_slices", st, 4);
       if ((s = oz_slice_a(false, A, lda, (int)m, (int)m, unit ? 2 : 1, Lsl, st)) != HSMA_OK) break;
     }
     // X_0 from the FP32-result solve of the rounded data
@@ -1227,7 +1208,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
           HsmaTraceScope ts("refine", st);
           scale_copy_kernel<<<g_launch_grid(m * n), 256, 0, st>>>(B0, R64, m * n, alpha, state);
         }
-        if ((s = oz_residual(Lsl, B, ldb, R64, m, Xsl, state, st)) != HSMA_OK) break;
+        if ((s = oz_residual(Lsl, B, ldb, R64, m, Xsl, ozs, state, st)) != HSMA_OK) break;
       } else {
         if ((s = fail(cudaMemcpy2DAsync(R64, sizeof(double) * m, B0, sizeof(double) * m, sizeof(double) * m, n,
                                         cudaMemcpyDeviceToDevice, st))) != HSMA_OK)
@@ -1304,17 +1285,18 @@ extern "C" HSMA_API hsma_status_t hsma_gemm_f64_emulated(int64_t M, int64_t N, i
     return HSMA_ERR_INVALID_ARG;
   if (M == 0 || N == 0 || K == 0) return HSMA_OK;
   if (A == nullptr || X == nullptr || C == nullptr) return HSMA_ERR_INVALID_ARG;
-  if (K > kOzMaxK || M > INT32_MAX || N > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
+  if (K > kEmuGemmMaxK || M > INT32_MAX || N > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Kp = oz_kp(K);
   const size_t a_b = oz_operand_bytes(M, Kp), x_b = oz_operand_bytes(N, Kp);
   void *ws = nullptr;
-  hsma_status_t s = hsma_ws_alloc(&ws, a_b + x_b, st);
+  hsma_status_t s = hsma_ws_alloc(&ws, a_b + x_b + oz_scratch_bytes(M, N), st);
   if (s != HSMA_OK) return s;
+  uint32_t *scratch = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(ws) + a_b + x_b);
   OzOperand Ao = oz_operand(ws, M, Kp), Xo = oz_operand(static_cast<unsigned char *>(ws) + a_b, N, Kp);
   s = oz_slice_a(false, A, lda, (int)M, (int)K, 0, Ao, st);
   if (s == HSMA_OK) s = oz_slice_x(X, ldx, (int)K, Ao.kexp, Xo, nullptr, st);
-  if (s == HSMA_OK) s = oz_product(Ao, Xo, C, ldc, 1, 0, 0, nullptr, "emulated_gemm", st);
+  if (s == HSMA_OK) s = oz_product(Ao, Xo, C, ldc, 1, 0, 0, scratch, nullptr, "emulated_gemm", st);
   hsma_status_t f = hsma_ws_free(ws, st);
   return s != HSMA_OK ? s : f;
 }

@@ -13,6 +13,7 @@
 
 #include "blocked.h"
 #include "common.cuh"
+#include "oz_tables.cuh"
 #include "tma.cuh"
 #include "trace.h"
 
@@ -66,33 +67,27 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 
 // Epilogues of the tensor-core product:
 //   TC_F32: C32 = beta*C32 - acc                    (the FP32-result update)
-//   TC_OZ:  C64 -/+= 2^(rexp[i] + cexp[j] + uexp[u]) * acc_u for every
-//           accumulation unit u of the tile (an emulated FP64 product; each
-//           acc_u holds an exact integer)
+//   TC_OZ:  C64 -/+= 2^(rexp[i] + cexp[j]) * S      (an emulated FP64 product:
+//           S, an integer, from its residues modulo the kOzP moduli of oz_tables.cuh)
 enum { TC_F32 = 0, TC_OZ = 1 };
 
-// Emulated FP64 products (see the Ozaki section below): kOzS slices per
-// operand, pairs p + q <= kOzS + 1.
-constexpr int kOzS = 10;
-constexpr int kOzPairs = kOzS * (kOzS + 1) / 2;
-constexpr int kOzMaxUnits = 64;
+constexpr int kTcMaxPairs = 8;
 
 struct TcArgs {
   float *C32;
   double *C64;
   int64_t ldc;
   float beta;      // TC_F32
-  int beta0;       // TC_OZ: 0 = the first unit overwrites C64 (old values not read)
+  int beta0;       // TC_OZ: 0 = the product overwrites C64 (old values not read)
   int negate;      // TC_OZ: add the product instead of subtracting it
   const int *rexp;  // TC_OZ: row exponents of A
   const int *cexp;  // TC_OZ: column exponents of B
+  uint32_t *scratch;  // TC_OZ: kOzTileWords words per CTA (residue bytes of its current tile)
   int M, N, K;
   int tri;          // row tile i0 needs k < i0 + TC_BM only
-  int nunits;       // accumulation units per tile (TC_F32: 1)
+  int npairs;       // TC_F32: slice pairs summed in the accumulator
   int band;         // tile rows per band of the tile order (set by the launcher)
-  uint8_t ubeg[kOzMaxUnits + 1];  // unit u accumulates pairs ubeg[u] .. ubeg[u+1]-1
-  int8_t uexp[kOzMaxUnits];       // TC_OZ: weight exponent of unit u
-  uint8_t pa[kOzPairs], pb[kOzPairs];  // slice of A and of B for each pair
+  uint8_t pa[kTcMaxPairs], pb[kTcMaxPairs];  // TC_F32: slice of A and of B for each pair
   const int *skip;  // device flag: when set, the launch does nothing
   unsigned int *err;
   uint64_t limit_ns;
@@ -130,24 +125,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
       : "r"(taddr));
 }
 
-// acc * 2^shift in FP64 for an FP32 accumulator value acc (bits f): the
-// exponent is rebased with integer operations, so the FP64 pipe only sees the
-// final addition; ldexp covers results outside the normal range.
-__device__ __forceinline__ double oz_scale(uint32_t f, int shift) {
-  if ((f & 0x7fffffffu) == 0) return 0.0;
-  const int E = (int)((f >> 23) & 0xffu) + (1023 - 127) + shift;
-  if (E >= 1 && E <= 2046)
-    return __hiloint2double((int)((f & 0x80000000u) | ((uint32_t)E << 20) | ((f & 0x7fffffu) >> 3)), (int)(f << 29));
-  return ldexp((double)__uint_as_float(f), shift);
-}
-
 // Persistent, warp-specialised product: warp 0 loads operand stages by TMA,
-// warp 1 issues the MMAs, warps 2..9 drain accumulators.  Work items are
-// (tile, accumulation unit); two accumulators of 256 tensor-memory columns
-// alternate between items, so the epilogue of one item runs while the next
-// item's products accumulate.  Tiles are dealt round-robin to the CTAs (one
-// per SM).  Operands are 3-D: (K, rows, slice); a unit sums the products of
-// its slice pairs over the whole K range in one accumulator.  Every CTA loads
+// warp 1 issues the MMAs, warps 2..9 drain accumulators.  A tile is a sequence
+// of accumulation units: one for TC_F32 (every slice pair over the whole K
+// range), and for TC_OZ one per modulus and K chunk of kOzChunk (the longest
+// whose FP32 sums of residue products stay exact).  Two accumulators of 256
+// tensor-memory columns alternate between units, so one unit's epilogue runs
+// while the next unit's products accumulate.  Tiles are dealt round-robin to
+// the CTAs (one per SM).  Operands are 3-D: (K, rows, slice).  Every CTA loads
 // its own A and B tiles with plain (single-CTA) TMA.
 constexpr int TC_WARPS = 10;
 constexpr int TC_EPI_WARPS = 8;
@@ -166,16 +151,16 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
   if (p.skip != nullptr && *(volatile const int *)p.skip != 0) return;
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int M = p.M, N = p.N, nunits = p.nunits;
+  const int M = p.M, N = p.N;
+  const int nslices = MODE == TC_OZ ? kOzP : p.npairs;  // passes over the K range per tile
   const int cid = blockIdx.x, ncl = gridDim.x;
   const int tiles_m = (M + TC_BM - 1) / TC_BM, tiles_n = (N + TC_BN - 1) / TC_BN;
   const int ntiles = tiles_m * tiles_n;
   // Tiles run in bands of p.band tile rows, column by column inside a band.
-  // For short K the host picks 16 tile rows, so the tiles in flight at once
-  // (one per SM) cover about 16 row tiles x 10 column tiles and their operand
-  // slices stay in L2 while every slice pair re-reads them; for
-  // long K one band spans all rows (column-major order), so the right operand's
-  // slices are shared by every row tile in flight.
+  // With 16 tile rows the tiles in flight at once (one per SM) cover about 16
+  // row tiles x 10 column tiles, the fewest operand rows; long TC_F32 products
+  // take one band over all rows (column-major order), so the right operand is
+  // shared by every row tile in flight.
   const int G = max(1, p.band);
   auto tile_k = [&](int t, int &m0, int &n0) {  // tile -> its origin and K-block count
     const int band = t / (G * tiles_n);
@@ -219,8 +204,8 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       for (int t = cid; t < ntiles && ok; t += ncl) {
         int m0, n0;
         const int nk = tile_k(t, m0, n0);
-        for (int q = 0; q < p.ubeg[nunits] && ok; ++q) {
-          const int sa = p.pa[q], sb = p.pb[q];
+        for (int q = 0; q < nslices && ok; ++q) {
+          const int sa = MODE == TC_OZ ? q : p.pa[q], sb = MODE == TC_OZ ? q : p.pb[q];
           for (int kb = 0; kb < nk; ++kb, ++it) {
             const int s = it % TC_STAGES;
             if (it >= TC_STAGES && !mbar_wait_bounded(&empty[s], ((it / TC_STAGES) - 1) & 1, p.limit_ns, p.err)) {
@@ -245,7 +230,10 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       for (int t = cid; t < ntiles && ok; t += ncl) {
         int m0, n0;
         const int nk = tile_k(t, m0, n0);
-        for (int u = 0; u < nunits && ok; ++u, ++i) {
+        const int total = nslices * nk;  // K blocks of the tile, slice by slice
+        for (int g0 = 0; g0 < total && ok; ++i) {
+          // the unit's K blocks: all of them, or (TC_OZ) the next chunk of this modulus
+          const int glen = MODE == TC_OZ ? min(kOzChunk / TC_BK, nk - g0 % nk) : total;
           const int b = i & 1;
           if (i >= 2 && !mbar_wait_bounded(&acc_empty[b], ((i >> 1) - 1) & 1, p.limit_ns, p.err)) {
             ok = false;
@@ -254,30 +242,29 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
           tc_fence_after();
           const uint32_t acc_cols = tmem + (uint32_t)(b * TC_TMEM_COLS);
           uint32_t accum = 0;
-          for (int q = p.ubeg[u]; q < p.ubeg[u + 1] && ok; ++q) {
-            for (int kb = 0; kb < nk; ++kb, ++it) {
-              const int s = it % TC_STAGES;
-              if (!mbar_wait_bounded(&full[s], (it / TC_STAGES) & 1, p.limit_ns, p.err)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              const uint32_t sa = smem_u32(smem + s * TC_STAGE_BYTES);
-              const uint64_t da = sw_desc(sa), db = sw_desc(sa + TC_A_BYTES);
-#pragma unroll
-              for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
-                    "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(tc_idesc()), "r"(accum)
-                    : "memory");
-                accum = 1u;
-              }
-              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                               smem_u32(&empty[s]))
-                           : "memory");
+          for (int kb = 0; kb < glen; ++kb, ++it) {
+            const int s = it % TC_STAGES;
+            if (!mbar_wait_bounded(&full[s], (it / TC_STAGES) & 1, p.limit_ns, p.err)) {
+              ok = false;
+              break;
             }
+            tc_fence_after();
+            const uint32_t sa = smem_u32(smem + s * TC_STAGE_BYTES);
+            const uint64_t da = sw_desc(sa), db = sw_desc(sa + TC_A_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < TC_BK / 16; ++kk) {
+              asm volatile(
+                  "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
+                  "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(tc_idesc()), "r"(accum)
+                  : "memory");
+              accum = 1u;
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             smem_u32(&empty[s]))
+                         : "memory");
           }
+          g0 += glen;
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                            smem_u32(&acc_full[b]))
                        : "memory");
@@ -293,14 +280,10 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
     __syncwarp();
   } else {
     // epilogue warps: thread = one row of the 128-row tile (its tensor-memory
-    // lane); two warps per lane quarter split the 256 columns.  The old values
-    // of the next 16-column chunk are loaded before this chunk's stores.  The
-    // units of a tile are drained in order by the same threads, so each
-    // read-modify-write of C sees the previous unit's stores.
+    // lane); two warps per lane quarter split the 256 columns.
     const int ew = warp - 2;
     const int quarter = warp & 3, half = ew >> 2;
     const int cbeg = half * (TC_BN / 2);
-    using V = typename std::conditional<MODE == TC_F32, float, double>::type;
     constexpr int CW = 16;  // columns per chunk: keeps ten warps within the register file
     int i = 0;
     bool ok = true;
@@ -308,23 +291,75 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       int m0, n0;
       const int nk = tile_k(t, m0, n0);
       const int row = m0 + quarter * 32 + lane;
-      const int rx = (MODE == TC_OZ && row < M) ? p.rexp[row] : 0;
-      for (int u = 0; u < nunits; ++u, ++i) {
+      if constexpr (MODE == TC_OZ) {
+        // Every unit: residues of the exact FP32 sums, four columns to a word of
+        // the CTA's scratch (a thread reads back only what it wrote; chunks of
+        // one modulus after the first add to the byte that is there).  After the
+        // last modulus: the integer from its residues, one addition to C each.
+        uint32_t *mine = p.scratch + (size_t)cid * kOzTileWords + (cbeg / 4) * TC_BM + quarter * 32 + lane;
+        const int cols = min(TC_BN / 2, N - n0 - cbeg);  // this warp's columns inside the matrix
+        for (int l = 0; l < kOzP && ok; ++l) {
+          const float mod = c_oz.modf[l], inv = c_oz.inv[l];
+          for (int g0 = 0; g0 < nk; g0 += kOzChunk / TC_BK, ++i) {
+            const int b = i & 1;
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i >> 1) & 1, p.limit_ns, p.err));
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll 2
+            for (int c0 = 0; c0 < cols; c0 += CW) {
+              uint32_t v[CW];
+              uint32_t *dst = mine + (l * (TC_BN / 4) + c0 / 4) * TC_BM;
+              tmem_ld16(tmem + (uint32_t)(b * TC_TMEM_COLS) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(cbeg + c0),
+                        v);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+              for (int w = 0; w < CW / 4; ++w) {
+                float r[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) r[j] = oz_residue(__uint_as_float(v[4 * w + j]), mod, inv);
+                if (g0 != 0) oz_add_bytes(r, dst[w * TC_BM], mod, inv);
+                dst[w * TC_BM] = oz_pack_bytes(r);
+              }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[b]);  // this warp is done with accumulator b
+          }
+        }
+        if (!ok) break;
+        if (row < M) {
+          const int rx = p.rexp[row] - 2 * kOzFrac;
+          double *crow = p.C64 + row + (int64_t)(n0 + cbeg) * p.ldc;
+  #pragma unroll 1
+          for (int c0 = 0; c0 < cols; c0 += 4) {
+            double old[4];
+  #pragma unroll
+            for (int j = 0; j < 4; ++j) old[j] = (p.beta0 != 0 && c0 + j < cols) ? crow[(int64_t)(c0 + j) * p.ldc] : 0.0;
+            uint32_t w[kOzP];
+  #pragma unroll
+            for (int l = 0; l < kOzP; ++l) w[l] = mine[(l * (TC_BN / 4) + c0 / 4) * TC_BM] ^ 0x80808080u;
+  #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              if (c0 + j < cols) {
+                const double x = oz_crt(w, j, rx + __ldg(p.cexp + n0 + cbeg + c0 + j));
+                crow[(int64_t)(c0 + j) * p.ldc] = p.negate ? old[j] + x : old[j] - x;
+              }
+            }
+          }
+        }
+      } else {
+        // the old values of the next 16-column chunk are loaded before this chunk's stores
         const int b = i & 1;
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i >> 1) & 1, p.limit_ns, p.err));
         if (!ok) break;
+        ++i;
         tc_fence_after();
-        const bool fresh = MODE == TC_OZ && u == 0 && p.beta0 == 0;
-        const int ushift = MODE == TC_OZ ? rx + p.uexp[u] : 0;
-        V old[CW], nxt[CW];
-        auto load_chunk = [&](int c0, V *dst) {
+        float old[CW], nxt[CW];
+        auto load_chunk = [&](int c0, float *dst) {
 #pragma unroll
           for (int j = 0; j < CW; ++j) {
             const int col = n0 + c0 + j;
-            if constexpr (MODE == TC_F32)
-              dst[j] = (p.beta != 0.0f && row < M && col < N) ? __ldcs(p.C32 + row + (int64_t)col * p.ldc) : 0.0f;
-            else
-              dst[j] = (!fresh && row < M && col < N) ? p.C64[row + (int64_t)col * p.ldc] : 0.0;
+            dst[j] = (p.beta != 0.0f && row < M && col < N) ? __ldcs(p.C32 + row + (int64_t)col * p.ldc) : 0.0f;
           }
         };
         load_chunk(cbeg, nxt);
@@ -334,41 +369,33 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
           for (int j = 0; j < CW; ++j) old[j] = nxt[j];
           if (c0 + CW < cbeg + TC_BN / 2) load_chunk(c0 + CW, nxt);
           uint32_t v[CW];
-          const uint32_t taddr =
-              tmem + (uint32_t)(b * TC_TMEM_COLS) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0;
-#pragma unroll
-          for (int h = 0; h < CW / 16; ++h) tmem_ld16(taddr + 16 * h, v + 16 * h);
+          tmem_ld16(tmem + (uint32_t)(b * TC_TMEM_COLS) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (row < M && nk > 0) {
 #pragma unroll
             for (int j = 0; j < CW; ++j) {
               const int col = n0 + c0 + j;
               if (col < N) {
-                if constexpr (MODE == TC_F32) {
-                  const float a = __uint_as_float(v[j]);
-                  const float y = (p.beta == 1.0f) ? (old[j] - a) : fmaf(p.beta, old[j], -a);
-                  __stcs(p.C32 + row + (int64_t)col * p.ldc, y);
-                  if (p.xs2 != nullptr && row < p.rows2) {
-                    __nv_bfloat16 hi, lo;
-                    split_bf16(y, hi, lo);
-                    __nv_bfloat16 *o = p.xs2 + (int64_t)col * p.ld2 + row;
-                    o[0] = hi;
-                    if (p.terms2 == 3) {
-                      o[p.nb2] = lo;
-                      o[2 * p.nb2] = hi;
-                    }
+                const float a = __uint_as_float(v[j]);
+                const float y = (p.beta == 1.0f) ? (old[j] - a) : fmaf(p.beta, old[j], -a);
+                __stcs(p.C32 + row + (int64_t)col * p.ldc, y);
+                if (p.xs2 != nullptr && row < p.rows2) {
+                  __nv_bfloat16 hi, lo;
+                  split_bf16(y, hi, lo);
+                  __nv_bfloat16 *o = p.xs2 + (int64_t)col * p.ld2 + row;
+                  o[0] = hi;
+                  if (p.terms2 == 3) {
+                    o[p.nb2] = lo;
+                    o[2 * p.nb2] = hi;
                   }
-                  if (p.xs3 != nullptr && row >= p.r3 && row < p.r3 + p.rows3) {
-                    __nv_bfloat16 x0, x1, x2;
-                    split3_bf16(y, x0, x1, x2);
-                    __nv_bfloat16 *o = p.xs3 + (int64_t)col * p.ld3 + (row - p.r3);
-                    o[0] = x0;
-                    o[p.per3] = x1;
-                    o[2 * p.per3] = x2;
-                  }
-                } else {
-                  const double x = oz_scale(v[j], ushift + __ldg(p.cexp + col));
-                  p.C64[row + (int64_t)col * p.ldc] = p.negate ? old[j] + x : old[j] - x;
+                }
+                if (p.xs3 != nullptr && row >= p.r3 && row < p.r3 + p.rows3) {
+                  __nv_bfloat16 x0, x1, x2;
+                  split3_bf16(y, x0, x1, x2);
+                  __nv_bfloat16 *o = p.xs3 + (int64_t)col * p.ld3 + (row - p.r3);
+                  o[0] = x0;
+                  o[p.per3] = x1;
+                  o[2 * p.per3] = x2;
                 }
               }
             }
@@ -416,8 +443,8 @@ struct SliceLayout {
 };
 
 // Launch the persistent product.  A: sa slices of M x K (row-major), B: sb
-// slices of N x K; the unit table of a0 names the slice pairs (TC_F32: one
-// unit, one pair, filled in here unless given).  One CTA per SM.
+// slices of N x K.  TC_F32: a0 names the slice pairs (one pair of slice 0 unless
+// given); TC_OZ: slice l of both holds residues modulo modulus l.  One CTA per SM.
 template <int MODE>
 hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, int sb, const TcArgs &a0,
                       const char *phase, cudaStream_t st, SliceLayout la = {}, SliceLayout lb = {}) {
@@ -447,15 +474,17 @@ hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, 
                       (uint64_t)lb.sst))
     return HSMA_ERR_CUDA;
   TcArgs a = a0;
-  if (MODE == TC_F32 && a.nunits == 0) {
-    a.nunits = 1;
-    a.ubeg[0] = 0;
-    a.ubeg[1] = 1;
-    a.pa[0] = a.pb[0] = 0;
+  if constexpr (MODE == TC_OZ) {
+    if (sa != kOzP || sb != kOzP || a.K > kOzMaxK || a.scratch == nullptr) return HSMA_ERR_INVALID_ARG;
+  } else {
+    if (a.npairs == 0) {
+      a.npairs = 1;
+      a.pa[0] = a.pb[0] = 0;
+    }
+    if (a.npairs > kTcMaxPairs) return HSMA_ERR_INVALID_ARG;
+    for (int q = 0; q < a.npairs; ++q)
+      if (a.pa[q] >= sa || a.pb[q] >= sb) return HSMA_ERR_INVALID_ARG;
   }
-  if (a.nunits < 1 || a.nunits > kOzMaxUnits) return HSMA_ERR_INVALID_ARG;
-  for (int q = 0; q < a.ubeg[a.nunits]; ++q)
-    if (a.pa[q] >= sa || a.pb[q] >= sb) return HSMA_ERR_INVALID_ARG;
   a.err = hsma_dev_error_ptr();
   if (a.err == nullptr) return HSMA_ERR_CUDA;
   if (a.limit_ns == 0) a.limit_ns = 4000000000ull;
@@ -465,7 +494,7 @@ hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, 
   if (dev < 0 || dev >= 64) return HSMA_ERR_UNSUPPORTED;
   if (nsm[dev] == 0) HSMA_CUDA_TRY(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
   const int ntiles = tiles_m * tiles_n;
-  a.band = a.K <= 2048 ? 16 : tiles_m;
+  a.band = MODE == TC_OZ || a.K <= 2048 ? 16 : tiles_m;
   const int grid = std::max(1, std::min(ntiles, nsm[dev]));
   HsmaTraceScope ts(phase, st);
   tc_gemm_kernel<MODE><<<grid, 32 * TC_WARPS, TC_SMEM, st>>>(ma, mb, a);

@@ -79,6 +79,23 @@ def test_emulated_gemm_fp64_accuracy(H, M, N, K):
         assert abs(got[i, j] - exact) <= 2.0 ** -50 * scale, (i, j, abs(got[i, j] - exact) / scale)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (127, 257, 63), (128, 256, 1024), (129, 255, 1025), (130, 3, 8192),
+                                    (5, 258, 8193), (257, 9, 16384)])
+def test_emulated_gemm_residue_edges(H, M, N, K):
+    """Edges of tiles, of the exact accumulation chunk (K = 1024) and of one product (K = 8192), with
+    full 53-bit significands of one sign (the largest sums the residues have to hold).  The integer
+    product is exact, rounded once per launch (at most 8192 of K) and once when added to a nonzero C:
+    one rounding up to K = 8192 (C is 0 here), three beyond."""
+    rng = np.random.default_rng(M + N + K)
+    A = np.asfortranarray(rng.integers(2 ** 52, 2 ** 53, (M, K)).astype(np.float64))
+    X = np.asfortranarray(rng.integers(2 ** 52, 2 ** 53, (K, N)).astype(np.float64))
+    A[0] = X[:, 0] = 2.0 ** 53 - 1
+    got = _gemm(H, A, X, np.zeros((M, N), order="F"))
+    for i, j in {(0, 0), (M - 1, N - 1), (M - 1, 0), (0, N - 1), (M // 2, N // 2)}:
+        exact = -sum(int(a) * int(x) for a, x in zip(A[i], X[:, j]))
+        assert abs(int(got[i, j]) - exact) * 2 ** 53 <= (1 if K <= 8192 else 3) * abs(exact), (i, j)
+
+
 def test_emulated_gemm_rejects_bad_arguments(H):
     assert H.hsma_gemm_f64_emulated(4, 4, 16385, 1, 4, 1, 16385, 1, 4, 0, check=False) == H.ERR_UNSUPPORTED
     assert H.hsma_gemm_f64_emulated(4, 4, 4, 1, 3, 1, 4, 1, 4, 0, check=False) == H.ERR_INVALID_ARG

@@ -910,13 +910,13 @@ hsma_status_t oz_slice_x(const double *X, int64_t ldx, int K, const int *kexp, O
 }
 
 // Scratch of the emulated products of up to rows x cols results: the residue
-// bytes of one tile per CTA.
+// bytes of two tiles per CTA.
 constexpr int kEmuGemmMaxK = 1 << 14;      // hsma_gemm_f64_emulated
 constexpr int kOzResidualMaxM = 1 << 14;   // refinement residuals
 
 size_t oz_scratch_bytes(int64_t rows, int64_t cols) {
-  const int64_t tiles = ((rows + TC_BM - 1) / TC_BM) * ((cols + TC_BN - 1) / TC_BN);
-  return (size_t)std::min<int64_t>(tiles, hsma_sm_count()) * kOzTileWords * sizeof(uint32_t);
+  const int64_t tiles = ((rows + TC_BM - 1) / TC_BM) * ((cols + 127) / 128);
+  return 2 * (size_t)std::min<int64_t>(tiles, hsma_sm_count()) * kOzTileWords * sizeof(uint32_t);
 }
 
 // C (M x N, column-major FP64) = (beta0 ? C : 0) -/+ L X in emulated FP64,

@@ -16,9 +16,11 @@
 // p_l, so that with c_l = (sum mod p_l)
 //     S = sum_l c_l P / p_l  (mod P).
 // The moduli are grouped by three (group products Q_g < 2^24): 32-bit integer
-// sums inside a group, six multiword terms n_g P / Q_g, and a multiple of P
-// found in FP32 from sum_g n_g / Q_g (|S| / P stays below 1/3, so rounding to
-// the nearest integer has a margin of 1/6).
+// sums n_g inside a group, then S / P = sum_g n_g / Q_g (mod 1) in 128-bit fixed
+// point, whose wrap-around takes off the multiple of P by itself (|S| / P stays
+// below 1/3).  Its error, 2^28 units of 2^-128, is 2^33 in S, far below the
+// 2^59 that rounding one operand entry costs; |S| below 2^37 counts as zero, so
+// that an exact zero stays one.
 #pragma once
 
 #include <stdint.h>
@@ -30,7 +32,13 @@ constexpr int kOzFrac = 59;         // fraction bits of the fixed-point operands
 constexpr int kOzChunk = 1024;      // K per exact FP32 sum
 constexpr int kOzMaxK = 8192;       // K per product: K 2^(2 kOzFrac) < P / 3
 constexpr int kOzGroups = 6;        // groups of three moduli (the last: two)
-constexpr int kOzTileWords = kOzP * (256 / 4) * 128;  // residue bytes of a 128 x 256 tile, in words
+// residue bytes of a 128 x 256 tile in words, per modulus and in all; a CTA's
+// scratch holds two tiles (one being written, one being converted)
+constexpr int kOzPlaneWords = (256 / 4) * 128;
+constexpr int kOzTileWords = kOzP * kOzPlaneWords;
+__device__ __forceinline__ size_t oz_scratch_at(int cta, int half, int col) {
+  return (size_t)(2 * cta + half) * kOzTileWords + (size_t)(col / 4) * 128;
+}
 
 struct OzTables {
   // slicing: balanced weights (2^15)^j of the four 15-bit limbs, for the left
@@ -38,12 +46,8 @@ struct OzTables {
   float wa[kOzP][4], wx[kOzP][4];
   float modf[kOzP], inv[kOzP];
   uint32_t gw[kOzP];             // Q_g / p_l
-  uint32_t W[kOzGroups][4];      // P / Q_g (below 2^128)
-  float qinv[kOzGroups];         // 1 / Q_g
-  uint32_t negP[5];              // 2^160 - P
-  uint32_t init[5];              // 16 P - sum_l 128 P / p_l (mod 2^160): undoes the offset of the
-                                 // stored bytes; 16 P keeps the multiple of P taken off positive
-  float init_f;                  // 16 - sum_l 128 / p_l
+  uint32_t F[kOzGroups][4];      // 2^128 / Q_g
+  uint32_t init[4];              // -sum_l 128 2^128 / p_l: undoes the offset of the stored bytes
 };
 
 constexpr uint32_t kOzMod[kOzP] = {256, 251, 249, 247, 245, 241, 239, 233, 229, 227, 223, 211, 199, 197, 193, 191, 187};
@@ -74,15 +78,17 @@ constexpr U160 u160_add(U160 a, U160 b) {
   return r;
 }
 
-constexpr U160 u160_neg(U160 a) {
+// round(2^128 num / den) for num < den < 2^26, four words
+constexpr U160 u128_fraction(uint32_t num, uint32_t den) {
   U160 r{};
-  uint64_t c = 1;
-  for (int i = 0; i < 5; ++i) {
-    c += (uint32_t)~a.w[i];
-    r.w[i] = (uint32_t)c;
-    c >>= 32;
+  uint64_t rem = num;
+  for (int i = 3; i >= 0; --i) {
+    rem <<= 32;
+    r.w[i] = (uint32_t)(rem / den);
+    rem %= den;
   }
-  return r;
+  U160 one{{2 * rem >= den ? 1u : 0u, 0, 0, 0, 0}};
+  return u160_add(r, one);
 }
 
 // representative of v modulo p in (-p/2, p/2]
@@ -90,19 +96,12 @@ constexpr int oz_balance(uint32_t v, uint32_t p) { return 2 * v > p ? (int)v - (
 
 constexpr OzTables oz_make_tables() {
   OzTables t{};
-  U160 P{{1, 0, 0, 0, 0}};
-  for (int l = 0; l < kOzP; ++l) P = u160_mul(P, kOzMod[l]);
   U160 off{};
-  float off_f = 0.0f;
   for (int l = 0; l < kOzP; ++l) {
     const uint32_t p = kOzMod[l];
-    U160 part{{1, 0, 0, 0, 0}};
-    uint32_t rest = 1;
+    uint32_t rest = 1;  // P / p_l mod p_l
     for (int k = 0; k < kOzP; ++k)
-      if (k != l) {
-        part = u160_mul(part, kOzMod[k]);
-        rest = rest * (kOzMod[k] % p) % p;
-      }
+      if (k != l) rest = rest * (kOzMod[k] % p) % p;
     uint32_t inv = 1;
     while (rest * inv % p != 1) ++inv;  // coprime moduli: ends below p
     uint32_t x = 1;
@@ -113,34 +112,34 @@ constexpr OzTables oz_make_tables() {
     }
     t.modf[l] = (float)p;
     t.inv[l] = 1.0f / (float)p;
-    off = u160_add(off, u160_mul(part, 128));
-    off_f -= 128.0f / (float)p;
+    off = u160_add(off, u128_fraction(128 % p, p));
   }
   for (int g = 0; g < kOzGroups; ++g) {
     uint32_t Q = 1;
-    U160 W{{1, 0, 0, 0, 0}};
-    for (int l = 0; l < kOzP; ++l) {
-      if (l / 3 == g)
-        Q *= kOzMod[l];
-      else
-        W = u160_mul(W, kOzMod[l]);
-    }
+    for (int l = 0; l < kOzP; ++l)
+      if (l / 3 == g) Q *= kOzMod[l];
     for (int l = 0; l < kOzP; ++l)
       if (l / 3 == g) t.gw[l] = Q / kOzMod[l];
-    for (int i = 0; i < 4; ++i) t.W[g][i] = W.w[i];
-    t.qinv[g] = 1.0f / (float)Q;
+    const U160 f = u128_fraction(1, Q);
+    for (int i = 0; i < 4; ++i) t.F[g][i] = f.w[i];
   }
-  const U160 nP = u160_neg(P), io = u160_add(u160_neg(off), u160_mul(P, 16));
-  for (int i = 0; i < 5; ++i) {
-    t.negP[i] = nP.w[i];
-    t.init[i] = io.w[i];
+  uint64_t c = 1;
+  for (int i = 0; i < 4; ++i) {
+    c += (uint32_t)~off.w[i];
+    t.init[i] = (uint32_t)c;
+    c >>= 32;
   }
-  t.init_f = off_f + 16.0f;
   return t;
 }
 
 constexpr OzTables kOzTables = oz_make_tables();
 __constant__ OzTables c_oz = kOzTables;
+
+constexpr U160 oz_product_of_moduli() {
+  U160 P{{1, 0, 0, 0, 0}};
+  for (int l = 0; l < kOzP; ++l) P = u160_mul(P, kOzMod[l]);
+  return P;
+}
 
 constexpr bool oz_moduli_ok() {
   for (int a = 0; a < kOzP; ++a)
@@ -153,12 +152,18 @@ constexpr bool oz_moduli_ok() {
       }
       if (x != 1) return false;
     }
-  U160 P{{1, 0, 0, 0, 0}};
-  for (int l = 0; l < kOzP; ++l) P = u160_mul(P, kOzMod[l]);
-  // 3 kOzMaxK 2^(2 kOzFrac) = 3 * 2^131 <= P < 2^133 (so every P / Q_g fits four words)
-  return P.w[4] >= 3u * (kOzMaxK >> 10) && P.w[4] < 32u;
+  // 3 kOzMaxK 2^(2 kOzFrac) = 3 * 2^131 <= P, and 2^132 <= P < 2^133
+  const U160 P = oz_product_of_moduli();
+  return P.w[4] >= 3u * (kOzMaxK >> 10) && P.w[4] >= 16u && P.w[4] < 32u;
 }
 static_assert(2 * kOzFrac + 10 == 128 && oz_moduli_ok(), "coprime moduli whose product covers the largest sum");
+
+// the leading 64 bits of P (2^132 <= P < 2^133)
+constexpr uint64_t oz_lead_p() {
+  const U160 P = oz_product_of_moduli();
+  return (uint64_t)P.w[4] << 59 | (uint64_t)P.w[3] << 27 | P.w[2] >> 5;
+}
+constexpr uint64_t kOzLeadP = oz_lead_p();
 
 // Balanced residue of an exact integer v, |v| <= 2^24: the quotient is rounded
 // with one FP32 rounding each for v / p and the sum with 1.5 2^23, so the result
@@ -187,76 +192,51 @@ __device__ __forceinline__ void oz_add_bytes(float (&r)[4], uint32_t w, float mo
   }
 }
 
-// The integer whose residues c_l + 128 are byte j of w[l], times 2^shift, as a
-// correctly rounded double (ldexp's rounding below the normal range).
-__device__ __forceinline__ double oz_crt(const uint32_t (&w)[kOzP], int j, int shift) {
-  uint64_t acc[5];
+// The integer S whose residues c_l + 128 are byte j of w[l]: the 64 leading bits
+// of S / P times those of P (relative error below 2^-61), rounded once to 53
+// bits.  Returned as a double in [1, 2) (or 2 after rounding up; 0 for S = 0)
+// with S's sign and the exponent of its leading bit in e.  Written without
+// branches so that the conversions of several results overlap.
+__device__ __forceinline__ uint64_t oz_crt(const uint32_t (&w)[kOzP], int j, int &e) {
+  uint64_t acc[4];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) acc[i] = c_oz.init[i];
-  float f = c_oz.init_f;
+  for (int i = 0; i < 4; ++i) acc[i] = c_oz.init[i];
 #pragma unroll
   for (int g = 0; g < kOzGroups; ++g) {
     uint32_t ng = 0;
 #pragma unroll
     for (int l = 3 * g; l < 3 * g + 3 && l < kOzP; ++l) ng += __byte_perm(w[l], 0u, 0x4440 | j) * c_oz.gw[l];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] += (uint64_t)ng * c_oz.W[g][i];
-    f = fmaf(__uint2float_rn(ng), c_oz.qinv[g], f);
+    for (int i = 0; i < 4; ++i) acc[i] += (uint64_t)ng * c_oz.F[g][i];
   }
-  // f = 16 + sum_l c_l / p_l to about 2^-18, within 1/3 of the multiple of P to
-  // take off; |c_l| <= p_l / 2 + 1% keeps it between 7 and 25
-  const uint32_t k = (uint32_t)__float2int_rn(f);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) acc[i] += (uint64_t)k * c_oz.negP[i];
-  uint32_t x[5];
-  uint64_t c = 0;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    c += acc[i];
-    x[i] = (uint32_t)c;
-    c >>= 32;
-  }
-  // sign and magnitude
-  const bool neg = (int32_t)x[4] < 0;
-  uint64_t lo = (uint64_t)x[1] << 32 | x[0], mid = (uint64_t)x[3] << 32 | x[2];
-  uint32_t hi = x[4];
-  if (neg) {
-    lo = ~lo + 1;
-    mid = ~mid + (lo == 0 ? 1 : 0);
-    hi = ~hi + ((lo | mid) == 0 ? 1u : 0u);
-  }
-  // the leading 64 bits from the top nonzero word on, and what lies below them
-  uint64_t top, next;
-  uint32_t rest = 0;
-  int pos;
-  if (hi != 0) {
-    top = (uint64_t)hi << 32 | (mid >> 32);
-    next = mid << 32 | lo >> 32;
-    rest = (uint32_t)lo;
-    pos = 159;
-  } else if (mid != 0) {
-    top = mid;
-    next = lo;
-    pos = 127;
-  } else {
-    top = lo;
-    next = 0;
-    pos = 63;
-  }
-  if (top == 0) return 0.0;
-  const int z = __clzll((long long)top);
-  const uint64_t mant = z != 0 ? top << z | next >> (64 - z) : top;
-  const bool sticky = ((next << z) | rest) != 0;
-  uint64_t r = mant >> 11;
-  const uint32_t rem = (uint32_t)mant & 0x7ffu;
-  if (rem > 0x400u || (rem == 0x400u && (sticky || (r & 1) != 0))) ++r;
-  const int e = pos - z + shift;  // exponent of the leading bit
-  double y;
-  if (e >= -1022 && e <= 1022)
-    y = __longlong_as_double((long long)(((uint64_t)(e + 1022) << 52) + r));  // r's bit 52 (or 53) carries in
-  else
-    y = ldexp((double)r, e - 52);
-  return neg ? -y : y;
+  acc[1] += acc[0] >> 32;
+  acc[2] += acc[1] >> 32;
+  acc[3] += acc[2] >> 32;
+  uint64_t lo = acc[1] << 32 | (uint32_t)acc[0], hi = acc[3] << 32 | (uint32_t)acc[2];
+  // magnitude (of a negative value less one unit of 2^-128, far below the error)
+  const uint32_t sign = (uint32_t)(hi >> 63);
+  const uint64_t flip = sign ? ~0ull : 0ull;
+  hi ^= flip;
+  lo ^= flip;
+  const bool small = hi == 0;
+  const bool zero = small && (lo >> 32) == 0;
+  hi = small ? lo : hi;
+  lo = small ? 0ull : lo;
+  const int z = __clzll((long long)hi);
+  const uint64_t m = hi << (z & 63) | (lo >> 1) >> (63 - (z & 63));
+  uint64_t h = __umul64hi(m, kOzLeadP);  // in [2^62, 2^64)
+  const uint32_t up = (uint32_t)(h >> 63);
+  e = 131 + (int)up - z - (small ? 64 : 0);
+  h <<= 1 - up;
+  const uint64_t r = (h >> 11) + ((h >> 10) & 1);
+  // r's bit 52 (or 53) carries into the exponent field
+  return zero ? 0ull : (((uint64_t)(sign << 11) + 1022) << 52) + r;
+}
+
+// y 2^e for y from oz_crt (ldexp's rounding below the normal range)
+__device__ __forceinline__ bool oz_scales(int e) { return e >= -1022 && e <= 1022; }
+__device__ __forceinline__ double oz_scaled(uint64_t y, int e) {
+  return __longlong_as_double((long long)(y == 0 ? 0ull : y + ((uint64_t)(int64_t)e << 52)));
 }
 
 }  // namespace

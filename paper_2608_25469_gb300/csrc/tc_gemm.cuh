@@ -32,17 +32,27 @@ namespace {
 #ifndef HSMA_TC_BK
 #define HSMA_TC_BK 64
 #endif
-constexpr int TC_BM = 128, TC_BN = 256, TC_BK = HSMA_TC_BK;
+constexpr int TC_BM = 128, TC_BK = HSMA_TC_BK;
 constexpr int TC_ROW_BYTES = TC_BK * 2;  // one K-row of a stage tile: the swizzle width
 static_assert(TC_ROW_BYTES == 64 || TC_ROW_BYTES == 128, "K-blocks of 32 or 64 BF16 values");
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;
-constexpr int TC_B_BYTES = TC_BN * TC_BK * 2;
-constexpr int TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
-constexpr int TC_STAGES = TC_BK == 32 ? 9 : 4;
-constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + 1024;
-static_assert(TC_SMEM <= 227 * 1024 - 256, "stages fit the shared memory of one CTA");
-static_assert(TC_STAGE_BYTES % 1024 == 0, "every stage starts on a swizzle-pattern boundary");
-constexpr uint32_t TC_TMEM_COLS = 256;
+constexpr uint32_t TC_TMEM_COLS = 512;  // all of the SM's tensor memory (one CTA per SM)
+
+// Tile of 128 x BN results: BN = 256 reads the fewest operand bytes per product,
+// BN = 128 gives twice the tiles when a launch has too few for the SMs.
+template <int BN>
+struct TcTile {
+  static constexpr int B_BYTES = BN * TC_BK * 2;
+  static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
+  static constexpr int STAGES = (BN == 256 ? 4 : 6) * (64 / TC_BK);
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
+  static constexpr int ACCS = TC_TMEM_COLS / BN;  // accumulators in tensor memory
+  // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M x N
+  static constexpr uint32_t IDESC =
+      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
+  static_assert(SMEM <= 227 * 1024 - 256, "stages fit the shared memory of one CTA");
+  static_assert(STAGE_BYTES % 1024 == 0, "every stage starts on a swizzle-pattern boundary");
+};
 
 // Shared-memory matrix descriptor: K-major operand, rows of TC_ROW_BYTES in
 // groups of 8 (8 * TC_ROW_BYTES apart), swizzled over the row width
@@ -55,11 +65,6 @@ __device__ __forceinline__ uint64_t sw_desc(uint32_t saddr) {
   d |= (uint64_t)1u << 46;                                // descriptor version
   d |= (uint64_t)(TC_ROW_BYTES == 128 ? 2u : 4u) << 61;   // swizzle mode
   return d;
-}
-
-// Instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M x N.
-__host__ __device__ constexpr uint32_t tc_idesc() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -125,27 +130,92 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
       : "r"(taddr));
 }
 
+// Conversion of ncols columns (a multiple of 4) from column c_beg on of a 128 x BN
+// tile at (m0, n0), rows 32 quarter + lane, from the residues in half h of the
+// CTA's scratch: four columns at a time, the next four's loads in flight.
+template <int BN>
+__device__ __forceinline__ void oz_convert(const TcArgs &p, int cid, int h, int m0, int n0, int quarter, int c_beg,
+                                           int ncols) {
+  const int rl = quarter * 32 + (threadIdx.x & 31), row = m0 + rl;
+  const int cols = min(ncols, p.N - n0 - c_beg);
+  if (row >= p.M || cols <= 0) return;
+  const uint32_t *mine = p.scratch + oz_scratch_at(cid, h, c_beg) + rl;
+  const int rx = p.rexp[row] - 2 * kOzFrac;
+  const int *cx = p.cexp + n0 + c_beg;
+  double *crow = p.C64 + row + (int64_t)(n0 + c_beg) * p.ldc;
+  uint32_t nw[kOzP];
+  double nold[4];
+  auto load4 = [&](int c0) {
+#pragma unroll
+    for (int l = 0; l < kOzP; ++l) nw[l] = mine[l * kOzPlaneWords + c0 / 4 * TC_BM];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      nold[j] = (p.beta0 != 0 && c0 + j < cols) ? crow[(int64_t)(c0 + j) * p.ldc] : 0.0;
+  };
+  load4(0);
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols; c0 += 4) {
+    uint32_t w[kOzP];
+    double old[4];
+    int e[4];
+    uint64_t y[4];
+    bool normal = true;
+#pragma unroll
+    for (int l = 0; l < kOzP; ++l) w[l] = nw[l] ^ 0x80808080u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) old[j] = nold[j];
+    if (c0 + 4 < cols) load4(c0 + 4);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      y[j] = oz_crt(w, j, e[j]);
+      e[j] += rx + __ldg(cx + min(c0 + j, cols - 1));
+      normal &= y[j] == 0 || oz_scales(e[j]);
+    }
+    double x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = oz_scaled(y[j], e[j]);
+    if (!normal) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = ldexp(__longlong_as_double((long long)y[j]), e[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c0 + j < cols) crow[(int64_t)(c0 + j) * p.ldc] = p.negate ? old[j] + x[j] : old[j] - x[j];
+  }
+}
+
 // Persistent, warp-specialised product: warp 0 loads operand stages by TMA,
-// warp 1 issues the MMAs, warps 2..9 drain accumulators.  A tile is a sequence
-// of accumulation units: one for TC_F32 (every slice pair over the whole K
-// range), and for TC_OZ one per modulus and K chunk of kOzChunk (the longest
-// whose FP32 sums of residue products stay exact).  Two accumulators of 256
-// tensor-memory columns alternate between units, so one unit's epilogue runs
-// while the next unit's products accumulate.  Tiles are dealt round-robin to
-// the CTAs (one per SM).  Operands are 3-D: (K, rows, slice).  Every CTA loads
-// its own A and B tiles with plain (single-CTA) TMA.
+// warp 1 issues the MMAs, warps 2..9 drain accumulators, and (TC_OZ) warps
+// 10..17 turn a finished tile's residues into FP64.  A tile is a sequence of
+// accumulation units: one for TC_F32 (every slice pair over the whole K range),
+// and for TC_OZ one per modulus and K chunk of kOzChunk (the longest whose FP32
+// sums of residue products stay exact).  The accumulators (512 tensor-memory
+// columns) rotate between units, so one unit's epilogue runs while the next
+// units' products accumulate.  Tiles are dealt round-robin to the CTAs (one per
+// SM).  Operands are 3-D: (K, rows, slice).  Every CTA loads its own A and B
+// tiles with plain (single-CTA) TMA.
 constexpr int TC_WARPS = 10;
 constexpr int TC_EPI_WARPS = 8;
+constexpr int TC_CRT_WARPS = 8;
 
 template <int MODE>
-__global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
-                                                                   const __grid_constant__ CUtensorMap mapB,
-                                                                   const __grid_constant__ TcArgs p) {
+constexpr int tc_threads() {
+  return 32 * (TC_WARPS + (MODE == TC_OZ ? TC_CRT_WARPS : 0));
+}
+
+template <int MODE, int BN>
+__global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
+                                                                        const __grid_constant__ CUtensorMap mapB,
+                                                                        const __grid_constant__ TcArgs p) {
+  using TL = TcTile<BN>;
+  constexpr int TC_BN = BN, TC_STAGES = TL::STAGES, TC_STAGE_BYTES = TL::STAGE_BYTES, NACC = TL::ACCS;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[TC_STAGES];
   __shared__ __align__(8) uint64_t empty[TC_STAGES];
-  __shared__ __align__(8) uint64_t acc_full[2];
-  __shared__ __align__(8) uint64_t acc_empty[2];
+  __shared__ __align__(8) uint64_t acc_full[NACC];
+  __shared__ __align__(8) uint64_t acc_empty[NACC];
+  __shared__ __align__(8) uint64_t res_full[2];   // TC_OZ: residues of a tile complete in scratch half
+  __shared__ __align__(8) uint64_t res_empty[2];  // ... and converted
   __shared__ __align__(8) uint64_t drained;
   __shared__ uint32_t tmem_base;
   if (p.skip != nullptr && *(volatile const int *)p.skip != 0) return;
@@ -178,16 +248,20 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < NACC; ++b) {
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], TC_EPI_WARPS);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&res_full[b], TC_EPI_WARPS);
+      mbar_init(&res_empty[b], TC_CRT_WARPS);
     }
     mbar_init(&drained, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"(2 * TC_TMEM_COLS)
+                 "r"(TC_TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -234,13 +308,13 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
         for (int g0 = 0; g0 < total && ok; ++i) {
           // the unit's K blocks: all of them, or (TC_OZ) the next chunk of this modulus
           const int glen = MODE == TC_OZ ? min(kOzChunk / TC_BK, nk - g0 % nk) : total;
-          const int b = i & 1;
-          if (i >= 2 && !mbar_wait_bounded(&acc_empty[b], ((i >> 1) - 1) & 1, p.limit_ns, p.err)) {
+          const int b = i % NACC;
+          if (i >= NACC && !mbar_wait_bounded(&acc_empty[b], (i / NACC - 1) & 1, p.limit_ns, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t acc_cols = tmem + (uint32_t)(b * TC_TMEM_COLS);
+          const uint32_t acc_cols = tmem + (uint32_t)(b * BN);
           uint32_t accum = 0;
           for (int kb = 0; kb < glen; ++kb, ++it) {
             const int s = it % TC_STAGES;
@@ -256,7 +330,7 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
               asm volatile(
                   "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                   "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
-                  "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(tc_idesc()), "r"(accum)
+                  "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(TL::IDESC), "r"(accum)
                   : "memory");
               accum = 1u;
             }
@@ -278,9 +352,9 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       mbar_wait_bounded(&drained, 0, p.limit_ns, p.err);
     }
     __syncwarp();
-  } else {
+  } else if (warp < TC_WARPS) {
     // epilogue warps: thread = one row of the 128-row tile (its tensor-memory
-    // lane); two warps per lane quarter split the 256 columns.
+    // lane); two warps per lane quarter split the columns.
     const int ew = warp - 2;
     const int quarter = warp & 3, half = ew >> 2;
     const int cbeg = half * (TC_BN / 2);
@@ -293,24 +367,27 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
       const int row = m0 + quarter * 32 + lane;
       if constexpr (MODE == TC_OZ) {
         // Every unit: residues of the exact FP32 sums, four columns to a word of
-        // the CTA's scratch (a thread reads back only what it wrote; chunks of
-        // one modulus after the first add to the byte that is there).  After the
-        // last modulus: the integer from its residues, one addition to C each.
-        uint32_t *mine = p.scratch + (size_t)cid * kOzTileWords + (cbeg / 4) * TC_BM + quarter * 32 + lane;
+        // this half of the CTA's scratch (chunks of one modulus after the first
+        // add to the byte that the same thread wrote).
+        const int ti = (t - cid) / ncl, h = ti & 1;
+        if (ti >= 2) {
+          ok = __all_sync(0xffffffffu, mbar_wait_bounded(&res_empty[h], ((ti >> 1) - 1) & 1, p.limit_ns, p.err));
+          if (!ok) break;
+        }
+        uint32_t *mine = p.scratch + oz_scratch_at(cid, h, cbeg) + quarter * 32 + lane;
         const int cols = min(TC_BN / 2, N - n0 - cbeg);  // this warp's columns inside the matrix
         for (int l = 0; l < kOzP && ok; ++l) {
           const float mod = c_oz.modf[l], inv = c_oz.inv[l];
           for (int g0 = 0; g0 < nk; g0 += kOzChunk / TC_BK, ++i) {
-            const int b = i & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i >> 1) & 1, p.limit_ns, p.err));
+            const int b = i % NACC;
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i / NACC) & 1, p.limit_ns, p.err));
             if (!ok) break;
             tc_fence_after();
+            uint32_t *dst = mine + l * kOzPlaneWords;
 #pragma unroll 2
-            for (int c0 = 0; c0 < cols; c0 += CW) {
+            for (int c0 = 0; c0 < cols; c0 += CW, dst += CW / 4 * TC_BM) {
               uint32_t v[CW];
-              uint32_t *dst = mine + (l * (TC_BN / 4) + c0 / 4) * TC_BM;
-              tmem_ld16(tmem + (uint32_t)(b * TC_TMEM_COLS) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(cbeg + c0),
-                        v);
+              tmem_ld16(tmem + (uint32_t)(b * BN) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(cbeg + c0), v);
               asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
               for (int w = 0; w < CW / 4; ++w) {
@@ -327,30 +404,12 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
           }
         }
         if (!ok) break;
-        if (row < M) {
-          const int rx = p.rexp[row] - 2 * kOzFrac;
-          double *crow = p.C64 + row + (int64_t)(n0 + cbeg) * p.ldc;
-  #pragma unroll 1
-          for (int c0 = 0; c0 < cols; c0 += 4) {
-            double old[4];
-  #pragma unroll
-            for (int j = 0; j < 4; ++j) old[j] = (p.beta0 != 0 && c0 + j < cols) ? crow[(int64_t)(c0 + j) * p.ldc] : 0.0;
-            uint32_t w[kOzP];
-  #pragma unroll
-            for (int l = 0; l < kOzP; ++l) w[l] = mine[(l * (TC_BN / 4) + c0 / 4) * TC_BM] ^ 0x80808080u;
-  #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              if (c0 + j < cols) {
-                const double x = oz_crt(w, j, rx + __ldg(p.cexp + n0 + cbeg + c0 + j));
-                crow[(int64_t)(c0 + j) * p.ldc] = p.negate ? old[j] + x : old[j] - x;
-              }
-            }
-          }
-        }
+        if (lane == 0) mbar_arrive(&res_full[h]);  // (after the last unit's __syncwarp)
+        if (t + ncl >= ntiles) oz_convert<BN>(p, cid, h, m0, n0, quarter, cbeg + TC_BN / 4, TC_BN / 4);
       } else {
         // the old values of the next 16-column chunk are loaded before this chunk's stores
-        const int b = i & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i >> 1) & 1, p.limit_ns, p.err));
+        const int b = i % NACC;
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], (i / NACC) & 1, p.limit_ns, p.err));
         if (!ok) break;
         ++i;
         tc_fence_after();
@@ -369,7 +428,7 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
           for (int j = 0; j < CW; ++j) old[j] = nxt[j];
           if (c0 + CW < cbeg + TC_BN / 2) load_chunk(c0 + CW, nxt);
           uint32_t v[CW];
-          tmem_ld16(tmem + (uint32_t)(b * TC_TMEM_COLS) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
+          tmem_ld16(tmem + (uint32_t)(b * BN) + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (row < M && nk > 0) {
 #pragma unroll
@@ -407,12 +466,28 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1) tc_gemm_kernel(const __grid_
         if (lane == 0) mbar_arrive(&acc_empty[b]);
       }
     }
+  } else if constexpr (MODE == TC_OZ) {
+    // Conversion warps (the rows and columns of the epilogue warps): a tile's
+    // integers from their residues, one addition to C each.  Run by the epilogue
+    // warps between units this held the accumulators for 110 us per 128 x 256
+    // tile, longer than the products of K = 1024 take.
+    const int cw = warp - TC_WARPS;
+    for (int t = cid, ti = 0; t < ntiles; t += ncl, ++ti) {
+      int m0, n0;
+      tile_k(t, m0, n0);
+      const int h = ti & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&res_full[h], (ti >> 1) & 1, p.limit_ns, p.err))) break;
+      // the CTA's last tile is shared with the epilogue warps, which are done
+      oz_convert<BN>(p, cid, h, m0, n0, cw & 3, (cw >> 2) * (TC_BN / 2), t + ncl >= ntiles ? TC_BN / 4 : TC_BN / 2);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&res_empty[h]);
+    }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TC_TMEM_COLS)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
                  : "memory");
   }
 }
@@ -445,18 +520,18 @@ struct SliceLayout {
 // Launch the persistent product.  A: sa slices of M x K (row-major), B: sb
 // slices of N x K.  TC_F32: a0 names the slice pairs (one pair of slice 0 unless
 // given); TC_OZ: slice l of both holds residues modulo modulus l.  One CTA per SM.
-template <int MODE>
-hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, int sb, const TcArgs &a0,
-                      const char *phase, cudaStream_t st, SliceLayout la = {}, SliceLayout lb = {}) {
+template <int MODE, int BN>
+hsma_status_t tc_gemm_tiled(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, int sb, const TcArgs &a0,
+                      const char *phase, cudaStream_t st, SliceLayout la, SliceLayout lb) {
   if (a0.M <= 0 || a0.N <= 0) return HSMA_OK;
   if (a0.K % TC_BK != 0 || a0.K <= 0) return HSMA_ERR_INVALID_ARG;
   static DeviceFlags attr;
   if (!attr.test()) {
     HSMA_CUDA_TRY(
-        cudaFuncSetAttribute(tc_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
+        cudaFuncSetAttribute(tc_gemm_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<BN>::SMEM));
     attr.set();
   }
-  const int tiles_m = (a0.M + TC_BM - 1) / TC_BM, tiles_n = (a0.N + TC_BN - 1) / TC_BN;
+  const int tiles_m = (a0.M + TC_BM - 1) / TC_BM, tiles_n = (a0.N + BN - 1) / BN;
   CUtensorMap ma, mb;
   auto dense = [&](SliceLayout l, int64_t rows) {
     if (l.rows == 0) l.rows = rows;
@@ -470,7 +545,7 @@ hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, 
   if (la.kext < a0.K || lb.kext < a0.K) return HSMA_ERR_INVALID_ARG;
   if (!make_slice_map(&ma, Ap, (uint64_t)la.kext, (uint64_t)la.rows, (uint64_t)sa, TC_BM, (uint64_t)la.ld,
                       (uint64_t)la.sst) ||
-      !make_slice_map(&mb, Bp, (uint64_t)lb.kext, (uint64_t)lb.rows, (uint64_t)sb, TC_BN, (uint64_t)lb.ld,
+      !make_slice_map(&mb, Bp, (uint64_t)lb.kext, (uint64_t)lb.rows, (uint64_t)sb, BN, (uint64_t)lb.ld,
                       (uint64_t)lb.sst))
     return HSMA_ERR_CUDA;
   TcArgs a = a0;
@@ -488,18 +563,25 @@ hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, 
   a.err = hsma_dev_error_ptr();
   if (a.err == nullptr) return HSMA_ERR_CUDA;
   if (a.limit_ns == 0) a.limit_ns = 4000000000ull;
-  static int nsm[64] = {0};
-  int dev = 0;
-  HSMA_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return HSMA_ERR_UNSUPPORTED;
-  if (nsm[dev] == 0) HSMA_CUDA_TRY(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
   const int ntiles = tiles_m * tiles_n;
   a.band = MODE == TC_OZ || a.K <= 2048 ? 16 : tiles_m;
-  const int grid = std::max(1, std::min(ntiles, nsm[dev]));
+  const int grid = std::max(1, std::min(ntiles, hsma_sm_count()));
   HsmaTraceScope ts(phase, st);
-  tc_gemm_kernel<MODE><<<grid, 32 * TC_WARPS, TC_SMEM, st>>>(ma, mb, a);
+  tc_gemm_kernel<MODE, BN><<<grid, tc_threads<MODE>(), TcTile<BN>::SMEM, st>>>(ma, mb, a);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
+}
+
+// Tile width: the one whose busiest CTA has the least to do, a tile of BN
+// columns counting BN plus TileCost (measured: a 128 x 256 tile costs 1.8 times
+// a 128 x 128 one).
+template <int MODE>
+hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, int sb, const TcArgs &a0,
+                      const char *phase, cudaStream_t st, SliceLayout la = {}, SliceLayout lb = {}) {
+  const int64_t tm = (a0.M + TC_BM - 1) / TC_BM, sms = hsma_sm_count();
+  auto cost = [&](int bn) { return (tm * ((a0.N + bn - 1) / bn) + sms - 1) / sms * (bn + 32); };
+  if (cost(128) < cost(256)) return tc_gemm_tiled<MODE, 128>(Ap, sa, Bp, sb, a0, phase, st, la, lb);
+  return tc_gemm_tiled<MODE, 256>(Ap, sa, Bp, sb, a0, phase, st, la, lb);
 }
 
 }  // namespace

@@ -47,18 +47,25 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 }
 
 // Wait for phase `parity` of an mbarrier, giving up after limit_ns
-// nanoseconds of wall time: then the error bit is set and false returned.
+// nanoseconds of wall time: then the error bit is set and false returned.  The
+// timer is read once per kWaitSpins polls only: its latency would be added to
+// every wait whose first poll fails.
+constexpr int kWaitSpins = 64;
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint64_t limit_ns,
                                                   unsigned int *err) {
-  if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
+  for (int k = 0; k < kWaitSpins; ++k)
+    if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
-  while (!mbar_try_wait(bar, parity)) {
+  for (;;) {
+#pragma unroll 1
+    for (int k = 0; k < kWaitSpins; ++k)
+      if (mbar_try_wait(bar, parity)) return true;
     if (global_timer_ns() - t0 > limit_ns) {
       atomicOr(err, HSMA_DEVERR_TIMEOUT);
       return false;
     }
   }
-  return true;
 }
 
 // 2-D tiled TMA load into shared memory, completing on an mbarrier.

@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
 // balanced by 2^-g_k, as out[l][row][k], rows' x Kp row-major per modulus (zero
 // beyond K').  One CTA per 32 source rows x 64 real columns: read as columns of
 // 32 rows, transposed through shared memory, written as pairs of consecutive k
-// (128 bytes per warp and modulus).  Tiles past the diagonal's 128-row tile,
+// (128 bytes per warp and modulus).  Tiles past the diagonal's 256-row tile,
 // which a triangular product does not read, are not written.
 template <bool CPLX>
 __global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restric
   __shared__ double sre[KT][33], sim[CPLX ? KT : 1][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 64, kc0 = k0 / W;
-  if (mode != 0 && k0 >= (W * i0 / TC_BM + 1) * TC_BM) return;
+  if (mode != 0 && k0 >= (W * i0 / TC_PM + 1) * TC_PM) return;
 #pragma unroll
   for (int q = 0; q < KT / 8; ++q) {
     double re, im;
@@ -915,8 +915,8 @@ constexpr int kEmuGemmMaxK = 1 << 14;      // hsma_gemm_f64_emulated
 constexpr int kOzResidualMaxM = 1 << 14;   // refinement residuals
 
 size_t oz_scratch_bytes(int64_t rows, int64_t cols) {
-  const int64_t tiles = ((rows + TC_BM - 1) / TC_BM) * ((cols + 127) / 128);
-  return 2 * (size_t)std::min<int64_t>(tiles, hsma_sm_count()) * kOzTileWords * sizeof(uint32_t);
+  const int64_t tiles = ((rows + TC_PM - 1) / TC_PM) * ((cols + 127) / 128);
+  return 2 * (size_t)std::min<int64_t>(2 * tiles, hsma_sm_count()) * kOzTileWords * sizeof(uint32_t);
 }
 
 // C (M x N, column-major FP64) = (beta0 ? C : 0) -/+ L X in emulated FP64,

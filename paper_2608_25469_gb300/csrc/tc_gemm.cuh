@@ -23,48 +23,92 @@ namespace {
 // tcgen05 BF16 x BF16 -> FP32 update:  C (M x N, column-major fp32) =
 // beta*C - A' B'^T with A' (M x K) and B' (N x K) row-major BF16 (K-major).
 // ---------------------------------------------------------------------------
-// K-block of a pipeline stage: 64 BF16 values (128-byte rows, 128-byte
-// swizzle, four 48 KB stages), or 32 (64-byte rows and swizzle, nine 24 KB
-// stages: more bytes in flight behind the stage being multiplied).  Measured
-// on GB300 the 32-wide ring is 20-25% slower on every product (emulated FP64
-// 16384^2 solve 209 -> 258 ms, FP32-result 8192 x 4096 update 1.10 -> 1.20 ms),
-// so the products are not bound by how many bytes the ring keeps in flight.
-#ifndef HSMA_TC_BK
-#define HSMA_TC_BK 64
-#endif
-constexpr int TC_BM = 128, TC_BK = HSMA_TC_BK;
-constexpr int TC_ROW_BYTES = TC_BK * 2;  // one K-row of a stage tile: the swizzle width
-static_assert(TC_ROW_BYTES == 64 || TC_ROW_BYTES == 128, "K-blocks of 32 or 64 BF16 values");
+constexpr int TC_BM = 128;             // rows of a tile per CTA
+constexpr int TC_PM = 2 * TC_BM;       // rows of a tile (a pair of CTAs)
+constexpr int TC_BK = 64;              // K-block of a pipeline stage: 128-byte rows, 128-byte swizzle
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;
 constexpr uint32_t TC_TMEM_COLS = 512;  // all of the SM's tensor memory (one CTA per SM)
 
-// Tile of 128 x BN results: BN = 256 reads the fewest operand bytes per product,
-// BN = 128 gives twice the tiles when a launch has too few for the SMs.
+// A pair of CTAs (a cluster on two SMs) forms 256 x BN results with one
+// cta_group::2 MMA stream: each CTA stages its 128 rows of A and half of B's
+// rows, and holds its 128 rows of the accumulators.  With one CTA per tile
+// (128 x 256) every K-block moved 48 KB into an SM's shared memory and 48 KB out
+// of it to the tensor core, 768 cycles at 128 bytes per cycle against the 512
+// its products take (712 measured); a pair moves 32 KB each way.
+// BN = 256 does the most products per operand byte, BN = 128 gives twice the
+// tiles when a launch has too few for the SMs.
 template <int BN>
 struct TcTile {
-  static constexpr int B_BYTES = BN * TC_BK * 2;
-  static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
-  static constexpr int STAGES = (BN == 256 ? 4 : 6) * (64 / TC_BK);
+  static constexpr int B_ROWS = BN / 2;  // rows of B staged per CTA
+  static constexpr int STAGE_BYTES = TC_A_BYTES + B_ROWS * TC_BK * 2;
+  static constexpr int STAGES = BN == 256 ? 6 : 8;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
   static constexpr int ACCS = TC_TMEM_COLS / BN;  // accumulators in tensor memory
   // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M x N
   static constexpr uint32_t IDESC =
-      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
-  static_assert(SMEM <= 227 * 1024 - 256, "stages fit the shared memory of one CTA");
+      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_PM >> 4) << 24);
+  static_assert(SMEM <= 227 * 1024 - 512, "stages fit the shared memory of one CTA");
   static_assert(STAGE_BYTES % 1024 == 0, "every stage starts on a swizzle-pattern boundary");
 };
 
-// Shared-memory matrix descriptor: K-major operand, rows of TC_ROW_BYTES in
-// groups of 8 (8 * TC_ROW_BYTES apart), swizzled over the row width
-// (layout codes: 2 = 128-byte, 4 = 64-byte swizzle).
+// Shared-memory matrix descriptor: K-major operand, rows of 128 bytes in groups
+// of 8 (1024 bytes apart), 128-byte swizzle.
 __device__ __forceinline__ uint64_t sw_desc(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1u << 16;                                // leading-dimension offset (unused when swizzled)
-  d |= (uint64_t)((8u * TC_ROW_BYTES) >> 4) << 32;        // stride between 8-row groups
-  d |= (uint64_t)1u << 46;                                // descriptor version
-  d |= (uint64_t)(TC_ROW_BYTES == 128 ? 2u : 4u) << 61;   // swizzle mode
+  d |= (uint64_t)1u << 16;            // leading-dimension offset (unused when swizzled)
+  d |= (uint64_t)(1024u >> 4) << 32;  // stride between 8-row groups
+  d |= (uint64_t)1u << 46;            // descriptor version
+  d |= (uint64_t)2u << 61;            // swizzle mode
   return d;
+}
+
+// Address, in the cluster's shared memory, of the same variable in CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// true in one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// every thread of both CTAs
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// arrive on an mbarrier of either CTA of the pair (address from cluster_addr)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+// arrive on the mbarrier at this offset in both CTAs once the pair's MMAs issued so far are done
+__device__ __forceinline__ void tc_commit_pair(uint64_t *bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
+// TMA load into this CTA's shared memory, completing on an mbarrier of the pair
+__device__ __forceinline__ void tma_load_3d_pair(void *dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
+      "%5}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z)
+      : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -89,7 +133,7 @@ struct TcArgs {
   const int *cexp;  // TC_OZ: column exponents of B
   uint32_t *scratch;  // TC_OZ: kOzTileWords words per CTA (residue bytes of its current tile)
   int M, N, K;
-  int tri;          // row tile i0 needs k < i0 + TC_BM only
+  int tri;          // row tile i0 needs k < i0 + TC_PM only
   int npairs;       // TC_F32: slice pairs summed in the accumulator
   int band;         // tile rows per band of the tile order (set by the launcher)
   uint8_t pa[kTcMaxPairs], pb[kTcMaxPairs];  // TC_F32: slice of A and of B for each pair
@@ -191,9 +235,13 @@ __device__ __forceinline__ void oz_convert(const TcArgs &p, int cid, int h, int 
 // and for TC_OZ one per modulus and K chunk of kOzChunk (the longest whose FP32
 // sums of residue products stay exact).  The accumulators (512 tensor-memory
 // columns) rotate between units, so one unit's epilogue runs while the next
-// units' products accumulate.  Tiles are dealt round-robin to the CTAs (one per
-// SM).  Operands are 3-D: (K, rows, slice).  Every CTA loads its own A and B
-// tiles with plain (single-CTA) TMA.
+// units' products accumulate.  Tiles are dealt round-robin to the pairs of CTAs
+// (one CTA per SM).  Operands are 3-D: (K, rows, slice).
+//
+// In a pair, both producers fill their own stage and signal the first CTA's
+// `full`; its MMA thread issues for both; its commits release the stage and hand
+// over the accumulator in both CTAs; both CTAs' epilogue warps return the
+// accumulator to the first CTA's acc_empty.  Everything else is per CTA.
 constexpr int TC_WARPS = 10;
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TC_CRT_WARPS = 8;
@@ -204,7 +252,7 @@ constexpr int tc_threads() {
 }
 
 template <int MODE, int BN>
-__global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
                                                                         const __grid_constant__ CUtensorMap mapB,
                                                                         const __grid_constant__ TcArgs p) {
   using TL = TcTile<BN>;
@@ -223,12 +271,13 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = p.M, N = p.N;
   const int nslices = MODE == TC_OZ ? kOzP : p.npairs;  // passes over the K range per tile
-  const int cid = blockIdx.x, ncl = gridDim.x;
-  const int tiles_m = (M + TC_BM - 1) / TC_BM, tiles_n = (N + TC_BN - 1) / TC_BN;
+  const uint32_t rank = cluster_rank();
+  const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;  // the pair and the number of pairs
+  const int tiles_m = (M + TC_PM - 1) / TC_PM, tiles_n = (N + TC_BN - 1) / TC_BN;
   const int ntiles = tiles_m * tiles_n;
   // Tiles run in bands of p.band tile rows, column by column inside a band.
-  // With 16 tile rows the tiles in flight at once (one per SM) cover about 16
-  // row tiles x 10 column tiles, the fewest operand rows; long TC_F32 products
+  // With 8 tile rows the tiles in flight at once (one per pair of SMs) cover
+  // about 8 row tiles x 10 column tiles, the fewest operand rows; long TC_F32 products
   // take one band over all rows (column-major order), so the right operand is
   // shared by every row tile in flight.
   const int G = max(1, p.band);
@@ -237,9 +286,9 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
     const int gb = min(G, tiles_m - band * G);
     const int idx = t - band * G * tiles_n;
     const int pm = band * G + idx % gb;
-    m0 = pm * TC_BM;
+    m0 = pm * TC_PM + (int)rank * TC_BM;  // this CTA's rows
     n0 = (idx / gb) * TC_BN;
-    const int kall = p.tri ? min(p.K, (pm + 1) * TC_BM) : p.K;
+    const int kall = p.tri ? min(p.K, (pm + 1) * TC_PM) : p.K;
     return (kall + TC_BK - 1) / TC_BK;
   };
 
@@ -250,7 +299,7 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
     }
     for (int b = 0; b < NACC; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], TC_EPI_WARPS);
+      mbar_init(&acc_empty[b], 2 * TC_EPI_WARPS);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&res_full[b], TC_EPI_WARPS);
@@ -260,98 +309,110 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
     fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                  "r"(TC_TMEM_COLS)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers are initialised and tensor memory allocated
   tc_fence_after();
   const uint32_t tmem = tmem_base;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // producer: TMA loads into a ring of stages, across items
-      int it = 0;
-      bool ok = true;
-      for (int t = cid; t < ntiles && ok; t += ncl) {
-        int m0, n0;
-        const int nk = tile_k(t, m0, n0);
-        for (int q = 0; q < nslices && ok; ++q) {
-          const int sa = MODE == TC_OZ ? q : p.pa[q], sb = MODE == TC_OZ ? q : p.pb[q];
-          for (int kb = 0; kb < nk; ++kb, ++it) {
-            const int s = it % TC_STAGES;
-            if (it >= TC_STAGES && !mbar_wait_bounded(&empty[s], ((it / TC_STAGES) - 1) & 1, p.limit_ns, p.err)) {
-              ok = false;
-              break;
-            }
+    // producer: TMA loads into a ring of stages, across tiles.  The whole warp
+    // runs the loop and one elected lane issues (here and below): as a branch of
+    // a single lane the MMA loop took 800 cycles per K block whatever the tile,
+    // this form 540 (BN = 128) to 560 (BN = 256, 512 of them products).
+    const uint32_t bar0 = cluster_addr(&full[0], 0);
+    int s = 0;
+    uint32_t phase = 1;  // the first round finds every stage empty
+    bool ok = true;
+    for (int t = cid; t < ntiles && ok; t += ncl) {
+      int m0, n0;
+      const int nk = tile_k(t, m0, n0);
+      for (int q = 0; q < nslices && ok; ++q) {
+        const int sa = MODE == TC_OZ ? q : p.pa[q], sb = MODE == TC_OZ ? q : p.pb[q];
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!mbar_wait_bounded(&empty[s], phase, p.limit_ns, p.err)) {
+            ok = false;
+            break;
+          }
+          if (elect_one()) {
             unsigned char *st = smem + s * TC_STAGE_BYTES;
-            mbar_arrive_expect_tx(&full[s], TC_STAGE_BYTES);
-            tma_load_3d(st, &mapA, &full[s], kb * TC_BK, m0, sa);
-            tma_load_3d(st + TC_A_BYTES, &mapB, &full[s], kb * TC_BK, n0, sb);
+            const uint32_t bar = bar0 + (uint32_t)s * 8u;
+            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * TC_STAGE_BYTES);
+            tma_load_3d_pair(st, &mapA, bar, kb * TC_BK, m0, sa);
+            tma_load_3d_pair(st + TC_A_BYTES, &mapB, bar, kb * TC_BK, n0 + (int)rank * TL::B_ROWS, sb);
+          }
+          __syncwarp();
+          if (++s == TC_STAGES) {
+            s = 0;
+            phase ^= 1;
           }
         }
       }
     }
-    __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer: per item, wait for a drained accumulator, then four K = 16
-      // steps per stage; each stage is released by a commit, the item by another
-      int it = 0, i = 0;
+    if (rank == 0) {
+      // MMA issuer (first CTA of the pair): per unit, wait for a drained
+      // accumulator, then four K = 16 steps per stage; each stage is released by
+      // a commit, the unit by another
+      const uint64_t desc0 = sw_desc(smem_u32(smem));
+      int s = 0, b = 0;
+      uint32_t phase = 0, acc_phase = 1;  // the first round finds every accumulator drained
       bool ok = true;
       for (int t = cid; t < ntiles && ok; t += ncl) {
         int m0, n0;
         const int nk = tile_k(t, m0, n0);
         const int total = nslices * nk;  // K blocks of the tile, slice by slice
-        for (int g0 = 0; g0 < total && ok; ++i) {
+        for (int g0 = 0; g0 < total && ok;) {
           // the unit's K blocks: all of them, or (TC_OZ) the next chunk of this modulus
           const int glen = MODE == TC_OZ ? min(kOzChunk / TC_BK, nk - g0 % nk) : total;
-          const int b = i % NACC;
-          if (i >= NACC && !mbar_wait_bounded(&acc_empty[b], (i / NACC - 1) & 1, p.limit_ns, p.err)) {
+          if (!mbar_wait_bounded(&acc_empty[b], acc_phase, p.limit_ns, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t acc_cols = tmem + (uint32_t)(b * BN);
-          uint32_t accum = 0;
-          for (int kb = 0; kb < glen; ++kb, ++it) {
-            const int s = it % TC_STAGES;
-            if (!mbar_wait_bounded(&full[s], (it / TC_STAGES) & 1, p.limit_ns, p.err)) {
+          for (int kb = 0; kb < glen; ++kb) {
+            if (!mbar_wait_bounded(&full[s], phase, p.limit_ns, p.err)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t sa = smem_u32(smem + s * TC_STAGE_BYTES);
-            const uint64_t da = sw_desc(sa), db = sw_desc(sa + TC_A_BYTES);
+            if (elect_one()) {
+              const uint64_t da = desc0 + (uint64_t)(s * (TC_STAGE_BYTES >> 4)), db = da + (TC_A_BYTES >> 4);
 #pragma unroll
-            for (int kk = 0; kk < TC_BK / 16; ++kk) {
-              asm volatile(
-                  "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
-                  "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(TL::IDESC), "r"(accum)
-                  : "memory");
-              accum = 1u;
+              for (int kk = 0; kk < TC_BK / 16; ++kk)
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                    "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
+                    "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(TL::IDESC), "r"(kb + kk)
+                    : "memory");
+              tc_commit_pair(&empty[s]);
+              if (kb == glen - 1) tc_commit_pair(&acc_full[b]);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&empty[s]))
-                         : "memory");
+            __syncwarp();
+            if (++s == TC_STAGES) {
+              s = 0;
+              phase ^= 1;
+            }
           }
           g0 += glen;
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(&acc_full[b]))
-                       : "memory");
+          if (++b == NACC) {
+            b = 0;
+            acc_phase ^= 1;
+          }
         }
       }
       // every issued product has finished before tensor memory is released,
       // also when a wait above gave up
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(&drained))
-                   : "memory");
+      if (elect_one()) tc_commit_pair(&drained);
+      __syncwarp();
       mbar_wait_bounded(&drained, 0, p.limit_ns, p.err);
     }
-    __syncwarp();
   } else if (warp < TC_WARPS) {
     // epilogue warps: thread = one row of the 128-row tile (its tensor-memory
     // lane); two warps per lane quarter split the columns.
@@ -374,7 +435,7 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
           ok = __all_sync(0xffffffffu, mbar_wait_bounded(&res_empty[h], ((ti >> 1) - 1) & 1, p.limit_ns, p.err));
           if (!ok) break;
         }
-        uint32_t *mine = p.scratch + oz_scratch_at(cid, h, cbeg) + quarter * 32 + lane;
+        uint32_t *mine = p.scratch + oz_scratch_at(blockIdx.x, h, cbeg) + quarter * 32 + lane;
         const int cols = min(TC_BN / 2, N - n0 - cbeg);  // this warp's columns inside the matrix
         for (int l = 0; l < kOzP && ok; ++l) {
           const float mod = c_oz.modf[l], inv = c_oz.inv[l];
@@ -400,12 +461,12 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[b]);  // this warp is done with accumulator b
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0));  // this warp is done with accumulator b
           }
         }
         if (!ok) break;
         if (lane == 0) mbar_arrive(&res_full[h]);  // (after the last unit's __syncwarp)
-        if (t + ncl >= ntiles) oz_convert<BN>(p, cid, h, m0, n0, quarter, cbeg + TC_BN / 4, TC_BN / 4);
+        if (t + ncl >= ntiles) oz_convert<BN>(p, blockIdx.x, h, m0, n0, quarter, cbeg + TC_BN / 4, TC_BN / 4);
       } else {
         // the old values of the next 16-column chunk are loaded before this chunk's stores
         const int b = i % NACC;
@@ -463,7 +524,7 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
         // this warp is done with accumulator b
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
+        if (lane == 0) mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0));
       }
     }
   } else if constexpr (MODE == TC_OZ) {
@@ -478,16 +539,17 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) tc_gemm_kernel(const __
       const int h = ti & 1;
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&res_full[h], (ti >> 1) & 1, p.limit_ns, p.err))) break;
       // the CTA's last tile is shared with the epilogue warps, which are done
-      oz_convert<BN>(p, cid, h, m0, n0, cw & 3, (cw >> 2) * (TC_BN / 2), t + ncl >= ntiles ? TC_BN / 4 : TC_BN / 2);
+      oz_convert<BN>(p, blockIdx.x, h, m0, n0, cw & 3, (cw >> 2) * (TC_BN / 2), t + ncl >= ntiles ? TC_BN / 4 : TC_BN / 2);
       __syncwarp();
       if (lane == 0) mbar_arrive(&res_empty[h]);
     }
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // no arrival or product of the other CTA is outstanding
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
                  : "memory");
   }
 }
@@ -504,7 +566,7 @@ bool make_slice_map(CUtensorMap *map, const void *base, uint64_t K, uint64_t row
   const cuuint32_t box[3] = {(cuuint32_t)TC_BK, box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, TC_ROW_BYTES == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -531,7 +593,7 @@ hsma_status_t tc_gemm_tiled(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16
         cudaFuncSetAttribute(tc_gemm_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<BN>::SMEM));
     attr.set();
   }
-  const int tiles_m = (a0.M + TC_BM - 1) / TC_BM, tiles_n = (a0.N + BN - 1) / BN;
+  const int tiles_m = (a0.M + TC_PM - 1) / TC_PM, tiles_n = (a0.N + BN - 1) / BN;
   CUtensorMap ma, mb;
   auto dense = [&](SliceLayout l, int64_t rows) {
     if (l.rows == 0) l.rows = rows;
@@ -545,7 +607,7 @@ hsma_status_t tc_gemm_tiled(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16
   if (la.kext < a0.K || lb.kext < a0.K) return HSMA_ERR_INVALID_ARG;
   if (!make_slice_map(&ma, Ap, (uint64_t)la.kext, (uint64_t)la.rows, (uint64_t)sa, TC_BM, (uint64_t)la.ld,
                       (uint64_t)la.sst) ||
-      !make_slice_map(&mb, Bp, (uint64_t)lb.kext, (uint64_t)lb.rows, (uint64_t)sb, BN, (uint64_t)lb.ld,
+      !make_slice_map(&mb, Bp, (uint64_t)lb.kext, (uint64_t)lb.rows, (uint64_t)sb, TcTile<BN>::B_ROWS, (uint64_t)lb.ld,
                       (uint64_t)lb.sst))
     return HSMA_ERR_CUDA;
   TcArgs a = a0;
@@ -564,22 +626,22 @@ hsma_status_t tc_gemm_tiled(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16
   if (a.err == nullptr) return HSMA_ERR_CUDA;
   if (a.limit_ns == 0) a.limit_ns = 4000000000ull;
   const int ntiles = tiles_m * tiles_n;
-  a.band = MODE == TC_OZ || a.K <= 2048 ? 16 : tiles_m;
-  const int grid = std::max(1, std::min(ntiles, hsma_sm_count()));
+  a.band = MODE == TC_OZ || a.K <= 2048 ? 8 : tiles_m;
+  const int grid = 2 * std::max(1, std::min(ntiles, hsma_sm_count() / 2));
   HsmaTraceScope ts(phase, st);
   tc_gemm_kernel<MODE, BN><<<grid, tc_threads<MODE>(), TcTile<BN>::SMEM, st>>>(ma, mb, a);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
 }
 
-// Tile width: the one whose busiest CTA has the least to do, a tile of BN
-// columns counting BN plus TileCost (measured: a 128 x 256 tile costs 1.8 times
-// a 128 x 128 one).
+// Tile width: the one whose busiest pair of CTAs has the least to do, a tile of
+// BN columns counting BN + 96 (a 256 x 128 tile takes about 0.64 of the time of
+// a 256 x 256 one).
 template <int MODE>
 hsma_status_t tc_gemm(const __nv_bfloat16 *Ap, int sa, const __nv_bfloat16 *Bp, int sb, const TcArgs &a0,
                       const char *phase, cudaStream_t st, SliceLayout la = {}, SliceLayout lb = {}) {
-  const int64_t tm = (a0.M + TC_BM - 1) / TC_BM, sms = hsma_sm_count();
-  auto cost = [&](int bn) { return (tm * ((a0.N + bn - 1) / bn) + sms - 1) / sms * (bn + 32); };
+  const int64_t tm = (a0.M + TC_PM - 1) / TC_PM, pairs = hsma_sm_count() / 2;
+  auto cost = [&](int bn) { return (tm * ((a0.N + bn - 1) / bn) + pairs - 1) / pairs * (bn + 96); };
   if (cost(128) < cost(256)) return tc_gemm_tiled<MODE, 128>(Ap, sa, Bp, sb, a0, phase, st, la, lb);
   return tc_gemm_tiled<MODE, 256>(Ap, sa, Bp, sb, a0, phase, st, la, lb);
 }

@@ -1,13 +1,15 @@
 // Large-case blocked solve (Section 4.3), fp64 and complex128.
 //
 // Phase 1 (Section 4.3, "parallel diagonal block inversion"): the N_B x N_B
-// diagonal blocks D_t are inverted independently, all in one launch.  Each CTA
-// produces a group of columns of D_t^{-1} by forward substitution against the
-// identity (Section 4.3.1): the columns of D_t are streamed through a two-slot
-// shared-memory buffer (Algorithm 2's double buffering: column k+1 is staged
-// while column k is used), so shared memory is O(N_B).  The columns of the
-// inverse live in registers: lane group g of a warp holds rows g, g+G, ...,
-// and the register window slides down by one slot every G steps.
+// diagonal blocks D_t are inverted independently: FP64 by doubling
+// (fp64_inverse.cu); the FP32 modes' base blocks (N_B = 32 or 64) by the column
+// substitution below, in one launch.  Each CTA produces a group of columns of
+// D_t^{-1} by forward substitution against the identity (Section 4.3.1): the
+// columns of D_t are streamed through a two-slot shared-memory buffer
+// (Algorithm 2's double buffering: column k+1 is staged while column k is
+// used), so shared memory is O(N_B).  The columns of the inverse live in
+// registers: lane group g of a warp holds rows g, g+G, ..., and the register
+// window slides down by one slot every G steps.
 //
 // Phase 2 (Section 4.3, "sequential GEMM update and solve"), for r = 0..k:
 //   X_r = D_r^{-1} B_r                       (solve product, triangular)
@@ -38,7 +40,7 @@ __device__ unsigned int g_hsma_dev_error = 0;
 namespace {
 
 // ---------------------------------------------------------------------------
-// Phase 1: diagonal-block inversion
+// Phase 1: diagonal-block inversion by substitution (FP32 base blocks)
 // ---------------------------------------------------------------------------
 constexpr int kInvSlots = 32;  // register slots per lane: N_B = 32 * G
 
@@ -538,28 +540,16 @@ hsma_status_t gemm(const GemmArgs<T> &p, const char *phase, cudaStream_t st, T *
   return gemm_tiled<T, TileWide>(p, phase, st, P, P_elems);
 }
 
-template <class T, int G>
-hsma_status_t launch_inverse_g(const T *A, int64_t lda, int64_t m, int unit, T *Dinv, cudaStream_t st) {
+template <int G>
+hsma_status_t launch_inverse_f32(const float *A, int64_t lda, int64_t m, int unit, float *Dinv, cudaStream_t st) {
   constexpr int NB = 32 * G, C = 32 / G;
   const int warps = std::min(8, NB / C);
   const int CT = warps * C;
   dim3 grid((unsigned)((m + NB - 1) / NB), (unsigned)(NB / CT));
   HsmaTraceScope ts("diag_inverse", st);
-  diag_inverse_kernel<T, G><<<grid, warps * 32, 0, st>>>(A, lda, m, unit, Dinv);
+  diag_inverse_kernel<float, G><<<grid, warps * 32, 0, st>>>(A, lda, m, unit, Dinv);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
-}
-
-template <class T>
-hsma_status_t launch_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, cudaStream_t st) {
-  switch (nb) {
-    case 32: return launch_inverse_g<T, 1>(A, lda, m, unit, Dinv, st);
-    case 64: return launch_inverse_g<T, 2>(A, lda, m, unit, Dinv, st);
-    case 128: return launch_inverse_g<T, 4>(A, lda, m, unit, Dinv, st);
-    case 256: return launch_inverse_g<T, 8>(A, lda, m, unit, Dinv, st);
-    case 512: return launch_inverse_g<T, 16>(A, lda, m, unit, Dinv, st);
-    default: return HSMA_ERR_UNSUPPORTED;
-  }
 }
 
 template <class T>
@@ -595,12 +585,14 @@ hsma_status_t blocked_impl(const HsmaBlockedCfg &cfg, const T *A, int64_t lda, T
   // partial products of split-K launches (only when n is small, unless split K is off)
   const size_t p_elems =
       cfg.split_k != HSMA_SPLITK_OFF && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
-  hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems, st);
+  const size_t inv_bytes = hsma_fp64_inverse_scratch(nb, m, sizeof(T));
+  hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems + inv_bytes, st);
   if (s != HSMA_OK) return s;
   T *Dinv = static_cast<T *>(ws);
+  T *Winv = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes + w_bytes + sizeof(T) * p_elems);
   T *W = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes);
   T *Pw = p_elems ? reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes + w_bytes) : nullptr;
-  s = launch_inverse<T>(nb, A, lda, m, unit, Dinv, st);
+  s = hsma_fp64_diag_inverse<T>(nb, A, lda, m, unit, Dinv, Winv, st);
   // W holds the current block row's right-hand side: copied from B for the
   // first block, written by the previous trailing update for the others, so
   // the solve product can write X_r straight into B_r.
@@ -695,16 +687,12 @@ unsigned int *hsma_dev_error_ptr() {
   return ptr[d];
 }
 
-hsma_status_t hsma_diag_inverse(int dtype, int nb, const void *A, int64_t lda, int64_t m, int unit, void *Dinv,
-                                cudaStream_t st) {
-  switch (dtype) {
-    case HSMA_C128:
-      return launch_inverse<cplx>(nb, static_cast<const cplx *>(A), lda, m, unit, static_cast<cplx *>(Dinv), st);
-    case HSMA_R32_BF16:
-      return launch_inverse<float>(nb, static_cast<const float *>(A), lda, m, unit, static_cast<float *>(Dinv), st);
-    default:
-      return launch_inverse<double>(nb, static_cast<const double *>(A), lda, m, unit, static_cast<double *>(Dinv),
-                                    st);
+hsma_status_t hsma_f32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
+                                    cudaStream_t st) {
+  switch (nb) {
+    case 32: return launch_inverse_f32<1>(A, lda, m, unit, Dinv, st);
+    case 64: return launch_inverse_f32<2>(A, lda, m, unit, Dinv, st);
+    default: return HSMA_ERR_UNSUPPORTED;
   }
 }
 

@@ -20,12 +20,18 @@ struct HsmaBlockedCfg {
 hsma_status_t hsma_blocked_solve(int dtype, const HsmaBlockedCfg &cfg, const void *A, int64_t lda, void *B,
                                  int64_t ldb, int64_t m, int64_t n, const double *alpha, int unit, cudaStream_t st);
 
-// Phase 1 alone: invert the N_B x N_B diagonal blocks of the lower triangle of
-// A (dtype HSMA_R64, HSMA_C128 or HSMA_R32_BF16 for float data) into Dinv
-// (ceil(m/nb) blocks of nb x nb, column-major, ld nb, zeros above the diagonal
-// and outside a partial last block).  nb in {32, 64, 128, 256, 512}.
-hsma_status_t hsma_diag_inverse(int dtype, int nb, const void *A, int64_t lda, int64_t m, int unit, void *Dinv,
-                                cudaStream_t st);
+// Phase 1 alone, FP64 (T = double, cplx): invert the N_B x N_B diagonal blocks of
+// the lower triangle of A into Dinv (ceil(m/nb) blocks of nb x nb, column-major,
+// ld nb, zeros above the diagonal and outside a partial last block).  nb in
+// {32, 64, 128, 256, 512}; W: hsma_fp64_inverse_scratch bytes of workspace.
+size_t hsma_fp64_inverse_scratch(int nb, int64_t m, size_t esize);
+template <class T>
+hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, T *W,
+                                     cudaStream_t st);
+
+// The same for float data by column substitution, nb in {32, 64}.
+hsma_status_t hsma_f32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
+                                    cudaStream_t st);
 
 // FP64 product used by the refinement residual: C = beta*C - L*X with L the
 // lower triangle of A (unit diagonal if unit), all column-major fp64 (m x m,

@@ -1,0 +1,126 @@
+// FP64 products on the tensor path (mma.sync m8n8k4 .f64, "DMMA") in small
+// output tiles, operands straight from global memory.
+//
+// A DMMA occupies its sub-partition's FP64 pipe for about 512 cycles on this
+// GPU, so operand traffic is negligible (an 8 x 8 tile reads 512 bytes per
+// DMMA, 1.2 TB/s over all SMs from the caches) and what counts is that every
+// sub-partition has DMMAs to do.  A CTA's four warps, one per sub-partition,
+// share one output tile and take every fourth K step; their sums are added in
+// shared memory in a fixed order.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "common.cuh"
+
+namespace {
+
+__device__ __forceinline__ void fp64_dmma(double (&d)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
+               : "+d"(d[0]), "+d"(d[1])
+               : "d"(a), "d"(b));
+}
+
+template <class T>
+struct Fp64Acc;
+template <>
+struct Fp64Acc<double> {
+  double v[2];
+  __device__ __forceinline__ void zero() { v[0] = v[1] = 0.0; }
+  __device__ __forceinline__ void mma(double a, double b) { fp64_dmma(v, a, b); }
+  __device__ __forceinline__ double get(int q) const { return v[q]; }
+};
+template <>
+struct Fp64Acc<cplx> {
+  double re[2], im[2];
+  __device__ __forceinline__ void zero() { re[0] = re[1] = im[0] = im[1] = 0.0; }
+  __device__ __forceinline__ void mma(cplx a, cplx b) {
+    fp64_dmma(re, a.re, b.re);
+    fp64_dmma(im, a.re, b.im);
+    fp64_dmma(re, -a.im, b.im);
+    fp64_dmma(im, a.im, b.re);
+  }
+  __device__ __forceinline__ cplx get(int q) const { return cplx{re[q], im[q]}; }
+};
+
+__device__ __forceinline__ double fp64_add(double a, double b) { return a + b; }
+__device__ __forceinline__ cplx fp64_add(cplx a, cplx b) { return cplx{a.re + b.re, a.im + b.im}; }
+
+__device__ __forceinline__ double fp64_neg(double a) { return -a; }
+__device__ __forceinline__ cplx fp64_neg(cplx a) { return cplx{-a.re, -a.im}; }
+
+constexpr int kFp64Warps = 4;
+
+// Rows m0 .. m0 + 8 WM - 1 and columns n0 .. n0 + 8 WN - 1 of A B over
+// k = kbeg .. kend - 1 (A: M x kend column-major, B: kend x N column-major;
+// entries outside read as zero).  All 128 threads take part; the tile is left in
+// red[0] (column-major, 8 WM rows) after a CTA barrier.
+template <class T, int WM, int WN>
+__device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, int64_t ldb,
+                                          int M, int N, int kbeg, int kend, int m0, int n0,
+                                          T (*red)[8 * WM * 8 * WN]) {
+  using E = Elem<T>;
+  constexpr int U = WM * WN >= 16 ? 2 : 4;  // K steps per load group; one group is in flight while another is multiplied
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  Fp64Acc<T> acc[WM][WN];
+#pragma unroll
+  for (int i = 0; i < WM; ++i)
+#pragma unroll
+    for (int j = 0; j < WN; ++j) acc[i][j].zero();
+  T a[2][U][WM], b[2][U][WN];
+  auto load = [&](int k0, int s) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = k0 + 4 * kFp64Warps * u + t;
+#pragma unroll
+      for (int i = 0; i < WM; ++i) {
+        const int r = m0 + 8 * i + g;
+        a[s][u][i] = (k < kend && r < M) ? E::ld(A + r + (int64_t)k * lda) : E::zero();
+      }
+#pragma unroll
+      for (int j = 0; j < WN; ++j) {
+        const int c = n0 + 8 * j + g;
+        b[s][u][j] = (k < kend && c < N) ? E::ld(B + k + (int64_t)c * ldb) : E::zero();
+      }
+    }
+  };
+  auto mul = [&](int k0, int s) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k0 + 4 * kFp64Warps * u >= kend) break;  // warp-uniform
+#pragma unroll
+      for (int i = 0; i < WM; ++i)
+#pragma unroll
+        for (int j = 0; j < WN; ++j) acc[i][j].mma(a[s][u][i], b[s][u][j]);
+    }
+  };
+  constexpr int kGroup = 4 * kFp64Warps * U;
+  int k0 = kbeg + 4 * warp;
+  load(k0, 0);
+  while (k0 < kend) {
+    load(k0 + kGroup, 1);
+    mul(k0, 0);
+    k0 += kGroup;
+    if (k0 >= kend) break;
+    load(k0 + kGroup, 0);
+    mul(k0, 1);
+    k0 += kGroup;
+  }
+#pragma unroll
+  for (int i = 0; i < WM; ++i)
+#pragma unroll
+    for (int j = 0; j < WN; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) red[warp][(8 * i + g) + (8 * j + 2 * t + q) * 8 * WM] = acc[i][j].get(q);
+  __syncthreads();
+  for (int e = threadIdx.x; e < 8 * WM * 8 * WN; e += 32 * kFp64Warps) {
+    T v = red[0][e];
+#pragma unroll
+    for (int w = 1; w < kFp64Warps; ++w) v = fp64_add(v, red[w][e]);
+    red[0][e] = v;
+  }
+  __syncthreads();
+}
+
+}  // namespace

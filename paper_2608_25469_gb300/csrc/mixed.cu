@@ -1005,8 +1005,8 @@ __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, do
 struct EmuLayout {
   int W = 1, h = 1, Kpb = 0, Kpp = 0;
   int64_t P = 0;
-  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0, sc_b = 0;
-  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b + sc_b; }
+  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0, sc_b = 0, iv_b = 0;
+  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b + sc_b + iv_b; }
 };
 
 EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
@@ -1025,13 +1025,14 @@ EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
   L.pd_b = al(oz_operand_bytes((int64_t)L.W * nb, L.Kpb));
   L.px_b = al(oz_operand_bytes(n, L.Kpp));
   L.sc_b = al(oz_scratch_bytes(L.W * m, n));
+  L.iv_b = hsma_fp64_inverse_scratch(nb, m, eb);
   return L;
 }
 
-hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *A, int64_t lda, double *B,
+hsma_status_t blocked_emulated(bool cplx_, int nb, int panel_cols, const double *A, int64_t lda, double *B,
                                int64_t ldb, int64_t m,
                                int64_t n, const double *alpha, int unit, cudaStream_t st) {
-  const EmuLayout E = emu_layout(cplx, nb, panel_cols, m, n);
+  const EmuLayout E = emu_layout(cplx_, nb, panel_cols, m, n);
   const int W = E.W;
   const int64_t P = E.P;
   const int Kpb = E.Kpb;
@@ -1060,17 +1061,21 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
     OzOperand Px = view(px_mem, n, Kp, n);
     {
       HsmaTraceScope ts("slices", st, 5);  // oz_slice_a: 4 kernels, oz_slice_x: 1
-      hsma_status_t e = oz_slice_a(cplx, A + W * (rb + c0 * lda), lda, (int)rows, k, 0, Pa, st);
+      hsma_status_t e = oz_slice_a(cplx_, A + W * (rb + c0 * lda), lda, (int)rows, k, 0, Pa, st);
       if (e == HSMA_OK) e = oz_slice_x(B + W * c0, (int64_t)W * ldb, W * k, Pa.kexp, Px, nullptr, st);
       if (e != HSMA_OK) return e;
     }
     return oz_product(Pa, Px, B + W * rb, (int64_t)W * ldb, 1, 0, 0, scratch, nullptr, phase, st);
   };
   do {
-    if ((s = hsma_diag_inverse(cplx ? HSMA_C128 : HSMA_R64, nb, A, lda, m, unit, Dinv, st)) != HSMA_OK) break;
-    if (alpha[0] != 1.0 || (cplx && alpha[1] != 0.0)) {
+    unsigned char *iv = px_mem + E.px_b + E.sc_b;
+    s = cplx_ ? hsma_fp64_diag_inverse<cplx>(nb, reinterpret_cast<const cplx *>(A), lda, m, unit,
+                                             reinterpret_cast<cplx *>(Dinv), reinterpret_cast<cplx *>(iv), st)
+              : hsma_fp64_diag_inverse<double>(nb, A, lda, m, unit, Dinv, reinterpret_cast<double *>(iv), st);
+    if (s != HSMA_OK) break;
+    if (alpha[0] != 1.0 || (cplx_ && alpha[1] != 0.0)) {
       HsmaTraceScope ts("copy", st);
-      scale_kernel<<<hsma_grid_rc(m, n), 256, 0, st>>>(B, ldb, m, n, alpha[0], cplx ? alpha[1] : 0.0, cplx);
+      scale_kernel<<<hsma_grid_rc(m, n), 256, 0, st>>>(B, ldb, m, n, alpha[0], cplx_ ? alpha[1] : 0.0, cplx_);
       if ((s = hsma_from_cuda(cudaGetLastError())) != HSMA_OK) break;
     }
     for (int64_t R0 = 0; R0 < m && s == HSMA_OK; R0 += P) {
@@ -1089,7 +1094,7 @@ hsma_status_t blocked_emulated(bool cplx, int nb, int panel_cols, const double *
         OzOperand Px = view(px_mem, n, Kpb, n);
         {
           HsmaTraceScope ts("slices", st, 5);
-          if ((s = oz_slice_a(cplx, Dinv + (size_t)W * r * nb * nb, nb, sr, sr, 1, Pd, st)) != HSMA_OK) break;
+          if ((s = oz_slice_a(cplx_, Dinv + (size_t)W * r * nb * nb, nb, sr, sr, 1, Pd, st)) != HSMA_OK) break;
           if ((s = oz_slice_x(Wb, (int64_t)W * nb, W * sr, Pd.kexp, Px, nullptr, st)) != HSMA_OK) break;
         }
         if ((s = oz_product(Pd, Px, B + W * r0, (int64_t)W * ldb, 0, 1, 1, scratch, nullptr, "solve_gemm",

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) inv_double_kernel(const float *__restrict
 hsma_status_t hsma_r32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
                                     cudaStream_t st) {
   if (nb < 2 * kInvBase || nb % (2 * kInvBase) != 0 || (nb & (nb - 1)) != 0)
-    return hsma_diag_inverse(HSMA_R32_BF16, nb, A, lda, m, unit, Dinv, st);
+    return hsma_f32_diag_inverse(nb, A, lda, m, unit, Dinv, st);
   const int64_t nblk = (m + nb - 1) / nb;
   const int64_t nbase = (m + kInvBase - 1) / kInvBase;
   auto al = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
@@ -138,7 +138,7 @@ hsma_status_t hsma_r32_diag_inverse(int nb, const float *A, int64_t lda, int64_t
   float *base = static_cast<float *>(ws);
   float *W = reinterpret_cast<float *>(static_cast<unsigned char *>(ws) + base_b);
   do {
-    if ((s = hsma_diag_inverse(HSMA_R32_BF16, kInvBase, A, lda, m, unit, base, st)) != HSMA_OK) break;
+    if ((s = hsma_f32_diag_inverse(kInvBase, A, lda, m, unit, base, st)) != HSMA_OK) break;
     int levels = 0;
     for (int h = kInvBase; h < nb; h *= 2) ++levels;
     HsmaTraceScope ts("diag_inverse", st, 1 + 2 * levels);

@@ -93,6 +93,19 @@ def test_planner_default_matches_oracle(H, code):
     assert oracle.backward_error(A, B, X, alpha) <= 1e-14
 
 
+@pytest.mark.parametrize("code", [I.R64, I.C128])
+@pytest.mark.parametrize("m,nb", [(33, 64), (4100, 512), (2050, 256), (2050, 64), (1055, 128)])
+def test_inverse_levels_parity(H, code, m, nb):
+    """Doubling levels of the diagonal inverses with every output tile size (by the number of
+    blocks) and partial pairs: a last block with no, one row of, or part of its second half."""
+    n = 3
+    A, B = I.gen_A(m, m, code), I.gen_B(m, m, n, code)
+    A[np.triu_indices(m, 1)] = np.nan
+    X = _run(H, code, A, B, 1.0, nb)
+    ref = oracle.solve(I.gen_A(m, m, code), B, 1.0)
+    assert oracle.forward_error(X, ref) <= TOL
+
+
 CFG_CASES = [(65, 7, 32), (300, 200, 128), (700, 50, 512), (1000, 9, 64), (513, 130, 256)]
 
 

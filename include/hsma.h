@@ -97,7 +97,8 @@ typedef enum { HSMA_PATH_AUTO = 0, HSMA_PATH_SMALL = 1, HSMA_PATH_BLOCKED = 2 } 
 #define HSMA_DEVERR_BAD_PIVOT 0x8u /* hsma_getrs_vbatched: a pivot outside [k+1, m]   */
 
 /* Blocked-path configuration values (hsma_opts_t / hsma_plan_t). */
-#define HSMA_TILE_64x64 1   /* FP64 tensor-product CTA tile, rows x columns of B */
+#define HSMA_TILE_64x64 1   /* FP64 tensor products with staged CTA tiles, rows x columns of B
+                               (0: small tiles of 8 to 32 rows, by the number of them) */
 #define HSMA_TILE_128x16 2
 #define HSMA_TILE_128x8 3
 #define HSMA_SPLITK_AUTO 1  /* split K across CTAs when the tiles leave SMs idle */
@@ -111,9 +112,8 @@ typedef struct {
   int32_t path;       /* hsma_path_t: SMALL (m <= 64) or BLOCKED                    */
   int32_t nb;         /* BLOCKED: diagonal block size (the paper's N_B)             */
   int32_t groups;     /* SMALL: row groups per warp G; a warp holds 32/G columns   */
-  int32_t tile;       /* BLOCKED FP64 products: HSMA_TILE_*, 0 = by n (128x8 for
-                         n <= 8, 128x16 for n <= 48, else 64x64)                  */
-  int32_t split_k;    /* BLOCKED: HSMA_SPLITK_*                                     */
+  int32_t tile;       /* BLOCKED FP64 products: HSMA_TILE_*, 0 = small tiles        */
+  int32_t split_k;    /* BLOCKED, HSMA_TILE_*: HSMA_SPLITK_*                        */
   int32_t looking;    /* BLOCKED: HSMA_LOOK_*                                       */
   int32_t panel_cols; /* emulated FP64 products: real columns per update panel     */
   int32_t reserved;

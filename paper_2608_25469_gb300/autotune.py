@@ -10,12 +10,11 @@ time).  At run time the planner picks the entry nearest to the input in
 
 Configuration space per dtype:
 
-* R64 / C128 with FP64 tensor products (DMMA): the diagonal block size N_B,
-  the product tile (64 x 64, 128 x 16, 128 x 8 rows x columns, or the rule by
-  n), split K (when the tiles leave SMs idle, or never) and the update
-  direction (right-looking, or the paper's left-looking form).  Searched in
-  stages: N_B with the default rest, then the tile, split K and direction one
-  at a time from the best so far (each stage keeps what it measured fastest).
+* R64 / C128 with FP64 tensor products (DMMA): the diagonal block size N_B
+  with each update direction (right-looking, or the paper's left-looking form),
+  products in small tiles (tile 0); then, from the fastest of these, the staged
+  tiles (64 x 64, 128 x 16, 128 x 8 rows x columns) and, for those, split K
+  (when the tiles leave SMs idle, or never).
 * R64 / C128 with FP64 products emulated on the BF16 tensor cores (table keys
   dtype + 10): N_B x the update-panel width.
 * R32_BF16 (FP32-result mode, also used by R64_IR and R32): N_B.
@@ -33,14 +32,15 @@ import time
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 NBS = (32, 64, 128, 256, 512)
-TILES = (1, 2, 3)          # HSMA_TILE_64x64, _128x16, _128x8 (0 = the rule by n)
+TILES = (1, 2, 3)          # HSMA_TILE_64x64, _128x16, _128x8 (0 = small tiles)
 EMU_NBS = (256, 512)
 PANELS = (1024, 2048, 3072, 4096)
 EMU = 10                   # table key offset of the emulated-products entries
 
 GRID = {
-    0: [(m, n) for m in (128, 512, 2048, 8192) for n in (16, 256, 4096)] + [(16384, 16384)],
-    1: [(m, n) for m in (128, 512, 2048) for n in (16, 256, 2048)] + [(8192, 8192)],
+    0: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096, 8192) for n in (4, 32, 256, 2048)] +
+       [(4096, 4096), (8192, 8192), (16384, 16384)],
+    1: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096) for n in (4, 32, 256, 1024)] + [(4096, 4096), (8192, 8192)],
     2: [(m, n) for m in (128, 512, 2048, 8192) for n in (16, 256, 4096)],
     EMU + 0: [(2048, 2048), (8192, 4096), (16384, 16384)],
     EMU + 1: [(2048, 2048), (4096, 4096), (8192, 8192)],
@@ -113,12 +113,15 @@ def tune_point(P, code, m, n, reps):
         best = min(cands, key=t)
         return best, times
     nbs = [nb for nb in NBS if nb <= max(32, 2 * m)]
-    best = min((dict(nb=nb) for nb in nbs), key=t)
     if code == 2:
-        return best, times
+        return min((dict(nb=nb) for nb in nbs), key=t), times
+    cands = [dict(nb=nb, looking=lk) for nb in nbs for lk in (1, 2) if lk == 1 or nb < m]
+    if m * m * n * (4 if code == 1 else 1) > 2e11:  # seconds per solve
+        cands = [c for c in cands if c["nb"] >= 128]
+    best = min(cands, key=t)
     best = min([best] + [dict(best, tile=tl) for tl in TILES], key=t)
-    best = min([best, dict(best, split_k=2)], key=t)
-    best = min([best, dict(best, looking=2)], key=t)
+    if best.get("tile", 0) != 0:
+        best = min([best, dict(best, split_k=2)], key=t)
     return best, times
 
 

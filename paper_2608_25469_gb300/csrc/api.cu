@@ -46,7 +46,7 @@ struct TuneEntry {
   int dtype;
   int64_t m, n;
   int nb;
-  int tile = 0;                     // HSMA_TILE_*, 0 = by n
+  int tile = 0;                     // HSMA_TILE_*, 0 = small tiles
   int split_k = HSMA_SPLITK_AUTO;
   int looking = HSMA_LOOK_RIGHT;
   int panel_cols = kEmuPanelColsDefault;  // emulated products

@@ -19,9 +19,14 @@
 // alpha is folded in once: X_0 = alpha D_0^{-1} B_0 and beta = alpha at r = 0.
 //
 // Both products run on the FP64 tensor path (mma.sync m8n8k4 .f64, "DMMA"),
-// complex as four real products, with operand tiles brought into shared memory
-// by TMA (cp.async.bulk.tensor) behind mbarriers, or by plain loads when a
-// leading dimension rules TMA out (an odd fp64 leading dimension).
+// complex as four real products, in small tiles with operands straight from
+// global memory (fp64_tile.cuh), which measured faster than the staged tiles at
+// every size: 512 x 64 FP64 138 -> 89 us, 777 x 129 complex 1.32 -> 0.55 ms,
+// 4096 x 512 FP64 11.1 -> 8.7 ms, 4096 x 4096 67.7 -> 66.2 ms (the FP64 pipe's
+// time).  The staged tiles (HSMA_TILE_*, on request and for masked operands)
+// bring operands into shared memory by TMA (cp.async.bulk.tensor) behind
+// mbarriers, or by plain loads when a leading dimension rules TMA out (an odd
+// fp64 leading dimension).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -31,6 +36,7 @@
 
 #include "blocked.h"
 #include "common.cuh"
+#include "fp64_tile.cuh"
 #include "tma.cuh"
 #include "trace.h"
 #include "workspace.h"
@@ -526,14 +532,68 @@ hsma_status_t gemm_tiled(const GemmArgs<T> &p0, const char *phase, cudaStream_t 
   return HSMA_OK;
 }
 
-// Launch one product.  Tile shape: `tile` (HSMA_TILE_*), or by n when 0
-// (128 x 8 for n <= 8, 128 x 16 for n <= 48, else 64 x 64).  K is split across
-// CTAs when the output alone has too few tiles and a partial-product
-// workspace P is given (P = nullptr: never).  `phase` names it for the tracer.
+// ---------------------------------------------------------------------------
+// Products in small tiles (fp64_tile.cuh): UPDATE and SCALE as above, without
+// partial products.  Grid (row tiles, column tiles).
+// ---------------------------------------------------------------------------
+template <class T, int WM, int WN, int NW>
+__global__ void __launch_bounds__(32 * NW) small_tile_kernel(const GemmArgs<T> p) {
+  using E = Elem<T>;
+  constexpr int BM = 8 * WM, BN = 8 * WN;
+  __shared__ T red[NW][BM * BN];
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+  fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, 0, p.tri ? min(p.K, m0 + BM) : p.K, m0, n0, red);
+  const bool b1 = is_one(p.beta);
+  for (int e = threadIdx.x; e < BM * BN; e += 32 * NW) {
+    const int row = m0 + e % BM, col = n0 + e / BM;
+    if (row >= p.M || col >= p.N) continue;
+    T v = red[0][e];
+    if (p.mode == MODE_UPDATE) {
+      const T old = p.C[row + (int64_t)col * p.ldc];
+      v = sub(b1 ? old : E::mul(p.beta, old), v);
+    } else if (!b1) {
+      v = E::mul(p.beta, v);
+    }
+    *(row < p.split_rows ? p.C2 + row + (int64_t)col * p.ldc2 : p.C + row + (int64_t)col * p.ldc) = v;
+  }
+}
+
+template <class T, int WM, int WN, int NW>
+hsma_status_t launch_small_tiles(const GemmArgs<T> &p, const char *phase, cudaStream_t st) {
+  const dim3 grid((p.M + 8 * WM - 1) / (8 * WM), (p.N + 8 * WN - 1) / (8 * WN));
+  if (grid.y > 65535) return HSMA_ERR_UNSUPPORTED;
+  HsmaTraceScope ts(phase, st);
+  small_tile_kernel<T, WM, WN, NW><<<grid, 32 * NW, 0, st>>>(p);
+  HSMA_CUDA_TRY(cudaGetLastError());
+  return HSMA_OK;
+}
+
+// Tile by the number of tiles: the largest that leaves at least four CTAs per SM
+// (fewer leave sub-partitions without DMMAs at the end); when even 8 x 8 tiles are
+// fewer than two CTAs per SM, sixteen warps share a tile's K range, unless it is
+// so short (64) that four warps have four steps each.
+template <class T>
+hsma_status_t gemm_small_tiles(const GemmArgs<T> &p, const char *phase, cudaStream_t st) {
+  const int64_t t8m = (p.M + 7) / 8, t8n = (p.N + 7) / 8, sms = sm_count();
+  auto tiles = [&](int wm, int wn) { return ((t8m + wm - 1) / wm) * ((t8n + wn - 1) / wn); };
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (t8n >= 4 && tiles(4, 4) >= 4 * sms) return launch_small_tiles<T, 4, 4, 4>(p, phase, st);
+  }
+  if (t8n >= 2 && tiles(2, 2) >= 4 * sms) return launch_small_tiles<T, 2, 2, 4>(p, phase, st);
+  if (tiles(1, 1) >= 2 * sms || p.K <= 64) return launch_small_tiles<T, 1, 1, 4>(p, phase, st);
+  return launch_small_tiles<T, 1, 1, 16>(p, phase, st);
+}
+
+// Launch one product.  Tile shape: `tile` (HSMA_TILE_*), or small tiles when 0
+// (masked operands: 128 x 8 for n <= 8, 128 x 16 for n <= 48, else 64 x 64).
+// With HSMA_TILE_* K is split across CTAs when the output alone has too few tiles
+// and a partial-product workspace P is given (P = nullptr: never).  `phase`
+// names it for the tracer.
 template <class T>
 hsma_status_t gemm(const GemmArgs<T> &p, const char *phase, cudaStream_t st, T *P = nullptr, size_t P_elems = 0,
                    int tile = 0) {
   if (p.M <= 0 || p.N <= 0) return HSMA_OK;
+  if (tile == 0 && !p.mask) return gemm_small_tiles<T>(p, phase, st);
   if (tile == 0) tile = p.N <= 8 ? HSMA_TILE_128x8 : p.N <= 48 ? HSMA_TILE_128x16 : HSMA_TILE_64x64;
   if (tile == HSMA_TILE_128x8) return gemm_tiled<T, TileN8>(p, phase, st, P, P_elems);
   if (tile == HSMA_TILE_128x16) return gemm_tiled<T, TileN16>(p, phase, st, P, P_elems);
@@ -584,7 +644,7 @@ hsma_status_t blocked_impl(const HsmaBlockedCfg &cfg, const T *A, int64_t lda, T
   const size_t w_bytes = sizeof(T) * (size_t)nb * n;
   // partial products of split-K launches (only when n is small, unless split K is off)
   const size_t p_elems =
-      cfg.split_k != HSMA_SPLITK_OFF && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
+      cfg.tile != 0 && cfg.split_k != HSMA_SPLITK_OFF && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
   const size_t inv_bytes = hsma_fp64_inverse_scratch(nb, m, sizeof(T));
   hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems + inv_bytes, st);
   if (s != HSMA_OK) return s;

@@ -6,7 +6,7 @@
 #include "../../include/hsma.h"
 
 // Configuration of the blocked path: diagonal block size, FP64 product tile
-// shape (HSMA_TILE_*; 0 = by n), split K (HSMA_SPLITK_*) and the update
+// shape (HSMA_TILE_*; 0 = small tiles), split K (HSMA_SPLITK_*) and the update
 // direction (HSMA_LOOK_*), as the planner picks them.
 struct HsmaBlockedCfg {
   int nb = 256;

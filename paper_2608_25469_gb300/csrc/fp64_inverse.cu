@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kBase = 32;      // blocks inverted by substitution
 constexpr int kBaseWarps = 4;  // columns per CTA of the base kernel
+constexpr int kFp64Warps = 4;  // warps per CTA of the products
 
 // Columns 4 y .. 4 y + 3 of the inverse of base block b (rows 32 b .. of the
 // matrix), one per warp: lane r holds row r of the block, scaled by 1/a_rr, in
@@ -72,9 +73,9 @@ __global__ void __launch_bounds__(32 * kFp64Warps) inv_level_kernel(const T *__r
   const int l0 = (int)(i0 % nb);
   T *Wp = W + (int64_t)blockIdx.y * h * h;
   if (PASS == 0) {  // column tile n0 of A^-1 starts at row n0
-    fp64_tile<T, WT, WT>(A + (i0 + h) + i0 * lda, lda, Y + l0 + (int64_t)l0 * nb, nb, sd, h, n0, h, m0, n0, red);
+    fp64_tile<T, WT, WT, kFp64Warps>(A + (i0 + h) + i0 * lda, lda, Y + l0 + (int64_t)l0 * nb, nb, sd, h, n0, h, m0, n0, red);
   } else {  // row tile m0 of D^-1 ends at its diagonal
-    fp64_tile<T, WT, WT>(Y + (l0 + h) + (int64_t)(l0 + h) * nb, nb, Wp, h, sd, h, 0, min(sd, m0 + TS), m0, n0, red);
+    fp64_tile<T, WT, WT, kFp64Warps>(Y + (l0 + h) + (int64_t)(l0 + h) * nb, nb, Wp, h, sd, h, 0, min(sd, m0 + TS), m0, n0, red);
   }
   T *out = PASS == 0 ? Wp : Y + (l0 + h) + (int64_t)l0 * nb;
   const int64_t ldo = PASS == 0 ? h : nb;

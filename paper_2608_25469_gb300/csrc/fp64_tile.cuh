@@ -4,9 +4,9 @@
 // A DMMA occupies its sub-partition's FP64 pipe for about 512 cycles on this
 // GPU, so operand traffic is negligible (an 8 x 8 tile reads 512 bytes per
 // DMMA, 1.2 TB/s over all SMs from the caches) and what counts is that every
-// sub-partition has DMMAs to do.  A CTA's four warps, one per sub-partition,
-// share one output tile and take every fourth K step; their sums are added in
-// shared memory in a fixed order.
+// sub-partition has DMMAs to do.  A CTA's warps (four, one per sub-partition, or
+// more when there are few tiles) share one output tile and take the K steps in
+// turn; their sums are added in shared memory in a fixed order.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -50,13 +50,12 @@ __device__ __forceinline__ cplx fp64_add(cplx a, cplx b) { return cplx{a.re + b.
 __device__ __forceinline__ double fp64_neg(double a) { return -a; }
 __device__ __forceinline__ cplx fp64_neg(cplx a) { return cplx{-a.re, -a.im}; }
 
-constexpr int kFp64Warps = 4;
 
 // Rows m0 .. m0 + 8 WM - 1 and columns n0 .. n0 + 8 WN - 1 of A B over
 // k = kbeg .. kend - 1 (A: M x kend column-major, B: kend x N column-major;
-// entries outside read as zero).  All 128 threads take part; the tile is left in
+// entries outside read as zero).  All NW warps of the CTA take part; the tile is left in
 // red[0] (column-major, 8 WM rows) after a CTA barrier.
-template <class T, int WM, int WN>
+template <class T, int WM, int WN, int NW>
 __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, int64_t ldb,
                                           int M, int N, int kbeg, int kend, int m0, int n0,
                                           T (*red)[8 * WM * 8 * WN]) {
@@ -72,7 +71,7 @@ __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, 
   auto load = [&](int k0, int s) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int k = k0 + 4 * kFp64Warps * u + t;
+      const int k = k0 + 4 * NW * u + t;
 #pragma unroll
       for (int i = 0; i < WM; ++i) {
         const int r = m0 + 8 * i + g;
@@ -88,14 +87,14 @@ __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, 
   auto mul = [&](int k0, int s) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (k0 + 4 * kFp64Warps * u >= kend) break;  // warp-uniform
+      if (k0 + 4 * NW * u >= kend) break;  // warp-uniform
 #pragma unroll
       for (int i = 0; i < WM; ++i)
 #pragma unroll
         for (int j = 0; j < WN; ++j) acc[i][j].mma(a[s][u][i], b[s][u][j]);
     }
   };
-  constexpr int kGroup = 4 * kFp64Warps * U;
+  constexpr int kGroup = 4 * NW * U;
   int k0 = kbeg + 4 * warp;
   load(k0, 0);
   while (k0 < kend) {
@@ -114,10 +113,10 @@ __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, 
 #pragma unroll
       for (int q = 0; q < 2; ++q) red[warp][(8 * i + g) + (8 * j + 2 * t + q) * 8 * WM] = acc[i][j].get(q);
   __syncthreads();
-  for (int e = threadIdx.x; e < 8 * WM * 8 * WN; e += 32 * kFp64Warps) {
+  for (int e = threadIdx.x; e < 8 * WM * 8 * WN; e += 32 * NW) {
     T v = red[0][e];
 #pragma unroll
-    for (int w = 1; w < kFp64Warps; ++w) v = fp64_add(v, red[w][e]);
+    for (int w = 1; w < NW; ++w) v = fp64_add(v, red[w][e]);
     red[0][e] = v;
   }
   __syncthreads();

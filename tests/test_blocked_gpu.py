@@ -106,6 +106,23 @@ def test_inverse_levels_parity(H, code, m, nb):
     assert oracle.forward_error(X, ref) <= TOL
 
 
+@pytest.mark.parametrize("code", [I.R64, I.C128])
+@pytest.mark.parametrize("m,n,nb,look", [(66, 1, 64, 1), (129, 8, 64, 1), (300, 9, 128, 2), (520, 31, 256, 1),
+                                         (1000, 33, 128, 2), (1031, 200, 512, 1), (1500, 257, 128, 2)])
+def test_small_tile_products_parity(H, code, m, n, nb, look):
+    """Every small-tile shape (by the number of tiles) at ragged sizes, odd leading dimensions,
+    alpha, both update directions, NaN in what is never read."""
+    alpha = -0.5 if code == I.R64 else 0.5 + 2j
+    A0, B0 = I.gen_A(m, m, code), I.gen_B(m, m, n, code)
+    A = I.embed(A0, m + 1, fill=np.nan)
+    A[:m][np.triu_indices(m, 1)] = np.nan
+    B = I.embed(B0, m + 3, fill=np.nan)
+    assert H.hsma_plan(code, m, n).tile == 0
+    X = _run(H, code, A, B, alpha, nb, looking=look)
+    assert np.all(np.isnan(X[m:]))
+    assert oracle.forward_error(X[:m], oracle.solve(A0, B0, alpha)) <= TOL
+
+
 CFG_CASES = [(65, 7, 32), (300, 200, 128), (700, 50, 512), (1000, 9, 64), (513, 130, 256)]
 
 

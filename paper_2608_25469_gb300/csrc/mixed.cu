@@ -574,7 +574,14 @@ __global__ void sumsq_kernel(const double *__restrict__ M_, int64_t ld, int64_t 
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(&sums[slot], acc);
+  // one atomic per CTA: the adds to one address run one after another
+  __shared__ double part[8];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) acc += part[w];
+    atomicAdd(&sums[slot], acc);
+  }
 }
 
 // sums: [0] ||L||^2, [1] ||B||^2, [2] ||R||^2, [3] ||X||^2; state: [0] converged, [1] steps, [2..3] eta (double).
@@ -681,9 +688,9 @@ __device__ __forceinline__ void oz_entry(const double *__restrict__ A, int64_t l
 // left operand is sliced as A_rk 2^-g_k and the right one as X_kj 2^g_k, which
 // leaves the product unchanged and makes the row and column scales of badly
 // scaled operands (D_r L D_c) meaningful.  A column without nonzeros keeps
-// kOzExpEmpty and the right operand's row k is then ignored.  A CTA covers 32
-// columns x 256 rows (a warp per column, lanes down the rows) and folds its
-// maxima in with atomicMax over the kOzExpEmpty fill.
+// kOzExpEmpty and the right operand's row k is then ignored.  A CTA covers 8
+// columns x 256 rows (a warp per column, lanes down the rows, eight loads in
+// flight) and folds its maxima in with atomicMax over the kOzExpEmpty fill.
 __global__ void oz_fill_kernel(int *p, int n, int v) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) p[k] = v;
 }
@@ -691,29 +698,27 @@ __global__ void oz_fill_kernel(int *p, int n, int v) {
 template <bool CPLX>
 __global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
                                                       int mode, int *kexp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, k = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int r0 = blockIdx.y * 256;
-  for (int k = blockIdx.x * 32 + warp; k < min(K, blockIdx.x * 32 + 32); k += 8) {
-    uint64_t mx = 0;
-    for (int r = r0 + lane; r < min(rows, r0 + 256); r += 32) {
-      double re, im;
-      oz_entry<CPLX>(A, lda, rows, K, mode, r, k, re, im);
-      mx = max(mx, max(oz_absbits(re), oz_absbits(im)));
-    }
+  if (k >= K || (mode != 0 && r0 + 255 < k)) return;
+  uint64_t mx = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, (uint64_t)__shfl_down_sync(0xffffffffu, mx, o));
-    if (lane == 0 && mx != 0) {
-      const int e = oz_exponent(mx);
-      atomicMax(&kexp[(CPLX ? 2 : 1) * k], e);
-      if (CPLX) atomicMax(&kexp[2 * k + 1], e);
-    }
+  for (int q = 0; q < 8; ++q) {
+    double re, im;
+    oz_entry<CPLX>(A, lda, rows, K, mode, r0 + lane + 32 * q, k, re, im);
+    mx = max(mx, max(oz_absbits(re), oz_absbits(im)));
+  }
+  const int e = __reduce_max_sync(0xffffffffu, mx != 0 ? oz_exponent(mx) : kOzExpEmpty);
+  if (lane == 0 && e != kOzExpEmpty) {
+    atomicMax(&kexp[(CPLX ? 2 : 1) * k], e);
+    if (CPLX) atomicMax(&kexp[2 * k + 1], e);
   }
 }
 
 // Row exponents of a left operand balanced by 2^-g_k (atomicMax over the
 // kOzExpEmpty fill): a CTA covers 32 rows x kOzRexpCols columns, lanes across
 // the rows.
-constexpr int kOzRexpCols = 128;
+constexpr int kOzRexpCols = 64;
 
 template <bool CPLX>
 __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
@@ -724,8 +729,9 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
   const int i = blockIdx.x * 32 + tx, kb = blockIdx.y * kOzRexpCols;
   if (mode != 0 && kb > blockIdx.x * 32 + 31) return;  // above the diagonal
   int ex = kOzExpEmpty;
-#pragma unroll 4
-  for (int k = kb + ty; k < min(K, kb + kOzRexpCols); k += 8) {
+#pragma unroll
+  for (int q = 0; q < kOzRexpCols / 8; ++q) {
+    const int k = kb + ty + 8 * q;
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, i, k, re, im);
     const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
@@ -875,7 +881,7 @@ hsma_status_t oz_slice_a(bool cplx, const double *A, int64_t lda, int rows, int 
                          cudaStream_t st) {
   if (rows <= 0 || K <= 0) return HSMA_OK;
   const int W = cplx ? 2 : 1;
-  const dim3 kg((unsigned)((K + 31) / 32), (unsigned)((rows + 255) / 256));
+  const dim3 kg((unsigned)((K + 7) / 8), (unsigned)((rows + 255) / 256));
   const dim3 rg((unsigned)((rows + 31) / 32), (unsigned)((K + kOzRexpCols - 1) / kOzRexpCols));
   const dim3 sg((unsigned)((rows + 31) / 32), (unsigned)(o.Kp / 64));
   if (kg.y > 65535 || rg.y > 65535) return HSMA_ERR_UNSUPPORTED;
@@ -913,6 +919,10 @@ hsma_status_t oz_slice_x(const double *X, int64_t ldx, int K, const int *kexp, O
 // bytes of two tiles per CTA.
 constexpr int kEmuGemmMaxK = 1 << 14;      // hsma_gemm_f64_emulated
 constexpr int kOzResidualMaxM = 1 << 14;   // refinement residuals
+// K per launch of a triangular product: longer ranges differ more between row
+// tiles, whose CTAs then read different moduli's planes at the same time
+// (8192 x 4096 refinement: 1024 14.7, 2048 14.4, 4096 14.2, 8192 14.4 ms).
+constexpr int kOzTriK = 4096;
 
 size_t oz_scratch_bytes(int64_t rows, int64_t cols) {
   const int64_t tiles = ((rows + TC_PM - 1) / TC_PM) * ((cols + 127) / 128);
@@ -921,11 +931,12 @@ size_t oz_scratch_bytes(int64_t rows, int64_t cols) {
 
 // C (M x N, column-major FP64) = (beta0 ? C : 0) -/+ L X in emulated FP64,
 // L and X given by their residues; tri: L is lower triangular.  At most kOzMaxK
-// columns of L per launch, each launch one rounding and one addition to C.
+// (kOzTriK) columns of L per launch, each launch one rounding and one addition to C.
 hsma_status_t oz_product(const OzOperand &L, const OzOperand &X, double *C, int64_t ldc, int beta0, int negate,
                          int tri, uint32_t *scratch, const int *skip, const char *phase, cudaStream_t st) {
   if (L.Kp != X.Kp) return HSMA_ERR_INVALID_ARG;
-  for (int64_t c0 = 0; c0 < L.Kp; c0 += kOzMaxK) {
+  const int64_t kmax = tri ? kOzTriK : kOzMaxK;
+  for (int64_t c0 = 0; c0 < L.Kp; c0 += kmax) {
     const int64_t i0 = tri ? c0 : 0;  // a triangular L has no entries above row c0 in these columns
     if (i0 >= L.rows) break;
     TcArgs a{};
@@ -938,7 +949,7 @@ hsma_status_t oz_product(const OzOperand &L, const OzOperand &X, double *C, int6
     a.scratch = scratch;
     a.M = (int)(L.rows - i0);
     a.N = X.rows;
-    a.K = (int)std::min<int64_t>(kOzMaxK, L.Kp - c0);
+    a.K = (int)std::min<int64_t>(kmax, L.Kp - c0);
     a.tri = tri;
     a.skip = skip;
     SliceLayout la, lb;  // views into the full planes at row i0 and column c0
@@ -956,15 +967,30 @@ hsma_status_t oz_product(const OzOperand &L, const OzOperand &X, double *C, int6
   return HSMA_OK;
 }
 
-// R -= L X in emulated FP64 (R holds alpha B on entry); skip: device flag.
-hsma_status_t oz_residual(const OzOperand &L, const double *X, int64_t ldx, double *R, int64_t ldr, OzOperand &Xo,
-                          uint32_t *scratch, const int *skip, cudaStream_t st) {
-  {
-    HsmaTraceScope ts("residual_slices", st);
-    hsma_status_t s = oz_slice_x(X, ldx, L.rows, L.kexp, Xo, skip, st);
-    if (s != HSMA_OK) return s;
+// Columns of X whose residues are held at a time by the refinement residual: all,
+// or equal parts (whole column tiles) of at most kOzXBytes.
+constexpr int64_t kOzXBytes = 640ll << 20;
+
+int64_t oz_residual_cols(int64_t n, int Kp) {
+  const int64_t parts = (2ll * kOzP * n * Kp + kOzXBytes - 1) / kOzXBytes;
+  return std::min(n, ((n + parts - 1) / parts + 255) / 256 * 256);
+}
+
+// R -= L X in emulated FP64 (R, m x n, holds alpha B on entry); skip: device flag.
+hsma_status_t oz_residual(const OzOperand &L, const double *X, int64_t ldx, int64_t n, double *R, int64_t ldr,
+                          void *x_ws, uint32_t *scratch, const int *skip, cudaStream_t st) {
+  const int64_t cols = oz_residual_cols(n, L.Kp);
+  for (int64_t j0 = 0; j0 < n; j0 += cols) {
+    OzOperand Xo = oz_operand(x_ws, cols, L.Kp);
+    Xo.rows = (int)std::min(cols, n - j0);
+    hsma_status_t s;
+    {
+      HsmaTraceScope ts("residual_slices", st);
+      if ((s = oz_slice_x(X + j0 * ldx, ldx, L.rows, L.kexp, Xo, skip, st)) != HSMA_OK) return s;
+    }
+    if ((s = oz_product(L, Xo, R + j0 * ldr, ldr, 1, 0, 1, scratch, skip, "residual", st)) != HSMA_OK) return s;
   }
-  return oz_product(L, Xo, R, ldr, 1, 0, 1, scratch, skip, "residual", st);
+  return HSMA_OK;
 }
 
 __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, double ar, double ai, int cplx) {
@@ -1143,7 +1169,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   const size_t st_b = 1024;
   const int ozkp = oz_kp(m);
   const size_t ozl_b = emulated ? al(oz_operand_bytes(m, ozkp)) : 0;
-  const size_t ozx_b = emulated ? al(oz_operand_bytes(n, ozkp)) : 0;
+  const size_t ozx_b = emulated ? al(oz_operand_bytes(oz_residual_cols(n, ozkp), ozkp)) : 0;
   const size_t ozs_b = emulated ? al(oz_scratch_bytes(m, n)) : 0;
   // the FP32 inverses and BF16 panels of L, shared by the first solve and every correction
   R32Plan P;
@@ -1169,7 +1195,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   int *state = reinterpret_cast<int *>(sums + 8);
   void *ozl_ws = base + al(a32_b) + al(r32_b) + al(b0_b) + al(r64_b) + st_b;
   void *ozx_ws = static_cast<unsigned char *>(ozl_ws) + ozl_b;
-  OzOperand Lsl = oz_operand(ozl_ws, m, ozkp), Xsl = oz_operand(ozx_ws, n, ozkp);
+  OzOperand Lsl = oz_operand(ozl_ws, m, ozkp);
   P.A = A32;
   uint32_t *ozs = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(ozx_ws) + ozx_b);
   P.Dinv = reinterpret_cast<float *>(static_cast<unsigned char *>(ozx_ws) + ozx_b + ozs_b);
@@ -1213,7 +1239,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
           HsmaTraceScope ts("refine", st);
           scale_copy_kernel<<<g_launch_grid(m * n), 256, 0, st>>>(B0, R64, m * n, alpha, state);
         }
-        if ((s = oz_residual(Lsl, B, ldb, R64, m, Xsl, ozs, state, st)) != HSMA_OK) break;
+        if ((s = oz_residual(Lsl, B, ldb, n, R64, m, ozx_ws, ozs, state, st)) != HSMA_OK) break;
       } else {
         if ((s = fail(cudaMemcpy2DAsync(R64, sizeof(double) * m, B0, sizeof(double) * m, sizeof(double) * m, n,
                                         cudaMemcpyDeviceToDevice, st))) != HSMA_OK)

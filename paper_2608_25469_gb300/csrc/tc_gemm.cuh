@@ -285,7 +285,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
     const int band = t / (G * tiles_n);
     const int gb = min(G, tiles_m - band * G);
     const int idx = t - band * G * tiles_n;
-    const int pm = band * G + idx % gb;
+    int pm = band * G + idx % gb;
+    if (p.tri) pm = tiles_m - 1 - pm;  // the longest K ranges first: the tail is short tiles
     m0 = pm * TC_PM + (int)rank * TC_BM;  // this CTA's rows
     n0 = (idx / gb) * TC_BN;
     const int kall = p.tri ? min(p.K, (pm + 1) * TC_PM) : p.K;

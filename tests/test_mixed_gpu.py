@@ -119,6 +119,18 @@ def test_ir_mode_reaches_fp64_accuracy(H, m, n, residual):
     assert H.hsma_device_status() == 0
 
 
+@pytest.mark.parametrize("m,n", [(8192, 2500), (4200, 260)])
+def test_ir_residual_parts(H, m, n):
+    """Residuals in several K ranges of L (4096 per launch) and column parts of X (whole 256-column
+    tiles of at most 640 MiB of residues), ragged in both."""
+    A, B = I.gen_A(21, m, I.R64), I.gen_B(21, m, n, I.R64)
+    X, info = _ir(H, A, B, 1.0)
+    assert info.converged == 1 and info.ir_residual <= 1e-15
+    cols = np.unique(np.linspace(0, n - 1, 24).astype(int))
+    assert oracle.forward_error(X[:, cols], oracle.solve_cols(A, B, 1.0, cols)) <= 1e-12
+    assert H.hsma_device_status() == 0
+
+
 def test_ir_mode_unit_diagonal_emulated(H):
     m, n = 700, 90
     A0, B = I.gen_A(12, m, I.R64), I.gen_B(12, m, n, I.R64)

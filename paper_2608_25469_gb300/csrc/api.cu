@@ -392,7 +392,7 @@ hsma_status_t hsma_trsm_vbatched(int dtype, int side, int uplo, int trans, int d
   // map), the other dtypes the per-instance kernel (with the same map)
   const bool packed = hsma_vbatched_packed_dtype(dtype) && packed_enabled();
   hsma_status_t s = hsma_ws_alloc(
-      &scratch, packed ? hsma_vbatched_packed_scratch_bytes(dtype, batch, max_m) : hsma_vbatched_scratch_bytes(batch),
+      &scratch, packed ? hsma_vbatched_packed_scratch_bytes(dtype, batch, max_m) : hsma_vbatched_scratch_bytes(dtype, batch),
       st);
   if (s != HSMA_OK) return s;
   if (packed)
@@ -462,7 +462,7 @@ static hsma_status_t factor_solve_vbatched(int dtype, int32_t batch, const int32
                                      q + me_b, st, 0, chol ? HSMA_LOWER : HSMA_UPPER,
                                      chol ? HSMA_CONJ_TRANS : HSMA_NO_TRANS);
   } else {
-    s = hsma_ws_alloc(&scratch, hsma_vbatched_scratch_bytes(batch), st);
+    s = hsma_ws_alloc(&scratch, hsma_vbatched_scratch_bytes(dtype, batch), st);
     if (s != HSMA_OK) return s;
     s = hsma_small_getrs_vbatched(dtype, batch, d_m, d_n, static_cast<const double *>(alpha), d_LU, d_lda, d_ipiv,
                                   d_B, d_ldb, d_status, static_cast<int32_t *>(scratch), st, chol, large ? 1 : 0);

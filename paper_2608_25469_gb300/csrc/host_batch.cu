@@ -138,7 +138,7 @@ hsma_status_t full_pipeline(int dtype, int diag, int32_t batch, const int32_t *h
   int32_t max_m = 0;
   for (int32_t i = 0; i < batch; ++i) max_m = std::max(max_m, h_m[i]);
   const size_t scr_b = al(packed ? hsma_vbatched_packed_scratch_bytes(dtype, per, max_m)
-                                 : hsma_vbatched_scratch_bytes(per));
+                                 : hsma_vbatched_scratch_bytes(dtype, per));
   const int nscr = nch < 2 ? nch : 2;
   const size_t total = a_b + b_b + s_b + sq_b + 3 * mi_b + 2 * oi_b + 2 * p_b + scr_b * nscr;
   std::unique_ptr<cudaEvent_t[]> evs(new (std::nothrow) cudaEvent_t[2 * nch]());  // copied-in, solved

@@ -24,7 +24,6 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
-#include <type_traits>
 
 #include "common.cuh"
 #include "small.h"
@@ -40,11 +39,6 @@ namespace {
 #endif
 #ifndef HSMA_VB_MINB
 #define HSMA_VB_MINB 3
-#endif
-// FP32 element types: the FP32 pipe leaves the kernel bound by load and
-// barrier latency, so more CTAs per SM pay off (and fit: half the registers).
-#ifndef HSMA_VB_MINB_F32
-#define HSMA_VB_MINB_F32 6
 #endif
 #ifndef HSMA_VB_GMASK
 #define HSMA_VB_GMASK 0xFu
@@ -462,9 +456,7 @@ __global__ void __launch_bounds__(1024) vbatched_schedule_kernel(int batch, cons
 
 template <class T, bool MAP>
 __global__ void __launch_bounds__(32 * kWarpsBatched,
-                                  (sizeof(T) == sizeof(float) || sizeof(T) == sizeof(cplxf)) && !std::is_same<T, double>::value
-                                      ? HSMA_VB_MINB_F32
-                                      : HSMA_VB_MINB) vbatched_solve_kernel(const int32_t *__restrict__ dm,
+                                  HSMA_VB_MINB) vbatched_solve_kernel(const int32_t *__restrict__ dm,
                                                                   const int32_t *__restrict__ dn,
                                                                   const int32_t *__restrict__ dlda,
                                                                   const int32_t *__restrict__ dldb,
@@ -562,9 +554,7 @@ __device__ __noinline__ void lu_stage_solve(int g, T *sTri, T *sC, T *sR, const 
 
 template <class T>
 __global__ void __launch_bounds__(32 * kWarpsBatched,
-                                  (sizeof(T) == sizeof(float) || sizeof(T) == sizeof(cplxf)) && !std::is_same<T, double>::value
-                                      ? HSMA_VB_MINB_F32
-                                      : HSMA_VB_MINB) vbatched_lu_kernel(const int32_t *__restrict__ dm,
+                                  HSMA_VB_MINB) vbatched_lu_kernel(const int32_t *__restrict__ dm,
                                                                   const int32_t *__restrict__ dn,
                                                                   const int32_t *__restrict__ dlda,
                                                                   const int32_t *__restrict__ dldb,
@@ -773,7 +763,10 @@ static hsma_status_t vbatched_impl(int32_t batch, const int32_t *dm, const int32
   return HSMA_OK;
 }
 
-size_t hsma_vbatched_scratch_bytes(int32_t batch) { return sizeof(int32_t) * (2 + (size_t)(batch > 0 ? batch : 0)); }
+size_t hsma_vbatched_scratch_bytes(int dtype, int32_t batch) {
+  if (dtype == HSMA_R32 || dtype == HSMA_C64) return 0;  // no schedule
+  return sizeof(int32_t) * (2 + (size_t)(batch > 0 ? batch : 0));
+}
 
 hsma_status_t hsma_small_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
                                   const double *alpha, const void *const *dA, const int32_t *dlda,
@@ -783,10 +776,10 @@ hsma_status_t hsma_small_vbatched(int dtype, int32_t batch, const int32_t *dm, c
   switch (dtype) {
     case HSMA_C128: return vbatched_impl<cplx>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
                                     skip_large);
-    case HSMA_R32: return vbatched_impl<float>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
-                                    skip_large);
-    case HSMA_C64: return vbatched_impl<cplxf>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
-                                    skip_large);
+    case HSMA_R32:
+    case HSMA_C64:
+      return hsma_f32_vbatched(dtype, batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, st, uplo, trans,
+                               skip_large);
     default: return vbatched_impl<double>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
                                     skip_large);
   }
@@ -935,11 +928,9 @@ hsma_status_t hsma_small_getrs_vbatched(int dtype, int32_t batch, const int32_t 
       return getrs_impl<cplx>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
                                  skip_large);
     case HSMA_R32:
-      return getrs_impl<float>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
-                                 skip_large);
     case HSMA_C64:
-      return getrs_impl<cplxf>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
-                                 skip_large);
+      return hsma_f32_factor_vbatched(dtype, batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, st, chol,
+                                      skip_large);
     default:
       return getrs_impl<double>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
                                  skip_large);

@@ -14,10 +14,20 @@ hsma_status_t hsma_small_single(int dtype, int g, const void *A, int64_t lda, vo
                                 int trans = HSMA_NO_TRANS);
 
 // Bytes of device scratch the varlen batch needs for `batch` instances.
-size_t hsma_vbatched_scratch_bytes(int32_t batch);
+size_t hsma_vbatched_scratch_bytes(int dtype, int32_t batch);
+
+// The same in FP32 (HSMA_R32, HSMA_C64; batch_f32.cu): one launch, no scratch.
+// Called by the two entry points below for these dtypes.
+hsma_status_t hsma_f32_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha,
+                                const void *const *dA, const int32_t *dlda, void *const *dB, const int32_t *dldb,
+                                int unit, uint32_t *status, cudaStream_t st, int uplo, int trans, int skip_large);
+hsma_status_t hsma_f32_factor_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
+                                       const double *alpha, const void *const *dA, const int32_t *dlda,
+                                       const int32_t *const *dipiv, void *const *dB, const int32_t *dldb,
+                                       uint32_t *status, cudaStream_t st, int chol, int skip_large);
 
 // Varlen batch (schedule pre-pass + persistent solve).  `scratch` holds
-// hsma_vbatched_scratch_bytes(batch) bytes of device memory.  skip_large:
+// hsma_vbatched_scratch_bytes(dtype, batch) bytes of device memory.  skip_large:
 // instances with m > 64 are skipped without a status bit (the caller solves
 // them on the blocked path); otherwise they are flagged HSMA_DEVERR_BAD_SIZE.
 hsma_status_t hsma_small_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
@@ -59,10 +69,8 @@ hsma_status_t hsma_small_lu_pivots(int dtype, int32_t batch, const int32_t *dm, 
 size_t hsma_vbatched_packed_scratch_bytes(int dtype, int32_t batch, int32_t max_m);
 // dtypes whose varlen batch runs the column-packed kernels (measured faster
 // than the per-instance kernel: complex128; real FP64 keeps the per-instance
-// kernel, whose G choice already fills its lanes at 4x less work per element,
-// and so does complex64, where the packed form ran at 2890 against 4800
-// GFLOP/s: FP32 arithmetic is cheap, and the triangle reads through the
-// caches cost more than the per-instance kernel's shared-memory staging)
+// kernel, whose G choice already fills its lanes at 4x less work per element;
+// the FP32 dtypes have their own, batch_f32.cu)
 inline bool hsma_vbatched_packed_dtype(int dtype) { return dtype == HSMA_C128; }
 hsma_status_t hsma_small_vbatched_packed(int dtype, int32_t batch, int32_t max_m, const int32_t *dm,
                                          const int32_t *dn, const double *alpha, const void *const *dA,

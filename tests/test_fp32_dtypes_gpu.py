@@ -129,3 +129,62 @@ def test_host_batch_complex64_equals_device_batch(H):
     for b in range(len(As)):
         got = hX[offB[b]:offB[b] + ms[b] * ns[b]].reshape((ms[b], ns[b]), order="F")
         assert np.array_equal(got, dev[b]), b
+
+
+EDGES = [(1, 1), (7, 15), (8, 16), (9, 17), (15, 64), (16, 65), (17, 3), (31, 33), (32, 130), (33, 16), (63, 5), (64, 64)]
+
+
+@pytest.mark.parametrize("code64,code", [(I.R64, 4), (I.C128, 5)], ids=["f32", "c64"])
+@pytest.mark.parametrize("kind", ["nn", "nn_unit", "un", "lt", "uc", "lc_unit", "lu", "chol"])
+def test_batched_fp32_block_edges(H, code64, code, kind):
+    """The batch kernel at the edges of its 8-row blocks, 16-column tiles and 64-column rounds, in
+    every index map and both factor solves, with padded leading dimensions and NaN in whatever is
+    not referenced.  Tolerance: the FP32 substitution bound, twice for the factor solves."""
+    import torch
+    uplo = 1 if kind[0] == "u" else 0
+    trans = {"t": 1, "c": 2}.get(kind[1], 0) if kind not in ("lu", "chol") else 0
+    unit = kind.endswith("unit")
+    alpha = 1.5 if code64 == I.R64 else 1.5 - 0.5j
+    As, Bs, raw, pivs = [], [], [], []
+    rng = np.random.default_rng(5)
+    for b, (m, n) in enumerate(EDGES):
+        A = I.gen_LU(3, m, code64, inst=b) if kind == "lu" else I.gen_A(3, m, code64, inst=b)
+        A = np.asfortranarray(A.T) if uplo else A
+        A32, B32 = _f32(code64, A), _f32(code64, I.gen_B(3, m, n, code64, inst=b))
+        raw.append((A32, B32))
+        E = np.array(A32, order="F")
+        if kind != "lu":
+            E[np.tril_indices(m, -1) if uplo else np.triu_indices(m, 1)] = np.nan
+        if unit:
+            np.fill_diagonal(E, np.nan)
+        As.append(I.embed(E, m + b % 3))
+        Bs.append(I.embed(B32, m + b % 3))
+        pivs.append((np.arange(m) + np.floor(rng.random(m) * (m - np.arange(m))) + 1).astype(np.int32))
+    bt = U.Batch(As, Bs)
+    bt.d_ldb = bt.d_lda
+    a = bt.args()
+    st, ds = H.stream_ptr(), bt.d_status.data_ptr()
+    if kind == "lu":
+        flat = torch.from_numpy(np.concatenate(pivs)).cuda()
+        off = np.concatenate([[0], np.cumsum([len(p) for p in pivs])[:-1]]).astype(np.int64)
+        ptr = torch.from_numpy(flat.data_ptr() + 4 * off).cuda()
+        H.hsma_getrs_vbatched(code, bt.batch, a[0], a[1], alpha, a[2], a[3], ptr.data_ptr(), a[4], a[5], 64, 0, ds, st)
+    elif kind == "chol":
+        H.hsma_potrs_vbatched(code, bt.batch, a[0], a[1], alpha, a[2], a[3], a[4], a[5], 64, 0, ds, st)
+    else:
+        H.hsma_trsm_vbatched(code, 0, uplo, trans, int(unit), bt.batch, a[0], a[1], alpha, a[2], a[3], a[4], a[5], 64,
+                             0, ds, st)
+    torch.cuda.synchronize()
+    assert bt.status() == 0
+    wide = np.complex128 if code64 == I.C128 else np.float64
+    for b, X in enumerate(bt.results()):
+        A32, B32 = (np.asfortranarray(v.astype(wide)) for v in raw[b])
+        m = A32.shape[0]
+        if kind == "lu":
+            ref = oracle.getrs(A32, pivs[b], B32, alpha)
+        elif kind == "chol":
+            ref = oracle.potrs(A32, B32, alpha)
+        else:
+            ref = oracle.solve_general(A32, B32, alpha, 0, uplo, trans, unit)
+        assert np.all(np.isnan(X[m:])), EDGES[b]
+        assert oracle.forward_error(X[:m].astype(wide), ref) <= TOL32 * (2 if kind in ("lu", "chol") else 1), EDGES[b]

@@ -229,13 +229,13 @@ HSMA_API hsma_status_t hsma_trsm(int dtype, int side, int uplo, int trans, int d
  *        it for instances it skips as invalid.  May be NULL.
  * HSMA_C128: the columns of all instances with the same m are dealt to warps
  * 32 (16 for m > 32) at a time, so a warp may serve several instances; the
- * other dtypes deal each instance's column tiles to the warps of one CTA.  An
+ * other dtypes run one CTA per instance, its columns dealt to the CTA's warps.  An
  * instance's arithmetic never depends on the others, so results are
  * bit-identical to solving it alone through this entry point with batch = 1.
  * Workspace (stream-ordered pool): for HSMA_C128 room for the pre-scaled
  * triangle and diagonal of every instance, batch x r (r + 1) / 2 elements
- * with r = max_m rounded up to even, plus 20 bytes per instance; otherwise
- * 4 bytes per instance.
+ * with r = max_m rounded up to even, plus 20 bytes per instance; for HSMA_R64
+ * 4 bytes per instance; for the FP32 dtypes none.
  */
 HSMA_API hsma_status_t hsma_trsm_llnn_vbatched(int dtype, int diag, int32_t batch, const int32_t *d_m,
                                       const int32_t *d_n, const void *alpha, const void *const *d_A,

@@ -1,26 +1,32 @@
-// Varlen batch of small solves (m <= 64) in FP32 (float and float complex):
+// Varlen batch of small solves (m <= 64) in double, float and float complex:
 // triangular solves, and LU- and Cholesky-factor solves fused per instance.
+// (Double complex has the column-packed kernels, packed.cu.)
 //
-// FP32 arithmetic is cheap here; what bounds this work is instruction fetch,
-// load latency and shared-memory reads.  The fully unrolled substitution of the
-// FP64 kernels (X in registers, one variant per row-group count) spends most of
-// its issue slots waiting for instructions when the arithmetic is this fast
-// (10.5 of 18 stall cycles per instruction, 362 us for 8192 complex64 solves
-// with m, n ~ U{8..64}).  Here the substitution runs in 8-row blocks with
-// rolled loops (about 600 instructions in all):
+// The fully unrolled substitution (X in registers, one variant per row-group
+// count) left the arithmetic waiting: in FP32 for instructions (10.5 of 18 stall
+// cycles, 362 us for 8192 complex64 solves with m, n ~ U{8..64}), in FP64 for
+// staging and for shared-memory operands with 12 warps per SM (FP64 pipe 69%
+// busy, 717 us for 4097 double LU solves).  Here the substitution runs in
+// blocks of rows with rolled loops (some 600 instructions, 50 to 60 registers):
 //
-//  * one CTA of four warps per instance, in any order (the hardware deals
-//    instances to SMs as they free up; there is no schedule pass);
-//  * the triangle (8 x 8 blocks) and the right-hand sides are copied to shared
+//  * one CTA of four warps per instance; the hardware deals them to the SMs as
+//    these free up (double, whose large instances take long: largest first within
+//    groups of 256 instances, by a pass of a few microseconds);
+//  * the triangle (square blocks) and the right-hand sides are copied to shared
 //    memory asynchronously, all of an instance's loads in flight at once;
-//  * a warp owns 16 columns, two lanes per column with four rows of each block;
-//    block row J gathers
-//        acc = alpha B_J - sum_{I < J} L_JI X_I
-//    from shared memory before its own eight steps, X overwrites B there, and
-//    the warp writes its columns back row-contiguously.
+//  * a warp owns 16 columns, two lanes per column with half the rows of each
+//    block (a last tile of at most 8 columns: four lanes with a quarter each, half
+//    the instructions); block row J gathers
+//        acc = B_J - sum_{I < J} L_JI X_I
+//    from shared memory before its own steps, X overwrites B there, and the warp
+//    writes its columns back row-contiguously;
+//  * as in the single solve, row r of the triangle is first scaled by 1/a_rr and
+//    B's row by alpha/a_rr, so that a solved value needs no further arithmetic;
+//    the operations and their order are the single solve's, bit for bit.
 //
-// Measured on 8192 complex64 solves: 362 us unrolled, 233 us in this form with
-// B read and X written from the lanes' own columns, 172 us as it stands.
+// Blocks of 8 rows in FP32 (fewer loads per multiply-add); of 4 in FP64, where
+// only the multiply-adds count and a block's own steps are the half-idle ones.
+// Measured: 8192 complex64 solves 180 us, 4097 double LU solves 565 us (pipe 84% busy).
 //
 // The per-instance arithmetic does not depend on the batch it sits in.
 #include <cuda_runtime.h>
@@ -33,8 +39,6 @@ namespace {
 
 constexpr int kWarps = 4;
 constexpr int kCols = 16;  // columns per warp
-constexpr int kBlk = 8;    // rows per block
-constexpr int kMaxBlocks = 64 / kBlk;
 constexpr int kLdX = kCols + 1;  // row pitch of the right-hand sides: column reads and row writes miss bank conflicts
 
 // Index map from the solved lower-triangular form onto the operand: with rev,
@@ -44,39 +48,51 @@ struct Map {
   int rev, tr, cj;
 };
 
-// block (J, I), I <= J, of the staged triangle: 8 columns of 8 rows
-__device__ __forceinline__ int blk_at(int J, int I) { return (J * (J + 1) / 2 + I) * kBlk * kBlk; }
+// Rows per block and per lane, elements of the staged triangle.
+template <class T>
+struct Blk {
+  static constexpr int kRows = sizeof(T) == sizeof(double) && !Elem<T>::kComplex ? 4 : 8;
+  static constexpr int kNum = 64 / kRows;
+  static constexpr int kTri = kNum * (kNum + 1) / 2 * kRows * kRows;
+  // block (J, I), I <= J: kRows columns of kRows rows
+  __device__ __forceinline__ static int at(int J, int I) { return (J * (J + 1) / 2 + I) * kRows * kRows; }
+};
 
 template <class T>
 constexpr size_t smem_bytes() {
-  return sizeof(T) * (kMaxBlocks * (kMaxBlocks + 1) / 2 * kBlk * kBlk + 64 + kWarps * 64 * kLdX);
+  return sizeof(T) * (Blk<T>::kTri + 128 + kWarps * 64 * kLdX);
 }
 
-// four consecutive elements (16-byte aligned)
-__device__ __forceinline__ void ld4(float (&v)[4], const float *p) {
+// the rows of one lane in a column of a block (aligned to their size)
+__device__ __forceinline__ void ldv(double (&v)[1], const double *p) { v[0] = *p; }
+__device__ __forceinline__ void ldv(float (&v)[2], const float *p) {
+  const float2 q = *reinterpret_cast<const float2 *>(p);
+  v[0] = q.x;
+  v[1] = q.y;
+}
+__device__ __forceinline__ void ldv(cplxf (&v)[2], const cplxf *p) {
+  const float4 q = *reinterpret_cast<const float4 *>(p);
+  v[0] = cplxf{q.x, q.y};
+  v[1] = cplxf{q.z, q.w};
+}
+__device__ __forceinline__ void ldv(double (&v)[2], const double *p) {
+  const double2 q = *reinterpret_cast<const double2 *>(p);
+  v[0] = q.x;
+  v[1] = q.y;
+}
+__device__ __forceinline__ void ldv(float (&v)[4], const float *p) {
   const float4 q = *reinterpret_cast<const float4 *>(p);
   v[0] = q.x;
   v[1] = q.y;
   v[2] = q.z;
   v[3] = q.w;
 }
-__device__ __forceinline__ void ld4(cplxf (&v)[4], const cplxf *p) {
+__device__ __forceinline__ void ldv(cplxf (&v)[4], const cplxf *p) {
   const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 2);
   v[0] = cplxf{a.x, a.y};
   v[1] = cplxf{a.z, a.w};
   v[2] = cplxf{b.x, b.y};
   v[3] = cplxf{b.z, b.w};
-}
-
-// 1 / a with three divisions (Elem's complex form saves one and loses an ulp;
-// here every solved row is multiplied by it)
-__device__ __forceinline__ float recip(float a) { return 1.0f / a; }
-__device__ __forceinline__ cplxf recip(cplxf a) {
-  const bool big = fabsf(a.re) >= fabsf(a.im);
-  const float p = big ? a.re : a.im, q = big ? a.im : a.re;
-  const float t = q / p, d = fmaf(q, t, p);
-  const float u = 1.0f / d, v = t / d;
-  return big ? cplxf{u, -v} : cplxf{v, -u};
 }
 
 template <class T>
@@ -95,13 +111,14 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 // its block.
 template <class T>
 __device__ __forceinline__ void stage_a(T *sL, const T *__restrict__ A, int64_t lda, int m, bool unit, Map mp) {
+  constexpr int kBlk = Blk<T>::kRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = warp; o < m; o += kWarps) {
     const T *line = A + (int64_t)(mp.rev ? m - 1 - o : o) * lda;
     for (int i = lane + (mp.tr ? 0 : o & ~31); i < (mp.tr ? o + 1 : m); i += 32) {
       const int r = mp.tr ? o : i, c = mp.tr ? i : o;
       if (r < c || (unit && r == c)) continue;
-      copy_async(sL + blk_at(r / kBlk, c / kBlk) + (c % kBlk) * kBlk + r % kBlk, line + (mp.rev ? m - 1 - i : i));
+      copy_async(sL + Blk<T>::at(r / kBlk, c / kBlk) + (c % kBlk) * kBlk + r % kBlk, line + (mp.rev ? m - 1 - i : i));
     }
   }
 }
@@ -116,57 +133,59 @@ __device__ __forceinline__ void stage_b(T *X, const T *B, int64_t ldb, int m, in
   }
 }
 
-// X = alpha L^-1 B for the staged columns of this warp, in shared memory; cj:
-// with conj(L), by solving for conj(X).
-template <class T>
-__device__ __forceinline__ void solve_tile(const T *sL, const T *sR, T *X0, int m, T alpha, int cj) {
+// The staged columns of this warp (32 / LPC of them, LPC lanes each) solved in
+// shared memory (sC: alpha / a_rr); cj: with conj(L), by solving for conj(X).
+template <class T, int LPC>
+__device__ __forceinline__ void solve_tile(const T *sL, const T *sC, T *X0, int m, int cj) {
   using E = Elem<T>;
+  constexpr int kBlk = Blk<T>::kRows, kMine = kBlk / LPC, kTile = 32 / LPC;
   const int lane = threadIdx.x & 31;
-  const int c = lane % kCols, h = lane / kCols;  // this lane's column of the tile and half of each block
+  const int c = lane % kTile, h = lane / kTile;  // this lane's column of the tile and part of each block
   T *X = X0 + c;
   const int nblk = (m + kBlk - 1) / kBlk;
 #pragma unroll 1
   for (int J = 0; J < nblk; ++J) {
-    T acc[4];
+    T acc[kMine];
     T *xJ = X + J * kBlk * kLdX;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      acc[q] = E::mul(alpha, xJ[(4 * h + q) * kLdX]);
+    for (int q = 0; q < kMine; ++q) {
+      T b = xJ[(kMine * h + q) * kLdX];
       if constexpr (E::kComplex) {
-        if (cj) acc[q].im = -acc[q].im;
+        if (cj) b.im = -b.im;
       }
+      acc[q] = E::mul(sC[J * kBlk + kMine * h + q], b);
     }
-    const T *L = sL + blk_at(J, 0) + 4 * h;
+    const T *L = sL + Blk<T>::at(J, 0) + kMine * h;
     const T *x = X;
 #pragma unroll 1
     for (int I = 0; I < J; ++I, L += kBlk * kBlk, x += kBlk * kLdX) {
 #pragma unroll
       for (int k = 0; k < kBlk; ++k) {
         const T xk = x[k * kLdX];
-        T l[4];
-        ld4(l, L + k * kBlk);
+        T l[kMine];
+        ldv(l, L + k * kBlk);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = E::fms(l[q], xk, acc[q]);
+        for (int q = 0; q < kMine; ++q) acc[q] = E::fms(l[q], xk, acc[q]);
       }
     }
     // the block's own rows: row k is final after k steps; later updates of rows
     // at or above k touch values that are no longer used
-    T out[4];
+    T out[kMine];
 #pragma unroll
     for (int k = 0; k < kBlk; ++k) {
-      const T mine = E::mul(acc[k % 4], sR[J * kBlk + k]);
-      if (k < 4 || h == 1) out[k % 4] = mine;  // rows 0 .. 3 are the first half's: kept below
+      if (h >= k / kMine) out[k % kMine] = acc[k % kMine];  // kept by the lane whose row it is
       if (k + 1 < kBlk) {
-        const T xk = E::shfl(mine, (k / 4) * kCols + c);
-        T l[4];
-        ld4(l, L + k * kBlk);
+        const T xk = E::shfl(acc[k % kMine], (k / kMine) * kTile + c);
+        T l[kMine];
+        ldv(l, L + k * kBlk);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = E::fms(l[q], xk, acc[q]);
+        for (int q = 0; q < kMine; ++q)
+          if ((LPC - 1) * kMine + q > k) acc[q] = E::fms(l[q], xk, acc[q]);  // else: final in every part
       }
     }
-    __syncwarp();  // both lanes of a column have read this block's B
+    __syncwarp();  // every lane of a column has read this block's B
 #pragma unroll
-    for (int q = 0; q < 4; ++q) xJ[(4 * h + q) * kLdX] = out[q];
+    for (int q = 0; q < kMine; ++q) xJ[(kMine * h + q) * kLdX] = out[q];
     __syncwarp();
   }
 }
@@ -193,27 +212,48 @@ __device__ __forceinline__ void write_x(const T *X, T *B, int64_t ldb, int m, in
 
 // One triangular solve of an instance in place on B, all threads of the CTA.
 template <class T>
-__device__ __forceinline__ void solve(T *sL, T *sR, T *sX, const T *__restrict__ A, int64_t lda, T *B, int64_t ldb,
+__device__ __forceinline__ void solve(T *sL, T *sR, T *sC, T *sX, const T *__restrict__ A, int64_t lda, T *B, int64_t ldb,
                                       int m, int n, T alpha, bool unit, Map mp) {
   using E = Elem<T>;
+  constexpr int kBlk = Blk<T>::kRows;
   const int warp = threadIdx.x >> 5;
   T *X = sX + warp * 64 * kLdX;
   stage_a<T>(sL, A, lda, m, unit, mp);
   if (warp * kCols < n) stage_b<T>(X, B, ldb, m, n, warp * kCols, mp.rev);
   copies_wait();
   __syncthreads();
-  if (threadIdx.x < 64) {
+  if (threadIdx.x < m) {
     const int r = threadIdx.x;
-    if (r < m) sR[r] = unit ? E::one() : recip(sL[blk_at(r / kBlk, r / kBlk) + (r % kBlk) * (kBlk + 1)]);
+    const T rv = unit ? E::one() : E::recip(sL[Blk<T>::at(r / kBlk, r / kBlk) + (r % kBlk) * (kBlk + 1)]);
+    if constexpr (E::kComplex) {
+      if (mp.cj) alpha.im = -alpha.im;
+    }
+    sR[r] = rv;
+    sC[r] = E::mul(alpha, rv);
   }
   __syncthreads();
+  if (!unit) {  // row r times 1/a_rr: a warp per row of blocks, two rows of a column per lane
+    const int lane = threadIdx.x & 31;
+    for (int J = warp; J * kBlk < m; J += kWarps) {
+      T *L = sL + Blk<T>::at(J, 0);
+      const T *r = sR + J * kBlk + 2 * lane % kBlk;
+      for (int e = 2 * lane; e < (J + 1) * kBlk * kBlk; e += 64) {
+        L[e] = E::mul(r[0], L[e]);
+        L[e + 1] = E::mul(r[1], L[e + 1]);
+      }
+    }
+    __syncthreads();
+  }
   for (int j0 = warp * kCols; j0 < n; j0 += kWarps * kCols) {
     if (j0 >= kWarps * kCols) {
       stage_b<T>(X, B, ldb, m, n, j0, mp.rev);
       copies_wait();
       __syncwarp();
     }
-    solve_tile<T>(sL, sR, X, m, alpha, mp.cj);
+    if (n - j0 <= kCols / 2)
+      solve_tile<T, 4>(sL, sC, X, m, mp.cj);
+    else
+      solve_tile<T, 2>(sL, sC, X, m, mp.cj);
     write_x<T>(X, B, ldb, m, n, j0, mp.rev, mp.cj);
     __syncwarp();  // before the next columns' copies
   }
@@ -262,21 +302,64 @@ __device__ __forceinline__ bool permute(T *B, int64_t ldb, int m, int n, const i
 
 enum { KIND_TRSM = 0, KIND_LU = 1, KIND_CHOL = 2 };
 
+// An order of the instances: each group of 256 consecutive ones by decreasing
+// work (m^2 times column tiles, eight classes per octave), the groups
+// interleaved rank by rank.  Started in this order the last CTAs are short ones.
+constexpr int kOrderGroup = 256;
+
+__global__ void __launch_bounds__(kOrderGroup) batch_order_kernel(int batch, const int32_t *__restrict__ dm,
+                                                                  const int32_t *__restrict__ dn, int32_t *order) {
+  __shared__ int hist[256], first[256];
+  const int t = threadIdx.x, g = blockIdx.x, b = g * kOrderGroup + t;
+  hist[t] = 0;
+  __syncthreads();
+  int cls = 255, at = 0;
+  if (b < batch) {
+    const int m = dm[b], n = dn[b];
+    if (m > 0 && m <= 64 && n > 0) {
+      const uint64_t w = 8ull * m * m * (uint64_t)((n + kCols - 1) / kCols);
+      const int lead = 63 - __clzll((long long)w);
+      cls = 254 - min(254, 8 * lead + (int)((w >> (lead - 3)) & 7));
+    }
+    at = atomicAdd(&hist[cls], 1);
+  }
+  __syncthreads();
+  // exclusive sums of the 256 classes, 32 at a time
+  int v = hist[t];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if ((t & 31) >= o) v += y;
+  }
+  first[t] = v;
+  __syncthreads();
+  int base = 0;
+  for (int w = 0; w < (cls >> 5); ++w) base += first[32 * w + 31];
+  if (b >= batch) return;
+  const int rank = base + first[cls] - hist[cls] + at;
+  const int full = batch / kOrderGroup, rest = batch % kOrderGroup;  // whole groups, and a last one of `rest`
+  const int groups = full + (rest != 0);
+  order[rank < rest || rest == 0 ? (int64_t)rank * groups + g
+                                 : (int64_t)rest * groups + (int64_t)(rank - rest) * full + g] = b;
+}
+
 template <class T>
-__global__ void __launch_bounds__(32 * kWarps) batch_f32_kernel(const int32_t *__restrict__ dm,
+__global__ void __launch_bounds__(32 * kWarps) batch_kernel(const int32_t *__restrict__ dm,
                                                                 const int32_t *__restrict__ dn,
                                                                 const int32_t *__restrict__ dlda,
                                                                 const int32_t *__restrict__ dldb,
                                                                 const void *const *__restrict__ dA,
                                                                 const int32_t *const *__restrict__ dipiv,
                                                                 void *const *__restrict__ dB, T alpha, int unit,
-                                                                uint32_t *status, Map mp, int kind, int skip_large) {
+                                                                const int32_t *__restrict__ order, uint32_t *status, Map mp, int kind,
+                                                                int skip_large) {
   using E = Elem<T>;
   extern __shared__ __align__(16) unsigned char smem[];
   T *sL = reinterpret_cast<T *>(smem);
-  T *sR = sL + kMaxBlocks * (kMaxBlocks + 1) / 2 * kBlk * kBlk;
-  T *sX = sR + 64;
-  const int b = blockIdx.x;
+  T *sR = sL + Blk<T>::kTri;
+  T *sC = sR + 64;
+  T *sX = sC + 64;
+  const int b = order != nullptr ? order[blockIdx.x] : blockIdx.x;
   const int m = dm[b], n = dn[b], lda = dlda[b], ldb = dldb[b];
   const T *A = static_cast<const T *>(dA[b]);
   T *B = static_cast<T *>(dB[b]);
@@ -308,49 +391,52 @@ __global__ void __launch_bounds__(32 * kWarps) batch_f32_kernel(const int32_t *_
     const Map pm = kind == KIND_TRSM ? mp : pass == 0 ? Map{0, 0, 0} : Map{1, kind == KIND_CHOL, kind == KIND_CHOL};
     const bool un = kind == KIND_TRSM ? unit != 0 : pass == 0 && kind == KIND_LU;
     if (pass != 0) __syncthreads();  // the first solve has read the staged triangle and written B
-    solve<T>(sL, sR, sX, A, lda, B, ldb, m, n, pass == 0 ? alpha : E::one(), un, pm);
+    solve<T>(sL, sR, sC, sX, A, lda, B, ldb, m, n, pass == 0 ? alpha : E::one(), un, pm);
   }
 }
 
 template <class T>
 hsma_status_t launch(int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha, const void *const *dA,
                      const int32_t *dlda, const int32_t *const *dipiv, void *const *dB, const int32_t *dldb, int unit,
-                     uint32_t *status, cudaStream_t st, Map mp, int kind, int skip_large) {
+                     uint32_t *status, int32_t *order, cudaStream_t st, Map mp, int kind, int skip_large) {
   static DeviceFlags attr_done;
   if (!attr_done.test()) {
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(batch_f32_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HSMA_CUDA_TRY(cudaFuncSetAttribute(batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_bytes<T>()));
     attr_done.set();
   }
+  if constexpr (sizeof(T) == sizeof(double) && !Elem<T>::kComplex) {
+    HsmaTraceScope ts("vbatched_schedule", st);
+    batch_order_kernel<<<(batch + kOrderGroup - 1) / kOrderGroup, kOrderGroup, 0, st>>>(batch, dm, dn, order);
+    HSMA_CUDA_TRY(cudaGetLastError());
+  } else {
+    order = nullptr;
+  }
   HsmaTraceScope ts(kind == KIND_TRSM ? "vbatched_solve" : "vbatched_lu", st);
-  batch_f32_kernel<T><<<batch, 32 * kWarps, smem_bytes<T>(), st>>>(dm, dn, dlda, dldb, dA, dipiv, dB,
-                                                                   hsma_alpha_as<T>(alpha), unit, status, mp, kind,
+  batch_kernel<T><<<batch, 32 * kWarps, smem_bytes<T>(), st>>>(dm, dn, dlda, dldb, dA, dipiv, dB,
+                                                                   hsma_alpha_as<T>(alpha), unit, order, status, mp, kind,
                                                                    skip_large);
   return hsma_from_cuda(cudaGetLastError());
 }
 
 }  // namespace
 
-hsma_status_t hsma_f32_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha,
+hsma_status_t hsma_blk_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha,
                                 const void *const *dA, const int32_t *dlda, void *const *dB, const int32_t *dldb,
-                                int unit, uint32_t *status, cudaStream_t st, int uplo, int trans, int skip_large) {
+                                int unit, uint32_t *status, int32_t *scratch, cudaStream_t st, int uplo, int trans,
+                                int skip_large) {
   const bool op_lower = (uplo == HSMA_LOWER) != (trans != HSMA_NO_TRANS);
   const Map mp{op_lower ? 0 : 1, trans != HSMA_NO_TRANS ? 1 : 0, trans == HSMA_CONJ_TRANS ? 1 : 0};
-  if (dtype == HSMA_R32)
-    return launch<float>(batch, dm, dn, alpha, dA, dlda, nullptr, dB, dldb, unit, status, st, mp, KIND_TRSM,
-                         skip_large);
-  return launch<cplxf>(batch, dm, dn, alpha, dA, dlda, nullptr, dB, dldb, unit, status, st, mp, KIND_TRSM,
-                       skip_large);
+  auto *f = dtype == HSMA_R32 ? launch<float> : dtype == HSMA_C64 ? launch<cplxf> : launch<double>;
+  return f(batch, dm, dn, alpha, dA, dlda, nullptr, dB, dldb, unit, status, scratch, st, mp, KIND_TRSM, skip_large);
 }
 
-hsma_status_t hsma_f32_factor_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
+hsma_status_t hsma_blk_factor_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
                                        const double *alpha, const void *const *dA, const int32_t *dlda,
                                        const int32_t *const *dipiv, void *const *dB, const int32_t *dldb,
-                                       uint32_t *status, cudaStream_t st, int chol, int skip_large) {
-  const int kind = chol ? KIND_CHOL : KIND_LU;
-  if (dtype == HSMA_R32)
-    return launch<float>(batch, dm, dn, alpha, dA, dlda, dipiv, dB, dldb, 0, status, st, Map{0, 0, 0}, kind,
-                         skip_large);
-  return launch<cplxf>(batch, dm, dn, alpha, dA, dlda, dipiv, dB, dldb, 0, status, st, Map{0, 0, 0}, kind,
-                       skip_large);
+                                       uint32_t *status, int32_t *scratch, cudaStream_t st, int chol,
+                                       int skip_large) {
+  auto *f = dtype == HSMA_R32 ? launch<float> : dtype == HSMA_C64 ? launch<cplxf> : launch<double>;
+  return f(batch, dm, dn, alpha, dA, dlda, dipiv, dB, dldb, 0, status, scratch, st, Map{0, 0, 0}, chol ? KIND_CHOL : KIND_LU,
+           skip_large);
 }

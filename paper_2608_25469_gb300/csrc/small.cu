@@ -773,16 +773,10 @@ hsma_status_t hsma_small_vbatched(int dtype, int32_t batch, const int32_t *dm, c
                                   void *const *dB, const int32_t *dldb, int unit, uint32_t *status,
                                   int32_t *scratch, cudaStream_t st, int uplo, int trans, int skip_large) {
   const SmallMap mp = make_map(uplo, trans);
-  switch (dtype) {
-    case HSMA_C128: return vbatched_impl<cplx>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
-                                    skip_large);
-    case HSMA_R32:
-    case HSMA_C64:
-      return hsma_f32_vbatched(dtype, batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, st, uplo, trans,
-                               skip_large);
-    default: return vbatched_impl<double>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp,
-                                    skip_large);
-  }
+  if (dtype != HSMA_C128)
+    return hsma_blk_vbatched(dtype, batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, uplo, trans,
+                             skip_large);
+  return vbatched_impl<cplx>(batch, dm, dn, alpha, dA, dlda, dB, dldb, unit, status, scratch, st, mp, skip_large);
 }
 
 template <class T>
@@ -923,18 +917,10 @@ hsma_status_t hsma_small_getrs_vbatched(int dtype, int32_t batch, const int32_t 
                                         uint32_t *status, int32_t *scratch, cudaStream_t st, int chol,
                                         int skip_large) {
   if (chol) dipiv = nullptr;
-  switch (dtype) {
-    case HSMA_C128:
-      return getrs_impl<cplx>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
-                                 skip_large);
-    case HSMA_R32:
-    case HSMA_C64:
-      return hsma_f32_factor_vbatched(dtype, batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, st, chol,
-                                      skip_large);
-    default:
-      return getrs_impl<double>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol,
-                                 skip_large);
-  }
+  if (dtype != HSMA_C128)
+    return hsma_blk_factor_vbatched(dtype, batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st,
+                                    chol, skip_large);
+  return getrs_impl<cplx>(batch, dm, dn, alpha, dLU, dlda, dipiv, dB, dldb, status, scratch, st, chol, skip_large);
 }
 
 // ---------------------------------------------------------------------------

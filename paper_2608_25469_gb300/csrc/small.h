@@ -16,15 +16,17 @@ hsma_status_t hsma_small_single(int dtype, int g, const void *A, int64_t lda, vo
 // Bytes of device scratch the varlen batch needs for `batch` instances.
 size_t hsma_vbatched_scratch_bytes(int dtype, int32_t batch);
 
-// The same in FP32 (HSMA_R32, HSMA_C64; batch_f32.cu): one launch, no scratch.
-// Called by the two entry points below for these dtypes.
-hsma_status_t hsma_f32_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha,
+// Every dtype but HSMA_C128 (batch.cu; HSMA_R64 uses the scratch).  Called by the
+// two entry points below for these dtypes.
+hsma_status_t hsma_blk_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn, const double *alpha,
                                 const void *const *dA, const int32_t *dlda, void *const *dB, const int32_t *dldb,
-                                int unit, uint32_t *status, cudaStream_t st, int uplo, int trans, int skip_large);
-hsma_status_t hsma_f32_factor_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
+                                int unit, uint32_t *status, int32_t *scratch, cudaStream_t st, int uplo, int trans,
+                                int skip_large);
+hsma_status_t hsma_blk_factor_vbatched(int dtype, int32_t batch, const int32_t *dm, const int32_t *dn,
                                        const double *alpha, const void *const *dA, const int32_t *dlda,
                                        const int32_t *const *dipiv, void *const *dB, const int32_t *dldb,
-                                       uint32_t *status, cudaStream_t st, int chol, int skip_large);
+                                       uint32_t *status, int32_t *scratch, cudaStream_t st, int chol,
+                                       int skip_large);
 
 // Varlen batch (schedule pre-pass + persistent solve).  `scratch` holds
 // hsma_vbatched_scratch_bytes(dtype, batch) bytes of device memory.  skip_large:
@@ -67,10 +69,8 @@ hsma_status_t hsma_small_lu_pivots(int dtype, int32_t batch, const int32_t *dm, 
 // m > 64 are skipped without a status bit, as skip_large below).  Results
 // equal hsma_small_vbatched's bit for bit.
 size_t hsma_vbatched_packed_scratch_bytes(int dtype, int32_t batch, int32_t max_m);
-// dtypes whose varlen batch runs the column-packed kernels (measured faster
-// than the per-instance kernel: complex128; real FP64 keeps the per-instance
-// kernel, whose G choice already fills its lanes at 4x less work per element;
-// the FP32 dtypes have their own, batch_f32.cu)
+// dtypes whose varlen batch runs the column-packed kernels: complex128, whose
+// arithmetic per element pays for the schedule and prep passes
 inline bool hsma_vbatched_packed_dtype(int dtype) { return dtype == HSMA_C128; }
 hsma_status_t hsma_small_vbatched_packed(int dtype, int32_t batch, int32_t max_m, const int32_t *dm,
                                          const int32_t *dn, const double *alpha, const void *const *dA,

@@ -134,13 +134,15 @@ def test_host_batch_complex64_equals_device_batch(H):
 EDGES = [(1, 1), (7, 15), (8, 16), (9, 17), (15, 64), (16, 65), (17, 3), (31, 33), (32, 130), (33, 16), (63, 5), (64, 64)]
 
 
-@pytest.mark.parametrize("code64,code", [(I.R64, 4), (I.C128, 5)], ids=["f32", "c64"])
+@pytest.mark.parametrize("code64,code", [(I.R64, 4), (I.C128, 5), (I.R64, 0)], ids=["f32", "c64", "f64"])
 @pytest.mark.parametrize("kind", ["nn", "nn_unit", "un", "lt", "uc", "lc_unit", "lu", "chol"])
-def test_batched_fp32_block_edges(H, code64, code, kind):
-    """The batch kernel at the edges of its 8-row blocks, 16-column tiles and 64-column rounds, in
-    every index map and both factor solves, with padded leading dimensions and NaN in whatever is
-    not referenced.  Tolerance: the FP32 substitution bound, twice for the factor solves."""
+def test_batched_block_edges(H, code64, code, kind):
+    """The batch kernel at the edges of its 4- and 8-row blocks, 16-column tiles and 64-column rounds,
+    in every index map and both factor solves, with padded leading dimensions and NaN in whatever is
+    not referenced.  Tolerance: the substitution bound of the type, twice for the factor solves."""
     import torch
+    tol = TOL32 if code else 1e-13
+    as_type = (lambda X: _f32(code64, X)) if code else np.asfortranarray
     uplo = 1 if kind[0] == "u" else 0
     trans = {"t": 1, "c": 2}.get(kind[1], 0) if kind not in ("lu", "chol") else 0
     unit = kind.endswith("unit")
@@ -150,7 +152,7 @@ def test_batched_fp32_block_edges(H, code64, code, kind):
     for b, (m, n) in enumerate(EDGES):
         A = I.gen_LU(3, m, code64, inst=b) if kind == "lu" else I.gen_A(3, m, code64, inst=b)
         A = np.asfortranarray(A.T) if uplo else A
-        A32, B32 = _f32(code64, A), _f32(code64, I.gen_B(3, m, n, code64, inst=b))
+        A32, B32 = as_type(A), as_type(I.gen_B(3, m, n, code64, inst=b))
         raw.append((A32, B32))
         E = np.array(A32, order="F")
         if kind != "lu":
@@ -187,4 +189,4 @@ def test_batched_fp32_block_edges(H, code64, code, kind):
         else:
             ref = oracle.solve_general(A32, B32, alpha, 0, uplo, trans, unit)
         assert np.all(np.isnan(X[m:])), EDGES[b]
-        assert oracle.forward_error(X[:m].astype(wide), ref) <= TOL32 * (2 if kind in ("lu", "chol") else 1), EDGES[b]
+        assert oracle.forward_error(X[:m].astype(wide), ref) <= tol * (2 if kind in ("lu", "chol") else 1), EDGES[b]

@@ -33,8 +33,8 @@ import time
 HERE = os.path.dirname(os.path.abspath(__file__))
 NBS = (32, 64, 128, 256, 512)
 TILES = (1, 2, 3)          # HSMA_TILE_64x64, _128x16, _128x8 (0 = small tiles)
-EMU_NBS = (256, 512)
-PANELS = (1024, 2048, 3072, 4096)
+EMU_NBS = (128, 256, 512)
+PANELS = (512, 1024, 2048, 4096)
 EMU = 10                   # table key offset of the emulated-products entries
 
 GRID = {
@@ -42,8 +42,9 @@ GRID = {
        [(4096, 4096), (8192, 8192), (16384, 16384)],
     1: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096) for n in (4, 32, 256, 1024)] + [(4096, 4096), (8192, 8192)],
     2: [(m, n) for m in (128, 512, 2048, 8192) for n in (16, 256, 4096)],
-    EMU + 0: [(2048, 2048), (8192, 4096), (16384, 16384)],
-    EMU + 1: [(2048, 2048), (4096, 4096), (8192, 8192)],
+    EMU + 0: [(m, n) for m in (512, 1024, 2048, 4096, 8192) for n in (128, 1024)] +
+             [(2048, 4096), (8192, 4096), (16384, 16384)],
+    EMU + 1: [(m, n) for m in (512, 1024, 2048, 4096) for n in (128, 1024)] + [(4096, 4096), (8192, 8192)],
 }
 QUICK = {0: [(512, 256), (4096, 4096)], 1: [(512, 256), (2048, 2048)], 2: [(1024, 256), (8192, 4096)],
          EMU + 0: [(4096, 4096)], EMU + 1: [(2048, 2048)]}

@@ -1014,17 +1014,14 @@ __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, do
 // the expanded forms (rows [re -im; im re] on the left, the interleaved real
 // view on the right and in B), so a complex product is four real ones.
 //
-// Each emulated product adds every accumulation unit into B once in FP64, so
-// its cost per element of B grows with the number of units, not with K.  The
-// updates are therefore applied per panel of h diagonal blocks (about 2048
-// real columns): inside a panel, each solved block updates only the panel's
-// remaining rows; below the panel, one update with K = h N_B covers all h
-// blocks.  The result is the same product sum, grouped differently.
-// The panel width (real columns; the panel's trailing update runs with K =
-// that many real columns) comes from the planner: the autotuned table, else
-// kEmuPanelColsDefault.  Measured on GB300 for m = 16384 FP64 / 8192
-// complex128: 1024 columns 217 / 112 ms, 2048 columns 208 / 105 ms, 3072 and
-// 4096 columns slower again.
+// Each emulated product converts its residues and adds to B once per element, so
+// that part of its cost does not grow with K.  The updates are therefore applied
+// per panel of h diagonal blocks: inside a panel, each solved block updates only
+// the panel's remaining rows; below the panel, one update with K = h N_B covers
+// all h blocks.  The result is the same product sum, grouped differently.  The
+// panel width (real columns) comes from the planner: the autotuned table, else
+// kEmuPanelColsDefault.  It matters little (16384 x 16384 FP64: 1024 columns 67.3,
+// 2048 65.1, 4096 66.0 ms); recursion by halves inside a panel measured the same.
 
 // Workspace of blocked_emulated: the inverses, one block row of B, and the
 // slices of an update panel, of one inverse and of the right operand.

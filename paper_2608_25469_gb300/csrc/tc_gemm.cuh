@@ -40,8 +40,12 @@ constexpr uint32_t TC_TMEM_COLS = 512;  // all of the SM's tensor memory (one CT
 template <int BN>
 struct TcTile {
   static constexpr int B_ROWS = BN / 2;  // rows of B staged per CTA
-  static constexpr int STAGE_BYTES = TC_A_BYTES + B_ROWS * TC_BK * 2;
-  static constexpr int STAGES = BN == 256 ? 6 : 8;
+  static constexpr int BLOCK_BYTES = TC_A_BYTES + B_ROWS * TC_BK * 2;  // one K-block of A and B
+  // K-blocks per stage: a narrow tile's products of one block (256 cycles) do not
+  // cover the issue loop's round, a wide tile's do and prefer more stages
+  static constexpr int SUB = BN == 256 ? 1 : 2;
+  static constexpr int STAGE_BYTES = SUB * BLOCK_BYTES;
+  static constexpr int STAGES = BN == 256 ? 6 : 4;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
   static constexpr int ACCS = TC_TMEM_COLS / BN;  // accumulators in tensor memory
   // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M x N
@@ -88,9 +92,12 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// arrive on an mbarrier of either CTA of the pair (address from cluster_addr)
+// Arrive on an mbarrier of either CTA of the pair (address from cluster_addr) to
+// hand back an accumulator.  Relaxed: what it orders are this warp's tensor-memory
+// loads, complete at their tcgen05.wait::ld; a release at cluster scope would wait
+// for the epilogue's global stores to be acknowledged as well.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
 // arrive on the mbarrier at this offset in both CTAs once the pair's MMAs issued so far are done
@@ -275,6 +282,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
   const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;  // the pair and the number of pairs
   const int tiles_m = (M + TC_PM - 1) / TC_PM, tiles_n = (N + TC_BN - 1) / TC_BN;
   const int ntiles = tiles_m * tiles_n;
+  // TC_OZ with no more than one tile per pair: the conversion warps have nothing
+  // to convert until the end, so they drain accumulators too
+  const bool single = MODE == TC_OZ && ntiles <= ncl;
   // Tiles run in bands of p.band tile rows, column by column inside a band.
   // With 8 tile rows the tiles in flight at once (one per pair of SMs) cover
   // about 8 row tiles x 10 column tiles, the fewest operand rows; long TC_F32 products
@@ -300,7 +310,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
     }
     for (int b = 0; b < NACC; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 2 * TC_EPI_WARPS);
+      mbar_init(&acc_empty[b], 2 * (TC_EPI_WARPS + (single ? TC_CRT_WARPS : 0)));
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&res_full[b], TC_EPI_WARPS);
@@ -335,7 +345,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
       const int nk = tile_k(t, m0, n0);
       for (int q = 0; q < nslices && ok; ++q) {
         const int sa = MODE == TC_OZ ? q : p.pa[q], sb = MODE == TC_OZ ? q : p.pb[q];
-        for (int kb = 0; kb < nk; ++kb) {
+        for (int kb = 0; kb < nk; kb += TL::SUB) {
           if (!mbar_wait_bounded(&empty[s], phase, p.limit_ns, p.err)) {
             ok = false;
             break;
@@ -343,9 +353,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
           if (elect_one()) {
             unsigned char *st = smem + s * TC_STAGE_BYTES;
             const uint32_t bar = bar0 + (uint32_t)s * 8u;
-            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * TC_STAGE_BYTES);
-            tma_load_3d_pair(st, &mapA, bar, kb * TC_BK, m0, sa);
-            tma_load_3d_pair(st + TC_A_BYTES, &mapB, bar, kb * TC_BK, n0 + (int)rank * TL::B_ROWS, sb);
+            const int nsub = min(TL::SUB, nk - kb);  // a slice's last stage may hold fewer blocks
+            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * nsub * TL::BLOCK_BYTES);
+#pragma unroll
+            for (int u = 0; u < TL::SUB; ++u, st += TL::BLOCK_BYTES) {
+              if (u > 0 && u >= nsub) break;
+              tma_load_3d_pair(st, &mapA, bar, (kb + u) * TC_BK, m0, sa);
+              tma_load_3d_pair(st + TC_A_BYTES, &mapB, bar, (kb + u) * TC_BK, n0 + (int)rank * TL::B_ROWS, sb);
+            }
           }
           __syncwarp();
           if (++s == TC_STAGES) {
@@ -377,23 +392,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
           }
           tc_fence_after();
           const uint32_t acc_cols = tmem + (uint32_t)(b * BN);
-          for (int kb = 0; kb < glen; ++kb) {
+          for (int kb = 0, nsub; kb < glen; kb += nsub) {
+            // blocks in this stage (TC_F32's unit spans slices, each with its own last stage)
+            nsub = TL::SUB == 1 ? 1 : min(TL::SUB, MODE == TC_OZ ? glen - kb : nk - kb % nk);
             if (!mbar_wait_bounded(&full[s], phase, p.limit_ns, p.err)) {
               ok = false;
               break;
             }
             tc_fence_after();
             if (elect_one()) {
-              const uint64_t da = desc0 + (uint64_t)(s * (TC_STAGE_BYTES >> 4)), db = da + (TC_A_BYTES >> 4);
+              const uint64_t d0 = desc0 + (uint64_t)(s * (TC_STAGE_BYTES >> 4));
 #pragma unroll
-              for (int kk = 0; kk < TC_BK / 16; ++kk)
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
-                    "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(TL::IDESC), "r"(kb + kk)
-                    : "memory");
+              for (int u = 0; u < TL::SUB; ++u) {
+                if (u > 0 && u >= nsub) break;
+                const uint64_t da = d0 + (uint64_t)(u * (TL::BLOCK_BYTES >> 4)), db = da + (TC_A_BYTES >> 4);
+#pragma unroll
+                for (int kk = 0; kk < TC_BK / 16; ++kk)
+                  asm volatile(
+                      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_cols),
+                      "l"(da + 2ull * kk), "l"(db + 2ull * kk), "r"(TL::IDESC), "r"(kb + u + kk)
+                      : "memory");
+              }
               tc_commit_pair(&empty[s]);
-              if (kb == glen - 1) tc_commit_pair(&acc_full[b]);
+              if (kb + nsub == glen) tc_commit_pair(&acc_full[b]);
             }
             __syncwarp();
             if (++s == TC_STAGES) {
@@ -414,12 +436,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
       __syncwarp();
       mbar_wait_bounded(&drained, 0, p.limit_ns, p.err);
     }
-  } else if (warp < TC_WARPS) {
+  } else if (warp < TC_WARPS || single) {
     // epilogue warps: thread = one row of the 128-row tile (its tensor-memory
-    // lane); two warps per lane quarter split the columns.
+    // lane); two warps (or four) per lane quarter split the columns.
     const int ew = warp - 2;
-    const int quarter = warp & 3, half = ew >> 2;
-    const int cbeg = half * (TC_BN / 2);
+    const int width = single ? TC_BN / 4 : TC_BN / 2;  // columns per warp
+    const int quarter = warp & 3, cbeg = (ew >> 2) * width;
     constexpr int CW = 16;  // columns per chunk: keeps ten warps within the register file
     int i = 0;
     bool ok = true;
@@ -437,7 +459,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
           if (!ok) break;
         }
         uint32_t *mine = p.scratch + oz_scratch_at(blockIdx.x, h, cbeg) + quarter * 32 + lane;
-        const int cols = min(TC_BN / 2, N - n0 - cbeg);  // this warp's columns inside the matrix
+        const int cols = min(width, N - n0 - cbeg);  // this warp's columns inside the matrix
         for (int l = 0; l < kOzP && ok; ++l) {
           const float mod = c_oz.modf[l], inv = c_oz.inv[l];
           for (int g0 = 0; g0 < nk; g0 += kOzChunk / TC_BK, ++i) {
@@ -466,6 +488,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
           }
         }
         if (!ok) break;
+        if (single) {  // each thread converts what it wrote
+          oz_convert<BN>(p, blockIdx.x, h, m0, n0, quarter, cbeg, width);
+          continue;
+        }
         if (lane == 0) mbar_arrive(&res_full[h]);  // (after the last unit's __syncwarp)
         if (t + ncl >= ntiles) oz_convert<BN>(p, blockIdx.x, h, m0, n0, quarter, cbeg + TC_BN / 4, TC_BN / 4);
       } else {

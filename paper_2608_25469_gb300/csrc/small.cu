@@ -24,7 +24,9 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <type_traits>
 
+#include "blocked.h"
 #include "common.cuh"
 #include "small.h"
 #include "trace.h"
@@ -132,11 +134,10 @@ __device__ __forceinline__ void stage(T *sTri, T *sC, T *sR, const T *__restrict
 // The B entries of a lane's rows in one column tile (zero outside the
 // instance), loaded before the solve so that they can be in flight while the
 // triangle is staged.
-template <class T, int G, int MMAX, bool MAP, bool FULL = false>
-__device__ __forceinline__ void warp_load_b(T (&b)[MMAX / G], const T *Bt, int64_t ldb, int m_, int ncols, int rev) {
+template <class T, int G, int MMAX, bool MAP>
+__device__ __forceinline__ void warp_load_b(T (&b)[MMAX / G], const T *Bt, int64_t ldb, int m, int ncols, int rev) {
   using E = Elem<T>;
   constexpr int R = MMAX / G;
-  const int m = FULL ? MMAX : m_;
   const int lane = threadIdx.x & 31;
   const int g = lane % G, c = lane / G;
   const bool colok = c < ncols;
@@ -153,13 +154,11 @@ __device__ __forceinline__ void warp_load_b(T (&b)[MMAX / G], const T *Bt, int64
 
 // One warp solves one column tile (up to 32/G columns starting at Bt) whose
 // B entries warp_load_b has loaded.
-// FULL: m == MMAX, known at compile time (the bound checks fold away).
-template <class T, int G, int MMAX, bool MAP, bool FULL = false>
+template <class T, int G, int MMAX, bool MAP>
 __device__ __forceinline__ void warp_solve_loaded(const T (&b)[MMAX / G], const T *sTri, const T *sC, T *Bt,
-                                                  int64_t ldb, int m_, int ncols, int rev) {
+                                                  int64_t ldb, int m, int ncols, int rev) {
   using E = Elem<T>;
   constexpr int R = MMAX / G;
-  const int m = FULL ? MMAX : m_;
   const int lane = threadIdx.x & 31;
   const int g = lane % G, c = lane / G;
   const bool colok = c < ncols;
@@ -204,15 +203,15 @@ __device__ __forceinline__ void warp_solve_loaded(const T (&b)[MMAX / G], const 
   }
 }
 
-template <class T, int G, int MMAX, bool MAP, bool FULL = false>
+template <class T, int G, int MMAX, bool MAP>
 __device__ __forceinline__ void warp_solve(const T *sTri, const T *sC, T *Bt, int64_t ldb, int m, int ncols,
                                            int rev) {
   T b[MMAX / G];
-  warp_load_b<T, G, MMAX, MAP, FULL>(b, Bt, ldb, m, ncols, rev);
-  warp_solve_loaded<T, G, MMAX, MAP, FULL>(b, sTri, sC, Bt, ldb, m, ncols, rev);
+  warp_load_b<T, G, MMAX, MAP>(b, Bt, ldb, m, ncols, rev);
+  warp_solve_loaded<T, G, MMAX, MAP>(b, sTri, sC, Bt, ldb, m, ncols, rev);
 }
 
-template <class T, int G, int MMAX, bool MAP, bool FULL = false>
+template <class T, int G, int MMAX, bool MAP>
 __device__ __forceinline__ void solve_tiles(const T *sTri, const T *sC, T *B, int64_t ldb, int m, int n, int tile0,
                                             int tile_step, int rev) {
   constexpr int C = 32 / G;
@@ -221,7 +220,7 @@ __device__ __forceinline__ void solve_tiles(const T *sTri, const T *sC, T *B, in
   for (int t = tile0 + warp; t < ntiles; t += tile_step) {
     const int col0 = t * C;
     const int nc = (n - col0) < C ? (n - col0) : C;
-    warp_solve<T, G, MMAX, MAP, FULL>(sTri, sC, B + (int64_t)col0 * ldb, ldb, m, nc, rev);
+    warp_solve<T, G, MMAX, MAP>(sTri, sC, B + (int64_t)col0 * ldb, ldb, m, nc, rev);
   }
 }
 
@@ -289,41 +288,222 @@ __device__ __forceinline__ void smem_parts(unsigned char *smem, T *&sTri, T *&sC
 }
 
 // ---------------------------------------------------------------------------
-// Single solve: CTA k stages the instance and its warps take column tiles
-// k*W, k*W+1, ... (W warps per CTA).  MAP = false is the paper's case (no
-// index remapping); FULL = true the m = MMAX case (no bound checks).
+// Single solve, G < 32: CTA k stages the instance and its warps take column
+// tiles k*W, k*W+1, ... (W warps per CTA).  MAP = false is the paper's case (no
+// index remapping).
 // ---------------------------------------------------------------------------
-template <class T, int G, int MMAX, bool MAP, bool FULL>
+template <class T, int G, int MMAX, bool MAP>
 __global__ void __launch_bounds__(32 * kWarpsSingle) small_single_kernel(const T *__restrict__ A, int64_t lda, T *B,
-                                                                 int64_t ldb, int m_, int n, T alpha, int unit,
+                                                                 int64_t ldb, int m, int n, T alpha, int unit,
                                                                  SmallMap mp) {
   extern __shared__ __align__(16) unsigned char smem[];
   T *sTri, *sC, *sR;
   smem_parts<T>(smem, sTri, sC, sR);
-  const int m = FULL ? MMAX : m_;
-  if constexpr (FULL && !MAP) {
-    // the warp's first column tile is loaded before staging, so its latency
-    // overlaps the staging (a one-pass staging with every triangle load in
-    // flight at once measured slower than this with warm caches: the kernel is
-    // bound by dependent FP64 work on one warp per sub-partition, not by memory)
-    constexpr int C = 32 / G;
-    const int ntiles = (n + C - 1) / C;
-    const int step = gridDim.x * kWarpsSingle;
-    const int t0 = blockIdx.x * kWarpsSingle + (threadIdx.x >> 5);
-    auto cols = [&](int t) { return (n - t * C) < C ? (n - t * C) : C; };
-    T b[MMAX / G];
-    if (t0 < ntiles) warp_load_b<T, G, MMAX, false, true>(b, B + (int64_t)t0 * C * ldb, ldb, m, cols(t0), 0);
-    stage<T, MMAX, kWarpsSingle, false>(sTri, sC, sR, A, lda, m, MMAX, alpha, unit != 0, mp);
-    for (int t = t0; t < ntiles; t += step) {
-      T *Bt = B + (int64_t)t * C * ldb;
-      if (t != t0) warp_load_b<T, G, MMAX, false, true>(b, Bt, ldb, m, cols(t), 0);
-      warp_solve_loaded<T, G, MMAX, false, true>(b, sTri, sC, Bt, ldb, m, cols(t), 0);
-    }
+  const int rows_used = ((m + G - 1) / G) * G;
+  stage<T, MMAX, kWarpsSingle, MAP>(sTri, sC, sR, A, lda, m, rows_used, alpha, unit != 0, mp);
+  solve_tiles<T, G, MMAX, MAP>(sTri, sC, B, ldb, m, n, blockIdx.x * kWarpsSingle, gridDim.x * kWarpsSingle, mp.rev);
+}
+
+// ---------------------------------------------------------------------------
+// Single solve, G = 32: a warp per column, the latency of one small solve.
+//
+// The chain of m - 1 dependent steps bounds it: per step a shuffle and the
+// multiply-adds of the values below, each 64 cycles of a sub-partition's FP64
+// pipe whatever its lanes do.  So a lane holds one real number per slot: a row
+// of a real column, or the real or imaginary part of a row of a complex one
+// (16 rows per slot, two multiply-adds each, instead of 32 rows and four: a
+// 37-row complex column takes 10.7k pipe cycles instead of 17.7k).  Finished
+// slots drop out: one rolled loop per slot, so that the code (a few hundred
+// instructions) does not have to be fetched as it runs.  The triangle is copied
+// to shared memory asynchronously while the diagonal's reciprocals are formed.
+// The operations and their order are those of the other variants.
+// ---------------------------------------------------------------------------
+constexpr int kColLd = 64;
+
+template <class T>
+__device__ __forceinline__ void small_copy_async(T *dst, const T *src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(T) == 16) {  // complex128 is 8-byte aligned only
+    const double *q = reinterpret_cast<const double *>(src);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(q) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8), "l"(q + 1) : "memory");
+  } else if constexpr (sizeof(T) == 8) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
   } else {
-    const int rows_used = ((m + G - 1) / G) * G;
-    stage<T, MMAX, kWarpsSingle, MAP>(sTri, sC, sR, A, lda, m, rows_used, alpha, unit != 0, mp);
-    solve_tiles<T, G, MMAX, MAP, FULL>(sTri, sC, B, ldb, m, n, blockIdx.x * kWarpsSingle,
-                                       gridDim.x * kWarpsSingle, mp.rev);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+  }
+}
+
+template <class T>
+struct Real {
+  using type = T;
+  __device__ __forceinline__ static T part(T v, int) { return v; }
+};
+template <>
+struct Real<cplx> {
+  using type = double;
+  __device__ __forceinline__ static double part(cplx v, int p) { return p ? v.im : v.re; }
+};
+template <>
+struct Real<cplxf> {
+  using type = float;
+  __device__ __forceinline__ static float part(cplxf v, int p) { return p ? v.im : v.re; }
+};
+
+template <class T>
+constexpr size_t small_column_smem() {
+  return sizeof(T) * (64 * kColLd + 128);
+}
+
+// The strictly lower elements (r, c) of an m x m matrix, dealt densely to the
+// threads: column p and column m - 2 - p together hold m of them.
+template <class Fn>
+__device__ __forceinline__ void for_strict_lower(int m, Fn fn) {
+  int p = 0, q = threadIdx.x;
+  while (q >= m) {
+    q -= m;
+    ++p;
+  }
+  while (2 * p < m - 1) {
+    const bool lead = q < m - 1 - p;
+    if (lead || 2 * p != m - 2) fn(lead ? p + 1 + q : q, lead ? p : m - 2 - p);
+    q += 32 * kWarpsSingle;
+    while (q >= m) {
+      q -= m;
+      ++p;
+    }
+  }
+}
+
+// The substitution of one column: NS slots per lane, known at compile time so
+// that the slots' multiply-adds of a step issue back to back.
+template <class T, int NS>
+__device__ __forceinline__ void column_steps(typename Real<T>::type (&s)[NS], const T *col, int m, int part,
+                                             int row0) {
+  using F = typename Real<T>::type;
+  constexpr int P = Elem<T>::kComplex ? 2 : 1, RS = 32 / P;
+#pragma unroll
+  for (int ph = 0; ph < NS; ++ph) {
+    const int last = min(m - 1, (ph + 1) * RS);  // the last row updates nothing
+#pragma unroll 4
+    for (int i = ph * RS; i < last; ++i, col += kColLd) {
+      const int src = (i - ph * RS) * P;
+      F u = __shfl_sync(0xffffffffu, s[ph], src), w = F(0);
+      if constexpr (P == 2) {  // s -= a x: part re takes (x.re, x.im), im takes (x.im, -x.re)
+        const F im = __shfl_sync(0xffffffffu, s[ph], src + 1);
+        w = part ? -u : im;
+        u = part ? im : u;
+      }
+      F y[NS];
+#pragma unroll
+      for (int t = ph; t < NS; ++t) {
+        if constexpr (P == 2)
+          y[t] = fma(-col[t * RS].re, u, s[t]);
+        else
+          y[t] = fma(-col[t * RS], u, s[t]);
+      }
+      if constexpr (P == 2) {
+#pragma unroll
+        for (int t = ph; t < NS; ++t) y[t] = fma(col[t * RS].im, w, y[t]);
+      }
+#pragma unroll
+      for (int t = ph; t < NS; ++t)
+        if (t > ph || row0 + t * RS > i) s[t] = y[t];
+    }
+  }
+}
+
+template <class T, bool MAP>
+__global__ void __launch_bounds__(32 * kWarpsSingle) small_column_kernel(const T *__restrict__ A, int64_t lda, T *B,
+                                                                         int64_t ldb, int m, int n, T alpha, int unit,
+                                                                         SmallMap mp) {
+  using E = Elem<T>;
+  using F = typename Real<T>::type;
+  constexpr int P = E::kComplex ? 2 : 1;  // real numbers per value
+  constexpr int RS = 32 / P, R = 64 / RS;  // rows per slot, slots
+  extern __shared__ __align__(16) unsigned char smem[];
+  T *sL = reinterpret_cast<T *>(smem);  // column i at i kColLd
+  T *sR = sL + 64 * kColLd, *sC = sR + 64;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int part = lane % P, row0 = lane / P;
+  const int rev = MAP ? mp.rev : 0, tr = MAP ? mp.tr : 0, cj = MAP ? mp.cj : 0;
+
+  // the diagonal entry this thread inverts and the warp's first column of B
+  T d = E::one();
+  if (tid < m && !unit) d = E::ld(A + (int64_t)(rev ? m - 1 - tid : tid) * (lda + 1));
+  const int step = gridDim.x * kWarpsSingle;
+  int j = blockIdx.x * kWarpsSingle + warp;
+  T b[R];
+  auto load_b = [&]() {
+    const T *col = B + (int64_t)j * ldb;
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int r = row0 + t * RS;
+      b[t] = E::zero();
+      if (r < m) b[t] = E::ld(col + (rev ? m - 1 - r : r));
+    }
+  };
+  if (j < n) load_b();
+  // the strictly lower part of the form (transposed reads: consecutive threads
+  // along a row of the form, which is a column of A)
+  for_strict_lower(m, [&](int r, int c) {
+    if (MAP && tr) {
+      const int t = r;
+      r = m - 1 - c;
+      c = m - 1 - t;
+    }
+    const int p = rev ? m - 1 - r : r, q = rev ? m - 1 - c : c;
+    small_copy_async(sL + c * kColLd + r, MAP && tr ? A + q + (int64_t)p * lda : A + p + (int64_t)q * lda);
+  });
+  if (tid < m) {
+    if constexpr (E::kComplex) {
+      if (cj) d.im = -d.im;
+    }
+    const T rv = unit ? E::one() : E::recip(d);
+    sR[tid] = rv;
+    sC[tid] = E::mul(alpha, rv);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  if (!unit || cj) {  // row r times 1/a_rr
+    for_strict_lower(m, [&](int r, int c) {
+      T v = sL[c * kColLd + r];
+      if constexpr (E::kComplex) {
+        if (cj) v.im = -v.im;
+      }
+      sL[c * kColLd + r] = E::mul(sR[r], v);
+    });
+    __syncthreads();
+  }
+
+  for (bool first = true; j < n; j += step, first = false) {
+    if (!first) load_b();
+    T *out = B + (int64_t)j * ldb;
+    auto run = [&](auto ns) {
+      constexpr int NS = decltype(ns)::value;
+      F s[NS];
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int r = row0 + t * RS;
+        s[t] = F(0);
+        if (r < m) s[t] = Real<T>::part(E::mul(sC[r], b[t]), part);
+      }
+      column_steps<T, NS>(s, sL + row0, m, part, row0);
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int r = row0 + t * RS;
+        if (r < m) reinterpret_cast<F *>(out + (rev ? m - 1 - r : r))[part] = s[t];
+      }
+    };
+    const int slots = (m + RS - 1) / RS;
+    if (slots == 1)
+      run(std::integral_constant<int, 1>{});
+    else if (slots == 2 || R == 2)
+      run(std::integral_constant<int, 2>{});
+    else if (slots == 3)
+      run(std::integral_constant<int, R < 3 ? 2 : 3>{});
+    else
+      run(std::integral_constant<int, R < 4 ? 2 : 4>{});
   }
 }
 
@@ -637,19 +817,18 @@ hsma_status_t set_smem_attrs() {
   return HSMA_OK;
 }
 
-template <class T, int G, int MMAX, bool MAP, bool FULL>
+template <class T, int G, int MMAX, bool MAP>
 hsma_status_t launch_single_v(const T *A, int64_t lda, T *B, int64_t ldb, int m, int n, T alpha, int unit,
                               int grid, cudaStream_t st, SmallMap mp) {
-  const size_t bytes = SmemLayout<T>::bytes(64);
+  constexpr auto *kernel = G == 32 ? small_column_kernel<T, MAP> : small_single_kernel<T, G == 32 ? 16 : G, MMAX, MAP>;
+  constexpr size_t bytes = G == 32 ? small_column_smem<T>() : SmemLayout<T>::bytes(64);
   static DeviceFlags attr_done;
   if (!attr_done.test()) {
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(small_single_kernel<T, G, MMAX, MAP, FULL>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     attr_done.set();
   }
   HsmaTraceScope ts("small_single", st);
-  small_single_kernel<T, G, MMAX, MAP, FULL><<<grid, 32 * kWarpsSingle, bytes, st>>>(A, lda, B, ldb, m, n, alpha,
-                                                                                       unit, mp);
+  kernel<<<grid, 32 * kWarpsSingle, bytes, st>>>(A, lda, B, ldb, m, n, alpha, unit, mp);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
 }
@@ -663,11 +842,8 @@ hsma_status_t launch_single_g(const T *A, int64_t lda, T *B, int64_t ldb, int m,
   const int cap = nsm * 16;
   if (grid > cap) grid = cap;
   const bool mapped = mp.rev != 0 || mp.tr != 0 || mp.cj != 0;
-  if (mapped) return launch_single_v<T, G, MMAX, true, false>(A, lda, B, ldb, m, n, alpha, unit, grid, st, mp);
-  if constexpr (G == 32 && MMAX == 64) {
-    if (m == MMAX) return launch_single_v<T, G, MMAX, false, true>(A, lda, B, ldb, m, n, alpha, unit, grid, st, mp);
-  }
-  return launch_single_v<T, G, MMAX, false, false>(A, lda, B, ldb, m, n, alpha, unit, grid, st, mp);
+  if (mapped) return launch_single_v<T, G, MMAX, true>(A, lda, B, ldb, m, n, alpha, unit, grid, st, mp);
+  return launch_single_v<T, G, MMAX, false>(A, lda, B, ldb, m, n, alpha, unit, grid, st, mp);
 }
 
 }  // namespace
@@ -683,9 +859,7 @@ static SmallMap make_map(int uplo, int trans) {
 template <class T>
 static hsma_status_t small_single_impl(int g, const void *A, int64_t lda, void *B, int64_t ldb, int m, int n,
                                        const double *alpha, int unit, cudaStream_t st, SmallMap mp) {
-  int dev = 0, nsm = 0;
-  HSMA_CUDA_TRY(cudaGetDevice(&dev));
-  HSMA_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const int nsm = hsma_sm_count();
   const bool cplx_ = Elem<T>::kComplex;
   if (g == 0) g = hsma_small_pick_g_single(m, n, cplx_, nsm);
   if (!hsma_small_g_ok(g, m, cplx_)) return HSMA_ERR_INVALID_ARG;

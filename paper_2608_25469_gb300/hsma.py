@@ -180,9 +180,13 @@ def _check(status: int, where: str):
         raise HsmaError(status, where)
 
 
+_Alpha = ctypes.c_double * 2
+
+
 def _alpha_buf(alpha):
+    """alpha as the two doubles the C ABI takes (passed as a pointer by ctypes)."""
     a = complex(alpha)
-    return (ctypes.c_double * 2)(a.real, a.imag)
+    return _Alpha(a.real, a.imag)
 
 
 def hsma_status_string(status: int) -> str:
@@ -195,7 +199,7 @@ def hsma_version() -> str:
 
 def hsma_trsm_llnn(dtype, diag, m, n, alpha, A, lda, B, ldb, stream=0, check=True) -> int:
     """Raw call; A and B are device pointers (ints).  Returns the status."""
-    s = _lib.hsma_trsm_llnn(dtype, diag, m, n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), A, lda, B, ldb,
+    s = _lib.hsma_trsm_llnn(dtype, diag, m, n, _alpha_buf(alpha), A, lda, B, ldb,
                             stream)
     if check:
         _check(s, "hsma_trsm_llnn")
@@ -204,7 +208,7 @@ def hsma_trsm_llnn(dtype, diag, m, n, alpha, A, lda, B, ldb, stream=0, check=Tru
 
 def hsma_trsm_llnn_ex(dtype, diag, m, n, alpha, A, lda, B, ldb, stream=0, opts: Opts | None = None,
                       info: Info | None = None, check=True) -> int:
-    s = _lib.hsma_trsm_llnn_ex(dtype, diag, m, n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), A, lda, B, ldb,
+    s = _lib.hsma_trsm_llnn_ex(dtype, diag, m, n, _alpha_buf(alpha), A, lda, B, ldb,
                                stream, ctypes.byref(opts) if opts is not None else None,
                                ctypes.byref(info) if info is not None else None)
     if check:
@@ -215,7 +219,7 @@ def hsma_trsm_llnn_ex(dtype, diag, m, n, alpha, A, lda, B, ldb, stream=0, opts: 
 def hsma_trsm(dtype, side, uplo, trans, diag, m, n, alpha, A, lda, B, ldb, stream=0, opts: Opts | None = None,
               info: Info | None = None, check=True) -> int:
     """BLAS triangular-solve variants: side LEFT/RIGHT, uplo LOWER/UPPER, trans NO_TRANS/TRANS/CONJ_TRANS."""
-    s = _lib.hsma_trsm(dtype, side, uplo, trans, diag, m, n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), A,
+    s = _lib.hsma_trsm(dtype, side, uplo, trans, diag, m, n, _alpha_buf(alpha), A,
                        lda, B, ldb, stream, ctypes.byref(opts) if opts is not None else None,
                        ctypes.byref(info) if info is not None else None)
     if check:
@@ -227,7 +231,7 @@ def hsma_trsm_vbatched(dtype, side, uplo, trans, diag, batch, d_m, d_n, alpha, d
                        max_n=0, d_status=0, stream=0, check=True) -> int:
     """Varlen batch of left-side variants (uplo, trans) with in-kernel index remapping."""
     s = _lib.hsma_trsm_vbatched(dtype, side, uplo, trans, diag, batch, d_m, d_n,
-                                ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), d_A, d_lda, d_B, d_ldb, max_m, max_n,
+                                _alpha_buf(alpha), d_A, d_lda, d_B, d_ldb, max_m, max_n,
                                 d_status or None, stream)
     if check:
         _check(s, "hsma_trsm_vbatched")
@@ -238,7 +242,7 @@ def hsma_getrs_vbatched(dtype, batch, d_m, d_n, alpha, d_LU, d_lda, d_ipiv, d_B,
                         d_status=0, stream=0, check=True) -> int:
     """Varlen batch of LU-factor solves in one launch: X = U^{-1} L^{-1} P^T (alpha B) per instance
     (packed getrf factors; d_ipiv: device array of per-instance pivot pointers, or 0 for none)."""
-    s = _lib.hsma_getrs_vbatched(dtype, batch, d_m, d_n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), d_LU,
+    s = _lib.hsma_getrs_vbatched(dtype, batch, d_m, d_n, _alpha_buf(alpha), d_LU,
                                  d_lda, d_ipiv or None, d_B, d_ldb, max_m, max_n, d_status or None, stream)
     if check:
         _check(s, "hsma_getrs_vbatched")
@@ -247,7 +251,7 @@ def hsma_getrs_vbatched(dtype, batch, d_m, d_n, alpha, d_LU, d_lda, d_ipiv, d_B,
 
 def hsma_getrs(dtype, m, n, alpha, LU, lda, ipiv, B, ldb, stream=0, opts: Opts | None = None, check=True) -> int:
     """One solve from LU factors (device pointers; ipiv: device int32 pivots or 0)."""
-    s = _lib.hsma_getrs(dtype, m, n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), LU, lda, ipiv or None, B, ldb,
+    s = _lib.hsma_getrs(dtype, m, n, _alpha_buf(alpha), LU, lda, ipiv or None, B, ldb,
                         stream or None, ctypes.byref(opts) if opts is not None else None)
     if check:
         _check(s, "hsma_getrs")
@@ -256,7 +260,7 @@ def hsma_getrs(dtype, m, n, alpha, LU, lda, ipiv, B, ldb, stream=0, opts: Opts |
 
 def hsma_potrs(dtype, m, n, alpha, L, lda, B, ldb, stream=0, opts: Opts | None = None, check=True) -> int:
     """One solve from a lower Cholesky factor (device pointers)."""
-    s = _lib.hsma_potrs(dtype, m, n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), L, lda, B, ldb,
+    s = _lib.hsma_potrs(dtype, m, n, _alpha_buf(alpha), L, lda, B, ldb,
                         stream or None, ctypes.byref(opts) if opts is not None else None)
     if check:
         _check(s, "hsma_potrs")
@@ -266,7 +270,7 @@ def hsma_potrs(dtype, m, n, alpha, L, lda, B, ldb, stream=0, opts: Opts | None =
 def hsma_potrs_vbatched(dtype, batch, d_m, d_n, alpha, d_L, d_lda, d_B, d_ldb, max_m=0, max_n=0, d_status=0,
                         stream=0, check=True) -> int:
     """Varlen batch of Cholesky-factor solves in one launch: X = L^{-H} L^{-1} (alpha B) per instance."""
-    s = _lib.hsma_potrs_vbatched(dtype, batch, d_m, d_n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), d_L,
+    s = _lib.hsma_potrs_vbatched(dtype, batch, d_m, d_n, _alpha_buf(alpha), d_L,
                                  d_lda, d_B, d_ldb, max_m, max_n, d_status or None, stream)
     if check:
         _check(s, "hsma_potrs_vbatched")
@@ -275,7 +279,7 @@ def hsma_potrs_vbatched(dtype, batch, d_m, d_n, alpha, d_L, d_lda, d_B, d_ldb, m
 
 def hsma_trsm_llnn_vbatched(dtype, diag, batch, d_m, d_n, alpha, d_A, d_lda, d_B, d_ldb, max_m=0, max_n=0,
                             d_status=0, stream=0, check=True) -> int:
-    s = _lib.hsma_trsm_llnn_vbatched(dtype, diag, batch, d_m, d_n, ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p),
+    s = _lib.hsma_trsm_llnn_vbatched(dtype, diag, batch, d_m, d_n, _alpha_buf(alpha),
                                      d_A, d_lda, d_B, d_ldb, max_m, max_n, d_status or None, stream)
     if check:
         _check(s, "hsma_trsm_llnn_vbatched")
@@ -286,7 +290,7 @@ def hsma_trsm_llnn_vbatched_noalloc(dtype, diag, batch, d_m, d_n, alpha, d_A, d_
                                     max_n=0, d_status=0, stream=0, check=True) -> int:
     """Allocation-free varlen batch: schedule scratch in a static device array (batch <= 65536)."""
     s = _lib.hsma_trsm_llnn_vbatched_noalloc(dtype, diag, batch, d_m, d_n,
-                                             ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), d_A, d_lda, d_B,
+                                             _alpha_buf(alpha), d_A, d_lda, d_B,
                                              d_ldb, max_m, max_n, d_status or None, stream)
     if check:
         _check(s, "hsma_trsm_llnn_vbatched_noalloc")
@@ -300,7 +304,7 @@ def hsma_trsm_llnn_vbatched_host(dtype, diag, batch, h_m, h_n, alpha, hA, h_offA
     def ptr(a):
         return a.ctypes.data if isinstance(a, np.ndarray) else a
     s = _lib.hsma_trsm_llnn_vbatched_host(dtype, diag, batch, ptr(h_m), ptr(h_n),
-                                          ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), ptr(hA), ptr(h_offA),
+                                          _alpha_buf(alpha), ptr(hA), ptr(h_offA),
                                           ptr(hB), ptr(h_offB), ptr(hX), chunks, stream)
     if check:
         _check(s, "hsma_trsm_llnn_vbatched_host")
@@ -313,7 +317,7 @@ def hsma_trsm_llnn_vbatched_host_tp(dtype, diag, batch, h_m, h_n, alpha, hAp, h_
     def ptr(a):
         return a.ctypes.data if isinstance(a, np.ndarray) else a
     s = _lib.hsma_trsm_llnn_vbatched_host_tp(dtype, diag, batch, ptr(h_m), ptr(h_n),
-                                             ctypes.cast(_alpha_buf(alpha), ctypes.c_void_p), ptr(hAp), ptr(h_offA),
+                                             _alpha_buf(alpha), ptr(hAp), ptr(h_offA),
                                              ptr(hB), ptr(h_offB), ptr(hX), chunks, stream)
     if check:
         _check(s, "hsma_trsm_llnn_vbatched_host_tp")
@@ -442,7 +446,19 @@ def from_device(t) -> np.ndarray:
     return np.asfortranarray(t.cpu().numpy().T)
 
 
+_torch = None
+
+
 def stream_ptr(stream=None) -> int:
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    """Raw handle of a torch stream (default: the current one)."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the raw handle without building a Stream object, where torch offers it
+    raw = getattr(_torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is not None:
+        return int(raw(_torch.cuda.current_device()))
+    return int(_torch.cuda.current_stream().cuda_stream)

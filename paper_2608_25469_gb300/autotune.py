@@ -38,9 +38,9 @@ PANELS = (512, 1024, 2048, 4096)
 EMU = 10                   # table key offset of the emulated-products entries
 
 GRID = {
-    0: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096, 8192) for n in (4, 32, 256, 2048)] +
+    0: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096, 8192) for n in (4, 32, 96, 256, 2048)] +
        [(4096, 4096), (8192, 8192), (16384, 16384)],
-    1: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096) for n in (4, 32, 256, 1024)] + [(4096, 4096), (8192, 8192)],
+    1: [(m, n) for m in (128, 256, 512, 1024, 2048, 4096) for n in (4, 32, 96, 256, 1024)] + [(4096, 4096), (8192, 8192)],
     2: [(m, n) for m in (128, 512, 2048, 8192) for n in (16, 256, 4096)],
     EMU + 0: [(m, n) for m in (512, 1024, 2048, 4096, 8192) for n in (128, 1024)] +
              [(2048, 4096), (8192, 4096), (16384, 16384)],

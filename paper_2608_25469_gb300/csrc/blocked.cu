@@ -1,15 +1,11 @@
 // Large-case blocked solve (Section 4.3), fp64 and complex128.
 //
 // Phase 1 (Section 4.3, "parallel diagonal block inversion"): the N_B x N_B
-// diagonal blocks D_t are inverted independently: FP64 by doubling
-// (fp64_inverse.cu); the FP32 modes' base blocks (N_B = 32 or 64) by the column
-// substitution below, in one launch.  Each CTA produces a group of columns of
-// D_t^{-1} by forward substitution against the identity (Section 4.3.1): the
-// columns of D_t are streamed through a two-slot shared-memory buffer
-// (Algorithm 2's double buffering: column k+1 is staged while column k is
-// used), so shared memory is O(N_B).  The columns of the inverse live in
-// registers: lane group g of a warp holds rows g, g+G, ..., and the register
-// window slides down by one slot every G steps.
+// diagonal blocks D_t are inverted independently by forward substitution against
+// the identity (Section 4.3.1) on base blocks of 32 rows (FP32: 64), joined by
+// doubling (fp64_inverse.cu, r32_inverse.cu).  Algorithm 2's column streaming
+// keeps shared memory at O(N_B) for one N_B-row substitution; here no block of
+// that size is substituted, and shared memory holds base blocks and tiles only.
 //
 // Phase 2 (Section 4.3, "sequential GEMM update and solve"), for r = 0..k:
 //   X_r = D_r^{-1} B_r                       (solve product, triangular)
@@ -44,94 +40,6 @@
 __device__ unsigned int g_hsma_dev_error = 0;
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// Phase 1: diagonal-block inversion by substitution (FP32 base blocks)
-// ---------------------------------------------------------------------------
-constexpr int kInvSlots = 32;  // register slots per lane: N_B = 32 * G
-
-template <class T, int G>
-__global__ void __launch_bounds__(256) diag_inverse_kernel(const T *__restrict__ A, int64_t lda, int64_t m, int unit,
-                                                            T *__restrict__ Dinv) {
-  using E = Elem<T>;
-  constexpr int R = kInvSlots, NB = 32 * G, C = 32 / G;
-  __shared__ T sRinv[NB];
-  __shared__ T sCol[2][NB];
-  const int nthr = blockDim.x, tid = threadIdx.x;
-  const int CT = (nthr / 32) * C;
-  const int64_t r0 = (int64_t)blockIdx.x * NB;
-  const int s = (int)((m - r0) < NB ? (m - r0) : NB);
-  const int j0 = blockIdx.y * CT;
-  T *Y = Dinv + (int64_t)blockIdx.x * NB * NB;
-  const T *D = A + r0 + r0 * lda;
-
-  for (int r = tid; r < NB; r += nthr) sRinv[r] = (r < s) ? (unit ? E::one() : E::recip(E::ld(D + r + (int64_t)r * lda))) : E::zero();
-  // zeros outside the computed region: whole columns >= s, rows < j0 and rows >= s
-  for (int e = tid; e < CT * NB; e += nthr) {
-    const int col = j0 + e / NB, row = e % NB;
-    if (col < NB && (col >= s || row < j0 || row >= s)) Y[row + (int64_t)col * NB] = E::zero();
-  }
-  __syncthreads();
-  if (j0 >= s) return;
-
-  const int warp = tid >> 5, lane = tid & 31;
-  const int g = lane % G, c = lane / G;
-  const int j = j0 + warp * C + c;
-  const bool colok = j < s;
-  const int q0 = j0 / G;
-
-  T x[R];
-#pragma unroll
-  for (int t = 0; t < R; ++t) x[t] = (colok && g + G * (t + q0) == j) ? sRinv[j] : E::zero();
-
-  // loader role: rows tid, tid + nthr (N_B <= 2 * nthr)
-  auto fetch = [&](int k, T *pf) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = tid + h * nthr;
-      pf[h] = (r > k && r < s && k < s) ? E::ld(D + r + (int64_t)k * lda) : E::zero();
-    }
-  };
-  auto put = [&](int k, const T *pf) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = tid + h * nthr;
-      if (r < NB) sCol[k & 1][r] = E::mul(sRinv[r < s ? r : 0], pf[h]);
-    }
-  };
-  T pf[2];
-  fetch(j0, pf);
-  put(j0, pf);
-  fetch(j0 + 1, pf);
-  __syncthreads();
-
-  for (int q = q0; q * G < s; ++q) {
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-      const int k = q * G + u;
-      if (k >= s) break;
-      if (k + 1 < s) put(k + 1, pf);
-      if (k + 2 < s) fetch(k + 2, pf);
-      const T *dc = sCol[k & 1];
-      const T xk = (G == 1) ? x[0] : E::shfl(x[0], c * G + u);
-      if (u < G - 1) {
-        const T nv = E::fms(dc[g + G * q], xk, x[0]);
-        if (g > u) x[0] = nv;
-      }
-#pragma unroll
-      for (int t = 1; t < R; ++t) {
-        if ((q + t) * G >= s) break;
-        x[t] = E::fms(dc[g + G * (q + t)], xk, x[t]);
-      }
-      __syncthreads();
-    }
-    const int row = g + G * q;
-    if (colok && row < s) Y[row + (int64_t)j * NB] = x[0];
-#pragma unroll
-    for (int t = 0; t < R - 1; ++t) x[t] = x[t + 1];
-    x[R - 1] = E::zero();
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Phase 2 products on the FP64 tensor path
@@ -534,14 +442,17 @@ hsma_status_t gemm_tiled(const GemmArgs<T> &p0, const char *phase, cudaStream_t 
 
 // ---------------------------------------------------------------------------
 // Products in small tiles (fp64_tile.cuh): UPDATE and SCALE as above, without
-// partial products.  Grid (row tiles, column tiles).
+// partial products.  Grid (column tiles, row tiles), row tiles from the last one
+// on: a triangular product's long K ranges start first and every SM gets its
+// share of long and short ones (256 x 2048 FP64: 224 -> 203 us, 4096 x 512
+// 8.68 -> 8.55 ms).
 // ---------------------------------------------------------------------------
 template <class T, int WM, int WN, int NW>
 __global__ void __launch_bounds__(32 * NW) small_tile_kernel(const GemmArgs<T> p) {
   using E = Elem<T>;
   constexpr int BM = 8 * WM, BN = 8 * WN;
   __shared__ T red[NW][BM * BN];
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+  const int m0 = (gridDim.y - 1 - blockIdx.y) * BM, n0 = blockIdx.x * BN;
   fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, 0, p.tri ? min(p.K, m0 + BM) : p.K, m0, n0, red);
   const bool b1 = is_one(p.beta);
   for (int e = threadIdx.x; e < BM * BN; e += 32 * NW) {
@@ -560,7 +471,7 @@ __global__ void __launch_bounds__(32 * NW) small_tile_kernel(const GemmArgs<T> p
 
 template <class T, int WM, int WN, int NW>
 hsma_status_t launch_small_tiles(const GemmArgs<T> &p, const char *phase, cudaStream_t st) {
-  const dim3 grid((p.M + 8 * WM - 1) / (8 * WM), (p.N + 8 * WN - 1) / (8 * WN));
+  const dim3 grid((p.N + 8 * WN - 1) / (8 * WN), (p.M + 8 * WM - 1) / (8 * WM));
   if (grid.y > 65535) return HSMA_ERR_UNSUPPORTED;
   HsmaTraceScope ts(phase, st);
   small_tile_kernel<T, WM, WN, NW><<<grid, 32 * NW, 0, st>>>(p);
@@ -598,18 +509,6 @@ hsma_status_t gemm(const GemmArgs<T> &p, const char *phase, cudaStream_t st, T *
   if (tile == HSMA_TILE_128x8) return gemm_tiled<T, TileN8>(p, phase, st, P, P_elems);
   if (tile == HSMA_TILE_128x16) return gemm_tiled<T, TileN16>(p, phase, st, P, P_elems);
   return gemm_tiled<T, TileWide>(p, phase, st, P, P_elems);
-}
-
-template <int G>
-hsma_status_t launch_inverse_f32(const float *A, int64_t lda, int64_t m, int unit, float *Dinv, cudaStream_t st) {
-  constexpr int NB = 32 * G, C = 32 / G;
-  const int warps = std::min(8, NB / C);
-  const int CT = warps * C;
-  dim3 grid((unsigned)((m + NB - 1) / NB), (unsigned)(NB / CT));
-  HsmaTraceScope ts("diag_inverse", st);
-  diag_inverse_kernel<float, G><<<grid, warps * 32, 0, st>>>(A, lda, m, unit, Dinv);
-  HSMA_CUDA_TRY(cudaGetLastError());
-  return HSMA_OK;
 }
 
 template <class T>
@@ -745,15 +644,6 @@ unsigned int *hsma_dev_error_ptr() {
   std::lock_guard<std::mutex> lk(mu);
   if (ptr[d] == nullptr && cudaGetSymbolAddress((void **)&ptr[d], g_hsma_dev_error) != cudaSuccess) ptr[d] = nullptr;
   return ptr[d];
-}
-
-hsma_status_t hsma_f32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
-                                    cudaStream_t st) {
-  switch (nb) {
-    case 32: return launch_inverse_f32<1>(A, lda, m, unit, Dinv, st);
-    case 64: return launch_inverse_f32<2>(A, lda, m, unit, Dinv, st);
-    default: return HSMA_ERR_UNSUPPORTED;
-  }
 }
 
 hsma_status_t hsma_residual_f64(const double *A, int64_t lda, int unit, const double *X, int64_t ldx, double *C,

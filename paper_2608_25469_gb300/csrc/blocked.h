@@ -29,10 +29,6 @@ template <class T>
 hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, T *W,
                                      cudaStream_t st);
 
-// The same for float data by column substitution, nb in {32, 64}.
-hsma_status_t hsma_f32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
-                                    cudaStream_t st);
-
 // FP64 product used by the refinement residual: C = beta*C - L*X with L the
 // lower triangle of A (unit diagonal if unit), all column-major fp64 (m x m,
 // m x n).  If skip is non-NULL and *skip != 0 on the device, the launch does

@@ -32,17 +32,29 @@ __global__ void build_perm_kernel(const int32_t *__restrict__ ipiv, int64_t m, i
   }
   __syncthreads();
   __shared__ int bad;
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  bool mine = false;
+  for (int64_t k = threadIdx.x; k < m; k += blockDim.x) {
+    const int64_t q = in_smem ? piv[k] : (int64_t)ipiv[k] - 1;
+    mine |= q < k || q >= m;
+  }
+  if (mine) bad = 1;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    bad = 0;
-    for (int64_t k = 0; k < m; ++k) {
-      const int64_t q = in_smem ? piv[k] : (int64_t)ipiv[k] - 1;
-      if (q < k || q >= m) {
-        bad = 1;
-        break;
+    if (!bad) {
+      // entry k is final once swapped, so step k writes it out and only moves the
+      // old p[k] down; the next entry is loaded before that store (and replaced
+      // by it when they coincide), which leaves one load's latency per step
+      int32_t cur = p[0];
+#pragma unroll 4
+      for (int64_t k = 0; k < m; ++k) {
+        const int64_t q = in_smem ? piv[k] : (int64_t)ipiv[k] - 1;
+        const int32_t t = p[q], next = k + 1 < m ? p[k + 1] : 0;
+        if (q != k) p[k] = t;
+        if (q != k) p[q] = cur;
+        cur = q == k + 1 ? cur : next;
       }
-      const int32_t t = p[k];
-      p[k] = p[q];
-      p[q] = t;
     }
     if (bad && err != nullptr) atomicOr(err, HSMA_DEVERR_BAD_PIVOT);
   }

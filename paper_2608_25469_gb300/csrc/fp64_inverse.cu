@@ -48,7 +48,10 @@ __global__ void __launch_bounds__(32 * kBaseWarps) inv_base_kernel(const T *__re
   T x = lane == j ? rv : E::zero();
 #pragma unroll
   for (int k = 0; k < kBase - 1; ++k) {
-    if (k >= j) x = E::fms(E::mul(rv, row[k]), E::shfl(x, k), x);  // warp-uniform
+    if (k >= j) {  // warp-uniform
+      const T y = E::fms(E::mul(rv, row[k]), E::shfl(x, k), x);
+      if (lane > k) x = y;
+    }
   }
   T *Y = Dinv + (r0 / nb) * (int64_t)nb * nb;
   const int l = (int)(r0 % nb);

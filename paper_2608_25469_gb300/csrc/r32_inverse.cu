@@ -3,7 +3,7 @@
 // mode the paper leaves to future work, Section 6), by doubling.
 //
 // Inverting a 512-row block by substitution is a 512-step dependent chain.
-// Here the substitution kernel inverts 64 x 64 blocks only (a 64-step chain),
+// Here substitution inverts 64 x 64 blocks only (a warp per column),
 // and each level joins adjacent h x h inverses into a 2h x 2h one: for
 //   T = [A 0; C D],   T^-1 = [A^-1 0; -D^-1 C A^-1  D^-1],
 // the new lower-left block takes two FP32 products, W = C A^-1 and then
@@ -28,20 +28,48 @@ constexpr int kInvBase = 64;  // blocks inverted by substitution
 constexpr int kDT = 64;       // output tile of the doubling products
 constexpr int kDK = 16;       // K step
 
-// Copy the inverse of base block b (64 x 64, contiguous) onto the diagonal of
-// its N_B-row outer block (ld N_B): one CTA per base block.
-__global__ void __launch_bounds__(256) inv_place_kernel(const float *__restrict__ base, int64_t m, int nb,
-                                                        float *Dinv) {
-  const int64_t b = blockIdx.x, r0 = b * kInvBase;
-  const int s = (int)std::min<int64_t>(kInvBase, m - r0);
-  const int64_t R = r0 / nb;
-  const int l = (int)(r0 % nb);
-  float *Y = Dinv + R * nb * nb;
-  const float *src = base + b * kInvBase * kInvBase;
-  for (int e = threadIdx.x; e < kInvBase * kInvBase; e += blockDim.x) {
-    const int i = e % kInvBase, j = e / kInvBase;
-    if (i < s && j < s) Y[(l + i) + (int64_t)(l + j) * nb] = src[i + j * kInvBase];
+// The inverse of base block b (BASE rows from BASE b of the matrix) onto the
+// diagonal of its N_B-row outer block (ld N_B), zeros above it and outside a
+// partial block: the block's strictly lower part is staged with its rows scaled by
+// 1/a_rr, and every warp substitutes one column (lane r holds rows r and r + 32):
+// a step is a shuffle and two multiply-adds.  (As a chain of 64 steps with a
+// barrier each over streamed columns, and a copy into place, 128 blocks took 39
+// us.)
+template <int BASE>
+__global__ void __launch_bounds__(256) inv_base_kernel(const float *__restrict__ A, int64_t lda, int64_t m, int nb,
+                                                       int unit, float *Dinv) {
+  constexpr int R = BASE / 32;
+  __shared__ float sL[BASE][BASE], sR[BASE];
+  const int tid = threadIdx.x, lane = tid & 31, j = blockIdx.y * 8 + (tid >> 5);
+  const int64_t r0 = (int64_t)blockIdx.x * BASE;
+  const int s = (int)min((int64_t)BASE, m - r0);
+  const float *D = A + r0 + r0 * lda;
+  if (tid < BASE) sR[tid] = tid < s ? (unit ? 1.0f : 1.0f / D[tid + (int64_t)tid * lda]) : 0.0f;
+  __syncthreads();
+#pragma unroll 4
+  for (int e = tid; e < BASE * BASE; e += 256) {
+    const int r = e % BASE, k = e / BASE;
+    sL[k][r] = (r > k && r < s) ? sR[r] * D[r + (int64_t)k * lda] : 0.0f;
   }
+  __syncthreads();
+  float x[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) x[t] = (lane + 32 * t == j && j < s) ? sR[j] : 0.0f;
+#pragma unroll
+  for (int ph = 0; ph < R; ++ph)
+#pragma unroll 8
+    for (int k = 32 * ph; k < 32 * ph + 32; ++k) {
+      const float xk = __shfl_sync(0xffffffffu, x[ph], k - 32 * ph);
+#pragma unroll
+      for (int t = ph; t < R; ++t) {
+        const float y = fmaf(-sL[k][lane + 32 * t], xk, x[t]);
+        if (t > ph || lane + 32 * t > k) x[t] = y;
+      }
+    }
+  float *Y = Dinv + (r0 / nb) * (int64_t)nb * nb;
+  const int l = (int)(r0 % nb);
+#pragma unroll
+  for (int t = 0; t < R; ++t) Y[(l + lane + 32 * t) + (int64_t)(l + j) * nb] = x[t];
 }
 
 // One 64 x 64 output tile of out = sign * P Q (P: M x K, Q: K x N, all
@@ -123,27 +151,29 @@ __global__ void __launch_bounds__(256) inv_double_kernel(const float *__restrict
 
 hsma_status_t hsma_r32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
                                     cudaStream_t st) {
-  if (nb < 2 * kInvBase || nb % (2 * kInvBase) != 0 || (nb & (nb - 1)) != 0)
-    return hsma_f32_diag_inverse(nb, A, lda, m, unit, Dinv, st);
   const int64_t nblk = (m + nb - 1) / nb;
+  if (nb == 32) {
+    HsmaTraceScope ts("diag_inverse", st);
+    inv_base_kernel<32><<<dim3((unsigned)nblk, 4), 256, 0, st>>>(A, lda, m, nb, unit, Dinv);
+    return hsma_from_cuda(cudaGetLastError());
+  }
+  if (nb < kInvBase || nb > 512 || (nb & (nb - 1)) != 0) return HSMA_ERR_UNSUPPORTED;
   const int64_t nbase = (m + kInvBase - 1) / kInvBase;
-  auto al = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
-  const size_t base_b = al(sizeof(float) * (size_t)nbase * kInvBase * kInvBase);
   // pair scratch: an outer block holds N_B / 2h pairs of h^2 floats at level
   // h, at most (N_B / 2)^2 in all (the last level)
-  const size_t w_b = al(sizeof(float) * (size_t)nblk * (nb / 2) * (nb / 2));
+  const size_t w_b = nb > kInvBase ? sizeof(float) * (size_t)nblk * (nb / 2) * (nb / 2) : 0;
   void *ws = nullptr;
-  hsma_status_t s = hsma_ws_alloc(&ws, base_b + w_b, st);
+  hsma_status_t s = hsma_ws_alloc(&ws, w_b, st);
   if (s != HSMA_OK) return s;
-  float *base = static_cast<float *>(ws);
-  float *W = reinterpret_cast<float *>(static_cast<unsigned char *>(ws) + base_b);
+  float *W = static_cast<float *>(ws);
   do {
-    if ((s = hsma_f32_diag_inverse(kInvBase, A, lda, m, unit, base, st)) != HSMA_OK) break;
     int levels = 0;
     for (int h = kInvBase; h < nb; h *= 2) ++levels;
     HsmaTraceScope ts("diag_inverse", st, 1 + 2 * levels);
-    if ((s = hsma_from_cuda(cudaMemsetAsync(Dinv, 0, sizeof(float) * (size_t)nblk * nb * nb, st))) != HSMA_OK) break;
-    inv_place_kernel<<<(unsigned)nbase, 256, 0, st>>>(base, m, nb, Dinv);
+    if (nb > kInvBase &&
+        (s = hsma_from_cuda(cudaMemsetAsync(Dinv, 0, sizeof(float) * (size_t)nblk * nb * nb, st))) != HSMA_OK)
+      break;
+    inv_base_kernel<kInvBase><<<dim3((unsigned)nbase, kInvBase / 8), 256, 0, st>>>(A, lda, m, nb, unit, Dinv);
     for (int h = kInvBase; h < nb; h *= 2) {
       const int64_t pairs = (m + 2 * h - 1) / (2 * h);
       if (pairs > 65535) {

@@ -210,6 +210,7 @@ def profile_traffic(name: str, files, work=None):
 
 
 SMALL_SOURCES = ["paper_2608_25469_gb300/csrc/small.cu", "paper_2608_25469_gb300/csrc/common.cuh"]
+BATCH_SOURCES = ["paper_2608_25469_gb300/csrc/batch.cu", "paper_2608_25469_gb300/csrc/common.cuh"]
 PACKED_SOURCES = ["paper_2608_25469_gb300/csrc/packed.cu", "paper_2608_25469_gb300/csrc/common.cuh"]
 
 
@@ -356,15 +357,15 @@ def run_batched(args, dist, device, c64=False):
     kernel_ms = solve_ms / max(solve_cnt, 1)
     achieved = flops / (kernel_ms * 1e-3) / 1e9
     name = "c64" if c64 else "c128"
-    # complex128 runs the column-packed batch; complex64 the per-instance kernel
-    traffic = (profile_traffic("vbatched_solve_c64_8192.txt", SMALL_SOURCES) if c64 else
+    # complex128 runs the column-packed batch; complex64 the blocked batch kernel
+    traffic = (profile_traffic("vbatched_solve_c64_8192.txt", BATCH_SOURCES) if c64 else
                profile_traffic("packed_solve_c128_8192.txt", PACKED_SOURCES, work=flops))
     if c64:
         # FP32 work is cheap here: the algorithmic bytes bind (HBM roofline, measured copy bandwidth)
         peaks, src = load_peaks()
         gbs = abytes / (kernel_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": round(gbs, 2), "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": round(gbs / peaks["hbm_gbs"], 4), "traffic": traffic, "kernel": "vbatched_solve_kernel<cplxf>",
+                "frac": round(gbs / peaks["hbm_gbs"], 4), "traffic": traffic, "kernel": "batch_kernel<cplxf>",
                 "kernel_ms": round(kernel_ms, 5), "kernel_gflops": round(achieved, 2),
                 "peak_source": f"HBM copy bandwidth, {src}"}
     else:
@@ -558,10 +559,10 @@ def run_batched_lu(args, dist, device):
                      "unit": "GFLOP/s", "frac": round(achieved / fp64_peak_gflops(), 4),
                      "traffic": (profile_traffic("packed_solve_lu_upper_c128_8192.txt", PACKED_SOURCES,
                                                  work=flops / 2) if cx else
-                                 profile_traffic("vbatched_lu_f64_8192.txt", SMALL_SOURCES)),
+                                 profile_traffic("vbatched_lu_f64_8192.txt", BATCH_SOURCES)),
                      "kernel": ("packed_solve_kernel<cplx> (two launches a step: unit lower, then upper "
                                 "through the index map; achieved over both)" if cx else
-                                "vbatched_lu_kernel<double> (interchanges, unit lower and upper in one launch)"),
+                                "batch_kernel<double> (interchanges, unit lower and upper in one launch)"),
                      "kernel_ms": round(kernel_ms, 5),
                      "peak_source": FP64_PEAK_SOURCE},
         "e2e": {"value": round(total * e2e_steps / (e2e_ms * 1e-3) / 1e9, 3), "unit": "GFLOP/s",
@@ -573,8 +574,10 @@ def run_batched_lu(args, dist, device):
 
 
 # the files that hold each profiled kernel (a summary's traffic is used only while they are unchanged)
-LARGE_SOURCES = ["paper_2608_25469_gb300/csrc/blocked.cu", "paper_2608_25469_gb300/csrc/tma.cuh"]
-EMU_SOURCES = ["paper_2608_25469_gb300/csrc/tc_gemm.cuh", "paper_2608_25469_gb300/csrc/tma.cuh"]
+LARGE_SOURCES = ["paper_2608_25469_gb300/csrc/blocked.cu", "paper_2608_25469_gb300/csrc/fp64_tile.cuh"]
+EMU_SOURCES = ["paper_2608_25469_gb300/csrc/tc_gemm.cuh", "paper_2608_25469_gb300/csrc/oz_tables.cuh",
+               "paper_2608_25469_gb300/csrc/tma.cuh"]
+OZ_MODULI = 17  # BF16 products of residues per emulated FP64 product
 # real columns per update panel of the emulated blocked solve when the plan reports none
 EMU_PANEL_COLS = 2048
 
@@ -707,7 +710,7 @@ def run_large(args, dist, device, code, m):
     upd_flops = (4.0 if cplx_ else 1.0) * float(n) * (m * m - m * nb)
     achieved = upd_flops / (upd_ms / max(args.steps, 1) * 1e-3) / 1e9
     if emulated:
-        # tensor work the emulated update products issue: 55 BF16 slice-pair
+        # tensor work the emulated update products issue: 17 BF16 residue
         # products of (W rows) x n x Kp each (W = 2 for complex); panels of h
         # blocks: per block an update of the panel's remaining rows (K = N_B),
         # per panel one update of the rows below it (K = h N_B)
@@ -719,8 +722,8 @@ def run_large(args, dist, device, code, m):
             PR = min(h * nb, m - R0)
             for r0 in range(R0, R0 + PR, nb):
                 sr = min(nb, m - r0)
-                bf16_flops += 55 * 2.0 * w * (R0 + PR - r0 - sr) * float(n) * kp(sr)
-            bf16_flops += 55 * 2.0 * w * (m - R0 - PR) * float(n) * kp(PR)
+                bf16_flops += OZ_MODULI * 2.0 * w * (R0 + PR - r0 - sr) * float(n) * kp(sr)
+            bf16_flops += OZ_MODULI * 2.0 * w * (m - R0 - PR) * float(n) * kp(PR)
         peaks, src = load_peaks()
         bf16_peak = peaks["bf16_tflops_sustained"] * 1e3
         bf16_rate = bf16_flops / (upd_ms / max(args.steps, 1) * 1e-3) / 1e9
@@ -748,7 +751,7 @@ def run_large(args, dist, device, code, m):
     return {
         "metric": METRIC, "value": round(value, 3), "unit": "GFLOP/s", "n_gpus": dist.world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_max / args.steps, 3), "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": ("c128" if cplx_ else "f64") + (" (emulated: bf16 slices)" if emulated else ""),
+        "scaling": "weak", "vs_baseline": None, "dtype": ("c128" if cplx_ else "f64") + (" (emulated: bf16 residues)" if emulated else ""),
         "data": "synthetic",
         "config": {"workload": f"{name}: one blocked solve m=n={m}, alpha=1, non-unit, N_B={nb}"
                                + (", FP64 products emulated on the BF16 tensor cores" if emulated else ""),
@@ -760,14 +763,14 @@ def run_large(args, dist, device, code, m):
                       "unit": "GFLOP/s", "frac": round(bf16_rate / bf16_peak, 4),
                       "traffic": profile_traffic(f"update_emulated_{name}.txt", EMU_SOURCES,
                                                  work=bf16_flops / max(upd_cnt / max(args.steps, 1), 1)),
-                      "kernel": "tc_gemm_kernel<TC_OZ> (update_gemm, tcgen05 BF16 slice pairs)",
+                      "kernel": "tc_gemm_kernel<TC_OZ> (update_gemm, tcgen05 BF16 residue products)",
                       "peak_source": f"bf16 tensor (sustained), {src}",
                       "fp64_equivalent_gflops": round(achieved, 1)} if emulated else
                      {"bound": "tensor", "achieved": round(achieved, 3), "peak": round(fp64_peak_gflops(), 1),
                       "unit": "GFLOP/s", "frac": round(achieved / fp64_peak_gflops(), 4),
                       "traffic": profile_traffic(f"update_gemm_{name}.txt", LARGE_SOURCES,
                                                  work=upd_flops / max(upd_cnt / max(args.steps, 1), 1)),
-                      "kernel": "gemm_kernel (update_gemm, DMMA m8n8k4)",
+                      "kernel": "small_tile_kernel (update_gemm, DMMA m8n8k4)",
                       "peak_source": FP64_PEAK_SOURCE + "; DMMA shares the FP64 budget"}),
         "phases_ms_per_step": {k: round(v[0] / args.steps, 3) for k, v in phases.items()},
         "phase_share": {k: round(v[0] / tot_phase, 4) for k, v in phases.items()} if tot_phase else None,
@@ -1145,8 +1148,8 @@ def serve_e2e(args, H, I, seed, t_arr, ms, ns, dts, emulated, device, count=2000
             "sources": "pinned host buffers (shared read-only inputs per dtype, one output region per request)"}
 
 
-def ir_residual_bf16_flops(m, n, chunk=1024, tile=128, pairs=55):
-    """BF16 slice-pair flops of one emulated refinement residual R = alpha B - L X: K chunks
+def ir_residual_bf16_flops(m, n, chunk=4096, tile=256, products=None):
+    """BF16 residue-product flops of one emulated refinement residual R = alpha B - L X: K chunks
     of `chunk` columns of L; a chunk starting at c0 multiplies rows c0.. of L, row tile t
     (of `tile` rows) needing K up to its own last row (64-padded)."""
     tot = 0.0
@@ -1157,7 +1160,7 @@ def ir_residual_bf16_flops(m, n, chunk=1024, tile=128, pairs=55):
         for pm in range(-(-M // tile)):
             rows = min(tile, M - pm * tile)
             kall = -(-min(K, (pm + 1) * tile) // 64) * 64
-            tot += pairs * 2.0 * rows * n * kall
+            tot += (products or OZ_MODULI) * 2.0 * rows * n * kall
     return tot
 
 
@@ -1251,7 +1254,7 @@ def run_mixed(args, dist, device, mode):
     else:
         evals = int(info.ir_iters) + 1  # residual evaluations that did work (one per check)
         res_fl = ir_residual_bf16_flops(m, n)
-        rcnt = counts.get("residual", 1)  # launches per step (one per K chunk and evaluation)
+        rcnt = counts.get("residual", 1)  # launches per step (one per K chunk, column part and evaluation)
         kernel_ms = phases.get("residual", 0.0) / max(rcnt, 1)
         ach = res_fl * evals / max(rcnt, 1) / (kernel_ms * 1e-3) / 1e9 if kernel_ms > 0 else 0.0
         pk = peaks["bf16_tflops_sustained"] * 1e3
@@ -1259,7 +1262,7 @@ def run_mixed(args, dist, device, mode):
                 "frac": round(ach / pk, 4),
                 "traffic": profile_traffic("residual_emulated_ir_8192x4096.txt", EMU_SOURCES,
                                            work=res_fl * evals / max(rcnt, 1)),
-                "kernel": "tc_gemm_kernel<TC_OZ> (residual: 55 BF16 slice pairs per K chunk of 1024)",
+                "kernel": "tc_gemm_kernel<TC_OZ> (residual: 17 BF16 residue products per K chunk of 4096)",
                 "kernel_ms": round(kernel_ms, 5), "residual_evaluations": evals,
                 "peak_source": f"bf16 tensor (measured sustained), {src}"}
         if "residual" in phases:

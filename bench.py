@@ -943,7 +943,7 @@ def run_single64(args, dist, device):
         "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(fp64_peak_gflops(), 1),
                      "unit": "GFLOP/s", "frac": round(achieved / fp64_peak_gflops(), 5),
                      "traffic": profile_traffic("small_single_fp64_64.txt", SMALL_SOURCES),
-                     "kernel": "small_single_kernel<double>",
+                     "kernel": "small_column_kernel<double>",
                      "peak_source": FP64_PEAK_SOURCE,
                      "note": "one 64 x 64 solve cannot fill the GPU: its bound is the 63-step dependent chain "
                              "(dependent_chain_estimate), not the FP64 throughput"},

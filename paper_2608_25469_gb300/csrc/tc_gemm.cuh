@@ -138,7 +138,7 @@ struct TcArgs {
   int negate;      // TC_OZ: add the product instead of subtracting it
   const int *rexp;  // TC_OZ: row exponents of A
   const int *cexp;  // TC_OZ: column exponents of B
-  uint32_t *scratch;  // TC_OZ: kOzTileWords words per CTA (residue bytes of its current tile)
+  uint32_t *scratch;  // TC_OZ: 2 kOzTileWords words per CTA (residue bytes of a tile being written and one being converted)
   int M, N, K;
   int tri;          // row tile i0 needs k < i0 + TC_PM only
   int npairs;       // TC_F32: slice pairs summed in the accumulator
@@ -339,6 +339,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
     const uint32_t bar0 = cluster_addr(&full[0], 0);
     int s = 0;
     uint32_t phase = 1;  // the first round finds every stage empty
+    uint32_t fills = 0;  // stages filled so far
     bool ok = true;
     for (int t = cid; t < ntiles && ok; t += ncl) {
       int m0, n0;
@@ -363,6 +364,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
             }
           }
           __syncwarp();
+          ++fills;
           if (++s == TC_STAGES) {
             s = 0;
             phase ^= 1;
@@ -370,6 +372,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
         }
       }
     }
+    // A CTA leaves with nothing outstanding: every stage has been released (so its
+    // loads have landed and the releases have arrived), and in the second CTA, where
+    // nobody else waits for them, the last commits have.
+    for (int k = 0; k < TC_STAGES && ok; ++k) {
+      ok = mbar_wait_bounded(&empty[s], phase, p.limit_ns, p.err);
+      if (++s == TC_STAGES) {
+        s = 0;
+        phase ^= 1;
+      }
+    }
+    // after a wait that gave up: the loads of the last fill of every stage
+    if (!ok && rank == 0)
+      for (uint32_t f = fills > TC_STAGES ? fills - TC_STAGES : 0; f < fills; ++f)
+        mbar_wait_bounded(&full[f % TC_STAGES], (f / TC_STAGES) & 1, p.limit_ns, p.err);
+    if (rank != 0) mbar_wait_bounded(&drained, 0, p.limit_ns, p.err);
   } else if (warp == 1) {
     if (rank == 0) {
       // MMA issuer (first CTA of the pair): per unit, wait for a drained
@@ -430,8 +447,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc_threads<MODE>(), 
           }
         }
       }
-      // every issued product has finished before tensor memory is released,
-      // also when a wait above gave up
+      // every issued product has finished before tensor memory is released, also
+      // when a wait above gave up (the second CTA's producer waits there)
       if (elect_one()) tc_commit_pair(&drained);
       __syncwarp();
       mbar_wait_bounded(&drained, 0, p.limit_ns, p.err);

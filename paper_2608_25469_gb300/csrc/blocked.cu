@@ -2,10 +2,9 @@
 //
 // Phase 1 (Section 4.3, "parallel diagonal block inversion"): the N_B x N_B
 // diagonal blocks D_t are inverted independently by forward substitution against
-// the identity (Section 4.3.1) on base blocks of 32 rows (FP32: 64), joined by
-// doubling (fp64_inverse.cu, r32_inverse.cu).  Algorithm 2's column streaming
-// keeps shared memory at O(N_B) for one N_B-row substitution; here no block of
-// that size is substituted, and shared memory holds base blocks and tiles only.
+// the identity (Section 4.3.1) in blocks of 32 rows, a warp per column of the
+// inverse (fp64_inverse.cu; FP32: 64-row blocks joined by doubling,
+// r32_inverse.cu).  As in Algorithm 2, shared memory is O(N_B): a column each.
 //
 // Phase 2 (Section 4.3, "sequential GEMM update and solve"), for r = 0..k:
 //   X_r = D_r^{-1} B_r                       (solve product, triangular)
@@ -453,7 +452,7 @@ __global__ void __launch_bounds__(32 * NW) small_tile_kernel(const GemmArgs<T> p
   constexpr int BM = 8 * WM, BN = 8 * WN;
   __shared__ T red[NW][BM * BN];
   const int m0 = (gridDim.y - 1 - blockIdx.y) * BM, n0 = blockIdx.x * BN;
-  fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, 0, p.tri ? min(p.K, m0 + BM) : p.K, m0, n0, red);
+  fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, p.tri ? min(p.K, m0 + BM) : p.K, m0, n0, red);
   const bool b1 = is_one(p.beta);
   for (int e = threadIdx.x; e < BM * BN; e += 32 * NW) {
     const int row = m0 + e % BM, col = n0 + e / BM;
@@ -544,14 +543,12 @@ hsma_status_t blocked_impl(const HsmaBlockedCfg &cfg, const T *A, int64_t lda, T
   // partial products of split-K launches (only when n is small, unless split K is off)
   const size_t p_elems =
       cfg.tile != 0 && cfg.split_k != HSMA_SPLITK_OFF && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
-  const size_t inv_bytes = hsma_fp64_inverse_scratch(nb, m, sizeof(T));
-  hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems + inv_bytes, st);
+  hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems, st);
   if (s != HSMA_OK) return s;
   T *Dinv = static_cast<T *>(ws);
-  T *Winv = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes + w_bytes + sizeof(T) * p_elems);
   T *W = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes);
   T *Pw = p_elems ? reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes + w_bytes) : nullptr;
-  s = hsma_fp64_diag_inverse<T>(nb, A, lda, m, unit, Dinv, Winv, st);
+  s = hsma_fp64_diag_inverse<T>(nb, A, lda, m, unit, Dinv, st);
   // W holds the current block row's right-hand side: copied from B for the
   // first block, written by the previous trailing update for the others, so
   // the solve product can write X_r straight into B_r.

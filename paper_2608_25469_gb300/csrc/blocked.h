@@ -23,11 +23,9 @@ hsma_status_t hsma_blocked_solve(int dtype, const HsmaBlockedCfg &cfg, const voi
 // Phase 1 alone, FP64 (T = double, cplx): invert the N_B x N_B diagonal blocks of
 // the lower triangle of A into Dinv (ceil(m/nb) blocks of nb x nb, column-major,
 // ld nb, zeros above the diagonal and outside a partial last block).  nb in
-// {32, 64, 128, 256, 512}; W: hsma_fp64_inverse_scratch bytes of workspace.
-size_t hsma_fp64_inverse_scratch(int nb, int64_t m, size_t esize);
+// {32, 64, 128, 256, 512}.
 template <class T>
-hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, T *W,
-                                     cudaStream_t st);
+hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, cudaStream_t st);
 
 // FP64 product used by the refinement residual: C = beta*C - L*X with L the
 // lower triangle of A (unit diagonal if unit), all column-major fp64 (m x m,

@@ -40,6 +40,8 @@ struct Elem<double> {
   __device__ __forceinline__ static double zero() { return 0.0; }
   __device__ __forceinline__ static double one() { return 1.0; }
   __device__ __forceinline__ static double mul(double a, double b) { return a * b; }
+  __device__ __forceinline__ static double add(double a, double b) { return a + b; }
+  __device__ __forceinline__ static double neg(double a) { return -a; }
   // s - a*x, one fused multiply-add
   __device__ __forceinline__ static double fms(double a, double x, double s) { return fma(-a, x, s); }
   __device__ __forceinline__ static double recip(double a) { return 1.0 / a; }
@@ -76,6 +78,8 @@ struct Elem<cplx> {
     r.im = fma(a.re, b.im, a.im * b.re);
     return r;
   }
+  __device__ __forceinline__ static cplx add(cplx a, cplx b) { return cplx{a.re + b.re, a.im + b.im}; }
+  __device__ __forceinline__ static cplx neg(cplx a) { return cplx{-a.re, -a.im}; }
   // s - a*x with four fused multiply-adds
   __device__ __forceinline__ static cplx fms(cplx a, cplx x, cplx s) {
     s.re = fma(-a.re, x.re, s.re);

@@ -1,31 +1,34 @@
 // FP64 inverses of the N_B x N_B diagonal blocks (phase 1 of the blocked
-// algorithm, Section 4.3) by doubling.
+// algorithm, Section 4.3): forward substitution against the identity
+// (Section 4.3.1) in blocks of 32 rows.
 //
-// Inverting an N_B-row block by substitution (Algorithm 2) is a chain of N_B
-// dependent steps, 0.3 ms at N_B = 256 and 1 ms at N_B = 512 on this GPU
-// whatever the number of blocks.  Here substitution inverts 32 x 32 blocks only,
-// one column per warp and lane-per-row, and each level joins adjacent h x h
-// inverses into a 2h x 2h one: for
-//   T = [A 0; C D],   T^-1 = [A^-1 0; -D^-1 C A^-1  D^-1],
-// W = C A^-1 and then -D^-1 W, for every pair of the level in one launch each,
-// with the known zeros of the triangular inverses left out.  The products are
-// small tiles on the FP64 tensor path; the tile size is the largest that still
-// gives every SM's sub-partitions work.
+// Substitution row by row (Algorithm 2) is a chain of N_B dependent steps, 0.3 ms at
+// N_B = 256 and 1 ms at N_B = 512 on this GPU whatever the number of blocks.
+// Here it inverts 32 x 32 base blocks only; below them a CTA carries one column
+// x of the inverse down the block rows,
+//   x_i = -D_ii^-1 (sum_{k < i} D_ik x_k),
+// with the column in shared memory and a lane per row: the sum is a run of
+// independent loads and multiply-adds, and what depends on the row before is
+// one 32-step product.  The CTAs need nothing from each other.
+//
+// Only inverses of 32-row blocks are multiplied, so D X - I stays at the level of
+// row-by-row substitution.  Joining inverses by doubling, -D22^-1 (D21 D11^-1),
+// costs the same multiply-adds but leaves the condition of the half-size blocks in
+// it: on LU factors of random matrices the residual of the solve was 1.3 (N_B =
+// 128) to 2.7 times (512) that of substitution, this form 1.0 to 1.1 times.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "blocked.h"
 #include "common.cuh"
-#include "fp64_tile.cuh"
 #include "trace.h"
-#include "workspace.h"
 
 namespace {
 
-constexpr int kBase = 32;      // blocks inverted by substitution
-constexpr int kBaseWarps = 4;  // columns per CTA of the base kernel
-constexpr int kFp64Warps = 4;  // warps per CTA of the products
+constexpr int kBase = 32;    // blocks inverted row by row
+constexpr int kInvWarps = 4;  // one per SM sub-partition
+constexpr int kMaxNb = 512;
 
 // Columns 4 y .. 4 y + 3 of the inverse of base block b (rows 32 b .. of the
 // matrix), one per warp: lane r holds row r of the block, scaled by 1/a_rr, in
@@ -33,10 +36,10 @@ constexpr int kFp64Warps = 4;  // warps per CTA of the products
 // one warp-wide multiply-add behind a shuffle (about 100 cycles, 400 complex);
 // several columns per warp would add their pipe time to every step.
 template <class T>
-__global__ void __launch_bounds__(32 * kBaseWarps) inv_base_kernel(const T *__restrict__ A, int64_t lda, int64_t m,
-                                                                   int nb, int unit, T *Dinv) {
+__global__ void __launch_bounds__(32 * kInvWarps) inv_base_kernel(const T *__restrict__ A, int64_t lda, int64_t m,
+                                                                  int nb, int unit, T *Dinv) {
   using E = Elem<T>;
-  const int lane = threadIdx.x & 31, j = blockIdx.y * kBaseWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, j = blockIdx.y * kInvWarps + (threadIdx.x >> 5);
   const int64_t r0 = (int64_t)blockIdx.x * kBase;
   const int s = (int)min((int64_t)kBase, m - r0);
   const T *D = A + r0 + r0 * lda;
@@ -55,88 +58,104 @@ __global__ void __launch_bounds__(32 * kBaseWarps) inv_base_kernel(const T *__re
   }
   T *Y = Dinv + (r0 / nb) * (int64_t)nb * nb;
   const int l = (int)(r0 % nb);
-  if (j < s && lane < s && lane >= j) Y[(l + lane) + (int64_t)(l + j) * nb] = x;
+  Y[(l + lane) + (int64_t)(l + j) * nb] = j < s && lane < s && lane >= j ? x : E::zero();
 }
 
-// Level h.  blockIdx.y = pair (rows 2 h y .. of the matrix), blockIdx.x = output
-// tile.  Pass 0: W = C A^-1 (ld h per pair); pass 1: the lower-left block of the
-// 2h inverse, -D^-1 W.  A partial last pair has a shorter D; a pair without a D
-// block does nothing.
-template <class T, int WT, int PASS>
-__global__ void __launch_bounds__(32 * kFp64Warps) inv_level_kernel(const T *__restrict__ A, int64_t lda, int64_t m,
-                                                                    int nb, int h, T *Dinv, T *W) {
-  constexpr int TS = 8 * WT;
-  __shared__ T red[kFp64Warps][TS * TS];
-  const int64_t i0 = (int64_t)blockIdx.y * 2 * h;
-  const int sd = (int)min((int64_t)h, m - i0 - h);
-  const int tiles = h / TS;
-  const int m0 = (blockIdx.x % tiles) * TS, n0 = (blockIdx.x / tiles) * TS;
-  if (m0 >= sd) return;
-  T *Y = Dinv + (i0 / nb) * (int64_t)nb * nb;
-  const int l0 = (int)(i0 % nb);
-  T *Wp = W + (int64_t)blockIdx.y * h * h;
-  if (PASS == 0) {  // column tile n0 of A^-1 starts at row n0
-    fp64_tile<T, WT, WT, kFp64Warps>(A + (i0 + h) + i0 * lda, lda, Y + l0 + (int64_t)l0 * nb, nb, sd, h, n0, h, m0, n0, red);
-  } else {  // row tile m0 of D^-1 ends at its diagonal
-    fp64_tile<T, WT, WT, kFp64Warps>(Y + (l0 + h) + (int64_t)(l0 + h) * nb, nb, Wp, h, sd, h, 0, min(sd, m0 + TS), m0, n0, red);
-  }
-  T *out = PASS == 0 ? Wp : Y + (l0 + h) + (int64_t)l0 * nb;
-  const int64_t ldo = PASS == 0 ? h : nb;
-  for (int e = threadIdx.x; e < TS * TS; e += 32 * kFp64Warps) {
-    const int i = m0 + e % TS, jc = n0 + e / TS;
-    if (i < sd) {
-      const T v = red[0][e];
-      out[i + (int64_t)jc * ldo] = PASS == 0 ? v : fp64_neg(v);
+// One column of the inverse of an outer block whose base blocks are in place; zeros
+// above the base block and past the matrix included.  The four warps take turns in
+// both products, kDepth columns of D at a time (the next kDepth in flight), and add
+// their parts through shared memory.  The FP64 pipe (64 cycles per warp-wide
+// multiply-add) bounds the longest column or, with many columns, the launch; a
+// block's longest columns start first.  A column per warp and one per two warps
+// leave the longest column's chain exposed: solves of 512 x 32 FP64 84 / 76 / 73 us
+// with 1 / 2 / 4 warps per column, emulated 512 x 128 (N_B = 512) 326 / 230 / 190 us
+// (joined by doubling 83 and 186 us; 8192 x 4096 emulated 7.53 -> 7.39 ms).
+template <class T>
+__global__ void __launch_bounds__(32 * kInvWarps) inv_columns_kernel(const T *__restrict__ A, int64_t lda, int64_t m,
+                                                                     int nb, T *Dinv) {
+  using E = Elem<T>;
+  constexpr int kDepth = 4, kPart = kBase / kInvWarps;
+  static_assert(2 * kDepth * kInvWarps == kBase && kPart == 2 * kDepth, "a block row is one turn of every warp");
+  __shared__ T sX[kInvWarps][kMaxNb];      // the column, a copy per warp
+  __shared__ T sSum[2][kInvWarps][kBase];  // the warps' parts of a sum and of a block row
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // block by block: CTAs that go to different SMs hold columns of nearly the same length
+  const int j = blockIdx.x % nb, blk = blockIdx.x / nb;
+  const int64_t r0 = (int64_t)blk * nb;
+  const int s = (int)min((int64_t)nb, m - r0);
+  const T *D = A + r0 + r0 * lda;
+  T *Y = Dinv + (int64_t)blk * nb * nb;
+  T *out = Y + (int64_t)j * nb, *x = sX[warp];
+  const int j0 = j & ~(kBase - 1);
+  for (int r = threadIdx.x; r < nb; r += 32 * kInvWarps)
+    if (r < j0 || j >= s || (r >= s && r >= j0 + kBase)) out[r] = E::zero();
+  if (j >= s) return;
+  auto sum_warps = [&](T v, int h) {  // in the same order in every warp
+    sSum[h][warp][lane] = v;
+    __syncthreads();
+    v = sSum[h][0][lane];
+#pragma unroll
+    for (int w = 1; w < kInvWarps; ++w) v = E::add(v, sSum[h][w][lane]);
+    return v;
+  };
+  x[j0 + lane] = out[j0 + lane];
+  __syncwarp();
+  for (int i0 = j0 + kBase; i0 < s; i0 += kBase) {
+    const T *d = D + min(i0 + lane, s - 1);  // lanes past the matrix repeat its last row
+    const T *inv = Y + (i0 + lane) + (int64_t)(i0 + kPart * warp) * nb;
+    T a[2][kDepth];
+    auto load = [&](int k0, int h) {  // columns before j meet zeros of x: not read
+#pragma unroll
+      for (int u = 0; u < kDepth; ++u) a[h][u] = k0 + u >= j ? E::ld(d + (int64_t)(k0 + u) * lda) : E::zero();
+    };
+    auto load_inv = [&](int k0, int h) {
+#pragma unroll
+      for (int u = 0; u < kDepth; ++u) a[h][u] = E::ld(inv + (int64_t)(k0 + u) * nb);
+    };
+    T acc = E::zero();
+    int k0 = j0 + kPart * warp;
+    load(k0, 0);
+    for (; k0 < i0; k0 += kBase) {
+      load(k0 + kDepth, 1);
+#pragma unroll
+      for (int u = 0; u < kDepth; ++u) acc = E::fms(a[0][u], x[k0 + u], acc);
+      if (k0 + kBase < i0)
+        load(k0 + kBase, 0);
+      else
+        load_inv(0, 0);
+#pragma unroll
+      for (int u = 0; u < kDepth; ++u) acc = E::fms(a[1][u], x[k0 + kDepth + u], acc);
     }
+    x[i0 + lane] = E::neg(sum_warps(acc, 0));
+    __syncwarp();
+    load_inv(kDepth, 1);
+    T y = E::zero();
+#pragma unroll
+    for (int u = 0; u < kPart; ++u) {
+      const int k = kPart * warp + u;
+      const T t = E::fms(a[u / kDepth][u % kDepth], x[i0 + k], y);
+      if (k <= lane) y = t;  // nothing above the diagonal is multiplied
+    }
+    y = sum_warps(y, 1);
+    __syncwarp();
+    x[i0 + lane] = y;
+    __syncwarp();
+    if (warp == 0 && i0 + lane < s) out[i0 + lane] = y;
   }
-}
-
-template <class T, int WT>
-void launch_level(const T *A, int64_t lda, int64_t m, int nb, int h, unsigned pairs, T *Dinv, T *W, cudaStream_t st) {
-  const unsigned tiles = (unsigned)(h / (8 * WT));
-  const dim3 grid(tiles * tiles, pairs);
-  inv_level_kernel<T, WT, 0><<<grid, 32 * kFp64Warps, 0, st>>>(A, lda, m, nb, h, Dinv, W);
-  inv_level_kernel<T, WT, 1><<<grid, 32 * kFp64Warps, 0, st>>>(A, lda, m, nb, h, Dinv, W);
 }
 
 }  // namespace
 
-size_t hsma_fp64_inverse_scratch(int nb, int64_t m, size_t esize) {
-  // the pairs of the last level, the largest: (N_B / 2)^2 per outer block
-  return nb > kBase ? esize * (size_t)((m + nb - 1) / nb) * (nb / 2) * (nb / 2) : 0;
-}
-
 template <class T>
-hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, T *W,
-                                     cudaStream_t st) {
-  if (nb < kBase || nb > 512 || (nb & (nb - 1)) != 0) return HSMA_ERR_UNSUPPORTED;
+hsma_status_t hsma_fp64_diag_inverse(int nb, const T *A, int64_t lda, int64_t m, int unit, T *Dinv, cudaStream_t st) {
+  if (nb < kBase || nb > kMaxNb || (nb & (nb - 1)) != 0) return HSMA_ERR_UNSUPPORTED;
   const int64_t nblk = (m + nb - 1) / nb, nbase = (m + kBase - 1) / kBase;
-  int levels = 0;
-  for (int h = kBase; h < nb; h *= 2) ++levels;
-  HsmaTraceScope ts("diag_inverse", st, 1 + 2 * levels);
-  // zeros above the diagonals and outside a partial block
-  HSMA_CUDA_TRY(cudaMemsetAsync(Dinv, 0, sizeof(T) * (size_t)nblk * nb * nb, st));
-  inv_base_kernel<T><<<dim3((unsigned)nbase, kBase / kBaseWarps), 32 * kBaseWarps, 0, st>>>(A, lda, m, nb, unit,
-                                                                                           Dinv);
-  for (int h = kBase; h < nb; h *= 2) {
-    const int64_t pairs = (m + 2 * h - 1) / (2 * h);
-    if (pairs > 65535) return HSMA_ERR_UNSUPPORTED;
-    const int64_t want = 4 * (int64_t)hsma_sm_count();  // CTAs for the SMs to share evenly
-    const int64_t t32 = pairs * (h / 32) * (h / 32);
-    bool done = false;
-    if constexpr (sizeof(T) == sizeof(double)) {  // complex: too many registers
-      if ((done = t32 >= want)) launch_level<T, 4>(A, lda, m, nb, h, (unsigned)pairs, Dinv, W, st);
-    }
-    if (done) continue;
-    if (4 * t32 >= want)
-      launch_level<T, 2>(A, lda, m, nb, h, (unsigned)pairs, Dinv, W, st);
-    else
-      launch_level<T, 1>(A, lda, m, nb, h, (unsigned)pairs, Dinv, W, st);
-  }
+  HsmaTraceScope ts("diag_inverse", st, nb > kBase ? 2 : 1);
+  inv_base_kernel<T><<<dim3((unsigned)nbase, kBase / kInvWarps), 32 * kInvWarps, 0, st>>>(A, lda, m, nb, unit, Dinv);
+  if (nb > kBase) inv_columns_kernel<T><<<(unsigned)(nblk * nb), 32 * kInvWarps, 0, st>>>(A, lda, m, nb, Dinv);
   return hsma_from_cuda(cudaGetLastError());
 }
 
-template hsma_status_t hsma_fp64_diag_inverse<double>(int, const double *, int64_t, int64_t, int, double *, double *,
+template hsma_status_t hsma_fp64_diag_inverse<double>(int, const double *, int64_t, int64_t, int, double *,
                                                       cudaStream_t);
-template hsma_status_t hsma_fp64_diag_inverse<cplx>(int, const cplx *, int64_t, int64_t, int, cplx *, cplx *,
-                                                    cudaStream_t);
+template hsma_status_t hsma_fp64_diag_inverse<cplx>(int, const cplx *, int64_t, int64_t, int, cplx *, cudaStream_t);

@@ -44,20 +44,13 @@ struct Fp64Acc<cplx> {
   __device__ __forceinline__ cplx get(int q) const { return cplx{re[q], im[q]}; }
 };
 
-__device__ __forceinline__ double fp64_add(double a, double b) { return a + b; }
-__device__ __forceinline__ cplx fp64_add(cplx a, cplx b) { return cplx{a.re + b.re, a.im + b.im}; }
-
-__device__ __forceinline__ double fp64_neg(double a) { return -a; }
-__device__ __forceinline__ cplx fp64_neg(cplx a) { return cplx{-a.re, -a.im}; }
-
-
 // Rows m0 .. m0 + 8 WM - 1 and columns n0 .. n0 + 8 WN - 1 of A B over
-// k = kbeg .. kend - 1 (A: M x kend column-major, B: kend x N column-major;
+// k < kend (A: M x kend column-major, B: kend x N column-major;
 // entries outside read as zero).  All NW warps of the CTA take part; the tile is left in
 // red[0] (column-major, 8 WM rows) after a CTA barrier.
 template <class T, int WM, int WN, int NW>
 __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, int64_t ldb,
-                                          int M, int N, int kbeg, int kend, int m0, int n0,
+                                          int M, int N, int kend, int m0, int n0,
                                           T (*red)[8 * WM * 8 * WN]) {
   using E = Elem<T>;
   constexpr int U = WM * WN >= 16 ? 2 : 4;  // K steps per load group; one group is in flight while another is multiplied
@@ -95,7 +88,7 @@ __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, 
     }
   };
   constexpr int kGroup = 4 * NW * U;
-  int k0 = kbeg + 4 * warp;
+  int k0 = 4 * warp;
   load(k0, 0);
   while (k0 < kend) {
     load(k0 + kGroup, 1);
@@ -116,7 +109,7 @@ __device__ __forceinline__ void fp64_tile(const T *__restrict__ A, int64_t lda, 
   for (int e = threadIdx.x; e < 8 * WM * 8 * WN; e += 32 * NW) {
     T v = red[0][e];
 #pragma unroll
-    for (int w = 1; w < NW; ++w) v = fp64_add(v, red[w][e]);
+    for (int w = 1; w < NW; ++w) v = E::add(v, red[w][e]);
     red[0][e] = v;
   }
   __syncthreads();

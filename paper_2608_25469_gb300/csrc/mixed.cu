@@ -1028,8 +1028,8 @@ __global__ void scale_kernel(double *B, int64_t ldb, int64_t rows, int64_t n, do
 struct EmuLayout {
   int W = 1, h = 1, Kpb = 0, Kpp = 0;
   int64_t P = 0;
-  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0, sc_b = 0, iv_b = 0;
-  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b + sc_b + iv_b; }
+  size_t dinv_b = 0, w_b = 0, pa_b = 0, pd_b = 0, px_b = 0, sc_b = 0;
+  size_t total() const { return dinv_b + w_b + pa_b + pd_b + px_b + sc_b; }
 };
 
 EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
@@ -1048,7 +1048,6 @@ EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
   L.pd_b = al(oz_operand_bytes((int64_t)L.W * nb, L.Kpb));
   L.px_b = al(oz_operand_bytes(n, L.Kpp));
   L.sc_b = al(oz_scratch_bytes(L.W * m, n));
-  L.iv_b = hsma_fp64_inverse_scratch(nb, m, eb);
   return L;
 }
 
@@ -1091,10 +1090,9 @@ hsma_status_t blocked_emulated(bool cplx_, int nb, int panel_cols, const double 
     return oz_product(Pa, Px, B + W * rb, (int64_t)W * ldb, 1, 0, 0, scratch, nullptr, phase, st);
   };
   do {
-    unsigned char *iv = px_mem + E.px_b + E.sc_b;
     s = cplx_ ? hsma_fp64_diag_inverse<cplx>(nb, reinterpret_cast<const cplx *>(A), lda, m, unit,
-                                             reinterpret_cast<cplx *>(Dinv), reinterpret_cast<cplx *>(iv), st)
-              : hsma_fp64_diag_inverse<double>(nb, A, lda, m, unit, Dinv, reinterpret_cast<double *>(iv), st);
+                                             reinterpret_cast<cplx *>(Dinv), st)
+              : hsma_fp64_diag_inverse<double>(nb, A, lda, m, unit, Dinv, st);
     if (s != HSMA_OK) break;
     if (alpha[0] != 1.0 || (cplx_ && alpha[1] != 0.0)) {
       HsmaTraceScope ts("copy", st);

@@ -521,6 +521,24 @@ cplx make_scalar<cplx>(const double *a) {
   return cplx{a[0], a[1]};
 }
 
+// Workspace of one blocked solve: the inverses, one block row of B and, for
+// HSMA_TILE_* with split K, partial products (only needed when n is small).
+struct BlockedLayout {
+  size_t dinv_b, w_b, p_elems, esize;
+  size_t total() const { return dinv_b + w_b + esize * p_elems; }
+};
+
+BlockedLayout blocked_layout(const HsmaBlockedCfg &cfg, size_t esize, int64_t m, int64_t n) {
+  BlockedLayout L;
+  const size_t nb = (size_t)cfg.nb, nblk = ((size_t)m + nb - 1) / nb;
+  L.esize = esize;
+  L.dinv_b = esize * nblk * nb * nb;
+  L.w_b = esize * nb * (size_t)n;
+  const bool split = cfg.tile != 0 && cfg.split_k != HSMA_SPLITK_OFF;
+  L.p_elems = split && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
+  return L;
+}
+
 // Blocked two-phase solve (Section 4.3).  Phase 1 inverts every diagonal
 // block; phase 2 walks the block rows r: X_r = D_r^{-1} W, where W holds the
 // block row's right-hand side after the updates, and the updates are either
@@ -538,16 +556,13 @@ hsma_status_t blocked_impl(const HsmaBlockedCfg &cfg, const T *A, int64_t lda, T
   const T al = make_scalar<T>(alpha);
   const T one = make_scalar<T>((const double[2]){1.0, 0.0});
   void *ws = nullptr;
-  const size_t dinv_bytes = sizeof(T) * (size_t)nblk * nb * nb;
-  const size_t w_bytes = sizeof(T) * (size_t)nb * n;
-  // partial products of split-K launches (only when n is small, unless split K is off)
-  const size_t p_elems =
-      cfg.tile != 0 && cfg.split_k != HSMA_SPLITK_OFF && (size_t)n * 64 < (size_t)2 * sm_count() * 64 * 64 ? partial_elems_max() : 0;
-  hsma_status_t s = hsma_ws_alloc(&ws, dinv_bytes + w_bytes + sizeof(T) * p_elems, st);
+  const BlockedLayout L = blocked_layout(cfg, sizeof(T), m, n);
+  const size_t p_elems = L.p_elems;
+  hsma_status_t s = hsma_ws_alloc(&ws, L.total(), st);
   if (s != HSMA_OK) return s;
   T *Dinv = static_cast<T *>(ws);
-  T *W = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes);
-  T *Pw = p_elems ? reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + dinv_bytes + w_bytes) : nullptr;
+  T *W = reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + L.dinv_b);
+  T *Pw = p_elems ? reinterpret_cast<T *>(static_cast<unsigned char *>(ws) + L.dinv_b + L.w_b) : nullptr;
   s = hsma_fp64_diag_inverse<T>(nb, A, lda, m, unit, Dinv, st);
   // W holds the current block row's right-hand side: copied from B for the
   // first block, written by the previous trailing update for the others, so
@@ -692,6 +707,10 @@ bool hsma_make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes, 
   CUresult r = enc(map, dt, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+size_t hsma_blocked_ws_bytes(int dtype, const HsmaBlockedCfg &cfg, int64_t m, int64_t n) {
+  return blocked_layout(cfg, dtype == HSMA_C128 ? sizeof(cplx) : sizeof(double), m, n).total();
 }
 
 hsma_status_t hsma_blocked_solve(int dtype, const HsmaBlockedCfg &cfg, const void *A, int64_t lda, void *B,

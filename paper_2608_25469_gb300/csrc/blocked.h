@@ -20,6 +20,9 @@ struct HsmaBlockedCfg {
 hsma_status_t hsma_blocked_solve(int dtype, const HsmaBlockedCfg &cfg, const void *A, int64_t lda, void *B,
                                  int64_t ldb, int64_t m, int64_t n, const double *alpha, int unit, cudaStream_t st);
 
+// Bytes of workspace that solve takes.
+size_t hsma_blocked_ws_bytes(int dtype, const HsmaBlockedCfg &cfg, int64_t m, int64_t n);
+
 // Phase 1 alone, FP64 (T = double, cplx): invert the N_B x N_B diagonal blocks of
 // the lower triangle of A into Dinv (ceil(m/nb) blocks of nb x nb, column-major,
 // ld nb, zeros above the diagonal and outside a partial last block).  nb in

@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "../../include/hsma.h"
+#include "blocked.h"
 #include "common.cuh"
 #include "gen.h"
 #include "mixed.h"
@@ -119,10 +120,13 @@ size_t request_bytes(const hsma_request_t &r, unsigned flags) {
   }
   if (r.m > 64) {
     hsma_plan_t p;
-    hsma_plan(r.dtype, r.m, r.n, &p);
-    const size_t nb = (size_t)(p.nb > 0 ? p.nb : 256);
-    const size_t nblk = ((size_t)r.m + nb - 1) / nb;
-    b += es * (nblk * nb * nb + nb * (size_t)r.n);  // Dinv + block-row copy
+    HsmaBlockedCfg cfg;
+    if (hsma_plan(r.dtype, r.m, r.n, &p) == HSMA_OK) {
+      cfg.nb = p.nb;
+      cfg.tile = p.tile;
+      cfg.split_k = p.split_k;
+    }
+    b += hsma_blocked_ws_bytes(r.dtype, cfg, r.m, r.n);
   }
   return b;
 }

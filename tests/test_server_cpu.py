@@ -111,3 +111,21 @@ def test_emulated_flag_accounts_for_its_workspace(H):
     assert H.hsma_server_drain(s, 30.0) == 0
     assert all(H.hsma_server_poll(s, t)[2] == 0 for t in ts)
     assert H.hsma_server_destroy(s) == 0
+
+
+def test_budget_counts_the_partial_products_of_split_products(H, tmp_path):
+    """A configuration table with staged tiles and split K makes the blocked solve take partial
+    products too (over 6 MB at 152 SMs): a budget without room for them admits no such request."""
+    need = 8 * 512 * 512 + 8 * 512 * 64 + 8 * (4 * 128 * 128 + 128 * 64)  # A, B, inverses, a block row
+    f = tmp_path / "table.txt"
+    for tile, split, status in ((0, 1, 0), (3, 2, 0), (3, 1, 3)):
+        f.write_text("0 512 64 128 %d %d 1 2048\n" % (tile, split))
+        assert H.hsma_tuning_load(str(f)) == 0
+        try:
+            s = H.hsma_server_create(need, 1, H.SERVER_FAKE_DEVICE)
+            t = H.hsma_server_submit(s, _req(H, 512, 64))
+            assert H.hsma_server_drain(s, 30.0) == 0
+            assert H.hsma_server_poll(s, t)[2] == status, (tile, split)
+            assert H.hsma_server_destroy(s) == 0
+        finally:
+            assert H.hsma_tuning_load(None) == 0

@@ -106,9 +106,10 @@ size_t request_bytes(const hsma_request_t &r, unsigned flags) {
   size_t b = es * (size_t)r.m * (size_t)r.m + es * (size_t)r.m * (size_t)r.n;
   if (r.ipiv_host != nullptr) b += sizeof(int32_t) * (size_t)r.m;
   if (r.m > 64 && r.kind != HSMA_REQ_TRSM) {
-    // the factor solves: permutation and a gathered copy of B, then two
-    // triangular solves one after the other (their workspaces never coexist)
-    b += sizeof(int32_t) * (size_t)r.m + es * (size_t)r.m * (size_t)r.n;
+    // the factor solves: the second triangular solve gathers its triangle and B in
+    // lower form beside its own workspace (the permutation with its copy of B and
+    // the first solve's workspace are freed before)
+    b += es * (size_t)r.m * (size_t)r.m + es * (size_t)r.m * (size_t)r.n + 512;
   }
   if (use_emulated(r, flags)) {
     hsma_opts_t o;

@@ -129,3 +129,19 @@ def test_budget_counts_the_partial_products_of_split_products(H, tmp_path):
             assert H.hsma_server_destroy(s) == 0
         finally:
             assert H.hsma_tuning_load(None) == 0
+
+
+@pytest.mark.parametrize("kind", ["GETRS", "POTRS"])
+def test_budget_counts_the_second_triangle_of_a_factor_solve(H, kind):
+    """The second triangular solve of a factor solve gathers its triangle and B into lower form."""
+    m, n = 512, 64
+    need = 8 * m * m + 8 * m * n + 8 * (4 * 128 * 128 + 128 * n)  # as a triangular solve
+    gathered = 8 * m * m + 8 * m * n
+    for budget, status in ((need + gathered + 1024, 0), (need + gathered - 8 * m * n, 3)):
+        s = H.hsma_server_create(budget, 1, H.SERVER_FAKE_DEVICE)
+        r = _req(H, m, n)
+        r.kind = getattr(H, "REQ_" + kind)
+        t = H.hsma_server_submit(s, r)
+        assert H.hsma_server_drain(s, 30.0) == 0
+        assert H.hsma_server_poll(s, t)[2] == status
+        assert H.hsma_server_destroy(s) == 0

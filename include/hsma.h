@@ -31,7 +31,8 @@
  *  - Quick returns: m == 0 or n == 0 is a no-op; alpha == 0 sets B := 0 and does
  *    not read A.
  *  - A singular A (a zero on the diagonal) is not detected; IEEE infinities and
- *    NaNs propagate, as in BLAS.
+ *    NaNs propagate, as in BLAS (emulated FP64 products write NaN for both: an
+ *    infinity too leaves them as NaN).
  *  - Workspace (diagonal-block inverses, refinement copies, batch schedules)
  *    is taken from a stream-ordered memory pool the library keeps per device
  *    (CUDA's default pool while `stream` is capturing a graph) on `stream`

@@ -613,6 +613,9 @@ __global__ void check_kernel(double *sums, int *state, double alpha_abs, double 
 // modulus gives the residues of the exact integer product, which is converted
 // to FP64 with one rounding and added to the result.  The fixed-point rounding
 // contributes at most 2^-59 of |row scale| |column scale| per product term.
+// Infinities and NaNs take no part in the scales or the residues: they mark their
+// row (left operand) or the rest of their column (right operand), where the result
+// is NaN (oz_tables.cuh).
 // ---------------------------------------------------------------------------
 constexpr int kOzExpEmpty = -1100;  // exponent of an all-zero row
 
@@ -664,6 +667,7 @@ __device__ __forceinline__ uint32_t oz_pair(float lo, float hi) {
 __device__ __forceinline__ uint64_t oz_absbits(double x) {
   return (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
+constexpr uint64_t kOzInfBits = 0x7ffull << 52;  // |x| of infinities and, above, NaNs
 
 // Entry (r, k) of the rows x K block of a column-major matrix (T = double, or
 // complex double as (re, im)) under a mode: 0 = the whole block; 1 = lower
@@ -706,7 +710,8 @@ __global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__
   for (int q = 0; q < 8; ++q) {
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, r0 + lane + 32 * q, k, re, im);
-    mx = max(mx, max(oz_absbits(re), oz_absbits(im)));
+    const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
+    if (ab < kOzInfBits) mx = max(mx, ab);
   }
   const int e = __reduce_max_sync(0xffffffffu, mx != 0 ? oz_exponent(mx) : kOzExpEmpty);
   if (lane == 0 && e != kOzExpEmpty) {
@@ -735,7 +740,10 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, i, k, re, im);
     const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
-    if (ab != 0) ex = max(ex, oz_exponent(ab) - kexp[W * k]);
+    if (ab >= kOzInfBits)
+      ex = kOzExpBad;
+    else if (ab != 0)
+      ex = max(ex, oz_exponent(ab) - kexp[W * k]);
   }
   red[ty][tx] = ex;
   __syncthreads();
@@ -781,7 +789,7 @@ __global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restric
     const int r = i0 + ii;
     if (r >= rows) break;
     const int e = rexp[W * r];
-    const bool zero = e == kOzExpEmpty;
+    const bool zero = e == kOzExpEmpty || e == kOzExpBad;
     float a0[4], a1[4];
     oz_limbs(zero ? 0 : oz_fixed(sre[CPLX ? tx : 2 * tx][ii], e + g0), a0);
     oz_limbs(zero ? 0 : oz_fixed(CPLX ? sim[tx][ii] : sre[2 * tx + 1][ii], e + g1), a1);
@@ -803,38 +811,50 @@ __global__ void __launch_bounds__(256) oz_slice_a_kernel(const double *__restric
 // Residues of a right operand: K x N column-major (complex: its real view with
 // 2K rows), balanced by 2^g_k (rows with g_k = kOzExpEmpty are ignored), as
 // out[l][j][k], N x Kp row-major per modulus (zero beyond K), plus the column
-// exponents.  One CTA per column: its largest exponent, then the residues, a
-// thread two consecutive k (128 bytes per warp and modulus).
+// exponents.  One CTA per column: its largest exponent and first infinity or NaN
+// (W = 2: either part of a complex entry), then the residues, a thread two
+// consecutive k (128 bytes per warp and modulus).
 __global__ void __launch_bounds__(256) oz_slice_x_kernel(const double *__restrict__ X, int64_t ldx, int K, int N,
-                                                         int Kp, const int *__restrict__ kexp, int *cexp,
+                                                         int Kp, int W, const int *__restrict__ kexp, int *cexp,
                                                          uint32_t *out, size_t pstride, const int *skip) {
   if (skip != nullptr && *(volatile const int *)skip) return;
-  __shared__ int red[8];
+  __shared__ int red[8], red_bad[8];
   const int tid = threadIdx.x;
   for (int64_t j = blockIdx.x; j < N; j += gridDim.x) {
     const double *x = X + j * ldx;
-    int ex = INT_MIN;
+    int ex = INT_MIN, bad = INT_MAX;
 #pragma unroll 4
     for (int k = tid; k < K; k += 256) {
       const uint64_t ab = oz_absbits(x[k]);
       const int g = kexp[k];
-      if (ab != 0 && g != kOzExpEmpty) ex = max(ex, oz_exponent(ab) + g);
+      if (ab >= kOzInfBits)
+        bad = min(bad, k);
+      else if (ab != 0 && g != kOzExpEmpty)
+        ex = max(ex, oz_exponent(ab) + g);
     }
     ex = __reduce_max_sync(0xffffffffu, ex);
-    if ((tid & 31) == 0) red[tid >> 5] = ex;
+    bad = __reduce_min_sync(0xffffffffu, bad);
+    if ((tid & 31) == 0) {
+      red[tid >> 5] = ex;
+      red_bad[tid >> 5] = bad;
+    }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < 8; ++w) ex = max(ex, red[w]);
-    __syncthreads();  // red is rewritten by the next column
+    for (int w = 0; w < 8; ++w) {
+      ex = max(ex, red[w]);
+      bad = min(bad, red_bad[w]);
+    }
+    __syncthreads();  // both are rewritten by the next column
     const int e = ex == INT_MIN ? 0 : ex;
-    if (tid == 0) cexp[j] = e;
+    if (tid == 0) cexp[j] = bad == INT_MAX ? e : oz_flag_column(e, bad - bad % W);
     uint32_t *o = out + (size_t)j * (Kp / 2);
     for (int k = 2 * tid; k < Kp; k += 512) {
       float a[2][4];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int g = k + h < K ? kexp[k + h] : kOzExpEmpty;
-        oz_limbs(g != kOzExpEmpty ? oz_fixed(x[k + h], e - g) : 0, a[h]);
+        const double v = g != kOzExpEmpty ? x[k + h] : 0.0;
+        oz_limbs(oz_absbits(v) < kOzInfBits ? oz_fixed(v, e - g) : 0, a[h]);
       }
 #pragma unroll
       for (int l = 0; l < kOzP; ++l)
@@ -905,11 +925,11 @@ hsma_status_t oz_slice_a(bool cplx, const double *A, int64_t lda, int rows, int 
 
 // Slice the K x N real matrix X (complex: its real view) into o (o.rows = N),
 // balanced by the K-balancing exponents of the left operand it multiplies.
-hsma_status_t oz_slice_x(const double *X, int64_t ldx, int K, const int *kexp, OzOperand &o, const int *skip,
-                         cudaStream_t st) {
+hsma_status_t oz_slice_x(bool cplx, const double *X, int64_t ldx, int K, const int *kexp, OzOperand &o,
+                         const int *skip, cudaStream_t st) {
   if (o.rows <= 0) return HSMA_OK;
   const int grid = std::min(o.rows, hsma_sm_count() * 16);
-  oz_slice_x_kernel<<<grid, 256, 0, st>>>(X, ldx, K, o.rows, o.Kp, kexp, o.exps,
+  oz_slice_x_kernel<<<grid, 256, 0, st>>>(X, ldx, K, o.rows, o.Kp, cplx ? 2 : 1, kexp, o.exps,
                                           reinterpret_cast<uint32_t *>(o.slices), (size_t)o.rows * o.Kp / 2, skip);
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
@@ -951,6 +971,7 @@ hsma_status_t oz_product(const OzOperand &L, const OzOperand &X, double *C, int6
     a.N = X.rows;
     a.K = (int)std::min<int64_t>(kmax, L.Kp - c0);
     a.tri = tri;
+    a.row0 = (int)i0;
     a.skip = skip;
     SliceLayout la, lb;  // views into the full planes at row i0 and column c0
     la.rows = L.rows - i0;
@@ -986,7 +1007,7 @@ hsma_status_t oz_residual(const OzOperand &L, const double *X, int64_t ldx, int6
     hsma_status_t s;
     {
       HsmaTraceScope ts("residual_slices", st);
-      if ((s = oz_slice_x(X + j0 * ldx, ldx, L.rows, L.kexp, Xo, skip, st)) != HSMA_OK) return s;
+      if ((s = oz_slice_x(false, X + j0 * ldx, ldx, L.rows, L.kexp, Xo, skip, st)) != HSMA_OK) return s;
     }
     if ((s = oz_product(L, Xo, R + j0 * ldr, ldr, 1, 0, 1, scratch, skip, "residual", st)) != HSMA_OK) return s;
   }
@@ -1084,7 +1105,7 @@ hsma_status_t blocked_emulated(bool cplx_, int nb, int panel_cols, const double 
     {
       HsmaTraceScope ts("slices", st, 5);  // oz_slice_a: 4 kernels, oz_slice_x: 1
       hsma_status_t e = oz_slice_a(cplx_, A + W * (rb + c0 * lda), lda, (int)rows, k, 0, Pa, st);
-      if (e == HSMA_OK) e = oz_slice_x(B + W * c0, (int64_t)W * ldb, W * k, Pa.kexp, Px, nullptr, st);
+      if (e == HSMA_OK) e = oz_slice_x(cplx_, B + W * c0, (int64_t)W * ldb, W * k, Pa.kexp, Px, nullptr, st);
       if (e != HSMA_OK) return e;
     }
     return oz_product(Pa, Px, B + W * rb, (int64_t)W * ldb, 1, 0, 0, scratch, nullptr, phase, st);
@@ -1116,7 +1137,7 @@ hsma_status_t blocked_emulated(bool cplx_, int nb, int panel_cols, const double 
         {
           HsmaTraceScope ts("slices", st, 5);
           if ((s = oz_slice_a(cplx_, Dinv + (size_t)W * r * nb * nb, nb, sr, sr, 1, Pd, st)) != HSMA_OK) break;
-          if ((s = oz_slice_x(Wb, (int64_t)W * nb, W * sr, Pd.kexp, Px, nullptr, st)) != HSMA_OK) break;
+          if ((s = oz_slice_x(cplx_, Wb, (int64_t)W * nb, W * sr, Pd.kexp, Px, nullptr, st)) != HSMA_OK) break;
         }
         if ((s = oz_product(Pd, Px, B + W * r0, (int64_t)W * ldb, 0, 1, 1, scratch, nullptr, "solve_gemm",
                             st)) != HSMA_OK)
@@ -1321,7 +1342,7 @@ extern "C" HSMA_API hsma_status_t hsma_gemm_f64_emulated(int64_t M, int64_t N, i
   uint32_t *scratch = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(ws) + a_b + x_b);
   OzOperand Ao = oz_operand(ws, M, Kp), Xo = oz_operand(static_cast<unsigned char *>(ws) + a_b, N, Kp);
   s = oz_slice_a(false, A, lda, (int)M, (int)K, 0, Ao, st);
-  if (s == HSMA_OK) s = oz_slice_x(X, ldx, (int)K, Ao.kexp, Xo, nullptr, st);
+  if (s == HSMA_OK) s = oz_slice_x(false, X, ldx, (int)K, Ao.kexp, Xo, nullptr, st);
   if (s == HSMA_OK) s = oz_product(Ao, Xo, C, ldc, 1, 0, 0, scratch, nullptr, "emulated_gemm", st);
   hsma_status_t f = hsma_ws_free(ws, st);
   return s != HSMA_OK ? s : f;

@@ -40,6 +40,15 @@ __device__ __forceinline__ size_t oz_scratch_at(int cta, int half, int col) {
   return (size_t)(2 * cta + half) * kOzTileWords + (size_t)(col / 4) * 128;
 }
 
+// Operands with infinities or NaNs: a row of the left operand that holds one has
+// the exponent kOzExpBad; a column of the right one whose first one is at k has
+// (k + 1) << 16 added to the low half of its exponent.  Either takes an entry's
+// exponent past kOzExpFlag (finite operands stay below 2^13), and the conversion
+// writes NaN: to the whole row, and to the column from row k on (a triangular
+// product does not multiply it above) or, of a full product, to all of it.
+constexpr int kOzExpBad = 1 << 20, kOzExpFlag = 1 << 14;
+__host__ __device__ constexpr int oz_flag_column(int e, int k) { return ((k + 1) << 16) | (e & 0xffff); }
+
 struct OzTables {
   // slicing: balanced weights (2^15)^j of the four 15-bit limbs, for the left
   // operand times (P / p_l)^-1, modulo p_l

@@ -141,6 +141,7 @@ struct TcArgs {
   uint32_t *scratch;  // TC_OZ: 2 kOzTileWords words per CTA (residue bytes of a tile being written and one being converted)
   int M, N, K;
   int tri;          // row tile i0 needs k < i0 + TC_PM only
+  int row0;         // TC_OZ, tri: row 0 and column 0 are this row and column of the operand
   int npairs;       // TC_F32: slice pairs summed in the accumulator
   int band;         // tile rows per band of the tile order (set by the launcher)
   uint8_t pa[kTcMaxPairs], pb[kTcMaxPairs];  // TC_F32: slice of A and of B for each pair
@@ -220,14 +221,22 @@ __device__ __forceinline__ void oz_convert(const TcArgs &p, int cid, int h, int 
     for (int j = 0; j < 4; ++j) {
       y[j] = oz_crt(w, j, e[j]);
       e[j] += rx + __ldg(cx + min(c0 + j, cols - 1));
-      normal &= y[j] == 0 || oz_scales(e[j]);
+      normal &= (y[j] == 0 && e[j] < kOzExpFlag) || oz_scales(e[j]);
     }
     double x[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) x[j] = oz_scaled(y[j], e[j]);
     if (!normal) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = ldexp(__longlong_as_double((long long)y[j]), e[j]);
+      for (int j = 0; j < 4; ++j) {
+        const int c = __ldg(cx + min(c0 + j, cols - 1));
+        bool bad = rx >= kOzExpFlag;
+        if (c >= kOzExpFlag) {
+          bad |= p.tri == 0 || row + p.row0 >= (c >> 16) - 1;
+          e[j] += (int)(int16_t)(c & 0xffff) - c;
+        }
+        x[j] = bad ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(__longlong_as_double((long long)y[j]), e[j]);
+      }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)

@@ -152,6 +152,54 @@ def test_emulated_blocked_unit_diagonal(H, code):
     assert oracle.forward_error(X, ref) <= TOL
 
 
+@pytest.mark.parametrize("M,N,K", [(300, 270, 100), (257, 40, 8200)])
+def test_emulated_gemm_non_finite_entries(H, M, N, K):
+    """An infinity or NaN makes its row of A and its column of X NaN in the result and nothing else."""
+    rng = np.random.default_rng(M)
+    A = np.asfortranarray(rng.integers(-1024, 1025, (M, K)).astype(np.float64))
+    X = np.asfortranarray(rng.integers(-1024, 1025, (K, N)).astype(np.float64))
+    exact = -(A.astype(np.int64) @ X.astype(np.int64)).astype(np.float64)
+    A[5, 3], A[M - 1, K - 1] = np.nan, -np.inf
+    X[9, 11], X[K - 1, N - 1] = np.inf, np.nan
+    got = _gemm(H, A, X, np.zeros((M, N), order="F"))
+    bad = np.zeros((M, N), bool)
+    bad[[5, M - 1]] = True
+    bad[:, [11, N - 1]] = True
+    assert np.all(np.isnan(got[bad]))
+    assert np.array_equal(got[~bad], exact[~bad])
+
+
+@pytest.mark.parametrize("code", [I.R64, I.C128, 5], ids=["f64", "c128", "c64"])
+@pytest.mark.parametrize("what", ["nan_b", "inf_b", "nan_a", "inf_a", "zero_diagonal"])
+@pytest.mark.parametrize("row,nb", [(333, 128), (511, 512), (1, 128)])
+def test_emulated_blocked_non_finite_propagates(H, code, what, row, nb):
+    """As in the substitution formula, an infinity or NaN of B reaches its column from its row on,
+    and one of A (or a zero on its diagonal) every column from its row on: nothing there comes out
+    finite, and everything else is as without it.  complex64 runs these products by default."""
+    import torch
+    m, n, col = 700, 40, 7
+    wide = I.C128 if code == 5 else code
+    A0, B0 = I.gen_A(3, m, wide), I.gen_B(3, m, n, wide)
+    A, B = A0.copy(order="F"), B0.copy(order="F")
+    v = {"nan": np.nan, "inf": np.inf}.get(what[:3], 0.0)
+    if what.endswith("_b"):
+        B[row, col] = v if wide == I.R64 else complex(0.5, v)  # the imaginary part alone
+    else:
+        A[row, row // 2 if what != "zero_diagonal" else row] = v
+    if code == 5:
+        dA, dB = H.to_device(A.astype(np.complex64)), H.to_device(B.astype(np.complex64))
+        H.hsma_trsm_llnn(5, 0, m, n, 1.0, dA.data_ptr(), m, dB.data_ptr(), m, H.stream_ptr())
+        torch.cuda.synchronize()
+        X = H.from_device(dB).astype(np.complex128)
+    else:
+        X = _run(H, code, A, B, 1.0, nb)
+    bad = np.zeros((m, n), bool)
+    bad[row:, col if what.endswith("_b") else slice(None)] = True
+    assert not np.any(np.isfinite(X[bad]))
+    ref = oracle.solve(A0, B0, 1.0)
+    assert np.linalg.norm((X - ref)[~bad]) <= (2e-5 if code == 5 else TOL) * np.linalg.norm(ref)
+
+
 def test_emulated_blocked_badly_scaled_rows(H):
     """Rows of A and B scaled by powers of two from 2^-300 to 2^300: the solution is unchanged
     and the per-row scales of the slices keep it at full accuracy (exponent rebasing falls back

@@ -137,9 +137,14 @@ typedef struct {
                           (DMMA, IEEE FP64 roundings); 1 = FP64 emulated on the
                           BF16 tensor cores: both operands rounded to 59-bit fixed
                           point per row / column scale, multiplied exactly through
-                          17 residues, one FP64 rounding per product (error below
-                          2^-59 of row max x column max per product term; N_B <=
-                          512, default 512)                                     */
+                          17 residues, one FP64 rounding per product (update
+                          products: error at most 2^-57 of row max x column max
+                          per term.  Solve products: 2^-59 of the scales below;
+                          a T = T_0 D whose columns differ by many powers of two
+                          can lose the small rows of a diagonal block's inverse,
+                          D^-1 T_0^-1, since its scales come from its columns;
+                          D T_0 does not.  N_B <= 512, default 512).  HSMA_C64
+                          above m = 64 always uses these products.              */
   int32_t tile;        /* BLOCKED FP64 products: HSMA_TILE_*; 0 = table         */
   int32_t split_k;     /* BLOCKED: HSMA_SPLITK_*; 0 = table                     */
   int32_t looking;     /* BLOCKED: HSMA_LOOK_*; 0 = table                       */
@@ -532,10 +537,12 @@ HSMA_API hsma_status_t hsma_gemm_bf16_update(int64_t M, int64_t N, int64_t K, co
  * direct use and testing): C -= A X with A (M x K), X (K x N) and C (M x N)
  * column-major FP64 (device pointers, leading dimensions lda, ldx, ldc).  Each
  * row of A and column of X is scaled by a power of two and rounded to 59-bit
- * fixed point; the integer product is formed exactly through its residues modulo
+ * fixed point (after a scale per k has been moved from A's column k to X's row k);
+ * the integer product is formed exactly through its residues modulo
  * 17 coprime moduli (BF16 products with exact FP32 sums) and subtracted from C
- * in FP64.  Error per entry: below 2^-59 x (max |A row|) x (max |X column|) x K,
- * plus two FP64 roundings per 8192 of K.  Errors: INVALID_ARG for negative sizes,
+ * in FP64.  Error per entry: at most 2^-57 x (max |A row|) x (max |X column|) x K,
+ * plus two FP64 roundings per 8192 of K.  A row of A or column of X with an
+ * infinity or NaN gives NaN.  Errors: INVALID_ARG for negative sizes,
  * short leading dimensions or null pointers; UNSUPPORTED for K > 16384 or
  * M, N beyond INT32_MAX.  Workspace comes from the library's stream-ordered
  * pool.

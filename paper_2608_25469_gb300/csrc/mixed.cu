@@ -605,19 +605,20 @@ __global__ void check_kernel(double *sums, int *state, double alpha_abs, double 
 // FP64 products emulated on the BF16 tensor cores (residue arithmetic in
 // oz_tables.cuh).
 //
-// Row i of the left operand is scaled by 2^-e_i and column j of the right
-// operand by 2^-f_j (powers of two with |entry| < 2^e), so every scaled entry
-// lies in (-1, 1).  It is rounded to the fixed-point integer I = a 2^(59 - e)
-// (bits below 2^-59 of the row or column scale are dropped) and stored as its
-// residues modulo kOzP moduli, exact in BF16.  One tensor-core product per
-// modulus gives the residues of the exact integer product, which is converted
-// to FP64 with one rounding and added to the result.  The fixed-point rounding
-// contributes at most 2^-59 of |row scale| |column scale| per product term.
+// Entry (i, k) of the left operand is scaled by 2^-(e_i + g_k) and entry (k, j) of
+// the right operand by 2^(g_k - f_j) (powers of two above every entry), so every
+// scaled entry lies in (-1, 1).  It is rounded to the fixed-point integer I = a 2^59
+// (bits below 2^-59 of the scale are dropped) and stored as its residues modulo kOzP
+// moduli, exact in BF16.  One tensor-core product per modulus gives the residues of
+// the exact integer product, which is converted to FP64 with one rounding and added
+// to the result.  The fixed-point rounding contributes at most 2^-59 2^(e_i + f_j)
+// per product term; for a full left operand (g_k <= 0) that is at most 2^-57 of the
+// largest entries of row i and of column j.
 // Infinities and NaNs take no part in the scales or the residues: they mark their
 // row (left operand) or the rest of their column (right operand), where the result
 // is NaN (oz_tables.cuh).
 // ---------------------------------------------------------------------------
-constexpr int kOzExpEmpty = -1100;  // exponent of an all-zero row
+constexpr int kOzExpEmpty = -(1 << 20);  // of an all-zero row or column: below every exponent and g_k (>= -2100)
 
 // e with |x| < 2^e, from the bits of |x| (x != 0)
 __device__ __forceinline__ int oz_exponent(uint64_t absbits) {
@@ -687,42 +688,26 @@ __device__ __forceinline__ void oz_entry(const double *__restrict__ A, int64_t l
   if (CPLX) im = A[W * (r + (int64_t)k * lda) + 1];
 }
 
-// K-balancing exponents: g_k with max_r |A_rk| < 2^g_k over the block (complex:
-// one g per complex column, stored for both real columns 2k and 2k+1).  The
-// left operand is sliced as A_rk 2^-g_k and the right one as X_kj 2^g_k, which
-// leaves the product unchanged and makes the row and column scales of badly
-// scaled operands (D_r L D_c) meaningful.  A column without nonzeros keeps
-// kOzExpEmpty and the right operand's row k is then ignored.  A CTA covers 8
-// columns x 256 rows (a warp per column, lanes down the rows, eight loads in
-// flight) and folds its maxima in with atomicMax over the kOzExpEmpty fill.
 __global__ void oz_fill_kernel(int *p, int n, int v) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) p[k] = v;
 }
 
-template <bool CPLX>
-__global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
-                                                      int mode, int *kexp) {
-  const int lane = threadIdx.x & 31, k = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int r0 = blockIdx.y * 256;
-  if (k >= K || (mode != 0 && r0 + 255 < k)) return;
-  uint64_t mx = 0;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    double re, im;
-    oz_entry<CPLX>(A, lda, rows, K, mode, r0 + lane + 32 * q, k, re, im);
-    const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
-    if (ab < kOzInfBits) mx = max(mx, ab);
-  }
-  const int e = __reduce_max_sync(0xffffffffu, mx != 0 ? oz_exponent(mx) : kOzExpEmpty);
-  if (lane == 0 && e != kOzExpEmpty) {
-    atomicMax(&kexp[(CPLX ? 2 : 1) * k], e);
-    if (CPLX) atomicMax(&kexp[2 * k + 1], e);
-  }
-}
+// Scales of a left operand: row exponents e_i and K-balancing exponents g_k with
+// |A_ik| < 2^(e_i + g_k) (complex: the same for both real rows and columns of an
+// entry).  The left operand is sliced as A_ik 2^-g_k and the right one as X_kj 2^g_k,
+// which leaves the product unchanged and takes the scales of badly scaled operands
+// (D_r L D_c) out.  One of the two is the plain maximum, the other the maximum relative
+// to it; the first then needs no second look, since every maximum is attained.
+//  * Full blocks: the rows first.  No row's large entries coarsen another row's, and
+//    as g_k <= 0 the columns of X keep exponents at or below their own.
+//  * Triangles: the columns first.  The inverse of a block of D_r L is graded along its
+//    columns, and its rows have different ones of them, so rows first would scale
+//    each row by a column that the rows above do not have.
+// A row or column without nonzeros keeps kOzExpEmpty; the right operand's row k is then
+// ignored.  Both kernels fold their maxima in with atomicMax over that fill.
 
-// Row exponents of a left operand balanced by 2^-g_k (atomicMax over the
-// kOzExpEmpty fill): a CTA covers 32 rows x kOzRexpCols columns, lanes across
-// the rows.
+// e_i, relative to g_k unless kexp is null: a CTA covers 32 rows x kOzRexpCols
+// columns, lanes across the rows.  kOzExpBad with an infinity or NaN.
 constexpr int kOzRexpCols = 64;
 
 template <bool CPLX>
@@ -743,7 +728,7 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
     if (ab >= kOzInfBits)
       ex = kOzExpBad;
     else if (ab != 0)
-      ex = max(ex, oz_exponent(ab) - kexp[W * k]);
+      ex = max(ex, oz_exponent(ab) - (kexp != nullptr ? kexp[W * k] : 0));
   }
   red[ty][tx] = ex;
   __syncthreads();
@@ -753,6 +738,32 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
       atomicMax(&rexp[W * i], ex);
       if (CPLX) atomicMax(&rexp[W * i + 1], ex);
     }
+  }
+}
+
+// g_k, relative to e_i unless rexp is null, over the finite entries: a CTA covers 8
+// columns x 256 rows (a warp per column, lanes down the rows, eight loads in flight).
+template <bool CPLX>
+__global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__ A, int64_t lda, int rows, int K,
+                                                      int mode, const int *__restrict__ rexp, int *kexp) {
+  constexpr int W = CPLX ? 2 : 1;
+  const int lane = threadIdx.x & 31, k = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int r0 = blockIdx.y * 256;
+  if (k >= K || (mode != 0 && r0 + 255 < k)) return;
+  int e = kOzExpEmpty;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int r = r0 + lane + 32 * q;
+    double re, im;
+    oz_entry<CPLX>(A, lda, rows, K, mode, r, k, re, im);
+    const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
+    const int er = rexp != nullptr && r < rows ? rexp[W * r] : 0;
+    if (ab != 0 && ab < kOzInfBits && er != kOzExpBad) e = max(e, oz_exponent(ab) - er);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0 && e != kOzExpEmpty) {
+    atomicMax(&kexp[W * k], e);
+    if (CPLX) atomicMax(&kexp[2 * k + 1], e);
   }
 }
 
@@ -910,15 +921,21 @@ hsma_status_t oz_slice_a(bool cplx, const double *A, int64_t lda, int rows, int 
   oz_fill_kernel<<<(nfill + 255) / 256, 256, 0, st>>>(o.exps, nfill, kOzExpEmpty);
   uint32_t *out = reinterpret_cast<uint32_t *>(o.slices);
   const size_t ps = (size_t)o.rows * o.Kp / 2;
-  if (cplx) {
-    oz_kexp_kernel<true><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp);
-    oz_rexp_kernel<true><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp, o.exps);
-    oz_slice_a_kernel<true><<<sg, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, out, ps);
-  } else {
-    oz_kexp_kernel<false><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp);
-    oz_rexp_kernel<false><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp, o.exps);
-    oz_slice_a_kernel<false><<<sg, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, out, ps);
-  }
+  auto launch = [&](auto c) {
+    constexpr bool C = decltype(c)::value;
+    if (mode == 0) {
+      oz_rexp_kernel<C><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, nullptr, o.exps);
+      oz_kexp_kernel<C><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, o.exps, o.kexp);
+    } else {
+      oz_kexp_kernel<C><<<kg, 256, 0, st>>>(A, lda, rows, K, mode, nullptr, o.kexp);
+      oz_rexp_kernel<C><<<rg, 256, 0, st>>>(A, lda, rows, K, mode, o.kexp, o.exps);
+    }
+    oz_slice_a_kernel<C><<<sg, 256, 0, st>>>(A, lda, rows, K, o.Kp, mode, o.kexp, o.exps, out, ps);
+  };
+  if (cplx)
+    launch(std::true_type{});
+  else
+    launch(std::false_type{});
   HSMA_CUDA_TRY(cudaGetLastError());
   return HSMA_OK;
 }

@@ -152,6 +152,41 @@ def test_emulated_blocked_unit_diagonal(H, code):
     assert oracle.forward_error(X, ref) <= TOL
 
 
+@pytest.mark.parametrize("grading", ["rows", "one_entry", "one_row", "one_column", "row_and_column", "extreme"])
+def test_emulated_gemm_scales_per_row(H, grading):
+    """Rows and columns of very different sizes: every entry within the documented bound, 2^-57 of its
+    own row's and column's largest entries per term, plus the rounding of the sum (added to zero)."""
+    from fractions import Fraction
+    M, N, K = 300, 40, 200
+    rng = np.random.default_rng(4)
+    A, X = rng.uniform(-1, 1, (M, K)), rng.uniform(-1, 1, (K, N))
+    if grading == "rows":
+        A *= np.exp2(-np.arange(M))[:, None] * np.tri(M, K)
+    elif grading == "one_entry":
+        A[0, 1] = 2.0 ** 100
+    elif grading == "one_row":
+        A[7] *= 2.0 ** 60
+    elif grading == "one_column":
+        A[:, 3] *= 2.0 ** 60
+    elif grading == "row_and_column":
+        c = np.exp2(rng.integers(-100, 101, K).astype(float))
+        A, X = A * np.exp2(rng.integers(-100, 101, M).astype(float))[:, None] * c, X / c[:, None]
+    else:  # ratios beyond the exponents of single numbers: 2^-1030 beside 2^1000 in A
+        A[:, ::2] *= 2.0 ** 1000
+        A[:, 1::2] *= 2.0 ** -1030
+        X[::2] *= 2.0 ** -1020
+        X[1::2] *= 2.0 ** 1010
+    A, X = np.asfortranarray(A), np.asfortranarray(X)
+    got = _gemm(H, A, X, np.zeros((M, N), order="F"))
+    for i, j in zip(rng.integers(0, M, 100), rng.integers(0, N, 100)):
+        a, x = [Fraction(v) for v in A[i]], [Fraction(v) for v in X[:, j]]
+        exact = -sum(p * q for p, q in zip(a, x))
+        off = abs(Fraction(got[i, j]) - exact)
+        assert off <= K * max(map(abs, a)) * max(map(abs, x)) / 2 ** 57 + abs(exact) / 2 ** 52, (i, j)
+        if grading != "one_entry":  # rows and columns of one size each once the scale per k is taken out
+            assert off <= sum(abs(p * q) for p, q in zip(a, x)) / 2 ** 50, (i, j)
+
+
 @pytest.mark.parametrize("M,N,K", [(300, 270, 100), (257, 40, 8200)])
 def test_emulated_gemm_non_finite_entries(H, M, N, K):
     """An infinity or NaN makes its row of A and its column of X NaN in the result and nothing else."""

@@ -39,7 +39,12 @@
  *    and released on the same stream; released workspace stays reserved in
  *    the pool, up to 4 GiB per device, for later calls.  HSMA_ERR_NO_MEMORY
  *    if the allocation fails.  Nothing is allocated on the small path of
- *    hsma_trsm_llnn.
+ *    hsma_trsm_llnn.  Emulated FP64 products hold 34 bytes per entry of the
+ *    operands being multiplied (a panel of A of panel_cols real columns, X's
+ *    rows in it; HSMA_R64_IR: the whole of A, X in parts of at most 640 MiB) and
+ *    up to 170 MB of residues of results.  Where that does not fit, the panel
+ *    is narrowed, HSMA_R64_IR forms its residual as with ir_residual = 1, and
+ *    hsma_gemm_f64_emulated works in parts of K (one more rounding each).
  *  - CUDA errors surfacing at enqueue time return HSMA_ERR_CUDA.
  *  - Thread safety: calls on different streams may run concurrently; the
  *    tuning table is read-only after hsma_tuning_load.

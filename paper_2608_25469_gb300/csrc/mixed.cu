@@ -1092,16 +1092,20 @@ EmuLayout emu_layout(bool cplx, int nb, int panel_cols, int64_t m, int64_t n) {
 hsma_status_t blocked_emulated(bool cplx_, int nb, int panel_cols, const double *A, int64_t lda, double *B,
                                int64_t ldb, int64_t m,
                                int64_t n, const double *alpha, int unit, cudaStream_t st) {
-  const EmuLayout E = emu_layout(cplx_, nb, panel_cols, m, n);
+  EmuLayout E = emu_layout(cplx_, nb, panel_cols, m, n);
   const int W = E.W;
-  const int64_t P = E.P;
-  const int Kpb = E.Kpb;
   if ((int64_t)W * m > INT32_MAX || n > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
-  const size_t eb = sizeof(double) * W;
-  const size_t dinv_b = E.dinv_b, w_b = E.w_b, pa_b = E.pa_b;
   void *ws = nullptr;
   hsma_status_t s = hsma_ws_alloc(&ws, E.total(), st);
+  while (s == HSMA_ERR_NO_MEMORY && E.h > 1) {  // a panel of fewer blocks
+    E = emu_layout(cplx_, nb, E.h / 2 * W * nb, m, n);
+    s = hsma_ws_alloc(&ws, E.total(), st);
+  }
   if (s != HSMA_OK) return s;
+  const int64_t P = E.P;
+  const int Kpb = E.Kpb;
+  const size_t eb = sizeof(double) * W;
+  const size_t dinv_b = E.dinv_b, w_b = E.w_b, pa_b = E.pa_b;
   unsigned char *base = static_cast<unsigned char *>(ws);
   double *Dinv = reinterpret_cast<double *>(base);
   double *Wb = reinterpret_cast<double *>(base + dinv_b);
@@ -1193,7 +1197,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   if (m > INT32_MAX || n > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
   // residual products: emulated FP64 on the BF16 tensor cores unless asked
   // otherwise or m is beyond what the residues of L are kept for
-  const bool emulated = res_mode == 0 && m <= kOzResidualMaxM;
+  bool emulated = res_mode == 0 && m <= kOzResidualMaxM;
   auto al = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
   const size_t a32_b = sizeof(float) * (size_t)m * m;
   const size_t r32_b = sizeof(float) * (size_t)m * n;
@@ -1201,9 +1205,6 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   const size_t r64_b = b0_b;
   const size_t st_b = 1024;
   const int ozkp = oz_kp(m);
-  const size_t ozl_b = emulated ? al(oz_operand_bytes(m, ozkp)) : 0;
-  const size_t ozx_b = emulated ? al(oz_operand_bytes(oz_residual_cols(n, ozkp), ozkp)) : 0;
-  const size_t ozs_b = emulated ? al(oz_scratch_bytes(m, n)) : 0;
   // the FP32 inverses and BF16 panels of L, shared by the first solve and every correction
   R32Plan P;
   P.nb = nb < 32 ? 32 : nb;
@@ -1214,10 +1215,18 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
   P.unit = unit;
   const size_t dinv_b = al(sizeof(float) * (size_t)((m + P.nb - 1) / P.nb) * P.nb * P.nb);
   const size_t pan_b = al(sizeof(__nv_bfloat16) * r32_panels_elems(P.nb, terms, m));
+  size_t ozl_b, ozx_b, ozs_b;
   void *ws = nullptr;
-  hsma_status_t s = hsma_ws_alloc(
-      &ws, al(a32_b) + al(r32_b) + al(b0_b) + al(r64_b) + st_b + ozl_b + ozx_b + ozs_b + dinv_b + pan_b,
-      st);
+  hsma_status_t s;
+  for (;;) {
+    ozl_b = emulated ? al(oz_operand_bytes(m, ozkp)) : 0;
+    ozx_b = emulated ? al(oz_operand_bytes(oz_residual_cols(n, ozkp), ozkp)) : 0;
+    ozs_b = emulated ? al(oz_scratch_bytes(m, n)) : 0;
+    s = hsma_ws_alloc(&ws, al(a32_b) + al(r32_b) + al(b0_b) + al(r64_b) + st_b + ozl_b + ozx_b + ozs_b + dinv_b + pan_b,
+                      st);
+    if (s != HSMA_ERR_NO_MEMORY || !emulated) break;
+    emulated = false;  // no room for the residues (34 m^2 bytes and more): FP64 tensor products
+  }
   if (s != HSMA_OK) return s;
   unsigned char *base = static_cast<unsigned char *>(ws);
   float *A32 = reinterpret_cast<float *>(base);
@@ -1351,16 +1360,27 @@ extern "C" HSMA_API hsma_status_t hsma_gemm_f64_emulated(int64_t M, int64_t N, i
   if (A == nullptr || X == nullptr || C == nullptr) return HSMA_ERR_INVALID_ARG;
   if (K > kEmuGemmMaxK || M > INT32_MAX || N > INT32_MAX) return HSMA_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int Kp = oz_kp(K);
-  const size_t a_b = oz_operand_bytes(M, Kp), x_b = oz_operand_bytes(N, Kp);
+  // residues of the whole K range, or without room for them of equal parts of it
+  int64_t part = oz_kp(K);
+  size_t a_b, x_b;
   void *ws = nullptr;
-  hsma_status_t s = hsma_ws_alloc(&ws, a_b + x_b + oz_scratch_bytes(M, N), st);
+  hsma_status_t s;
+  for (;;) {
+    a_b = oz_operand_bytes(M, (int)part);
+    x_b = oz_operand_bytes(N, (int)part);
+    s = hsma_ws_alloc(&ws, a_b + x_b + oz_scratch_bytes(M, N), st);
+    if (s != HSMA_ERR_NO_MEMORY || part == TC_BK) break;
+    part = oz_kp(part / 2);
+  }
   if (s != HSMA_OK) return s;
   uint32_t *scratch = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(ws) + a_b + x_b);
-  OzOperand Ao = oz_operand(ws, M, Kp), Xo = oz_operand(static_cast<unsigned char *>(ws) + a_b, N, Kp);
-  s = oz_slice_a(false, A, lda, (int)M, (int)K, 0, Ao, st);
-  if (s == HSMA_OK) s = oz_slice_x(false, X, ldx, (int)K, Ao.kexp, Xo, nullptr, st);
-  if (s == HSMA_OK) s = oz_product(Ao, Xo, C, ldc, 1, 0, 0, scratch, nullptr, "emulated_gemm", st);
+  for (int64_t k0 = 0; k0 < K && s == HSMA_OK; k0 += part) {
+    const int k = (int)std::min(part, K - k0), Kp = oz_kp(k);
+    OzOperand Ao = oz_operand(ws, M, Kp), Xo = oz_operand(static_cast<unsigned char *>(ws) + a_b, N, Kp);
+    s = oz_slice_a(false, A + k0 * lda, lda, (int)M, k, 0, Ao, st);
+    if (s == HSMA_OK) s = oz_slice_x(false, X + k0, ldx, k, Ao.kexp, Xo, nullptr, st);
+    if (s == HSMA_OK) s = oz_product(Ao, Xo, C, ldc, 1, 0, 0, scratch, nullptr, "emulated_gemm", st);
+  }
   hsma_status_t f = hsma_ws_free(ws, st);
   return s != HSMA_OK ? s : f;
 }

@@ -44,8 +44,9 @@ cudaMemPool_t library_pool(int dev) {
   return pools[dev];
 }
 
-long fault_after() {
-  const char *e = std::getenv("HSMA_FAULT_ALLOC_AFTER");
+// a fault-injection setting, -1 when it is not set
+long fault_setting(const char *name) {
+  const char *e = std::getenv(name);
   if (e == nullptr || *e == '\0') return -1;
   return std::atol(e);
 }
@@ -53,9 +54,10 @@ long fault_after() {
 
 hsma_status_t hsma_ws_alloc(void **p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
-  const long lim = fault_after();
+  const long lim = fault_setting("HSMA_FAULT_ALLOC_AFTER"), most = fault_setting("HSMA_FAULT_ALLOC_ABOVE");
   const long k = g_allocs.fetch_add(1);
   if (lim >= 0 && k >= lim) return HSMA_ERR_NO_MEMORY;
+  if (most >= 0 && bytes > (size_t)most) return HSMA_ERR_NO_MEMORY;
   if (bytes == 0) return HSMA_OK;
   // under stream capture the allocation becomes a graph memory node from the
   // default pool, as before; otherwise it comes from the library's pool

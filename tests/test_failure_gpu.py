@@ -154,3 +154,56 @@ def test_host_batch_alloc_failure(H, monkeypatch):
     for b in range(len(As)):
         got = hX[offB[b]:offB[b] + ms[b] * ns[b]].reshape((ms[b], ns[b]), order="F")
         assert oracle.forward_error(got, oracle.solve(As[b], Bs[b], 1.0)) <= 1e-13, b
+
+
+@pytest.mark.parametrize("code", [I.R64, I.C128])
+def test_emulated_solve_narrows_its_panel_without_memory(H, code, monkeypatch):
+    """A panel of 2048 real columns needs 158 MB (complex 314) at m = 2048; one block of 128 columns
+    fits in 64 MB (96), and nothing fits in 1 MB."""
+    import torch
+    m, n = 2048, 32
+    A, B = I.gen_A(8, m, code), I.gen_B(8, m, n, code)
+    dA = H.to_device(A)
+    opts = H.Opts()
+    opts.fp64_products, opts.nb, opts.panel_cols = 1, 128, 2048
+    ref = oracle.solve(A, B, 1.0)
+    for limit, status in (((64 if code == I.R64 else 96) << 20, H.OK), (1 << 20, H.ERR_NO_MEMORY)):
+        dB = H.to_device(B)
+        monkeypatch.setenv("HSMA_FAULT_ALLOC_ABOVE", str(limit))
+        got = H.hsma_trsm_llnn_ex(code, 0, m, n, 1.0, dA.data_ptr(), m, dB.data_ptr(), m, H.stream_ptr(), opts=opts,
+                                  check=False)
+        monkeypatch.delenv("HSMA_FAULT_ALLOC_ABOVE")
+        torch.cuda.synchronize()
+        assert got == status
+        X = H.from_device(dB)
+        assert oracle.forward_error(X, ref) <= 1e-12 if status == H.OK else np.array_equal(X, B)
+
+
+def test_refinement_without_room_for_residues(H, monkeypatch):
+    """m = 1024: residues of A take 36 MB; the rest of the call fits in 32 MB."""
+    import torch
+    m, n = 1024, 16
+    A, B = I.gen_A(6, m, I.R64), I.gen_B(6, m, n, I.R64)
+    dA, dB = H.to_device(A), H.to_device(B)
+    monkeypatch.setenv("HSMA_FAULT_ALLOC_ABOVE", str(32 << 20))
+    info = H.Info()
+    H.hsma_trsm_llnn_ex(H.R64_IR, 0, m, n, 1.0, dA.data_ptr(), m, dB.data_ptr(), m, H.stream_ptr(), info=info)
+    monkeypatch.delenv("HSMA_FAULT_ALLOC_ABOVE")
+    torch.cuda.synchronize()
+    assert info.converged == 1
+    assert oracle.forward_error(H.from_device(dB), oracle.solve(A, B, 1.0)) <= 1e-12
+
+
+def test_emulated_gemm_in_parts_of_k_without_memory(H, monkeypatch):
+    """Integers, so that the result is exact whatever the parts: K = 3000 in parts that fit in 32 MB."""
+    import torch
+    M, N, K = 600, 70, 3000
+    rng = np.random.default_rng(2)
+    A = np.asfortranarray(rng.integers(-1024, 1025, (M, K)).astype(np.float64))
+    X = np.asfortranarray(rng.integers(-1024, 1025, (K, N)).astype(np.float64))
+    dA, dX, dC = H.to_device(A), H.to_device(X), H.to_device(np.zeros((M, N), order="F"))
+    monkeypatch.setenv("HSMA_FAULT_ALLOC_ABOVE", str(32 << 20))
+    H.hsma_gemm_f64_emulated(M, N, K, dA.data_ptr(), M, dX.data_ptr(), K, dC.data_ptr(), M, H.stream_ptr())
+    monkeypatch.delenv("HSMA_FAULT_ALLOC_ABOVE")
+    torch.cuda.synchronize()
+    assert np.array_equal(H.from_device(dC), -(A.astype(np.int64) @ X.astype(np.int64)).astype(np.float64))

@@ -495,7 +495,8 @@ hsma_status_t gemm_small_tiles(const GemmArgs<T> &p, const char *phase, cudaStre
 }
 
 // Launch one product.  Tile shape: `tile` (HSMA_TILE_*), or small tiles when 0
-// (masked operands: 128 x 8 for n <= 8, 128 x 16 for n <= 48, else 64 x 64).
+// (masked operands and launches with a skip flag, which the small tiles do not
+// know: 128 x 8 for n <= 8, 128 x 16 for n <= 48, else 64 x 64).
 // With HSMA_TILE_* K is split across CTAs when the output alone has too few tiles
 // and a partial-product workspace P is given (P = nullptr: never).  `phase`
 // names it for the tracer.
@@ -503,7 +504,7 @@ template <class T>
 hsma_status_t gemm(const GemmArgs<T> &p, const char *phase, cudaStream_t st, T *P = nullptr, size_t P_elems = 0,
                    int tile = 0) {
   if (p.M <= 0 || p.N <= 0) return HSMA_OK;
-  if (tile == 0 && !p.mask) return gemm_small_tiles<T>(p, phase, st);
+  if (tile == 0 && !p.mask && p.skip == nullptr) return gemm_small_tiles<T>(p, phase, st);
   if (tile == 0) tile = p.N <= 8 ? HSMA_TILE_128x8 : p.N <= 48 ? HSMA_TILE_128x16 : HSMA_TILE_64x64;
   if (tile == HSMA_TILE_128x8) return gemm_tiled<T, TileN8>(p, phase, st, P, P_elems);
   if (tile == HSMA_TILE_128x16) return gemm_tiled<T, TileN16>(p, phase, st, P, P_elems);

@@ -95,14 +95,6 @@ __device__ __forceinline__ void ldv(cplxf (&v)[4], const cplxf *p) {
   v[3] = cplxf{b.z, b.w};
 }
 
-template <class T>
-__device__ __forceinline__ void copy_async(T *dst, const T *src) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(T) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Start copying the lower-triangular form: a warp per stored column (row with

@@ -182,18 +182,6 @@ __device__ __forceinline__ cplx add(cplx a, cplx b) { return cplx{a.re + b.re, a
 __device__ __forceinline__ bool is_one(double a) { return a == 1.0; }
 __device__ __forceinline__ bool is_one(cplx a) { return a.re == 1.0 && a.im == 0.0; }
 
-// out = beta*C - v (UPDATE) or beta*v (SCALE)
-template <class T>
-__device__ __forceinline__ void finish_elem(int mode, T beta, bool b1, T *cp, T v) {
-  using E = Elem<T>;
-  if (mode == MODE_UPDATE) {
-    const T old = *cp;
-    *cp = sub(b1 ? old : E::mul(beta, old), v);
-  } else {
-    *cp = b1 ? v : E::mul(beta, v);
-  }
-}
-
 template <class T, class TL>
 __device__ __forceinline__ void epilogue(const GemmArgs<T> &p, const Acc<T, TL> &acc, int m0, int n0, int wm, int wn,
                                          int g, int t) {

@@ -162,6 +162,21 @@ struct Elem<cplxf> {
   __device__ __forceinline__ static bool is_zero(cplxf a) { return a.re == 0.0f && a.im == 0.0f; }
 };
 
+// Copy one element from global to shared memory asynchronously.
+template <class T>
+__device__ __forceinline__ void copy_async(T *dst, const T *src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(T) == 16) {  // complex128 is 8-byte aligned only
+    const double *q = reinterpret_cast<const double *>(src);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(q) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8), "l"(q + 1) : "memory");
+  } else if constexpr (sizeof(T) == 8) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+  } else {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+  }
+}
+
 // alpha (host double, or double[2] for complex) in the element type
 template <class T>
 inline T hsma_alpha_as(const double *a);

@@ -326,20 +326,6 @@ __global__ void __launch_bounds__(32 * kWarpsSingle) small_single_kernel(const T
 constexpr int kColLd = 64;
 
 template <class T>
-__device__ __forceinline__ void small_copy_async(T *dst, const T *src) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(T) == 16) {  // complex128 is 8-byte aligned only
-    const double *q = reinterpret_cast<const double *>(src);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(q) : "memory");
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8), "l"(q + 1) : "memory");
-  } else if constexpr (sizeof(T) == 8) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-  } else {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-  }
-}
-
-template <class T>
 struct Real {
   using type = T;
   __device__ __forceinline__ static T part(T v, int) { return v; }
@@ -468,7 +454,7 @@ __global__ void __launch_bounds__(32 * kWarpsSingle) small_column_kernel(const T
       c = m - 1 - t;
     }
     const int p = rev ? m - 1 - r : r, q = rev ? m - 1 - c : c;
-    small_copy_async(sL + c * kColLd + r, MAP && tr ? A + q + (int64_t)p * lda : A + p + (int64_t)q * lda);
+    copy_async(sL + c * kColLd + r, MAP && tr ? A + q + (int64_t)p * lda : A + p + (int64_t)q * lda);
   });
   if (tid < m) {
     if constexpr (E::kComplex) {

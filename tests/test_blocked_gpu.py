@@ -140,9 +140,35 @@ def test_inverse_accuracy_on_lu_factors(H, code, factor, m, nb):
     assert np.exp(np.mean(np.log(ratios))) <= 1.25, ratios
 
 
+SMALL_TILE_CASES = [(66, 1, 64, 1), (129, 8, 64, 1), (300, 9, 128, 2), (520, 31, 256, 1), (1000, 33, 128, 2),
+                    (1031, 200, 512, 1), (1500, 257, 128, 2), (1031, 517, 128, 1), (2051, 515, 128, 1)]
+
+
+def _small_tiles(code, m, n, nb, look, sms):
+    """The tile (in units of 8 x 8) and warps per CTA of every product of one blocked solve."""
+    cdiv = lambda a, b: -(-a // b)
+    products = []
+    for r0 in range(0, m, nb):
+        sr = min(nb, m - r0)
+        products.append((sr, sr))
+        if look == 2 and r0 > 0:
+            products.append((sr, r0))
+        elif look == 1 and r0 + sr < m:
+            products.append((m - r0 - sr, sr))
+    shapes = set()
+    for M, K in products:
+        tiles = lambda w: cdiv(cdiv(M, 8), w) * cdiv(cdiv(n, 8), w)
+        if code == I.R64 and cdiv(n, 8) >= 4 and tiles(4) >= 4 * sms:
+            shapes.add((4, 4))
+        elif cdiv(n, 8) >= 2 and tiles(2) >= 4 * sms:
+            shapes.add((2, 4))
+        else:
+            shapes.add((1, 4 if tiles(1) >= 2 * sms or K <= 64 else 16))
+    return shapes
+
+
 @pytest.mark.parametrize("code", [I.R64, I.C128])
-@pytest.mark.parametrize("m,n,nb,look", [(66, 1, 64, 1), (129, 8, 64, 1), (300, 9, 128, 2), (520, 31, 256, 1),
-                                         (1000, 33, 128, 2), (1031, 200, 512, 1), (1500, 257, 128, 2)])
+@pytest.mark.parametrize("m,n,nb,look", SMALL_TILE_CASES)
 def test_small_tile_products_parity(H, code, m, n, nb, look):
     """Every small-tile shape (by the number of tiles) at ragged sizes, odd leading dimensions,
     alpha, both update directions, NaN in what is never read."""
@@ -155,6 +181,15 @@ def test_small_tile_products_parity(H, code, m, n, nb, look):
     X = _run(H, code, A, B, alpha, nb, looking=look)
     assert np.all(np.isnan(X[m:]))
     assert oracle.forward_error(X[:m], oracle.solve(A0, B0, alpha)) <= TOL
+
+
+@pytest.mark.parametrize("code", [I.R64, I.C128])
+def test_small_tile_cases_cover_every_shape(H, code):
+    """The cases above select every compiled shape on this device."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    got = set().union(*(_small_tiles(code, *c, sms) for c in SMALL_TILE_CASES))
+    assert got == {(2, 4), (1, 4), (1, 16)} | ({(4, 4)} if code == I.R64 else set())
 
 
 CFG_CASES = [(65, 7, 32), (300, 200, 128), (700, 50, 512), (1000, 9, 64), (513, 130, 256)]

@@ -96,6 +96,25 @@ def test_emulated_gemm_residue_edges(H, M, N, K):
         assert abs(int(got[i, j]) - exact) * 2 ** 60 <= (1 if K <= 8192 else 3) * 129 * abs(exact), (i, j)
 
 
+@pytest.mark.parametrize("width,over,K", [(128, 0, 70), (128, 1, 70), (256, 0, 70), (256, 1, 70), (128, 1, 1030),
+                                          (256, 0, 1030)])
+def test_emulated_gemm_one_and_several_tiles_per_pair(H, width, over, K):
+    """As many tiles as pairs of CTAs (every warp drains its pair's only tile) and the fewest beyond
+    (conversion warps work beside the draining ones) of both tile widths.  The wide tile is chosen for
+    one round and again once narrow ones would take four, at half as many tiles again."""
+    import torch
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    tm = pairs + over if width == 128 else (pairs if not over else 3 * pairs // 2 + 1)
+    cost = lambda bn, n: -(-tm * -(-n // bn) // pairs) * (bn + 96)
+    M, N = 256 * tm - 3, width - 1
+    assert (cost(128, N) < cost(256, N)) == (width == 128) and (tm <= pairs) == (over == 0)
+    rng = np.random.default_rng(M)
+    A = np.asfortranarray(rng.integers(-1024, 1025, (M, K)).astype(np.float64))
+    X = np.asfortranarray(rng.integers(-1024, 1025, (K, N)).astype(np.float64))
+    got = _gemm(H, A, X, np.zeros((M, N), order="F"))
+    assert np.array_equal(got, -(A @ X))  # integers below 2^53: exact
+
+
 def test_emulated_gemm_rejects_bad_arguments(H):
     assert H.hsma_gemm_f64_emulated(4, 4, 16385, 1, 4, 1, 16385, 1, 4, 0, check=False) == H.ERR_UNSUPPORTED
     assert H.hsma_gemm_f64_emulated(4, 4, 4, 1, 3, 1, 4, 1, 4, 0, check=False) == H.ERR_INVALID_ARG

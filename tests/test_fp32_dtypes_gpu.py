@@ -190,3 +190,38 @@ def test_batched_block_edges(H, code64, code, kind):
             ref = oracle.solve_general(A32, B32, alpha, 0, uplo, trans, unit)
         assert np.all(np.isnan(X[m:])), EDGES[b]
         assert oracle.forward_error(X[:m].astype(wide), ref) <= tol * (2 if kind in ("lu", "chol") else 1), EDGES[b]
+
+
+@pytest.mark.parametrize("code64,code", [(I.R64, 4), (I.C128, 5), (I.R64, 0)], ids=["f32", "c64", "f64"])
+@pytest.mark.parametrize("uplo", [0, 1], ids=["lower", "upper"])
+@pytest.mark.parametrize("what", ["nan_b", "inf_b", "zero_diagonal"])
+def test_batched_non_finite_propagates(H, code64, code, uplo, what):
+    """An infinity or NaN of B reaches its column from its row on (in the order of the substitution), a
+    zero on the diagonal every column; nothing else changes by a bit, the other instances neither."""
+    import torch
+    sizes = [(64, 40), (13, 5), (37, 17)]
+    as_type = (lambda X: _f32(code64, X)) if code else np.asfortranarray
+    out = []
+    for planted in (False, True):
+        As, Bs = [], []
+        for b, (m, n) in enumerate(sizes):
+            A = I.gen_A(3, m, code64, inst=b)
+            As.append(as_type(np.asfortranarray(A.T) if uplo else A).copy(order="F"))
+            Bs.append(as_type(I.gen_B(3, m, n, code64, inst=b)).copy(order="F"))
+        if planted and what == "zero_diagonal":
+            As[0][21, 21] = 0
+        elif planted:
+            Bs[0][21, 33] = np.nan if what == "nan_b" else np.inf
+        bt = U.Batch(As, Bs)
+        a = bt.args()
+        H.hsma_trsm_vbatched(code, 0, uplo, 0, 0, bt.batch, a[0], a[1], 1.5, a[2], a[3], a[4], a[5], 64, 0,
+                             bt.d_status.data_ptr(), H.stream_ptr())
+        torch.cuda.synchronize()
+        assert bt.status() == 0
+        out.append(bt.results())
+    bad = np.zeros(sizes[0], bool)
+    bad[slice(None, 22) if uplo else slice(21, None), slice(None) if what == "zero_diagonal" else 33] = True
+    clean, got = out
+    assert not np.any(np.isfinite(got[0][bad]))
+    assert np.array_equal(got[0][~bad], clean[0][~bad])
+    assert all(np.array_equal(p, q) for p, q in zip(got[1:], clean[1:]))

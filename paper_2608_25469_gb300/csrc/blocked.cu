@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(32 * NW) small_tile_kernel(const GemmArgs<T> p
   constexpr int BM = 8 * WM, BN = 8 * WN;
   __shared__ T red[NW][BM * BN];
   const int m0 = (gridDim.y - 1 - blockIdx.y) * BM, n0 = blockIdx.x * BN;
-  fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, p.tri ? min(p.K, m0 + BM) : p.K, m0, n0, red);
+  fp64_tile<T, WM, WN, NW>(p.A, p.lda, p.Bm, p.ldb, p.M, p.N, p.K, p.tri, m0, n0, red);
   const bool b1 = is_one(p.beta);
   for (int e = threadIdx.x; e < BM * BN; e += 32 * NW) {
     const int row = m0 + e % BM, col = n0 + e / BM;

@@ -140,6 +140,23 @@ def test_inverse_accuracy_on_lu_factors(H, code, factor, m, nb):
     assert np.exp(np.mean(np.log(ratios))) <= 1.25, ratios
 
 
+def test_solve_products_round_once_at_the_size_of_the_result(H):
+    """m = 512 with two blocks, left-looking, on the seeded recipe, where the diagonal dominates: an
+    entry sees the rounding of 1/a_ii and of the solve product, in the second block that of the update
+    too, each at most u = 2^-53 relative and of root mean square at most u / sqrt(3).  The mean over
+    both blocks, sqrt(2.5 / 3) u, bounds the error from the exact solution; partial sums added to a
+    partial sum that holds the diagonal's term give 1.4 times that bound."""
+    m, n, nb = 512, 24, 256
+    A, B = I.gen_A(21, m, I.R64), I.gen_B(21, m, n, I.R64)
+    X = _run(H, I.R64, A, B, 1.0, nb, looking=2).astype(np.longdouble)
+    exact = B.astype(np.longdouble)
+    for k in range(m):
+        exact[k] /= A[k, k]
+        exact[k + 1:] -= np.outer(A[k + 1:, k].astype(np.longdouble), exact[k])
+    err = float(np.sqrt(((X - exact) ** 2).sum() / (exact ** 2).sum()))
+    assert err <= np.sqrt(2.5 / 3.0) * 2.0 ** -53, err
+
+
 SMALL_TILE_CASES = [(66, 1, 64, 1), (129, 8, 64, 1), (300, 9, 128, 2), (520, 31, 256, 1), (1000, 33, 128, 2),
                     (1031, 200, 512, 1), (1500, 257, 128, 2), (1031, 517, 128, 1), (2051, 515, 128, 1)]
 

@@ -227,9 +227,10 @@ HSMA_API hsma_status_t hsma_trsm(int dtype, int side, int uplo, int trans, int d
  * batch  number of instances (>= 0).
  * d_m, d_n, d_lda, d_ldb: DEVICE arrays of `batch` int32 sizes.
  * d_A, d_B: DEVICE arrays of `batch` device pointers.
- * max_m  host upper bound on every m_i, or 0 for "unknown" (taken as 64); up
- *        to 64 it sizes the workspace, and an instance with m_i > max_m is
- *        skipped and flagged HSMA_DEVERR_BAD_SIZE.  max_m > 64 admits
+ * max_m  host upper bound on every m_i, or 0 for "unknown" (taken as 64).  For
+ *        HSMA_C128 it sizes the workspace, and an instance with m_i > max_m is
+ *        skipped and flagged HSMA_DEVERR_BAD_SIZE; the other dtypes flag m_i >
+ *        64 only.  max_m > 64 admits
  *        instances of any size: the call then reads the batch's sizes and
  *        pointers back to the host (it waits for the stream once, so it is
  *        not capturable), runs the instances with m_i <= 64 as the batch and
@@ -406,14 +407,14 @@ HSMA_API hsma_status_t hsma_trsm_llnn_vbatched_host_tp(int dtype, int diag, int3
  * that array (about 256 KB) until the process exits.  Limit: batch <= 65536
  * instances; a larger batch returns HSMA_ERR_UNSUPPORTED without launching.
  * The first call on a device looks up the array's device address (one
- * cudaGetSymbolAddress per device, made with that device current) and, like
- * the first varlen batch of any kind, copies a 32 KB table of per-size
- * schedule entries into a second static array; make that first call before
- * any stream capture (a capturing first call computes the entries in the
- * kernel instead).  The call itself allocates and frees nothing.  All calls share the one array: each call resets the counters it
- * needs, but calls whose work overlaps on the GPU (on different streams, or
- * from different threads, without ordering between them) race on the array
- * and must be serialised by the caller.
+ * cudaGetSymbolAddress per device, made with that device current) and, for
+ * HSMA_C128, copies a 32 KB table of per-size schedule entries into a second
+ * static array; make that first call before any stream capture (a capturing
+ * first call computes the entries in the kernel instead).  The call itself
+ * allocates and frees nothing.  All calls of HSMA_C128 and HSMA_R64 share the
+ * one array: each call resets what it needs, but calls whose work overlaps on
+ * the GPU (on different streams, or from different threads, without ordering
+ * between them) race on the array and must be serialised by the caller.
  */
 HSMA_API hsma_status_t hsma_trsm_llnn_vbatched_noalloc(int dtype, int diag, int32_t batch, const int32_t *d_m,
                                                        const int32_t *d_n, const void *alpha,

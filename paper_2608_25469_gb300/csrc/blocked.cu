@@ -16,7 +16,7 @@
 // Both products run on the FP64 tensor path (mma.sync m8n8k4 .f64, "DMMA"),
 // complex as four real products, in small tiles with operands straight from
 // global memory (fp64_tile.cuh), which measured faster than the staged tiles at
-// every size: 512 x 64 FP64 138 -> 89 us, 777 x 129 complex 1.32 -> 0.55 ms,
+// every size (staged -> small): 512 x 64 FP64 138 -> 89 us, 777 x 129 complex 1.32 -> 0.55 ms,
 // 4096 x 512 FP64 11.1 -> 8.7 ms, 4096 x 4096 67.7 -> 66.2 ms (the FP64 pipe's
 // time).  The staged tiles (HSMA_TILE_*, on request and for masked operands)
 // bring operands into shared memory by TMA (cp.async.bulk.tensor) behind

@@ -298,7 +298,10 @@ __host__ __device__ inline int hsma_small_pick_g_batched(int m, int n, bool cplx
 // Device constants of this GPU's FP64 pipe used by the latency-aware choice
 // for a single solve: a warp-wide FP64 instruction occupies a sub-partition
 // for 64 cycles; a dependent step costs one FP64 latency plus, for G > 1, a
-// shuffle round trip.
+// shuffle round trip.  The instructions counted are those of the kernels with
+// whole rows per lane (G < 32); the G = 32 kernel issues about 60% of them for
+// complex types, and FP32 types have a shorter pipe, so the model leans towards
+// narrower layouts there.
 __host__ __device__ inline double hsma_small_time_model(int m, int n, int g, bool cplx_, int nsm) {
   const double tile = (double)hsma_small_tile_instr(m, g, cplx_);
   const int C = 32 / g;

@@ -5,8 +5,8 @@
 // FP32-result mode (HSMA_R32_BF16): phase 1 inverts the diagonal blocks in
 // FP32; phase 2 forms X_r = D_r^{-1} B_r and applies the trailing update
 // B_{r+1:} -= A_{r+1:,r} X_r on the 5th-generation tensor cores: operands in
-// BF16, products accumulated in FP32 in tensor memory (tcgen05.mma kind::f16,
-// 128 x 256 tiles, TMA loads with 128-byte swizzle).  The solve product cuts
+// BF16, products accumulated in FP32 in tensor memory (tcgen05.mma kind::f16 on
+// pairs of CTAs, tc_gemm.cuh).  The solve product cuts
 // both operands into three BF16 slices (24 significant bits, exact for FP32)
 // and sums the six slice pairs with p + q <= 2 in one accumulator (the
 // refinement's correction solves use FP32 FMAs instead).  With three

@@ -14,7 +14,7 @@ hsma_status_t hsma_mixed_ir(int nb, const hsma_opts_t *opts, const double *A, in
                             int64_t m, int64_t n, double alpha, int unit, cudaStream_t st, hsma_info_t *info);
 
 // Blocked FP64 / complex FP64 solve with the solve and trailing-update
-// products emulated in FP64 on the BF16 tensor cores (exact integer slices);
+// products emulated in FP64 on the BF16 tensor cores (exact through residues);
 // trailing updates are applied per panel of about panel_cols real columns.
 hsma_status_t hsma_blocked_emulated(int dtype, int nb, int panel_cols, const void *A, int64_t lda, void *B,
                                     int64_t ldb, int64_t m, int64_t n, const double *alpha, int unit,
@@ -36,13 +36,13 @@ constexpr int kEmulatedTableDtype(int dtype) { return dtype + 10; }
 hsma_status_t hsma_c64_blocked(int nb, int panel_cols, const void *A, int64_t lda, void *B, int64_t ldb, int64_t m,
                                int64_t n, const double *alpha, int unit, cudaStream_t st);
 
-// The planner's choice for one solve with the given options (hsma_plan with
-// opts; api.cu).
 // FP32 inverses of the nb x nb diagonal blocks of L (m x m, lda) into Dinv
 // (ceil(m / nb) blocks of nb x nb, ld nb, zeros above each diagonal and
 // outside a partial block): 64 x 64 blocks by substitution, joined by doubling
-// when nb is a power of two >= 128 (r32_inverse.cu), else substitution at nb.
+// (r32_inverse.cu).  nb: a power of two, 32 to 512.
 hsma_status_t hsma_r32_diag_inverse(int nb, const float *A, int64_t lda, int64_t m, int unit, float *Dinv,
                                     cudaStream_t st);
 
+// The planner's choice for one solve with the given options (hsma_plan with
+// opts; api.cu).
 hsma_status_t hsma_make_plan(int dtype, int64_t m, int64_t n, const hsma_opts_t *opts, hsma_plan_t *out);

@@ -9,10 +9,11 @@
 // takes 32/G consecutive columns of that stream, which may belong to several
 // instances, so every warp tile is full except the last one of each m.
 //
-//  1. schedule (one CTA): validates the instances, groups them by m, orders
-//     the groups by the cost of one warp tile (longest first), and writes
-//     per position in that order the instance and its first column in the
-//     stream (staged triangles lie position by position);
+//  1. schedule (a count pass and a place pass over the whole grid): validates
+//     the instances, groups them by m, orders the groups by the cost of one
+//     warp tile (longest first), and writes per position in that order the
+//     instance and its first column in the stream (staged triangles lie
+//     position by position);
 //  2. prep (all SMs, one warp per instance): 1/a_rr, alpha/a_rr and the
 //     strict lower triangle with row r pre-multiplied by 1/a_rr, packed by
 //     columns into a workspace (the same products the shared-memory staging

@@ -15,9 +15,12 @@
 // runs beside it.
 //
 // With HSMA_SERVER_FP64_EMULATED the blocked requests with m >= 384 use FP64
-// products emulated on the BF16 tensor cores (the fp64_products option); below
-// that the FP64 tensor products of a few block steps take no longer than the
-// emulated path's extra slicing launches.
+// products emulated on the BF16 tensor cores (the fp64_products option).  Below
+// that they do not pay up to n = 512.  Above, it depends on n (ms, FP64 / emulated
+// products; n = 4, 128, 512): m = 512 0.07 / 0.17, 0.10 / 0.19, 0.20 / 0.19; m = 1024
+// 0.12 / 0.33, 0.24 / 0.39, 0.62 / 0.39; m = 4096 0.56 / 1.46, 2.5 / 1.8, 8.5 / 1.8;
+// complex128 at 1024 0.29 / 0.57, 0.73 / 0.72, 2.3 / 0.75.  The requests with many
+// columns, where the emulated products win, are the ones that hold a server up.
 //
 // A fake-device mode (HSMA_SERVER_FAKE_DEVICE) runs the same admission and
 // queue logic with no GPU: each "launch" completes after a modelled time.

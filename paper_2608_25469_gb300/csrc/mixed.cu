@@ -622,8 +622,9 @@ constexpr int kOzExpEmpty = -(1 << 20);  // of an all-zero row or column: below 
 
 // e with |x| < 2^e, from the bits of |x| (x != 0)
 __device__ __forceinline__ int oz_exponent(uint64_t absbits) {
-  const int ea = (int)(absbits >> 52);
-  return ea != 0 ? ea - 1022 : 64 - __clzll((long long)absbits) - 1074;
+  const int ea = (int)((uint32_t)(absbits >> 32) >> 20);
+  if (ea == 0) return 64 - __clzll((long long)absbits) - 1074;  // subnormal: rare, a branch of its own
+  return ea - 1022;
 }
 
 // round(a 2^(kOzFrac - e)) for |a| < 2^e (ties away from zero)
@@ -668,7 +669,8 @@ __device__ __forceinline__ uint32_t oz_pair(float lo, float hi) {
 __device__ __forceinline__ uint64_t oz_absbits(double x) {
   return (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
-constexpr uint64_t kOzInfBits = 0x7ffull << 52;  // |x| of infinities and, above, NaNs
+// an infinity or NaN, from the bits of |x|
+__device__ __forceinline__ bool oz_non_finite(uint64_t absbits) { return (uint32_t)(absbits >> 32) >= 0x7ff00000u; }
 
 // Entry (r, k) of the rows x K block of a column-major matrix (T = double, or
 // complex double as (re, im)) under a mode: 0 = the whole block; 1 = lower
@@ -719,17 +721,18 @@ __global__ void __launch_bounds__(256) oz_rexp_kernel(const double *__restrict__
   const int i = blockIdx.x * 32 + tx, kb = blockIdx.y * kOzRexpCols;
   if (mode != 0 && kb > blockIdx.x * 32 + 31) return;  // above the diagonal
   int ex = kOzExpEmpty;
+  uint64_t mx = 0;
 #pragma unroll
   for (int q = 0; q < kOzRexpCols / 8; ++q) {
     const int k = kb + ty + 8 * q;
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, i, k, re, im);
     const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
-    if (ab >= kOzInfBits)
-      ex = kOzExpBad;
-    else if (ab != 0)
-      ex = max(ex, oz_exponent(ab) - (kexp != nullptr ? kexp[W * k] : 0));
+    mx = max(mx, ab);
+    if (kexp != nullptr && ab != 0) ex = max(ex, oz_exponent(ab) - kexp[W * k]);
   }
+  if (kexp == nullptr && mx != 0) ex = oz_exponent(mx);
+  if (oz_non_finite(mx)) ex = kOzExpBad;
   red[ty][tx] = ex;
   __syncthreads();
   if (ty == 0) {
@@ -751,15 +754,21 @@ __global__ void __launch_bounds__(256) oz_kexp_kernel(const double *__restrict__
   const int r0 = blockIdx.y * 256;
   if (k >= K || (mode != 0 && r0 + 255 < k)) return;
   int e = kOzExpEmpty;
+  uint64_t mx = 0;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int r = r0 + lane + 32 * q;
     double re, im;
     oz_entry<CPLX>(A, lda, rows, K, mode, r, k, re, im);
     const uint64_t ab = max(oz_absbits(re), oz_absbits(im));
-    const int er = rexp != nullptr && r < rows ? rexp[W * r] : 0;
-    if (ab != 0 && ab < kOzInfBits && er != kOzExpBad) e = max(e, oz_exponent(ab) - er);
+    if (rexp == nullptr) {
+      if (!oz_non_finite(ab)) mx = max(mx, ab);
+    } else if (ab != 0) {  // (r < rows)
+      const int er = rexp[W * r];
+      if (er != kOzExpBad) e = max(e, oz_exponent(ab) - er);
+    }
   }
+  if (mx != 0) e = oz_exponent(mx);
   e = __reduce_max_sync(0xffffffffu, e);
   if (lane == 0 && e != kOzExpEmpty) {
     atomicMax(&kexp[W * k], e);
@@ -838,7 +847,7 @@ __global__ void __launch_bounds__(256) oz_slice_x_kernel(const double *__restric
     for (int k = tid; k < K; k += 256) {
       const uint64_t ab = oz_absbits(x[k]);
       const int g = kexp[k];
-      if (ab >= kOzInfBits)
+      if (oz_non_finite(ab))
         bad = min(bad, k);
       else if (ab != 0 && g != kOzExpEmpty)
         ex = max(ex, oz_exponent(ab) + g);
@@ -865,7 +874,7 @@ __global__ void __launch_bounds__(256) oz_slice_x_kernel(const double *__restric
       for (int h = 0; h < 2; ++h) {
         const int g = k + h < K ? kexp[k + h] : kOzExpEmpty;
         const double v = g != kOzExpEmpty ? x[k + h] : 0.0;
-        oz_limbs(oz_absbits(v) < kOzInfBits ? oz_fixed(v, e - g) : 0, a[h]);
+        oz_limbs(oz_non_finite(oz_absbits(v)) ? 0 : oz_fixed(v, e - g), a[h]);
       }
 #pragma unroll
       for (int l = 0; l < kOzP; ++l)

@@ -32,7 +32,10 @@
  *    not read A.
  *  - A singular A (a zero on the diagonal) is not detected; IEEE infinities and
  *    NaNs propagate, as in BLAS (emulated FP64 products write NaN for both: an
- *    infinity too leaves them as NaN).
+ *    infinity too leaves them as NaN).  On the blocked path (m > 64) one in B
+ *    may also reach rows above its own in the same tile of a solve product, where
+ *    it meets the zeros of a triangular inverse: up to 7 rows with FP64 products
+ *    (HSMA_TILE_*: 127), 255 with FP32 results, none with emulated products.
  *  - Workspace (diagonal-block inverses, refinement copies, batch schedules)
  *    is taken from a stream-ordered memory pool the library keeps per device
  *    (CUDA's default pool while `stream` is capturing a graph) on `stream`

@@ -157,6 +157,28 @@ def test_solve_products_round_once_at_the_size_of_the_result(H):
     assert err <= np.sqrt(2.5 / 3.0) * 2.0 ** -53, err
 
 
+@pytest.mark.parametrize("code", [I.R64, I.C128])
+@pytest.mark.parametrize("n", [3, 600])
+@pytest.mark.parametrize("what,row", [("nan_b", 300), ("inf_b", 511), ("zero_diagonal", 389)])
+def test_blocked_non_finite_propagates(H, code, n, what, row):
+    """An infinity or NaN of B reaches its column from its row on, and at most 7 rows above (the 8 x 8
+    part of the inverse that holds its row); a zero on the diagonal every column from its row on."""
+    m, nb, col = 640, 256, 2
+    A0, B0 = I.gen_A(5, m, code), I.gen_B(5, m, n, code)
+    A, B = A0.copy(order="F"), B0.copy(order="F")
+    if what == "zero_diagonal":
+        A[row, row] = 0
+    else:
+        B[row, col] = np.nan if what == "nan_b" else np.inf
+    X = _run(H, code, A, B, 1.0, nb)
+    reach = slice(None) if what == "zero_diagonal" else col
+    assert not np.any(np.isfinite(X[row:, reach]))
+    bad = np.zeros((m, n), bool)
+    bad[row if what == "zero_diagonal" else row // 8 * 8:, reach] = True
+    ref = oracle.solve(A0, B0, 1.0)
+    assert np.linalg.norm((X - ref)[~bad]) <= TOL * np.linalg.norm(ref)
+
+
 SMALL_TILE_CASES = [(66, 1, 64, 1), (129, 8, 64, 1), (300, 9, 128, 2), (520, 31, 256, 1), (1000, 33, 128, 2),
                     (1031, 200, 512, 1), (1500, 257, 128, 2), (1031, 517, 128, 1), (2051, 515, 128, 1)]
 

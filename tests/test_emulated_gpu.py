@@ -62,7 +62,7 @@ def _two_prod(a, b):
 def test_emulated_gemm_fp64_accuracy(H, M, N, K):
     """Random FP64 data with rows and columns of X scaled over 2^-30..2^30, up to the exactness
     bound K = 2^14.  Sampled entries against the correctly rounded C0 - A X (exact products,
-    math.fsum): error within 2^-50 (|C0| + |A||X|), far below one dropped slice pair (~2^-30)."""
+    math.fsum): error within 2^-50 (|C0| + |A||X|)."""
     import math
     rng = np.random.default_rng(K)
     A = np.asfortranarray(rng.uniform(-1, 1, (M, K)) * np.exp2(rng.integers(-30, 30, (M, 1))))

@@ -108,7 +108,7 @@ def _ir(H, A, B, alpha, **kw):
 @pytest.mark.parametrize("m,n", [(1000, 300), (300, 1000), (129, 1), (2000, 64)])
 def test_ir_mode_reaches_fp64_accuracy(H, m, n, residual):
     """FP64-result mode; residual products emulated on the BF16 tensor cores (exact
-    integer slices) or FP64 tensor products."""
+    integer products through residues) or FP64 tensor products."""
     A, B = I.gen_A(9, m, I.R64), I.gen_B(9, m, n, I.R64)
     X, info = _ir(H, A, B, 1.5, ir_residual=residual)
     assert info.converged == 1 and 1 <= info.ir_iters <= 10
